@@ -208,6 +208,10 @@ def _prepare_steps(c, rng, gen):
     s["cur"], s["nxt"] = _routing(L, K), _routing(L, K)
     # the routing of this token, predicted from the token before it
     edg.prerouter_topk(desc, s["W"], _states(gen, L, H), L, *s["cur"])
+    # a decoder keeps each layer's buffers: x, the routing it executes, its head, the routing it predicts, y
+    (ci, cg), (ni, ng) = s["cur"], s["nxt"]
+    s["calls"] = [(l, s["X"][l], ci[l], cg[l], s["W"][l], ni[(l + 1) % L], ng[(l + 1) % L], None, s["Y"][l], s["ws"])
+                  for l in range(L)]
     return s
 
 
@@ -271,7 +275,7 @@ def _prepare_stack(c, rng, gen):
     X = X.to(torch.bfloat16)
     dec = StackDecoder(desc, store, _heads(c, L, gen), prefetch=True)
     dec.prime(X[NX - 1])
-    return dict(store=store, keep=keep, dec=dec, X=X, Y=_out(c, L, H), t=0)
+    return dict(store=store, keep=keep, dec=dec, X=list(X), Y=_out(c, L, H), t=0)
 
 
 def _prepare_ffn(c, rng, gen):
@@ -289,6 +293,8 @@ def _prepare_ffn(c, rng, gen):
         rank = torch.argsort(torch.rand((L, 1, c["E"]), generator=gen, device="cuda"), dim=-1).float() + 1
         gumbel = -torch.log(-torch.log(torch.rand((L, T, c["E"]), generator=gen, device="cuda").clamp(1e-9, 1 - 1e-7)))
         s["logits"] = (-1.1 * torch.log(rank) + gumbel).contiguous()
+    s["layers"] = [(s["inds"][l], s["gates"][l], s["X"][l], s["W" if c["router"] == "head" else "logits"][l], pool[l],
+                    s["loras"][l][0], s["Y"][l]) for l in range(L)]
     return s
 
 
@@ -322,11 +328,9 @@ def run(state):
 
 
 def _run_steps(s, c):
-    L, (ci, cg), (ni, ng) = c["layers"], s["cur"], s["nxt"]
-    for l in range(L):
-        n = (l + 1) % L
-        edg.moe_layer_decode(s["store"], l, s["X"][l], ci[l], cg[l], s["W"][l], ni[n], ng[n], None, s["Y"][l], s["ws"])
-    return s["Y"], ni, ng
+    for call in s["calls"]:
+        edg.moe_layer_decode(s["store"], *call)
+    return s["Y"], s["nxt"][0], s["nxt"][1]
 
 
 def _run_chain(s, c):
@@ -341,20 +345,19 @@ def _run_burst(s, c):
 
 def _run_stack(s, c):
     t = s["t"]
-    s["dec"].step(t, s["X"][t % s["X"].shape[0]], s["Y"])
+    s["dec"].step(t, s["X"][t % len(s["X"])], s["Y"])
     s["t"] = t + 1
     return s["Y"], s["dec"].inds[(t + 1) % 2], s["dec"].gates[(t + 1) % 2]
 
 
 def _run_ffn(s, c):
-    for l in range(c["layers"]):
-        inds, gates = s["inds"][l], s["gates"][l]
-        if c["router"] == "head":
-            edg.prerouter_topk_tokens(s["desc"], s["W"][l], s["X"][l], c["T"], inds, gates)
+    T, head = c["T"], c["router"] == "head"
+    for inds, gates, x, router, pool, lora, y in s["layers"]:
+        if head:
+            edg.prerouter_topk_tokens(s["desc"], router, x, T, inds, gates)
         else:
-            edg.softmax_topk_rows(s["desc"], s["logits"][l], c["T"], inds, gates)
-        edg.moe_expert_ffn_int4_lora(s["desc"], s["pool"][l], s["table"], c["T"], inds, None, gates, s["X"][l], s["loras"][l][0],
-                                     s["Y"][l], s["ws"])
+            edg.softmax_topk_rows(s["desc"], router, T, inds, gates)
+        edg.moe_expert_ffn_int4_lora(s["desc"], pool, s["table"], T, inds, None, gates, x, lora, y, s["ws"])
     return s["Y"], s["inds"], s["gates"]
 
 
