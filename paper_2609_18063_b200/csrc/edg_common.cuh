@@ -98,18 +98,33 @@ struct WorkspaceLayout {
     size_t lone_bytes;// what a batch-1 call that never chains needs: everything up to the first set of partials
     // grouped path (T > 1) only:
     size_t o;         // [T*K][H] float             : gate-weighted output of every (token, choice) pair
-    size_t o_part;    // [T*K][4][H] float          : the same per quarter of the intermediate dimension (small groups only)
-    size_t xt;        // [T*K/8 + n_slots] tile records of the streaming small-group kernel: x fragments, block sums, projections, pair table
     size_t pair_slot; // [T*K] int32                : resolved slot of every pair (-1: skipped)
     size_t pair_ad;   // [T*K] int32                : adapter of every pair
     size_t counts;    // [n_slots] int32            : pairs per slot
     size_t n_tiles;   // int32
-    size_t tiles;     // [T*K/8 + n_slots][2] int32 : (slot, first position) of every tile of 8 or 64 pairs
+    size_t tiles;     // [T*K/128 + n_slots][2] int32 : (slot, first position) of every tile of 128 pairs
     size_t lists;     // [n_slots][T] int32         : pairs of every slot, ascending
     size_t hq;        // [T*K/128 + n_slots][I/32][2][128 x 32] fp16: h of every 128-token tile as tensor-core operand tiles (value, residual)
     size_t xq;        // [T*K/128 + n_slots][H/32][128 x 32] fp16: the gathered token states of every tile as operand tiles
+    // streaming form of the grouped path (run_grouped_ffn):
+    size_t g_tiles;   // [tiles] {slot, first position, pairs, adapter}
+    size_t g_done;    // [tiles] int32              : finished row tiles of every tile's h
+    size_t g_order;   // [T*K] int32                : pairs sorted by slot
+    size_t g_cnt;     // [2][n_slots] int32         : counters of the sort, for pools beyond 8192 slots
+    size_t g_u;       // [tiles][2][cap][rank16] fp16 : sigma A_gate x, sigma A_up x
+    size_t g_xq;      // [tiles][cap * H] fp16      : token states in operand order
+    size_t g_hq;      // [tiles][2 * cap * I] fp16  : h, value and residual, in operand order
     size_t bytes;
 };
+
+// pairs a tile of the streaming form holds, and how many tiles T tokens can make
+int grouped_tile_cap(const edg_layer_desc& d, int T);
+inline size_t grouped_max_tiles(const edg_layer_desc& d, int T) {
+    const size_t P = (size_t)T * d.K, cap = (size_t)grouped_tile_cap(d, T);
+    return P / cap + 1 + (P < (size_t)d.n_slots ? P : (size_t)d.n_slots);
+}
+// Whether T tokens go through the tcgen05 tiles (umma_*) or through the streaming form.
+bool grouped_use_umma(const edg_layer_desc& d, int T);
 
 __host__ __device__ inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -127,25 +142,30 @@ inline WorkspaceLayout workspace_layout(const edg_layer_desc& d, int T) {
     const size_t one_set = (size_t)kDownSlices * (d.K + 1) * d.H * sizeof(float);   // K routed experts and the shared expert
     W.lone_bytes = W.partial + one_set;
     size_t end = round_up(W.partial + (size_t)kHandoffRing * one_set, 256);
-    W.o_part = W.xt = end;
     W.o = W.pair_slot = W.pair_ad = W.counts = W.n_tiles = W.tiles = W.lists = W.hq = W.xq = end;
+    W.g_tiles = W.g_done = W.g_order = W.g_cnt = W.g_u = W.g_xq = W.g_hq = end;
     if (T > 1) {
         const size_t P = (size_t)T * d.K;
         W.o = end;                 end = round_up(W.o + P * d.H * sizeof(float), 256);
-        const bool small = P <= 8 * (size_t)d.n_slots;
-        W.o_part = end;            end = round_up(W.o_part + (small ? P * 4 * d.H * sizeof(float) : 0), 256);
-        // a tile record: 8 tokens of fp16 state, two sums per 32 activations and token, 2 x rank projections per token, pair table
-        const size_t rr = d.rank > 0 ? (size_t)d.rank : 8;
-        const size_t tile_rec = (size_t)8 * d.H * 2 + 2 * 8 * (size_t)(d.H / 32) * 4 + 8 * 2 * rr * 4 + 128;
-        W.xt = end;                end = round_up(W.xt + (small ? (P / 8 + 1 + d.n_slots) * tile_rec : 0), 256);
         W.pair_slot = end;         end = round_up(W.pair_slot + P * 4, 256);
-        W.pair_ad = end;           end = round_up(W.pair_ad + P * 4, 256);
-        W.counts = end;            end = round_up(W.counts + (size_t)d.n_slots * 4, 256);
         W.n_tiles = end;           end += 256;
-        W.tiles = end;             end = round_up(W.tiles + (P / 8 + 1 + d.n_slots) * 8, 256);
-        W.lists = end;             end = round_up(W.lists + (size_t)d.n_slots * T * 4, 256);
-        W.hq = end;                end = round_up(W.hq + ((P + 127) / 128 + d.n_slots) * (size_t)(d.I / 32) * 2 * 8192, 256);
-        W.xq = end;                end = round_up(W.xq + ((P + 127) / 128 + d.n_slots) * (size_t)(d.H / 32) * 8192, 256);
+        if (grouped_use_umma(d, T)) {
+            W.pair_ad = end;       end = round_up(W.pair_ad + P * 4, 256);
+            W.counts = end;        end = round_up(W.counts + (size_t)d.n_slots * 4, 256);
+            W.tiles = end;         end = round_up(W.tiles + (P / 128 + 1 + d.n_slots) * 8, 256);
+            W.lists = end;         end = round_up(W.lists + (size_t)d.n_slots * T * 4, 256);
+            W.hq = end;            end = round_up(W.hq + ((P + 127) / 128 + d.n_slots) * (size_t)(d.I / 32) * 2 * 8192, 256);
+            W.xq = end;            end = round_up(W.xq + ((P + 127) / 128 + d.n_slots) * (size_t)(d.H / 32) * 8192, 256);
+        } else {
+            const size_t tiles = grouped_max_tiles(d, T), cap = (size_t)grouped_tile_cap(d, T), r16 = (r + 15) / 16 * 16;
+            W.g_tiles = end;       end = round_up(W.g_tiles + tiles * 16, 256);
+            W.g_done = end;        end = round_up(W.g_done + tiles * 4, 256);
+            W.g_order = end;       end = round_up(W.g_order + P * 4, 256);
+            W.g_cnt = end;         end = round_up(W.g_cnt + (d.n_slots > 8192 ? 2 * (size_t)d.n_slots * 4 : 0), 256);
+            W.g_u = end;           end = round_up(W.g_u + tiles * 2 * cap * r16 * 2, 256);
+            W.g_xq = end;          end = round_up(W.g_xq + tiles * cap * d.H * 2, 256);
+            W.g_hq = end;          end = round_up(W.g_hq + tiles * cap * d.I * 4, 256);
+        }
     }
     W.bytes = end;
     return W;

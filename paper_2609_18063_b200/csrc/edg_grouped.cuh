@@ -1,4 +1,4 @@
-// Parameters shared by the grouped (T > 1) kernels: the mma.sync tiles for small groups and the
+// Parameters shared by the grouped (T > 1) kernels: the streaming form for small groups and the
 // tcgen05 tiles for large ones.
 #pragma once
 
@@ -29,20 +29,23 @@ struct GroupedParams {
     uint8_t* hq;              // h of every 128-token tile as fp16 operand tiles (tcgen05 path)
     uint8_t* xq;              // the gathered token states of every tile as fp16 operand tiles (tcgen05 path)
     int T, H, I, E, K, group, rank, n_adapters, n_slots, out_dtype;
-    int ntok;                 // tokens per tile of this call (8, 64 or 128)
+    int ntok;                 // tokens per tile of the tcgen05 engine (128)
     float sigma;
     RecordLayout L;
 };
 
 // tcgen05 path for large groups (prefill): tiles of 128 tokens
 constexpr int kUmmaTokens = 128;
+// Where the 128-token tiles overtake the streaming form (us, streaming against tcgen05): 256 experts, 87 pairs per slot 920 : 947,
+// 128 1297 : 1166; 64 experts, 62 361 : 384, 125 667 : 675, 256 1286 : 1203; H 1024, I 256, 250 85 : 131, 1024 243 : 218.
+constexpr int kUmmaPairsPerSlot = 96;
 bool umma_grouped_supported(const edg_layer_desc& d);
 cudaError_t launch_umma_gate_up(const GroupedParams& p, int max_tiles, cudaStream_t st);
 cudaError_t launch_umma_down(const GroupedParams& p, int max_tiles, cudaStream_t st);
 
-// streaming path for small groups (batched decode): tiles of 8 tokens through the batch-1 kernel's pipeline
-bool grouped_stream_supported(const edg_layer_desc& d);
-int32_t run_grouped_stream(const edg_layer_desc* d, const GroupedParams& g, float* o_part, uint8_t* xt, int max_tiles, cudaStream_t st);
+// streaming form for small and middling groups (edg_grouped_ffn.cu)
+int32_t run_grouped_ffn(const edg_layer_desc* d, const GroupedParams& p, const WorkspaceLayout& W, uint8_t* ws, cudaStream_t st);
+cudaError_t launch_sum_choices(const GroupedParams& p, cudaStream_t st);
 
 // adapter projections for many tokens / pairs on the tensor cores (one shared adapter); false = shape not covered
 bool launch_lora_ax_tokens(const edg_layer_desc* d, const void* x, const edg_lora* lora, float* u_gu, int T, cudaStream_t st);

@@ -83,4 +83,24 @@ __device__ __forceinline__ void dequant_word_b(uint32_t w, uint32_t (&out)[4]) {
     out[3] = lop3_and_or(w2, 0x00F000F0u, 0x54005400u);
 }
 
+// The exact form: (w & 0x000F000F) read as fp16 is the subnormal q * 2^-24, (w & 0x00F000F0) is q * 2^-20, so one HFMA2
+// per pair of codes gives (q - z) * 2^-9 without rounding (subnormal inputs are exact numbers to it; zero points are
+// multiples of 1/128) -- nine instructions a word, and no bias or zero point to remove afterwards.
+// mz = neg_zero_x of the row's (scale, zero) pair; sums of products are scaled back by kUnscaleX.
+constexpr float kUnscaleX = 512.f;
+__device__ __forceinline__ __half2 neg_zero_x(__half2 sz) { return __hmul2(__high2half2(sz), u32_as_h2(0x98009800u)); }   // -z * 2^-9
+__device__ __forceinline__ void dequant_word_x(uint32_t w, __half2 mz, uint32_t (&out)[4]) {
+    const __half2 e15 = u32_as_h2(0x78007800u), e11 = u32_as_h2(0x68006800u);      // 2^15, 2^11
+    const uint32_t w2 = w >> 8;
+    out[0] = h2_as_u32(__hfma2(u32_as_h2(w & 0x000F000Fu), e15, mz));
+    out[1] = h2_as_u32(__hfma2(u32_as_h2(w & 0x00F000F0u), e11, mz));
+    out[2] = h2_as_u32(__hfma2(u32_as_h2(w2 & 0x000F000Fu), e15, mz));
+    out[3] = h2_as_u32(__hfma2(u32_as_h2(w2 & 0x00F000F0u), e11, mz));
+}
+// a += s * c, two values in one instruction
+__device__ __forceinline__ void fma2(float& a0, float& a1, float s, float c0, float c1) {
+    asm("{\n.reg .b64 a, s, c;\nmov.b64 a, {%0, %1};\nmov.b64 s, {%2, %2};\nmov.b64 c, {%3, %4};\nfma.rn.f32x2 a, s, c, a;\nmov.b64 {%0, %1}, a;\n}"
+        : "+f"(a0), "+f"(a1) : "f"(s), "f"(c0), "f"(c1));
+}
+
 }  // namespace edg

@@ -1,0 +1,85 @@
+"""The grouped path where it can go wrong: edges of its tiles (8, 16 and 32 pairs) and of its units (narrow layers whose last unit
+is partly empty), down slices of 32, 64 and 128 columns, every scale group, ranks that are no multiple of 8 or 16, adapters per
+expert, the sort for pools beyond what shared memory counts, and the first sizes that take the tcgen05 tiles.  Every token
+against the oracle; bars as everywhere (fp32 sums of exact int4 x bf16 products; the adapter's fp16 operands)."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2609_18063_b200 as edg
+from oracle import moe_oracle as orc
+from paper_2609_18063_b200 import layer_io
+from workloads import synth
+
+from _gpu_util import DeviceLayer, out_tensor, x_dev
+from test_gpu_grouped import _check_tokens, _ffn_tokens
+
+pytestmark = pytest.mark.gpu
+
+
+def _layer(H, I, group, rank, E, K, n_adapters=1):
+    cfg = dataclasses.replace(synth.CONFIGS["cfg1"], name=f"H{H}I{I}g{group}r{rank}", H=H, I=I, group=group, rank=rank, E=E, K=K,
+                              n_slots=E, n_adapters=n_adapters, seed=23)
+    return DeviceLayer(cfg)
+
+
+def _routing(rng, T, E, K, pop=None):
+    inds = np.stack([np.sort(rng.choice(E, K, replace=False, p=pop)) for _ in range(T)]).astype(np.int32)
+    return inds, rng.dirichlet(np.ones(K), size=T).astype(np.float32)
+
+
+@pytest.mark.parametrize("H,I,group,rank,E,K,n_adapters,T", [
+    (256, 128, 32, 5, 4, 1, 1, 2),          # slices of 32 columns, odd rank, one unit of each kind and that one half empty
+    (512, 256, 64, 8, 8, 2, 8, 17),         # tiles of up to 8: runs of 8 and 9 pairs
+    (1024, 256, 32, 24, 8, 2, 1, 33),       # tiles of up to 16, second 16 ranks partly empty
+    (2048, 512, 128, 16, 4, 2, 4, 50),      # tiles of up to 32: three columns and a remainder of one pair
+    (1024, 1024, 64, 64, 4, 1, 1, 97),      # slices of two stages, the largest rank
+    (4096, 512, 64, 0, 4, 2, 1, 70),        # wide state, no adapter
+])
+def test_streaming_form_at_tile_edges(H, I, group, rank, E, K, n_adapters, T):
+    L = _layer(H, I, group, rank, E, K, n_adapters)
+    X = synth.hidden_states(L.cfg, T, stream=61)
+    inds_h, gates_h = _routing(np.random.default_rng(5), T, E, K, np.array([0.6] + [0.4 / (E - 1)] * (E - 1)))
+    assert T * K <= 96 * E
+    Y = _ffn_tokens(L, L.desc, X, torch.from_numpy(inds_h).cuda(), torch.from_numpy(gates_h).cuda(), T)
+    _check_tokens(L, X, inds_h, gates_h, Y, range(T))
+    assert np.array_equal(Y, _ffn_tokens(L, L.desc, X, torch.from_numpy(inds_h).cuda(), torch.from_numpy(gates_h).cuda(), T))
+
+
+@pytest.mark.parametrize("n_adapters", [1, 16])
+def test_first_size_of_the_tensor_memory_tiles(n_adapters):
+    """97 pairs per slot on the small layer: groups of 32, rank 8, ragged tiles, an expert that spans many tiles."""
+    L = _layer(1024, 256, 32, 8, 16, 2, n_adapters)
+    T = 776 + 1
+    X = synth.hidden_states(L.cfg, T, stream=62)
+    inds_h, gates_h = _routing(np.random.default_rng(6), T, 16, 2, np.array([0.3] + [0.7 / 15] * 15))
+    assert T * 2 > 96 * 16
+    Y = _ffn_tokens(L, L.desc, X, torch.from_numpy(inds_h).cuda(), torch.from_numpy(gates_h).cuda(), T)
+    _check_tokens(L, X, inds_h, gates_h, Y, list(range(0, T, 9)) + [T - 1])
+
+
+def test_pool_with_more_slots_than_shared_memory_counts():
+    """26,000 slots: the sort keeps its counters in the workspace.  Three experts live in the first, a middle and the last slot."""
+    cfg = _layer(256, 128, 32, 8, 4, 2).cfg
+    S, T = 26000, 9
+    desc = edg.make_desc(cfg, n_slots=S)
+    R = edg.record_bytes(desc)
+    pool = torch.empty((S, R), dtype=torch.uint8, device="cuda")
+    where = [0, 13001, 25999, 7]
+    for e, s in enumerate(where):
+        pool[s] = torch.from_numpy(edg.pack_expert(desc, synth.expert_tensors(cfg, 0, e))).cuda()
+    table = torch.tensor(where, dtype=torch.int32, device="cuda")
+    lora, keep = layer_io.lora_to_device(desc, [synth.lora_tensors(cfg, 0, 0)])
+    X = synth.hidden_states(cfg, T, stream=63)
+    inds_h, gates_h = _routing(np.random.default_rng(7), T, 4, 2)
+    ws, y = layer_io.new_workspace(desc, T), out_tensor(desc, T)
+    edg.moe_expert_ffn_int4_lora(desc, pool, table, T, torch.from_numpy(inds_h).cuda(), None, torch.from_numpy(gates_h).cuda(), x_dev(X),
+                                 lora, y, ws)
+    torch.cuda.synchronize()
+    assert edg.workspace_status(ws) == 0
+    for t in range(T):
+        ref = orc.moe_ffn(X[t], inds_h[t], gates_h[t].astype(np.float64), lambda e: synth.expert_tensors(cfg, 0, e),
+                          lambda e: synth.lora_tensors(cfg, 0, 0), cfg.lora_scale, cfg.group)
+        assert orc.max_abs(y[t].cpu().numpy(), ref) <= 2e-2 and orc.rel_l2(y[t].cpu().numpy(), ref) <= 1e-3
