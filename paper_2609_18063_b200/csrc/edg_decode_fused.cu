@@ -16,9 +16,9 @@
 //   * Issuing a bulk copy costs its lane some 50 ns and the lanes of a warp take turns, so the 16
 //     copies of a load are dealt to the four warps behind a CTA barrier, and the score of small
 //     copies for the adapter slices is issued while the quarter's weights are still in flight.
-//   * Both projections run on mma.sync.m16n8k16 fragments: the codes masked straight into biased
-//     fp16 (1024 + q or 64 + q, five instructions a word), the activations as column 0 of the B
-//     tile; bias, zero point and scale are applied in fp32 per 64-code block.  The loops over K
+//   * Both projections run on mma.sync.m16n8k16 fragments: the codes masked straight into fp16 --
+//     subnormal, or biased in dependent chains (edg_mma.cuh), five instructions a word -- the activations
+//     as column 0 of the B tile; zero point and scale are applied in fp32 per 64-code block.  The loops over K
 //     blocks are rolled and the operands live in shared memory on purpose: a CTA runs most of this
 //     code once, and instruction fetch competes with the weight stream.
 //   * The rank-r LoRA projections A.x are split over the CTAs of a cluster and exchanged through
@@ -373,7 +373,7 @@ __device__ __noinline__ void head_publish(const FusedParams& p, uint8_t* smem, f
 constexpr int kPreRed = 32;       // s_red rows 0..31: adapter projections, 32..39: head rows
 constexpr int kMaxPre = 8 * kFW;  // head rows per head CTA (up to four batches of two per warp)
 
-template <int NCW, int DCH, int TG, int TD, int CPB>
+template <int NCW, int DCH, int TG, int TD, int CPB, bool EX>
 __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_constant__ FusedParams p) {
     extern __shared__ __align__(128) uint8_t smem[];
     const int cl = blockIdx.x / kC;                // cluster: an expert, or some quarters of it
@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
             const uint4 v = *reinterpret_cast<const uint4*>(p.x + t * 8);
             const float f[8] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y),
                                 bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w)};
-            s_xb[t] = permute8(f);
+            s_xb[t] = EX ? permute8_s(f) : permute8(f);
             // fp16 is exact for bf16 inputs in the normal range; sum what the MMA will see
 #pragma unroll
             for (int e = 0; e < 8; e += 2) {
@@ -547,8 +547,8 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
         sum = group_sum<4 * CPB>(sum);
         sodd = group_sum<4 * CPB>(sodd);
         if (on && (t % (4 * CPB)) == 0) {
-            s_xsum[t / (4 * CPB)] = sum + sodd;
-            s_xbias[t / (4 * CPB)] = fmaf(1024.f, sum, 64.f * sodd);
+            s_xsum[t / (4 * CPB)] = EX ? (sum + sodd) * kScaleS : sum + sodd;
+            if (!EX) s_xbias[t / (4 * CPB)] = fmaf(1024.f, sum, 64.f * sodd);
         }
     }
     };
@@ -763,7 +763,13 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         uint4 xb = make_uint4(0, 0, 0, 0);
-                        if (g8 == 0) xb = xbp[j * 4];
+                        if (g8 == 0) {
+                            xb = xbp[j * 4];
+                            if (EX) {                          // undo the 2^-4 of the odd positions
+                                xb.y = h2_as_u32(__hmul2(u32_as_h2(xb.y), __float2half2_rn(16.f)));
+                                xb.w = h2_as_u32(__hmul2(u32_as_h2(xb.w), __float2half2_rn(16.f)));
+                            }
+                        }
                         mma16816(c, lw[j].x, lw2[j].x, lw[j].y, lw2[j].y, __byte_perm(xb.x, xb.y, 0x5410), __byte_perm(xb.z, xb.w, 0x5410));
                         mma16816(c, lw[j].z, lw2[j].z, lw[j].w, lw2[j].w, __byte_perm(xb.x, xb.y, 0x7632), __byte_perm(xb.z, xb.w, 0x7632));
                     }
@@ -1002,22 +1008,22 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                             for (int mt = 0; mt < NT; ++mt) {
                                 const uint8_t* cw = cbase + mt * S.mat_codes + i * 256;
                                 uint32_t alo[4], ahi[4];
-                                dequant_word_b(*reinterpret_cast<const uint32_t*>(cw), alo);
-                                dequant_word_b(*reinterpret_cast<const uint32_t*>(cw + 128), ahi);
+                                dequant_code_word<EX>(*reinterpret_cast<const uint32_t*>(cw), alo);
+                                dequant_code_word<EX>(*reinterpret_cast<const uint32_t*>(cw + 128), ahi);
                                 if (u == 0) mma16816_zero(cfr[mt], alo[0], ahi[0], alo[1], ahi[1], xb.x, xb.y);
                                 else mma16816(cfr[mt], alo[0], ahi[0], alo[1], ahi[1], xb.x, xb.y);
                                 mma16816(cfr[mt], alo[2], ahi[2], alo[3], ahi[3], xb.z, xb.w);
                             }
                         }
                         const int gi = ((ch0 + ib * CPB) * 32) >> p.gshift;
-                        const float xs = s_xsum[(vw * NCW) / CPB + ib], xbias = s_xbias[(vw * NCW) / CPB + ib];
+                        const float xs = s_xsum[(vw * NCW) / CPB + ib], xbias = EX ? 0.f : s_xbias[(vw * NCW) / CPB + ib];
 #pragma unroll
                         for (int mt = 0; mt < NT; ++mt) {
                             const uint8_t* zw = st + S.sz0 + mt * S.mat_sz + gi * 64 + g8 * 4;
                             const __half2 z0 = u32_as_h2(*reinterpret_cast<const uint32_t*>(zw));
                             const __half2 z1 = u32_as_h2(*reinterpret_cast<const uint32_t*>(zw + 32));
-                            a_lo[mt] = fmaf(__low2float(z0), fmaf(-__high2float(z0), xs, cfr[mt][0] - xbias), a_lo[mt]);
-                            a_hi[mt] = fmaf(__low2float(z1), fmaf(-__high2float(z1), xs, cfr[mt][2] - xbias), a_hi[mt]);
+                            a_lo[mt] = fmaf(__low2float(z0), fmaf(-__high2float(z0), xs, EX ? cfr[mt][0] : cfr[mt][0] - xbias), a_lo[mt]);
+                            a_hi[mt] = fmaf(__low2float(z1), fmaf(-__high2float(z1), xs, EX ? cfr[mt][2] : cfr[mt][2] - xbias), a_hi[mt]);
                         }
                     }
                     // the second half of the K range follows into the same stages as soon as all
@@ -1031,8 +1037,8 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                 if (t4 == 0) {
 #pragma unroll
                     for (int mt = 0; mt < NT; ++mt) {
-                        s_part[warp * 2 * rows_gu + mt * 16 + g8] = a_lo[mt];
-                        s_part[warp * 2 * rows_gu + mt * 16 + 8 + g8] = a_hi[mt];
+                        s_part[warp * 2 * rows_gu + mt * 16 + g8] = EX ? a_lo[mt] * kUnscaleS : a_lo[mt];
+                        s_part[warp * 2 * rows_gu + mt * 16 + 8 + g8] = EX ? a_hi[mt] * kUnscaleS : a_hi[mt];
                     }
                 }
             }
@@ -1110,7 +1116,7 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                 const float4 a = *reinterpret_cast<const float4*>(hq + i * 32 + q * 8);
                 const float4 b = *reinterpret_cast<const float4*>(hq + i * 32 + q * 8 + 4);
                 const float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-                s_hb[tid] = lo ? permute8_lo(f) : permute8(f);
+                s_hb[tid] = EX ? (lo ? permute8_lo_s(f) : permute8_s(f)) : (lo ? permute8_lo(f) : permute8(f));
             } else if (tid >= 64 && tid < 64 + DCH / CPB) {
                 const int j = tid - 64;
                 float v = 0.f, vo = 0.f;
@@ -1118,8 +1124,8 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                     v += hq[j * 32 * CPB + e];
                     vo += hq[j * 32 * CPB + e + 1];
                 }
-                s_hsum[j] = v + vo;
-                s_hbias[j] = fmaf(1024.f, v, 64.f * vo);
+                s_hsum[j] = EX ? (v + vo) * kScaleS : v + vo;
+                if (!EX) s_hbias[j] = fmaf(1024.f, v, 64.f * vo);
             }
             __syncthreads();
             // this buffer's barrier is used again two quarters on: arm it before anyone can send
@@ -1148,23 +1154,23 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                                 const int ti = warp + kFW * (ps * TD + tt);
                                 const uint8_t* cw = dbase + (ti * DCH + i) * 256;
                                 uint32_t alo[4], ahi[4];
-                                dequant_word_b(*reinterpret_cast<const uint32_t*>(cw), alo);
-                                dequant_word_b(*reinterpret_cast<const uint32_t*>(cw + 128), ahi);
+                                dequant_code_word<EX>(*reinterpret_cast<const uint32_t*>(cw), alo);
+                                dequant_code_word<EX>(*reinterpret_cast<const uint32_t*>(cw + 128), ahi);
                                 if (u == 0) mma16816_zero(cfr[tt], alo[0], ahi[0], alo[1], ahi[1], hb.x, hb.y);
                                 else mma16816(cfr[tt], alo[0], ahi[0], alo[1], ahi[1], hb.x, hb.y);
                                 mma16816(cfr[tt], alo[2], ahi[2], alo[3], ahi[3], hb.z, hb.w);
                             }
                         }
                         const int gi = (ib * CPB * 32) >> p.gshift;
-                        const float hs = s_hsum[ib], hbias = s_hbias[ib];
+                        const float hs = s_hsum[ib], hbias = EX ? 0.f : s_hbias[ib];
 #pragma unroll
                         for (int tt = 0; tt < TD; ++tt) {
                             const int ti = warp + kFW * (ps * TD + tt);
                             const uint8_t* zw = dsz + (ti * gps + gi) * 64 + g8 * 4;
                             const __half2 z0 = u32_as_h2(*reinterpret_cast<const uint32_t*>(zw));
                             const __half2 z1 = u32_as_h2(*reinterpret_cast<const uint32_t*>(zw + 32));
-                            acc_lo[tt] = fmaf(__low2float(z0), fmaf(-__high2float(z0), hs, cfr[tt][0] + cfr[tt][1] - hbias), acc_lo[tt]);
-                            acc_hi[tt] = fmaf(__low2float(z1), fmaf(-__high2float(z1), hs, cfr[tt][2] + cfr[tt][3] - hbias), acc_hi[tt]);
+                            acc_lo[tt] = fmaf(__low2float(z0), fmaf(-__high2float(z0), hs, EX ? cfr[tt][0] + cfr[tt][1] : cfr[tt][0] + cfr[tt][1] - hbias), acc_lo[tt]);
+                            acc_hi[tt] = fmaf(__low2float(z1), fmaf(-__high2float(z1), hs, EX ? cfr[tt][2] + cfr[tt][3] : cfr[tt][2] + cfr[tt][3] - hbias), acc_hi[tt]);
                         }
                     }
                     if (t4 == 0) {
@@ -1172,8 +1178,9 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                         for (int tt = 0; tt < TD; ++tt) {
                             const int ti = warp + kFW * (ps * TD + tt);
                             // (the first quarter of an expert starts the sums)
-                            s_o[ti * 16 + g8] = it ? s_o[ti * 16 + g8] + acc_lo[tt] : acc_lo[tt];
-                            s_o[ti * 16 + 8 + g8] = it ? s_o[ti * 16 + 8 + g8] + acc_hi[tt] : acc_hi[tt];
+                            const float vl = EX ? acc_lo[tt] * kUnscaleS : acc_lo[tt], vh = EX ? acc_hi[tt] * kUnscaleS : acc_hi[tt];
+                            s_o[ti * 16 + g8] = it ? s_o[ti * 16 + g8] + vl : vl;
+                            s_o[ti * 16 + 8 + g8] = it ? s_o[ti * 16 + 8 + g8] + vh : vh;
                         }
                     }
                 }
@@ -1346,9 +1353,9 @@ bool fused_supported(const edg_layer_desc& d) {
     return fused_smem(d.H, d.I, d.E, d.group, d.rank).total <= kFusedSmemLimit;
 }
 
-template <int NCW, int DCH, int TG, int TD, int CPB>
-static cudaError_t launch_fused(const FusedParams& p, size_t smem, bool pdl, cudaStream_t st) {
-    auto kern = fused_layer_kernel<NCW, DCH, TG, TD, CPB>;
+template <int NCW, int DCH, int TG, int TD, int CPB, bool EX>
+static cudaError_t launch_form(const FusedParams& p, size_t smem, bool pdl, cudaStream_t st) {
+    auto kern = fused_layer_kernel<NCW, DCH, TG, TD, CPB, EX>;
     static bool configured = false;       // per-process, per-instantiation one-time attributes
     if (!configured) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmemLimit);
@@ -1373,6 +1380,14 @@ static cudaError_t launch_fused(const FusedParams& p, size_t smem, bool pdl, cud
     cfg.attrs = at;
     cfg.numAttrs = pdl ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, p);
+}
+
+// Steps of a dependent chain (they write the next hidden state) keep the biased code arithmetic, all others take the subnormal
+// form (edg_mma.cuh): the 1280-step burst of the 35B-class layer 4.42 -> 4.25 ms, two subtractions per scaled block fewer.
+template <int NCW, int DCH, int TG, int TD, int CPB>
+static cudaError_t launch_fused(const FusedParams& p, size_t smem, bool pdl, cudaStream_t st) {
+    return p.x_next == nullptr ? launch_form<NCW, DCH, TG, TD, CPB, true>(p, smem, pdl, st)
+                               : launch_form<NCW, DCH, TG, TD, CPB, false>(p, smem, pdl, st);
 }
 
 // One fused launch for a batch-1 layer-step.  W_pre may be null (no prediction).

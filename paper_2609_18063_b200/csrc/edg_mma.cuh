@@ -70,17 +70,45 @@ __device__ __forceinline__ uint4 permute8(const float (&v)[8]) {
     return r;
 }
 
-// The cheapest form: the code words masked straight into fp16 with a bias -- codes 0, 2, 4, 6 of a
-// word as 1024 + q, codes 1, 3, 5, 7 as 64 + q (their nibble sits four bits higher in the
-// mantissa) -- five instructions a word.  The dot product then carries 1024 * (sum of the
-// activations at even positions) + 64 * (sum at odd positions), exactly representable products
-// summed in fp32, which the caller subtracts per scaled block along with the zero-point term.
+// The cheapest form: the code words masked straight into fp16 subnormals -- codes 0, 2, 4, 6 of a word are q * 2^-24, codes 1, 3,
+// 5, 7 (their nibble sits four bits higher) q * 2^-20 -- five instructions a word and nothing to remove: the tensor cores take
+// subnormal operands exactly.  The activations at odd positions carry the missing 2^-4 (permute8_s), sums of products come
+// out as 2^-24 of the dot product with the codes, in which unit the caller removes the zero point
+// (fma(-z, 2^-24 * sum of the activations, c)); kUnscaleS brings the end result back.  1e-6 relative on a layer's output.
+constexpr float kScaleS = 5.9604644775390625e-8f;      // 2^-24
+constexpr float kUnscaleS = 16777216.f;                // 2^24
+__device__ __forceinline__ void dequant_word_s(uint32_t w, uint32_t (&out)[4]) {
+    const uint32_t w2 = w >> 8;
+    out[0] = w & 0x000F000Fu;
+    out[1] = w & 0x00F000F0u;
+    out[2] = w2 & 0x000F000Fu;
+    out[3] = w2 & 0x00F000F0u;
+}
+// permute8 and permute8_lo with the activations at odd positions scaled by 2^-4
+__device__ __forceinline__ uint4 permute8_s(const float (&v)[8]) {
+    const float f[8] = {v[0], v[1] * 0.0625f, v[2], v[3] * 0.0625f, v[4], v[5] * 0.0625f, v[6], v[7] * 0.0625f};
+    return permute8(f);
+}
+__device__ __forceinline__ uint4 permute8_lo_s(const float (&v)[8]) {
+    const float f[8] = {v[0], v[1] * 0.0625f, v[2], v[3] * 0.0625f, v[4], v[5] * 0.0625f, v[6], v[7] * 0.0625f};
+    return permute8_lo(f);
+}
+// The biased form: codes 0, 2, 4, 6 of a word as 1024 + q, codes 1, 3, 5, 7 as 64 + q, five instructions a word too.  The dot
+// product then carries 1024 * (sum of the activations at even positions) + 64 * (sum at odd positions), which the caller
+// subtracts per scaled block along with the zero-point term.  Its fp32 sums of 10^4-sized terms cost 2e-5 relative on a
+// layer's output; it stays for chains of dependent steps, whose state is rounded to bf16 and fed back: there another
+// rounding can tip a near-tie of the routing further on, and a chain is to reproduce what it produced before.
 __device__ __forceinline__ void dequant_word_b(uint32_t w, uint32_t (&out)[4]) {
     const uint32_t w2 = w >> 8;
     out[0] = lop3_and_or(w, 0x000F000Fu, 0x64006400u);
     out[1] = lop3_and_or(w, 0x00F000F0u, 0x54005400u);
     out[2] = lop3_and_or(w2, 0x000F000Fu, 0x64006400u);
     out[3] = lop3_and_or(w2, 0x00F000F0u, 0x54005400u);
+}
+// EX: the subnormal form, else the biased one
+template <bool EX> __device__ __forceinline__ void dequant_code_word(uint32_t w, uint32_t (&o)[4]) {
+    if (EX) dequant_word_s(w, o);
+    else dequant_word_b(w, o);
 }
 
 // The exact form: (w & 0x000F000F) read as fp16 is the subnormal q * 2^-24, (w & 0x00F000F0) is q * 2^-20, so one HFMA2
