@@ -141,8 +141,8 @@ int32_t edg_ffn_workspace_bytes(const edg_layer_desc* desc, int32_t T, size_t* b
  * Synchronises `stream`. */
 int32_t edg_workspace_status(const void* workspace, void* stream, int32_t* status);
 
-/* Tracing: with a dev buffer of (CTAs in the grid) x 32 uint64 (the batch-1 layer kernel launches
- * at most 16 (K + 1) + E / 16 + 3 CTAs), every CTA stamps the GPU's nanosecond timer
+/* Tracing: with a dev buffer of (CTAs in the grid) x 32 uint64, every CTA of the batch-1 layer kernel -- which then always runs in
+ * its throughput form, of at most 16 (K + 1) + E / 16 + 3 CTAs -- stamps the GPU's nanosecond timer
  * at its phase boundaries, in slot 0 start, 1 first copies issued, 2 adapter projections sent,
  * 3 first weights landed, 4 gate/up of the first quarter done, 5 peers' projections in, 6 h sent,
  * 7 h of the quarter in, 8 partial output written, 9 end, 10 slot taken, 12 head row summed,

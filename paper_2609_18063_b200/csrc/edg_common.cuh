@@ -114,8 +114,17 @@ struct WorkspaceLayout {
     size_t g_u;       // [tiles][2][cap][rank16] fp16 : sigma A_gate x, sigma A_up x
     size_t g_xq;      // [tiles][cap * H] fp16      : token states in operand order
     size_t g_hq;      // [tiles][2 * cap * I] fp16  : h, value and residual, in operand order
+    // the form of the batch-1 step that runs alone or as a link of a dependent chain (edg_step.cu):
+    size_t step;      // kStepCtrlBytes: start counter at 0, lists of deferred units from kStepDeferOff (starts as zeros)
+    size_t step_x;    // exchange buffers: h and A_down h partials (4 of them), x + y (16); a word not written holds 0xFFFFFFFF
     size_t bytes;
 };
+
+constexpr int kStepStates = 16;
+constexpr size_t kStepDeferOff = 256, kStepCtrlBytes = kStepDeferOff + kStepStates * (2048 / 16 + 2) * 4;
+int sm_count();
+size_t step_region_words(const edg_layer_desc& d);
+size_t step_exchange_words(const edg_layer_desc& d);
 
 // pairs a tile of the streaming form holds, and how many tiles T tokens can make
 int grouped_tile_cap(const edg_layer_desc& d, int T);
@@ -142,6 +151,8 @@ inline WorkspaceLayout workspace_layout(const edg_layer_desc& d, int T) {
     const size_t one_set = (size_t)kDownSlices * (d.K + 1) * d.H * sizeof(float);   // K routed experts and the shared expert
     W.lone_bytes = W.partial + one_set;
     size_t end = round_up(W.partial + (size_t)kHandoffRing * one_set, 256);
+    W.step = end;     end = round_up(W.step + kStepCtrlBytes, 256);
+    W.step_x = end;   end = round_up(W.step_x + step_region_words(d) * sizeof(float), 256);
     W.o = W.pair_slot = W.pair_ad = W.counts = W.n_tiles = W.tiles = W.lists = W.hq = W.xq = end;
     W.g_tiles = W.g_done = W.g_order = W.g_cnt = W.g_u = W.g_xq = W.g_hq = end;
     if (T > 1) {
@@ -186,6 +197,12 @@ struct FusedExtras {
 };
 
 bool fused_supported(const edg_layer_desc& d);
+// The batch-1 layer-step that runs alone or as a link of a dependent chain (edg_step.cu).
+unsigned long long* trace_buffer();      // set by edg_set_trace_buffer, or null
+bool step_supported(const edg_layer_desc& d, bool shared);
+int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* slots, const int32_t* table, const int32_t* experts,
+                 const float* gates, const void* x, const edg_lora* lora, void* y, const void* W_pre, int32_t* inds_next, float* gates_next,
+                 float* logits_next, void* workspace, int flag_in, int flag_out, int stale, cudaStream_t st, const FusedExtras& extras);
 // One fused launch for a batch-1 layer-step (edg_decode_fused.cu).  W_pre may be null (no prediction).
 int32_t run_fused_layer(const edg_layer_desc* d, const void* slot_pool, const int32_t* slots, const int32_t* table,
                         const int32_t* experts, const float* gates, const void* x, const edg_lora* lora, void* y,

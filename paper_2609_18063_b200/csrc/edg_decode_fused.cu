@@ -43,7 +43,7 @@
 #include <cooperative_groups.h>
 
 #include "edg_mma.cuh"
-#include "edg_ptx.cuh"
+#include "edg_head.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -55,7 +55,6 @@ constexpr int kFW = 4;            // warps per CTA
 constexpr int kStages = 2;        // copy stages per CTA: a quarter of the gate/up K range each, or half of the down block
 constexpr int kMaxRank = 64;
 constexpr int kMaxEpc = 4;         // experts a cluster may take, one after the other
-constexpr int kTraceMarks = 32;
 constexpr int kRing = kHandoffRing;   // chained layer-steps in flight: hand-off slots for logits, reduce scratch, counters
 
 // ---------------------------------------------------------------- shared-memory carve-up
@@ -171,14 +170,6 @@ __device__ __forceinline__ void trace_mark(const FusedParams& p, int m) {
     }
 }
 
-__device__ __forceinline__ void trace_stamp(const FusedParams& p, int m) {
-    if (p.trace != nullptr) {
-        unsigned long long t;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-        p.trace[(size_t)blockIdx.x * kTraceMarks + m] = t;
-    }
-}
-
 // four consecutive outputs (i a multiple of 4)
 __device__ __forceinline__ void store_y4(void* y, int out_dtype, size_t i, float4 v) {
     if (out_dtype == EDG_F32) {
@@ -277,89 +268,6 @@ __device__ __noinline__ float head_row_partial(const void* W_pre, int pre_dtype,
         }
     }
     return acc;
-}
-
-__device__ __noinline__ void topk_large(float* work, int E, int K, int lane, int32_t* inds, float* gates) {
-    warp_softmax_topk(work, E, K, lane, inds, gates);
-}
-
-// One warp publishes head logits -- lane l owns logit `e` with value `v` when `own` is set -- into the
-// ring slot the next layer-step reads, and if they were the last ones of the head, computes the
-// top-k: the (expert, gate) pairs go behind the logits of the ring slot, where a chained next step
-// picks them up, and into the caller's inds_next / gates_next.  `state` is the lane's entry of
-// the ring slot as it was when the kernel started: a slot is written again only after the step
-// that read it has ended and has reset it.
-__device__ __noinline__ void head_publish(const FusedParams& p, uint8_t* smem, float v, int e, bool own, int lane, uint32_t state) {
-    int mine = 0;
-    const int ring = p.flag_out >= 0 ? p.flag_out : 0;
-    float* logits_ws = p.logits_ws + (size_t)ring * (p.E + kPairWords);
-    int32_t* pre_counter = p.pre_counter + ring;
-    if (own) {
-        if (p.flag_out >= 0) {
-            uint32_t it = 0;
-            while (state != kNotYet && ++it < kSpinLimit) state = ld_relaxed_gpu_u32(&logits_ws[e]);
-            if (state != kNotYet) atomicExch(p.status, EDG_E_TIMEOUT);
-            // "the step that last read this slot is over" travels on to the reader of this logit
-            asm volatile("fence.acq_rel.gpu;" ::: "memory");
-        }
-        st_relaxed_gpu_u32(&logits_ws[e], __float_as_uint(v));
-        mine = 1;
-    }
-    const int n_mine = __popc(__ballot_sync(0xFFFFFFFFu, mine));
-    __syncwarp();
-    int last = 0;
-    // the counting atomic releases this warp's logits and acquires everyone else's
-    if (lane == 0) last = (atom_add_acq_rel_gpu(pre_counter, n_mine) + n_mine == p.E) ? 1 : 0;
-    last = __shfl_sync(0xFFFFFFFFu, last, 0);
-    if (!last) return;
-    if (lane == 0) {
-        atomicSub(pre_counter, p.E);      // commutes with the arrivals of the head that uses this slot next
-        trace_stamp(p, 16);
-    }
-    float* work = reinterpret_cast<float*>(smem + p.S.s_topk);
-#pragma unroll 1
-    for (int i0 = 0; i0 < p.E; i0 += 256) {                     // 8 independent loads per lane and pass
-        float v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int i = i0 + u * 32 + lane;
-            v[u] = i < p.E ? __ldcg(&logits_ws[i]) : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int i = i0 + u * 32 + lane;
-            if (i < p.E) {
-                work[i] = v[u];
-                if (p.logits_next != nullptr) p.logits_next[i] = v[u];
-            }
-        }
-    }
-    __syncwarp();
-    int32_t* s_i = reinterpret_cast<int32_t*>(smem + p.S.s_topk) + p.E;        // [K] winners, then [K] gates
-    float* s_g = reinterpret_cast<float*>(s_i + 32);
-    if (lane == 0) trace_stamp(p, 17);
-    if (p.E <= 256) warp_softmax_topk_reg<8>(work, p.E, p.K, lane, s_i, s_g);
-    else topk_large(work, p.E, p.K, lane, s_i, s_g);
-    __syncwarp();
-    if (lane == 0) trace_stamp(p, 25);
-    if (lane < p.K) {
-        // the hand-off proper, first: (expert, gate) as one word per choice behind the logits of the
-        // ring slot, released after everything the publishers of the logits had observed.  The
-        // step that takes them resets the slot only after all of its CTAs have read them, i.e.
-        // after this warp has long finished with the logits.
-        if (p.flag_out >= 0) {
-            __threadfence();
-            if (lane == 0) trace_stamp(p, 26);
-            st_relaxed_gpu_u64(reinterpret_cast<unsigned long long*>(logits_ws + p.E) + lane,
-                               ((unsigned long long)__float_as_uint(s_g[lane]) << 32) | (uint32_t)s_i[lane]);
-        }
-        p.inds_next[lane] = s_i[lane];
-        p.gates_next[lane] = s_g[lane];
-        // (each entry is final by itself: the host polls the mirror until all K are >= 0)
-        if (p.inds_mirror != nullptr)
-            asm volatile("st.relaxed.sys.global.s32 [%0], %1;" ::"l"(p.inds_mirror + lane), "r"(s_i[lane]) : "memory");
-    }
-    if (lane == 0) trace_stamp(p, 15);
 }
 
 // ---------------------------------------------------------------- the fused kernel
@@ -799,7 +707,7 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                 const float v_lo = __shfl_sync(0xFFFFFFFFu, lo_, (lane & 7) * 4);
                 const float v_hi = __shfl_sync(0xFFFFFFFFu, hi_, (lane & 7) * 4);
                 if (warp == 0) trace_mark(p, 12);
-                head_publish(p, smem, lane < 8 ? v_lo : v_hi, mrow0 + lane, lane < 16, lane, pre_state);
+                publish_logits(p, reinterpret_cast<float*>(smem + p.S.s_topk), lane < 8 ? v_lo : v_hi, mrow0 + lane, lane < 16, lane, pre_state);
                 if (warp == 0) trace_mark(p, 13);
             }
         }
@@ -861,7 +769,7 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
             }
             // both rows in one go: lane 0 publishes the first, lane 1 the second
             const uint32_t st2 = __shfl_sync(0xFFFFFFFFu, ps2, 0);
-            head_publish(p, smem, lane == 1 ? v2 : v, lane == 1 ? pe2 : pe, lane == 0 || (lane == 1 && prow2), lane,
+            publish_logits(p, reinterpret_cast<float*>(smem + p.S.s_topk), lane == 1 ? v2 : v, lane == 1 ? pe2 : pe, lane == 0 || (lane == 1 && prow2), lane,
                          lane == 1 ? st2 : ps);
             if (warp == 0) trace_mark(p, 13);
         }
@@ -891,7 +799,7 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
         float v = 0.f;
         if (own)
             for (int w = 0; w < kFW; ++w) v += s_red[(kPreRed + lane) * kFW + w];
-        head_publish(p, smem, v, e, own, lane, pre_state);
+        publish_logits(p, reinterpret_cast<float*>(smem + p.S.s_topk), v, e, own, lane, pre_state);
     }
 
     read_take();
@@ -1337,6 +1245,7 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
 // ---------------------------------------------------------------- host side
 
 static unsigned long long* g_trace = nullptr;     // set by edg_set_trace_buffer
+unsigned long long* trace_buffer() { return g_trace; }
 
 constexpr size_t kFusedSmemLimit = 56 * 1024;     // four CTAs per SM
 

@@ -810,14 +810,14 @@ cudaError_t launch_pdl(void (*kern)(Args...), dim3 grid, int threads, size_t sme
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-int device_sms() {
+}  // namespace
+
+int sm_count() {
     int dev = 0, n = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
     return n;
 }
-
-}  // namespace
 
 // Pairs a tile holds.  A tile's weights are read once whatever it holds; its MMA time grows with its columns of 8.
 int grouped_tile_cap(const edg_layer_desc& d, int T) {
@@ -910,7 +910,7 @@ int32_t run_grouped_ffn(const edg_layer_desc* d, const GroupedParams& g, const W
     ta.slots = g.slots; ta.table = g.table; ta.experts = g.experts; ta.x = g.x; ta.xq = xq; ta.u = u; ta.lora = g.lora;
     ta.H = H; ta.K = g.K; ta.rank = g.rank; ta.r16 = p.r16; ta.cap = cap; ta.adapters = ga.adapters; ta.sigma = g.sigma;
     EDG_CUDA_TRY(launch_pdl(tile_operands_kernel, dim3((unsigned)grouped_max_tiles(*d, g.T), cap / 8 + 2 * p.r16 / 16), 256, 0, st, ta));
-    const int sms = device_sms();
+    const int sms = sm_count();
     if (cap == 8) EDG_CUDA_TRY(launch_pdl(g.group >= 64 ? grouped_ffn_kernel<2, 1> : grouped_ffn_kernel<1, 1>, dim3(sms), GThreads, smem, st, p, cgu, zgu, cd, zd));
     else EDG_CUDA_TRY(launch_pdl(g.group >= 64 ? grouped_ffn_kernel<2, 4> : grouped_ffn_kernel<1, 4>, dim3(sms), GThreads, smem, st, p, cgu, zgu, cd, zd));
     EDG_CUDA_TRY(launch_sum_choices(g, st));

@@ -140,6 +140,7 @@ struct edg_store {
     // chaining of consecutive batch-1 layer-steps: when a call consumes the routing that the
     // previous call on the same stream and workspace produced, its kernel is launched as a
     // programmatic dependent of that one and waits on a device flag instead of the kernel's end
+    bool chain_latency = false;            // that step ran in the latency form
     const void* chain_x_next = nullptr;    // the hidden state the last batch-1 layer-step produces for its successor, or null
     const void* chain_inds = nullptr;
     const void* chain_ws = nullptr;
@@ -632,15 +633,25 @@ static int32_t layer_decode(edg_store* s, int32_t layer, const void* x,
             const edg::WorkspaceLayout W = edg::workspace_layout(s->d, 1);
             EDG_CUDA_TRY(cudaMemsetAsync(w8 + edg::kCtrlCounters, 0, edg::kCtrlBytes - edg::kCtrlCounters, st));
             EDG_CUDA_TRY(cudaMemsetAsync(w8 + W.logits, 0xFF, (size_t)edg::kHandoffRing * (s->d.E + edg::kPairWords) * sizeof(float), st));
+            EDG_CUDA_TRY(cudaMemsetAsync(w8 + W.step, 0, edg::kStepCtrlBytes, st));
+            EDG_CUDA_TRY(cudaMemsetAsync(w8 + W.step_x, 0xFF, edg::step_region_words(s->d) * sizeof(float), st));
             EDG_CUDA_TRY(cudaMemsetAsync(w8 + W.dep, 0, (size_t)edg::kHandoffRing * edg::kDepWords * sizeof(float), st));
             s->ring_ws = workspace;
             s->ring_next = 0;
             s->pub_slot = -1;
         }
-        const bool chain = chained && !fresh;
-        const int flag_in = chain ? s->chain_flag : -1;              // ring slot this step's logits arrive in
+        bool chain = chained && !fresh;
         // a chained step whose x is the state the previous step is still producing waits for it on the device
-        const bool dep_chain = chain && s->chain_x_next != nullptr && s->chain_x_next == x;
+        bool dep_chain = chain && s->chain_x_next != nullptr && s->chain_x_next == x;
+        // A step that shares the GPU with dozens of others, chained through the routing alone, runs in the throughput form; one
+        // that is alone, or a link of a dependent chain, in the latency form.  (A step that writes the next hidden state while
+        // its own is at hand already starts a dependent chain: it is launched alone, its successors wait for it.)
+        const bool shared = !s->shared_rec.empty() && s->shared_rec[layer] != nullptr;
+        const bool latency_ok = edg::step_supported(s->d, shared) && edg::trace_buffer() == nullptr;     // (only the other form is traced)
+        if (dep_chain && latency_ok != s->chain_latency) chain = dep_chain = false;                      // the forms hand x on in ways of their own
+        if (latency_ok && chain && !dep_chain && x_next != nullptr) chain = false;
+        const bool latency = latency_ok && (!chain || dep_chain);
+        const int flag_in = chain ? s->chain_flag : -1;              // ring slot this step's logits arrive in
         int stale = -1;
         if (!chain && s->pub_slot >= 0) stale = s->pub_slot;         // nobody will read that head's logits
         s->pub_slot = -1;
@@ -652,11 +663,14 @@ static int32_t layer_decode(edg_store* s, int32_t layer, const void* x,
         extras.x_next = x_next;
         extras.eps = eps;
         extras.dep_wait = dep_chain ? flag_in : -1;
-        if (!s->shared_rec.empty() && s->shared_rec[layer] != nullptr) {
+        if (shared) {
             extras.shared_rec = s->shared_rec[layer];
             extras.shared_lora = s->shared_has_lora[layer] ? &s->shared_lora[layer] : nullptr;
         }
-        rc = edg::run_fused_layer(&s->d, pool, slot_arg, table, expert_arg, gates_cur, x,
+        if (latency)
+            rc = edg::run_step(&s->d, pool, slot_arg, table, expert_arg, gates_cur, x, (lora && s->d.rank > 0) ? lora : nullptr, y,
+                               W_pre_next, inds_next, gates_next, logits_next_opt, workspace, flag_in, flag_out, stale, st, extras);
+        else rc = edg::run_fused_layer(&s->d, pool, slot_arg, table, expert_arg, gates_cur, x,
                                   (lora && s->d.rank > 0) ? lora : nullptr, y, W_pre_next, inds_next, gates_next,
                                   logits_next_opt, workspace, flag_in, flag_out, ring, stale, st, &extras);
         if (W_pre_next != nullptr) s->pub_slot = flag_out;
@@ -668,6 +682,7 @@ static int32_t layer_decode(edg_store* s, int32_t layer, const void* x,
             s->step_done_valid = true;
         }
         s->chain_x_next = x_next;
+        s->chain_latency = latency;
         s->chain_inds = W_pre_next != nullptr ? inds_next : nullptr;
         s->chain_ws = workspace;
         s->chain_stream = stream;
