@@ -121,7 +121,7 @@ struct WorkspaceLayout {
 };
 
 constexpr int kStepStates = 16;
-constexpr size_t kStepDeferOff = 256, kStepCtrlBytes = kStepDeferOff + kStepStates * (2048 / 16 + 2) * 4;
+constexpr size_t kStepDeferOff = 256, kStepCtrlBytes = kStepDeferOff + kStepStates * (2048 / 16 + 4) * 4;
 int sm_count();
 size_t step_region_words(const edg_layer_desc& d);
 size_t step_exchange_words(const edg_layer_desc& d);

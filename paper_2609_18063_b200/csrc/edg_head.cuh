@@ -20,6 +20,34 @@ static __device__ __noinline__ void topk_large(float* work, int E, int K, int la
     warp_softmax_topk(work, E, K, lane, inds, gates);
 }
 
+// The top-k of the logits in `work` by one warp, into the caller's inds_next / gates_next and, first, as one (expert, gate) word per
+// choice into `pair` (this lane's word of the ring slot, or null), where a chained next step picks them up.  FENCE: what the
+// publishers of the logits had observed travels on with them.  `work`: E floats and 256 bytes for the winners.
+template <bool FENCE, typename P>
+__device__ __noinline__ void emit_routing(const P& p, float* work, int lane, unsigned long long* pair) {
+    __syncwarp();
+    int32_t* s_i = reinterpret_cast<int32_t*>(work) + p.E;        // [K] winners, then [K] gates
+    float* s_g = reinterpret_cast<float*>(s_i + 32);
+    if (p.E <= 256) warp_softmax_topk_reg<8>(work, p.E, p.K, lane, s_i, s_g);
+    else topk_large(work, p.E, p.K, lane, s_i, s_g);
+    __syncwarp();
+    if (lane == 0) trace_stamp(p, 25);
+    if (lane < p.K) {
+        // the step that takes the pairs resets the slot only after all of its CTAs have read them, i.e.
+        // after this warp has long finished with the logits
+        if (pair != nullptr) {
+            if (FENCE) __threadfence();
+            if (lane == 0) trace_stamp(p, 26);
+            st_relaxed_gpu_u64(pair, ((unsigned long long)__float_as_uint(s_g[lane]) << 32) | (uint32_t)s_i[lane]);
+        }
+        p.inds_next[lane] = s_i[lane];
+        p.gates_next[lane] = s_g[lane];
+        // (each entry is final by itself: the host polls the mirror until all K are >= 0)
+        if (p.inds_mirror != nullptr)
+            asm volatile("st.relaxed.sys.global.s32 [%0], %1;" ::"l"(p.inds_mirror + lane), "r"(s_i[lane]) : "memory");
+    }
+}
+
 // One warp publishes head logits -- lane l owns logit `e` with value `v` when `own` is set -- into the
 // ring slot the next layer-step reads, and if they were the last ones of the head, computes the
 // top-k: the (expert, gate) pairs go behind the logits of the ring slot, where a chained next step
@@ -72,30 +100,8 @@ __device__ __noinline__ void publish_logits(const P& p, float* work, float v, in
         }
     }
     __syncwarp();
-    int32_t* s_i = reinterpret_cast<int32_t*>(work) + p.E;        // [K] winners, then [K] gates
-    float* s_g = reinterpret_cast<float*>(s_i + 32);
     if (lane == 0) trace_stamp(p, 17);
-    if (p.E <= 256) warp_softmax_topk_reg<8>(work, p.E, p.K, lane, s_i, s_g);
-    else topk_large(work, p.E, p.K, lane, s_i, s_g);
-    __syncwarp();
-    if (lane == 0) trace_stamp(p, 25);
-    if (lane < p.K) {
-        // the hand-off proper, first: (expert, gate) as one word per choice behind the logits of the
-        // ring slot, released after everything the publishers of the logits had observed.  The
-        // step that takes them resets the slot only after all of its CTAs have read them, i.e.
-        // after this warp has long finished with the logits.
-        if (p.flag_out >= 0) {
-            __threadfence();
-            if (lane == 0) trace_stamp(p, 26);
-            st_relaxed_gpu_u64(reinterpret_cast<unsigned long long*>(logits_ws + p.E) + lane,
-                               ((unsigned long long)__float_as_uint(s_g[lane]) << 32) | (uint32_t)s_i[lane]);
-        }
-        p.inds_next[lane] = s_i[lane];
-        p.gates_next[lane] = s_g[lane];
-        // (each entry is final by itself: the host polls the mirror until all K are >= 0)
-        if (p.inds_mirror != nullptr)
-            asm volatile("st.relaxed.sys.global.s32 [%0], %1;" ::"l"(p.inds_mirror + lane), "r"(s_i[lane]) : "memory");
-    }
+    emit_routing<true>(p, work, lane, p.flag_out >= 0 ? reinterpret_cast<unsigned long long*>(logits_ws + p.E) + lane : nullptr);
     if (lane == 0) trace_stamp(p, 15);
 }
 

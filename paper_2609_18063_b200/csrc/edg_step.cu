@@ -40,11 +40,11 @@ constexpr int kStepMaxK = 16;
 constexpr int kStepMaxRank = 64;
 constexpr uint32_t kEpochStarts = 8192;       // what one grid adds to the start counter in total
 constexpr uint32_t kWaitStarted = 256;        // polls before a CTA whose grid is not fully resident gives its rows away
-constexpr int kStepBufs = 4;
+constexpr int kStepBufs = 4, kStateCopies = 8;
 
 // byte offsets in shared memory; h .. udi lie inside the union, used once the gate/up weights are
 struct StepSmem {
-    uint32_t un, codes_warp, sz, sz_warp, xb, x, xsum, xbias, bgu, ad, bd, u4, uf, hl, sel, red, total;
+    uint32_t un, sz, sz_tile, xb, x, xsum, xbias, bgu, ad, bd, u4, uf, hl, sel, red, bar, total;
     uint32_t h, hb, hsum, hbias, part, udi;
 };
 
@@ -66,11 +66,12 @@ struct StepParams {
     uint16_t* x_next;
     unsigned long long* trace;                // (this form is not traced: null)
     uint32_t* starts;                         // the start counter
-    float* hx;                                // [kStepBufs][hx_words]: h; the A_down h partials of every expert CTA; the A x partials
-    float* vx;                                // [kStepStates][H]: x + y of a dependent chain
-    int32_t* defer;                           // [kStepStates][H/16 + 2]: number, then (unit + 1) of those left to the last starter
-    uint32_t hx_words, ud_off, ux_off;
+    float* hx;                                // [kStepBufs][hx_words]: h; the A_down h partials of every expert CTA; the A x partials; head logits
+    float* vx;                                // [kStepStates][kStateCopies][H]: x + y of a dependent chain
+    int32_t* defer;                           // [kStepStates][H/16 + 4]: number, then (unit + 1) of those left to the last starter
+    uint32_t hx_words, ud_off, ux_off, lx_off;
     int I, E, K, Kt, group, gshift, rank, rank_shared, rmax, n_adapters, n_slots, pre_dtype, out_dtype;
+    int cta_route, cta_state;                 // CTAs that compute the routing for the next step and the caller's x_next, or -1
     int n_gu, n_dn, n_exp, n_head, n_headc;   // CTAs with gate/up, with down work, the larger of both; tiles of 16 head rows, CTAs for them
     int flag_in, flag_out, stale, dep;        // dep: x arrives in band from the step before
     float sigma, eps;
@@ -145,7 +146,6 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g8 = lane >> 2, t4 = lane & 3;
     const int cta = blockIdx.x, crank = cta % 4;
     const bool has_gu = cta < p.n_gu, has_dn = cta < p.n_dn, has_head = cta >= p.n_exp && cta - p.n_exp < p.n_headc;
-    const bool finisher = p.x_next != nullptr && cta == p.n_exp;         // writes x_next
     const int kpos = cta / 16, n0 = ((cta % 16) / 4) * sw + crank * RG;  // this CTA's expert, and its first row of h
     const bool is_shared = kpos >= p.K;
     const edg_lora& lo = is_shared ? p.shared_lora : p.lora;
@@ -164,9 +164,14 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
     int* s_ad = s_slot + 40;
     int* s_misc = s_slot + 60;                                           // [0] epoch, [1] this CTA started last, [2], [3] scratch
     float* s_red = reinterpret_cast<float*>(smem + S.red);               // [64]
+    uint64_t* bar_w = reinterpret_cast<uint64_t*>(smem + S.bar);         // gate/up weights
+    constexpr int MP = CPB == 2 ? 2 : 1, VP = MP;                        // row tiles, and items of the down projection, at once
+    constexpr int CT = NCK * TW * 256;                                   // bytes of a row tile's codes
 
     // ---- start: count this CTA in, let the next kernel come
     if (tid == 0) {
+        mbar_init(bar_w, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         uint32_t old;
         asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(p.starts) : "memory");
         const bool last = old % kEpochStarts == gridDim.x - 1;
@@ -181,8 +186,29 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         pdl_launch_dependents();
     }
     if (p.flag_in < 0) pdl_wait_prior_grid();                            // a step on its own: everything queued before it has happened
-    uint4 xv8 = make_uint4(0, 0, 0, 0);
-    if (!p.dep && tid < H / 8) xv8 = __ldcg(reinterpret_cast<const uint4*>(p.x + tid * 8));
+    // eight values of the state (value i of them): the B words of the MMAs, the block sums
+    auto take_x = [&](int i, uint4 v) {
+        const float f[8] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y), bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w)};
+        s_xb[i] = EX ? permute8_s(f) : permute8(f);
+        float sum = 0.f, sodd = 0.f;
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) {
+            sum += __half2float(__float2half_rn(f[e]));
+            sodd += __half2float(__float2half_rn(f[e + 1]));
+        }
+        sum = group_sum<4 * CPB>(sum);
+        sodd = group_sum<4 * CPB>(sodd);
+        if (i % (4 * CPB) == 0) {
+            s_xsum[i / (4 * CPB)] = EX ? (sum + sodd) * kScaleS : sum + sodd;
+            if (!EX) s_xbias[i / (4 * CPB)] = fmaf(1024.f, sum, 64.f * sodd);
+        }
+    };
+    if (!p.dep && tid >= TThreads - H / 8) {                             // (by the last warps: the first is after the routing)
+        const int i = tid - (TThreads - H / 8);
+        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(p.x + i * 8));
+        *reinterpret_cast<uint4*>(s_x + i * 8) = v;
+        take_x(i, v);
+    }
     const bool head_mma = p.pre_dtype == EDG_F16 && p.E % 16 == 0;
     auto load_head = [&](int tile) {                                     // row by row, padded by 16 bytes against bank conflicts
         const uint8_t* src = static_cast<const uint8_t*>(p.W_pre) + (size_t)tile * 16 * H * 2;
@@ -190,7 +216,6 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         for (int i = tid; i < 16 * (H / 8); i += TThreads) cp16(un + (i / (H / 8)) * (H * 2 + 16) + (i % (H / 8)) * 16, src + (size_t)i * 16);
     };
     if (has_head && head_mma) load_head(cta - p.n_exp);
-    cp_commit();
     if (p.stale >= 0 && cta == 0)
         for (int i = tid; i < p.E + kPairWords; i += TThreads) st_relaxed_gpu_u32(&p.logits_ws[(size_t)p.stale * (p.E + kPairWords) + i], kNotYet);
 
@@ -225,33 +250,23 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         }
         if (lane == p.K && p.Kt > p.K) { slot = 0; vg = 1.f; }           // the shared expert: always on, weight 1
         if (lane < p.Kt) { s_slot[lane] = slot; s_gate[lane] = vg; s_ad[lane] = ad; }
+        // all of this CTA's gate/up weights: a row tile's codes and its (scale, zero) pairs are one run each
+        const int mine = __shfl_sync(0xFFFFFFFFu, slot, has_gu ? kpos : 0);
+        if (has_gu && mine >= 0) {
+            if (lane == 0) mbar_expect_tx(bar_w, NT * (CT + S.sz_tile));
+            __syncwarp();
+            const uint8_t* rec = is_shared ? p.shared_rec : p.pool + (size_t)mine * p.L.bytes;
+            const int mt = lane % NT, n = n0 + 16 * (mt % TG);
+            if (lane < NT) bulk_g2s(un + mt * CT, rec + (mt / TG ? p.L.codes_up : p.L.codes_gate) + code_off(H, n, 0), CT, bar_w);
+            else if (lane < 2 * NT) bulk_g2s(smem + S.sz + mt * S.sz_tile, rec + (mt / TG ? p.L.sz_up : p.L.sz_gate) + sz_off(H, p.group, n, 0), S.sz_tile, bar_w);
+        }
     }
     __syncthreads();
     const uint32_t epoch = (uint32_t)s_misc[0];
     auto record = [&](int k) { return k >= p.K ? p.shared_rec : p.pool + (size_t)s_slot[k] * p.L.bytes; };
     const bool valid = has_gu && s_slot[kpos] >= 0;
-    const int gsh = p.gshift, gpw = max(1, (NCK * 32) >> gsh);           // scale groups of a row that a warp touches
-    uint8_t* my_codes = un + warp * S.codes_warp;
-    uint8_t* my_sz = smem + S.sz + warp * S.sz_warp;
-    const int ad_k = has_gu ? s_ad[kpos] : 0;
+    const int gsh = p.gshift, ad_k = has_gu ? s_ad[kpos] : 0;
 
-    // ---- all of this CTA's gate/up weights, by the warps that will use them
-    if (valid) {
-        const uint8_t* rec = record(kpos);
-#pragma unroll
-        for (int mt = 0; mt < NT; ++mt) {
-            const uint8_t* src = rec + (mt / TG ? p.L.codes_up : p.L.codes_gate) + code_off(H, n0 + 16 * (mt % TG), warp * NCK);
-#pragma unroll
-            for (int i = 0; i < NCK / 2; ++i) cp16(my_codes + mt * NCK * 256 + (i * 32 + lane) * 16, src + (i * 32 + lane) * 16);
-        }
-        const int g0 = (warp * NCK * 32) >> gsh;
-        const int lg = 31 - __clz(gpw * 4);
-        for (int i = lane; i < NT << lg; i += 32) {
-            const int mt = i >> lg, o = (i & (gpw * 4 - 1)) * 16;
-            cp16(my_sz + mt * gpw * 64 + o, rec + (mt / TG ? p.L.sz_up : p.L.sz_gate) + sz_off(H, p.group, n0 + 16 * (mt % TG), g0) + o);
-        }
-    }
-    cp_commit();
     // ---- the adapter's slices: this CTA's rows of B_gate and B_up, its columns of A_down, B_down rows of its output rows
     if (valid && r > 0) {
         const int per = RG * r / 8;                                      // 16-byte pieces of one matrix's rows
@@ -275,18 +290,14 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
     };
     if (has_dn) load_bd(cta);
     cp_commit();
-    // ---- its down weights are announced to the L2
-    if (has_dn) {
-        constexpr int lines = DCH * 2;                                   // 128-byte lines of a row tile's codes in one slice
-        for (int i = tid; i < p.Kt * 4 * lines; i += TThreads) {
-            const int k = i / (4 * lines), c = (i / lines) % 4;
-            if (s_slot[k] >= 0)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(record(k) + p.L.codes_down + (size_t)c * ((size_t)H * sw / 2) + code_off(sw, cta * 16, 0) + (i % lines) * 128));
-        }
-        for (int i = tid; i < p.Kt * 4; i += TThreads)
-            if (s_slot[i / 4] >= 0)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(record(i / 4) + p.L.sz_down + down_sz_off(H, p.I, p.group, cta * 16, (i % 4) * (sw >> gsh))));
-    }
+    // ---- its down weights are announced to the L2, an (expert, quarter of I) per lane
+    if (has_dn && warp == 1)
+        for (int i = lane; i < p.Kt * 4; i += 32)
+            if (s_slot[i >> 2] >= 0) {
+                const uint8_t* rec = record(i >> 2);
+                bulk_prefetch_l2(rec + p.L.codes_down + (size_t)(i & 3) * ((size_t)H * sw / 2) + code_off(sw, cta * 16, 0), DCH * 256);
+                bulk_prefetch_l2(rec + p.L.sz_down + down_sz_off(H, p.I, p.group, cta * 16, (i & 3) * (sw >> gsh)), (sw >> gsh) * 64);
+            }
     // ---- rows of A_gate, A_up of every set: four tasks (the four warps of the throughput form) per row, all CTAs share them
     const int set_tasks = 8 * p.rank, n_task = sets * set_tasks + 8 * p.rank_shared;
     auto a_row = [&](int set, int q) {                                   // lane's first values of task q of a set
@@ -296,7 +307,9 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         return static_cast<const uint16_t*>(up ? l.A_up : l.A_gate) + row * H + ((q & 3) * 32 + lane) * 8;
     };
     auto task_set = [&](int task) { return task >= sets * set_tasks ? sets : (sets == 1 ? 0 : task / set_tasks); };
-    const int task0 = warp * gridDim.x + cta;
+    // (the CTAs without expert work first, then the last warps of the others)
+    const int spare = (int)gridDim.x - p.n_exp;
+    const int task0 = cta >= p.n_exp ? (TW - 1 - warp) * spare + cta - p.n_exp : TW * spare + (TW - 1 - warp) * p.n_exp + cta;
     uint4 pa[NCK / 2];
     if (task0 < n_task) {
         const int set = task_set(task0);
@@ -306,15 +319,10 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
     }
     // A_down h partials this thread adds up (tid -> (expert and quarter, rank))
     const int udq = p.rmax > 0 ? tid / p.rmax : 0, udj = tid - udq * p.rmax, udn = p.rmax > 0 ? TThreads / p.rmax : 1;
-    const int e_own = (cta - p.n_exp) * 16 + lane;
-    uint32_t pre_state = kNotYet;
-    if (has_head && warp == 0 && lane < 16 && e_own < p.E && p.flag_out >= 0)
-        pre_state = ld_relaxed_gpu_u32(&p.logits_ws[(size_t)p.flag_out * (p.E + kPairWords) + e_own]);
-
     // ---- the hidden state
     if (p.dep) {
         const bool on = tid * 4 < H;
-        const float* src = p.vx + (size_t)((epoch + kStepStates - 1) % kStepStates) * H + 4 * tid;
+        const float* src = p.vx + (size_t)((epoch + kStepStates - 1) % kStepStates * kStateCopies + cta % kStateCopies) * H + 4 * tid;
         uint4 w = make_uint4(0, 0, 0, 0);
         bool got = !on;
         for (uint32_t it = 0; !got && it < kSpinLimit; ++it) {
@@ -337,36 +345,19 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         }
         __syncthreads();
     }
-    if (tid < H / 8) {                                                   // eight values a thread: B words, block sums
-        const uint4 v = p.dep ? *reinterpret_cast<const uint4*>(s_x + tid * 8) : xv8;
-        if (!p.dep) *reinterpret_cast<uint4*>(s_x + tid * 8) = v;
-        const float f[8] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y), bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w)};
-        s_xb[tid] = EX ? permute8_s(f) : permute8(f);
-        float sum = 0.f, sodd = 0.f;
-#pragma unroll
-        for (int e = 0; e < 8; e += 2) {
-            sum += __half2float(__float2half_rn(f[e]));
-            sodd += __half2float(__float2half_rn(f[e + 1]));
-        }
-        sum = group_sum<4 * CPB>(sum);
-        sodd = group_sum<4 * CPB>(sodd);
-        if (tid % (4 * CPB) == 0) {
-            s_xsum[tid / (4 * CPB)] = EX ? (sum + sodd) * kScaleS : sum + sodd;
-            if (!EX) s_xbias[tid / (4 * CPB)] = fmaf(1024.f, sum, 64.f * sodd);
-        }
-    }
-    // (every CTA of the step before has used its exchange buffers up: they are cleared for the step three epochs on)
-    {
-        float* hc = p.hx + (size_t)((epoch + kStepBufs - 1) % kStepBufs) * p.hx_words;
-        float* vc = p.vx + (size_t)((epoch + kStepStates / 2) % kStepStates) * H;
-        const uint32_t all = gridDim.x * TThreads;
-        for (uint32_t i = tid * gridDim.x + cta; i < p.hx_words; i += all) st_relaxed_gpu_u32(hc + i, kNotYet);
-        for (uint32_t i = tid * gridDim.x + cta; i < (uint32_t)H; i += all) st_relaxed_gpu_u32(vc + i, kNotYet);
-        if (cta == 0 && tid == 0) st_relaxed_gpu(p.defer + (size_t)((epoch + kStepStates / 2) % kStepStates) * (p.n_dn + 2), 0);
-    }
-    __syncthreads();
-
+    if (p.dep && tid < H / 8) take_x(tid, *reinterpret_cast<const uint4*>(s_x + tid * 8));
+    if (p.dep) __syncthreads();
     float* hx = p.hx + (size_t)(epoch % kStepBufs) * p.hx_words;
+    auto all_started = [&]() {
+        uint32_t c;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(p.starts) : "memory");
+        return c / kEpochStarts != epoch;
+    };
+    // after `it` polls without success: give up when the grid is not fully resident, go on with a flagged result at the very end
+    auto tired = [&](uint32_t it, bool& give_up, bool& got) {
+        if ((it % kWaitStarted) == kWaitStarted - 1 && !all_started()) give_up = true;
+        if (it >= kSpinLimit) { atomicExch(p.status, EDG_E_TIMEOUT); got = true; }
+    };
     // ---- this warp's share of A x
     auto a_dot = [&](int set, int q, bool first) {
         float v = 0.f;
@@ -383,49 +374,120 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         if (lane == 0) st_relaxed_gpu_u32(hx + p.ux_off + (size_t)set * 8 * p.rmax + (q & 3) * 2 * p.rmax + (q >> 2), __float_as_uint(v));
     }
     if (valid) {
-        // ---- gate/up on the tensor cores; per (row, scaled block) the scale and what it multiplies stay in the tile's own region
-        cp_wait<1>();
-        __syncwarp();
+        // ---- gate/up on the tensor cores, a gate tile and its up tile at once where the registers allow it; per (row, scaled block)
+        // the scale and what it multiplies stay in the region the codes came in
+        mbar_wait(bar_w, 0, p.status);
         const uint4* xbp = s_xb + warp * NCK * 4 + t4;
 #pragma unroll 1
-        for (int mt = 0; mt < NT; ++mt) {
-            uint8_t* cb = my_codes + mt * NCK * 256;
-            const uint8_t* zb = my_sz + mt * gpw * 64 + g8 * 4;
-            float t_lo[NBW], t_hi[NBW], s_lo[NBW], s_hi[NBW];
+        for (int t = 0; t < NT / MP; ++t) {
+            float c[MP][NBW][4];
 #pragma unroll
-            for (int b = 0; b < NBW; ++b) {
-                float c[4];
+            for (int u = 0; u < CPB; ++u)
 #pragma unroll
-                for (int u = 0; u < CPB; ++u) {
+                for (int b = 0; b < NBW; ++b) {
                     const int i = b * CPB + u;
                     uint4 xb = make_uint4(0, 0, 0, 0);
                     if (g8 == 0) xb = xbp[i * 4];
-                    uint32_t alo[4], ahi[4];
-                    dequant_code_word<EX>(*reinterpret_cast<const uint32_t*>(cb + i * 256 + g8 * 16 + t4 * 4), alo);
-                    dequant_code_word<EX>(*reinterpret_cast<const uint32_t*>(cb + i * 256 + 128 + g8 * 16 + t4 * 4), ahi);
-                    if (u == 0) mma16816_zero(c, alo[0], ahi[0], alo[1], ahi[1], xb.x, xb.y);
-                    else mma16816(c, alo[0], ahi[0], alo[1], ahi[1], xb.x, xb.y);
-                    mma16816(c, alo[2], ahi[2], alo[3], ahi[3], xb.z, xb.w);
-                }
-                const int gi = (b * CPB * 32) >> gsh, blk = (warp * NCK) / CPB + b;
-                const __half2 z0 = u32_as_h2(*reinterpret_cast<const uint32_t*>(zb + gi * 64));
-                const __half2 z1 = u32_as_h2(*reinterpret_cast<const uint32_t*>(zb + gi * 64 + 32));
-                const float xs = s_xsum[blk], xbias = EX ? 0.f : s_xbias[blk];
-                s_lo[b] = __low2float(z0); s_hi[b] = __low2float(z1);
-                t_lo[b] = fmaf(-__high2float(z0), xs, EX ? c[0] : c[0] - xbias);
-                t_hi[b] = fmaf(-__high2float(z1), xs, EX ? c[2] : c[2] - xbias);
-            }
-            __syncwarp();                                                // every lane is done with this tile's codes
-            if (t4 == 0) {
-                float2* ts = reinterpret_cast<float2*>(cb);              // [block][16 rows, rotated] (scale, term)
-                const int at = (g8 + 4 * (warp >> 1)) & 15;
 #pragma unroll
-                for (int b = 0; b < NBW; ++b) { ts[b * 16 + at] = make_float2(s_lo[b], t_lo[b]); ts[b * 16 + (at ^ 8)] = make_float2(s_hi[b], t_hi[b]); }
+                    for (int m = 0; m < MP; ++m) {
+                        const uint8_t* cb = un + (m * TG + t) * CT + (warp * NCK + i) * 256 + g8 * 16 + t4 * 4;
+                        uint32_t alo[4], ahi[4];
+                        dequant_code_word<EX>(*reinterpret_cast<const uint32_t*>(cb), alo);
+                        dequant_code_word<EX>(*reinterpret_cast<const uint32_t*>(cb + 128), ahi);
+                        if (u == 0) mma16816_zero(c[m][b], alo[0], ahi[0], alo[1], ahi[1], xb.x, xb.y);
+                        else mma16816(c[m][b], alo[0], ahi[0], alo[1], ahi[1], xb.x, xb.y);
+                        mma16816(c[m][b], alo[2], ahi[2], alo[3], ahi[3], xb.z, xb.w);
+                    }
+                }
+            __syncwarp();                                                // every lane is done with these tiles' codes
+            if (t4 == 0) {
+                const int at = (g8 + 4 * (warp >> 1)) & 15;              // rotated against bank conflicts
+#pragma unroll
+                for (int b = 0; b < NBW; ++b) {
+                    const int blk = warp * NBW + b;
+                    const float xs = s_xsum[blk], xbias = EX ? 0.f : s_xbias[blk];
+#pragma unroll
+                    for (int m = 0; m < MP; ++m) {
+                        const uint8_t* zb = smem + S.sz + (m * TG + t) * S.sz_tile + ((blk * CPB * 32) >> gsh) * 64 + g8 * 4;
+                        const __half2 z0 = u32_as_h2(*reinterpret_cast<const uint32_t*>(zb)), z1 = u32_as_h2(*reinterpret_cast<const uint32_t*>(zb + 32));
+                        float2* ts = reinterpret_cast<float2*>(un + (m * TG + t) * CT + warp * NCK * 256) + b * 16;      // [16 rows] (scale, term)
+                        ts[at] = make_float2(__low2float(z0), fmaf(-__high2float(z0), xs, EX ? c[m][b][0] : c[m][b][0] - xbias));
+                        ts[at ^ 8] = make_float2(__low2float(z1), fmaf(-__high2float(z1), xs, EX ? c[m][b][2] : c[m][b][2] - xbias));
+                    }
+                }
             }
         }
     }
+    // A x of this expert: the four tasks of a row, from whoever has computed them
+    bool miss = false;
+    if (valid && tid >= 256 && tid - 256 < 2 * r) {
+        const float* ux = hx + p.ux_off + (size_t)(is_shared ? sets : (p.n_adapters == 1 ? 0 : kpos)) * 8 * p.rmax + (tid - 256);
+        uint32_t u[4];
+        bool got = false;
+        for (uint32_t it = 0; !got && !miss; ++it) {
+#pragma unroll
+            for (int w = 0; w < 4; ++w) u[w] = ld_relaxed_gpu_u32(ux + w * 2 * p.rmax);
+            got = u[0] != kNotYet && u[1] != kNotYet && u[2] != kNotYet && u[3] != kNotYet;
+            if (!got) tired(it, miss, got);
+        }
+        s_uf[tid - 256] = ((__uint_as_float(u[0]) + __uint_as_float(u[1])) + __uint_as_float(u[2])) + __uint_as_float(u[3]);
+    }
     cp_wait<0>();
-    __syncthreads();
+    if (__syncthreads_or(miss)) {                                    // not all of this grid is resident: all of them here
+        const int set = is_shared ? sets : (p.n_adapters == 1 ? 0 : kpos);
+#pragma unroll 1
+        for (int q = warp; q < 8 * r; q += TW) {
+            const float u = a_dot(set, q, false);
+            if (lane == 0) s_u4[(q & 3) * 2 * kStepMaxRank + (q >> 2)] = u;
+        }
+        __syncthreads();
+        if (tid < 2 * r) {
+            float u = 0.f;
+            for (int w = 0; w < 4; ++w) u += s_u4[w * 2 * kStepMaxRank + tid];
+            s_uf[tid] = u;
+        }
+        __syncthreads();
+    }
+
+    // ---- finish gate/up: four chains per row (as the four warps of the throughput form), adapter, SiLU, product
+    if (has_gu) {
+        if (tid < 2 * RG * 4) {
+            float v = 0.f;
+            const int slot = tid >> 2, w = tid & 3, m = slot & 1, i = slot >> 1, mt = m * TG + (i >> 4), row = i & 15;
+            if (valid) {
+                constexpr int NB = 2 * NBW;                              // blocks of one half of a chain
+#pragma unroll
+                for (int half = 0; half < 2; ++half)
+#pragma unroll
+                    for (int j = 0; j < NB; ++j) {
+                        const int blk = (w + 4 * half) * NB + j;         // block of the row; NBW of them per warp here
+                        const float2 st = reinterpret_cast<const float2*>(un + mt * CT + (blk / NBW) * NCK * 256)[(blk % NBW) * 16 + ((row + 4 * w) & 15)];
+                        v = fmaf(st.x, st.y, v);
+                    }
+                if (EX) v *= kUnscaleS;
+            }
+            const float p1 = __shfl_down_sync(0xFFFFFFFFu, v, 1), p2 = __shfl_down_sync(0xFFFFFFFFu, v, 2), p3 = __shfl_down_sync(0xFFFFFFFFu, v, 3);
+            v = ((v + p1) + p2) + p3;
+            if (valid && r > 0 && w == 0)
+                v = fmaf(p.sigma, b_dot(reinterpret_cast<const uint16_t*>(smem + S.bgu) + (m * RG + i) * r, s_uf + m * r, r), v);
+            const float up = __shfl_down_sync(0xFFFFFFFFu, v, 4);
+            if ((tid & 7) == 0) {
+                const float h = valid ? silu_f(v) * up : 0.f;
+                s_hl[i] = h;
+                st_relaxed_gpu_u32(hx + (size_t)kpos * p.I + n0 + i, __float_as_uint(h));
+            }
+        }
+        __syncthreads();
+        if (r > 0 && warp * 8 < r) {                                     // partial of A_down h over this CTA's rows, four lanes per rank
+            const uint16_t* A = reinterpret_cast<const uint16_t*>(smem + S.ad);
+            const int j = tid >> 2, part = tid & 3;                      // (TThreads / 4 ranks in one go: kStepMaxRank and more)
+            float u = 0.f;
+            if (j < r && valid)
+                for (int n = part; n < RG; n += 4) u = fmaf(bf16_bits_to_float(A[j * RG + n]), s_hl[n], u);
+            u = group_sum<4>(u);
+            if (j < r && part == 0) st_relaxed_gpu_u32(hx + p.ud_off + (size_t)cta * p.rmax + j, __float_as_uint(u));
+        }
+    }
 
     // ---- the down weights of this CTA's output rows: the first two items of every warp are on their way from here on
     constexpr int kPre = 2;
@@ -450,88 +512,15 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         for (int u = 0; u < kPre; ++u) load_item(cta, warp + u * TW, dw[u], dz[u]);
     }
 
-    auto all_started = [&]() {
-        uint32_t c;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(p.starts) : "memory");
-        return c / kEpochStarts != epoch;
-    };
-    // after `it` polls without success: give up when the grid is not fully resident, go on with a flagged result at the very end
-    auto tired = [&](uint32_t it, bool& give_up, bool& got) {
-        if ((it % kWaitStarted) == kWaitStarted - 1 && !all_started()) give_up = true;
-        if (it >= kSpinLimit) { atomicExch(p.status, EDG_E_TIMEOUT); got = true; }
-    };
-    // ---- finish gate/up: four chains per row (as the four warps of the throughput form), adapter, SiLU, product
-    if (has_gu) {
-        float v = 0.f;
-        if (tid < 2 * RG * 4) {
-            const int slot = tid >> 2, w = tid & 3, m = slot & 1, i = slot >> 1, mt = m * TG + (i >> 4), row = i & 15;
-            if (valid) {
-                constexpr int NB = 2 * NBW;                              // blocks of one half of a chain
-#pragma unroll
-                for (int half = 0; half < 2; ++half)
-#pragma unroll
-                    for (int j = 0; j < NB; ++j) {
-                        const int blk = (w + 4 * half) * NB + j;         // block of the row; NBW of them per warp here
-                        const float2 st = reinterpret_cast<const float2*>(un + (blk / NBW) * S.codes_warp + mt * NCK * 256)[(blk % NBW) * 16 + ((row + 4 * w) & 15)];
-                        v = fmaf(st.x, st.y, v);
-                    }
-                if (EX) v *= kUnscaleS;
-            }
-            const float p1 = __shfl_down_sync(0xFFFFFFFFu, v, 1), p2 = __shfl_down_sync(0xFFFFFFFFu, v, 2), p3 = __shfl_down_sync(0xFFFFFFFFu, v, 3);
-            v = ((v + p1) + p2) + p3;
-        }
-        // A x of this expert: the four tasks of a row, from whoever has computed them
-        bool miss = false;
-        if (valid && tid >= 256 && tid - 256 < 2 * r) {
-            const float* ux = hx + p.ux_off + (size_t)(is_shared ? sets : (p.n_adapters == 1 ? 0 : kpos)) * 8 * p.rmax + (tid - 256);
-            uint32_t u[4];
-            bool got = false;
-            for (uint32_t it = 0; !got && !miss; ++it) {
-#pragma unroll
-                for (int w = 0; w < 4; ++w) u[w] = ld_relaxed_gpu_u32(ux + w * 2 * p.rmax);
-                got = u[0] != kNotYet && u[1] != kNotYet && u[2] != kNotYet && u[3] != kNotYet;
-                if (!got) tired(it, miss, got);
-            }
-            s_uf[tid - 256] = ((__uint_as_float(u[0]) + __uint_as_float(u[1])) + __uint_as_float(u[2])) + __uint_as_float(u[3]);
-        }
-        if (__syncthreads_or(miss)) {                                    // not all of this grid is resident: all of them here
-            const int set = is_shared ? sets : (p.n_adapters == 1 ? 0 : kpos);
-#pragma unroll 1
-            for (int q = warp; q < 8 * r; q += TW) {
-                const float u = a_dot(set, q, false);
-                if (lane == 0) s_u4[(q & 3) * 2 * kStepMaxRank + (q >> 2)] = u;
-            }
-            __syncthreads();
-            if (tid < 2 * r) {
-                float u = 0.f;
-                for (int w = 0; w < 4; ++w) u += s_u4[w * 2 * kStepMaxRank + tid];
-                s_uf[tid] = u;
-            }
-            __syncthreads();
-        }
-        if (tid < 2 * RG * 4) {
-            const int slot = tid >> 2, m = slot & 1, i = slot >> 1;
-            if (valid && r > 0 && (tid & 3) == 0)
-                v = fmaf(p.sigma, b_dot(reinterpret_cast<const uint16_t*>(smem + S.bgu) + (m * RG + i) * r, s_uf + m * r, r), v);
-            const float up = __shfl_down_sync(0xFFFFFFFFu, v, 4);
-            if ((tid & 7) == 0) {
-                const float h = valid ? silu_f(v) * up : 0.f;
-                s_hl[i] = h;
-                st_relaxed_gpu_u32(hx + (size_t)kpos * p.I + n0 + i, __float_as_uint(h));
-            }
-        }
-        __syncthreads();
-        if (r > 0 && warp * 8 < r) {                                     // partial of A_down h over this CTA's rows, four lanes per rank
-            const uint16_t* A = reinterpret_cast<const uint16_t*>(smem + S.ad);
-            const int j = tid >> 2, part = tid & 3;                      // (TThreads / 4 ranks in one go: kStepMaxRank and more)
-            float u = 0.f;
-            if (j < r && valid)
-                for (int n = part; n < RG; n += 4) u = fmaf(bf16_bits_to_float(A[j * RG + n]), s_hl[n], u);
-            u = group_sum<4>(u);
-            if (j < r && part == 0) st_relaxed_gpu_u32(hx + p.ud_off + (size_t)cta * p.rmax + j, __float_as_uint(u));
-        }
+    // (every CTA of the step before has used its exchange buffers up: they are cleared for the step three epochs on)
+    {
+        float* hc = p.hx + (size_t)((epoch + kStepBufs - 1) % kStepBufs) * p.hx_words;
+        float* vc = p.vx + (size_t)((epoch + kStepStates / 2) % kStepStates) * kStateCopies * H;
+        const uint32_t all = gridDim.x * TThreads;
+        for (uint32_t i = tid * gridDim.x + cta; i < p.hx_words; i += all) st_relaxed_gpu_u32(hc + i, kNotYet);
+        for (uint32_t i = tid * gridDim.x + cta; i < (uint32_t)H * kStateCopies; i += all) st_relaxed_gpu_u32(vc + i, kNotYet);
+        if (cta == 0 && tid == 0) st_relaxed_gpu(p.defer + (size_t)((epoch + kStepStates / 2) % kStepStates) * (p.n_dn + 4), 0);
     }
-
     // ---- the head's rows, in tiles of 16
     if (has_head) {
 #pragma unroll 1
@@ -540,8 +529,8 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
             const bool own = warp == 0 && lane < 16 && e0 + lane < p.E;
             float lg = 0.f;
             if (tile >= p.n_headc) {                                     // (the first tile has been on its way since the start)
+                __syncthreads();
                 if (head_mma) { load_head(tile); cp_commit(); cp_wait<0>(); }
-                if (own && p.flag_out >= 0) pre_state = ld_relaxed_gpu_u32(&p.logits_ws[(size_t)p.flag_out * (p.E + kPairWords) + e0 + lane]);
                 __syncthreads();
             }
             if (head_mma) {
@@ -605,8 +594,7 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
                 if (warp == 0 && lane < 16)
                     for (int w = 0; w < 4; ++w) lg += s_red[lane * 4 + w];
             }
-            if (warp == 0) publish_logits(p, reinterpret_cast<float*>(un), lg, e0 + lane, own, lane, pre_state);
-            __syncthreads();                                             // (the union is used again)
+            if (own) st_relaxed_gpu_u32(hx + p.lx_off + e0 + lane, __float_as_uint(lg));
         }
     }
 
@@ -671,65 +659,73 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
             }
             __syncthreads();
         }
+        auto delta = [&](int item) {                                     // adapter delta of row `warp` for an (expert, quarter)
+            const int k = item >> 2, rk = k >= p.K ? p.rank_shared : p.rank, set = k >= p.K ? sets : (p.n_adapters == 1 ? 0 : k);
+            return b_dot(reinterpret_cast<const uint16_t*>(smem + S.bd) + (size_t)set * 16 * p.rmax + warp * rk, s_udi + item * (p.rmax + 1), rk);
+        };
+        const float dl0 = p.rmax > 0 && lane < n_items ? delta(lane) : 0.f;
 #pragma unroll 1
-        for (int it = 0; it * TW < n_items; ++it) {
-            const int item = warp + it * TW;
-            if (!own || it >= kPre) load_item(d, item, dw[0], dz[0]);
-            else if (it == 1) {
+        for (int i0 = warp; i0 < n_items; i0 += kPre * TW) {
+            if (!own || i0 != warp) {
 #pragma unroll
-                for (int i = 0; i < DCH; ++i) { dw[0][i][0] = dw[1][i][0]; dw[0][i][1] = dw[1][i][1]; }
-#pragma unroll
-                for (int b = 0; b < NBQ; ++b) { dz[0][b][0] = dz[1][b][0]; dz[0][b][1] = dz[1][b][1]; }
+                for (int v = 0; v < kPre; ++v) load_item(d, i0 + v * TW, dw[v], dz[v]);
             }
-            if (item >= n_items) break;
-            float acc_lo = 0.f, acc_hi = 0.f;
 #pragma unroll
-            for (int b = 0; b < NBQ; ++b) {
-                float c[4];
+            for (int v0 = 0; v0 < kPre; v0 += VP) {
+                float c[VP][NBQ][4];
 #pragma unroll
-                for (int u = 0; u < CPB; ++u) {
-                    const int i = b * CPB + u;
-                    uint4 hb = make_uint4(0, 0, 0, 0);
-                    if (g8 < 2) hb = s_hb[((item * DCH + i) * 2 + g8) * 4 + t4];
-                    uint32_t alo[4], ahi[4];
-                    dequant_code_word<EX>(dw[0][i][0], alo);
-                    dequant_code_word<EX>(dw[0][i][1], ahi);
-                    if (u == 0) mma16816_zero(c, alo[0], ahi[0], alo[1], ahi[1], hb.x, hb.y);
-                    else mma16816(c, alo[0], ahi[0], alo[1], ahi[1], hb.x, hb.y);
-                    mma16816(c, alo[2], ahi[2], alo[3], ahi[3], hb.z, hb.w);
+                for (int u = 0; u < CPB; ++u)
+#pragma unroll
+                    for (int b = 0; b < NBQ; ++b)
+#pragma unroll
+                        for (int v = 0; v < VP; ++v) {
+                            const int i = b * CPB + u, item = min(i0 + (v0 + v) * TW, n_items - 1);
+                            uint4 hb = make_uint4(0, 0, 0, 0);
+                            if (g8 < 2) hb = s_hb[((item * DCH + i) * 2 + g8) * 4 + t4];
+                            uint32_t alo[4], ahi[4];
+                            dequant_code_word<EX>(dw[v0 + v][i][0], alo);
+                            dequant_code_word<EX>(dw[v0 + v][i][1], ahi);
+                            if (u == 0) mma16816_zero(c[v][b], alo[0], ahi[0], alo[1], ahi[1], hb.x, hb.y);
+                            else mma16816(c[v][b], alo[0], ahi[0], alo[1], ahi[1], hb.x, hb.y);
+                            mma16816(c[v][b], alo[2], ahi[2], alo[3], ahi[3], hb.z, hb.w);
+                        }
+#pragma unroll
+                for (int v = 0; v < VP; ++v) {
+                    const int item = i0 + (v0 + v) * TW;
+                    if (t4 == 0 && item < n_items) {
+                        float acc_lo = 0.f, acc_hi = 0.f;
+#pragma unroll
+                        for (int b = 0; b < NBQ; ++b) {
+                            const __half2 z0 = u32_as_h2(dz[v0 + v][b][0]), z1 = u32_as_h2(dz[v0 + v][b][1]);
+                            const float hs = s_hsum[item * NBQ + b], hbias = EX ? 0.f : s_hbias[item * NBQ + b];
+                            acc_lo = fmaf(__low2float(z0), fmaf(-__high2float(z0), hs, EX ? c[v][b][0] + c[v][b][1] : c[v][b][0] + c[v][b][1] - hbias), acc_lo);
+                            acc_hi = fmaf(__low2float(z1), fmaf(-__high2float(z1), hs, EX ? c[v][b][2] + c[v][b][3] : c[v][b][2] + c[v][b][3] - hbias), acc_hi);
+                        }
+                        s_part[item * 17 + g8] = EX ? acc_lo * kUnscaleS : acc_lo;
+                        s_part[item * 17 + 8 + g8] = EX ? acc_hi * kUnscaleS : acc_hi;
+                    }
                 }
-                const __half2 z0 = u32_as_h2(dz[0][b][0]), z1 = u32_as_h2(dz[0][b][1]);
-                const float hs = s_hsum[item * NBQ + b], hbias = EX ? 0.f : s_hbias[item * NBQ + b];
-                acc_lo = fmaf(__low2float(z0), fmaf(-__high2float(z0), hs, EX ? c[0] + c[1] : c[0] + c[1] - hbias), acc_lo);
-                acc_hi = fmaf(__low2float(z1), fmaf(-__high2float(z1), hs, EX ? c[2] + c[3] : c[2] + c[3] - hbias), acc_hi);
-            }
-            if (t4 == 0) {
-                s_part[item * 17 + g8] = EX ? acc_lo * kUnscaleS : acc_lo;
-                s_part[item * 17 + 8 + g8] = EX ? acc_hi * kUnscaleS : acc_hi;
             }
         }
         __syncthreads();
         // warp w: row w; lane: (expert, quarter).  Adapter delta, gate weight, then the sum in order.
         float yv = 0.f;
         for (int b0 = 0; b0 < n_items; b0 += 32) {
-            const int item = b0 + lane, k = item >> 2;
+            const int item = b0 + lane;
             float o = 0.f;
-            if (item < n_items && s_slot[k] >= 0) {
-                const int rk = k >= p.K ? p.rank_shared : p.rank, set = k >= p.K ? sets : (p.n_adapters == 1 ? 0 : k);
-                const float dl = b_dot(reinterpret_cast<const uint16_t*>(smem + S.bd) + (size_t)set * 16 * p.rmax + warp * rk, s_udi + item * (p.rmax + 1), rk);
-                o = s_gate[k] * fmaf(p.sigma, dl, s_part[item * 17 + warp]);
-            }
+            if (item < n_items && s_slot[item >> 2] >= 0) o = s_gate[item >> 2] * fmaf(p.sigma, b0 == 0 ? dl0 : delta(item), s_part[item * 17 + warp]);
             const int n = min(32, n_items - b0);
 #pragma unroll 8
             for (int i = 0; i < n; ++i) yv += __shfl_sync(0xFFFFFFFFu, o, i);
         }
+        const int row = d * 16 + warp;
+        if (p.x_next != nullptr && lane < kStateCopies)
+            st_relaxed_gpu_u32(p.vx + (size_t)(epoch % kStepStates * kStateCopies + lane) * H + row,
+                               __float_as_uint(bf16_bits_to_float(s_x[row]) + round_as(yv, p.out_dtype)));
         if (lane == 0) {
-            const int row = d * 16 + warp;
             if (p.out_dtype == EDG_F32) store_out<float>(static_cast<float*>(p.y), row, yv);
             else if (p.out_dtype == EDG_F16) store_out<__half>(static_cast<__half*>(p.y), row, yv);
             else store_out<bf16_t>(static_cast<bf16_t*>(p.y), row, yv);
-            if (p.x_next != nullptr)
-                st_relaxed_gpu_u32(p.vx + (size_t)(epoch % kStepStates) * H + row, __float_as_uint(bf16_bits_to_float(s_x[row]) + round_as(yv, p.out_dtype)));
         }
         __syncthreads();
         return true;
@@ -740,7 +736,7 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         bool give_up = false, got = !on;
         for (uint32_t it = 0; !got && !give_up; ++it) {
-            const uint4 w = ld_relaxed16(p.vx + (size_t)(epoch % kStepStates) * H + 4 * tid);
+            const uint4 w = ld_relaxed16(p.vx + (size_t)(epoch % kStepStates * kStateCopies + cta % kStateCopies) * H + 4 * tid);
             got = there(w);
             v = make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
             if (!got) { __nanosleep(32); tired(it, give_up, got); }
@@ -755,16 +751,67 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         __syncthreads();
         return true;
     };
-    // A CTA's own unit (its rows, or the caller's x_next: unit n_dn); then, if it is the one that started last, what others have left to
+    // the routing of the next step, by one warp, as soon as all logits are there
+    auto route = [&]() -> bool {
+        bool give_up = false;
+        if (warp == 0) {
+            float* work = reinterpret_cast<float*>(un);
+            float* slot = p.logits_ws + (size_t)max(p.flag_out, 0) * (p.E + kPairWords);
+            unsigned long long* pr = reinterpret_cast<unsigned long long*>(slot + p.E) + lane;
+            unsigned long long was = ~0ull;
+            if (p.flag_out >= 0 && lane < p.K) was = ld_relaxed_gpu_u64(pr);
+#pragma unroll 1
+            for (int i0 = 0; i0 < p.E && !give_up; i0 += 256) {          // 8 independent loads per lane and pass
+                uint32_t v[8];
+                bool got = false;
+                for (uint32_t it = 0; !got && !give_up; ++it) {
+                    bool all = true;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int i = i0 + u * 32 + lane;
+                        v[u] = i < p.E ? ld_relaxed_gpu_u32(hx + p.lx_off + i) : 0u;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) all = all && v[u] != kNotYet;
+                    got = __all_sync(0xFFFFFFFFu, all);
+                    if (!got) tired(it, give_up, got);
+                    give_up = __any_sync(0xFFFFFFFFu, give_up);
+                    got = __all_sync(0xFFFFFFFFu, got);
+                }
+                if (give_up) break;
+                // the step that last read this slot of the ring has reset it
+                for (uint32_t it = 0; was != ~0ull && it < kSpinLimit; ++it) was = ld_relaxed_gpu_u64(pr);
+                if (was != ~0ull) atomicExch(p.status, EDG_E_TIMEOUT);
+                __syncwarp();
+                // (the logits move on into the ring slot, beside the routing made of them)
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int i = i0 + u * 32 + lane;
+                    if (i < p.E) {
+                        work[i] = __uint_as_float(v[u]);
+                        if (p.flag_out >= 0) st_relaxed_gpu_u32(slot + i, v[u]);
+                        st_relaxed_gpu_u32(hx + p.lx_off + i, kNotYet);
+                        if (p.logits_next != nullptr) p.logits_next[i] = __uint_as_float(v[u]);
+                    }
+                }
+            }
+            if (!give_up) {
+                emit_routing<false>(p, work, lane, p.flag_out >= 0 ? pr : nullptr);
+            }
+        }
+        return !__syncthreads_or(give_up);
+    };
+    // A CTA's own units (its rows, or the routing: n_dn + 1, and the caller's x_next: n_dn); then, if it is the one that started last, what others have left to
     // it.  An entry of the list is claimed by an atomic: by the last starter, or by the one that left it, if it finds
     // afterwards that the last one has started -- then nothing stands in the way of waiting any more.
-    int32_t* defer = p.defer + (size_t)(epoch % kStepStates) * (p.n_dn + 2);
-    int unit = finisher ? p.n_dn : (has_dn ? cta : -1), left = -1, next = 0;
+    int32_t* defer = p.defer + (size_t)(epoch % kStepStates) * (p.n_dn + 4);
+    int unit = has_dn ? cta : (cta == p.cta_route ? p.n_dn + 1 : (cta == p.cta_state ? p.n_dn : -1)), left = -1, next = 0;
+    int then = cta == p.cta_route && cta == p.cta_state ? p.n_dn : -1;
     bool own = true;
 #pragma unroll 1
     for (;;) {
         if (unit >= 0) {
-            if (!(unit == p.n_dn ? finish_state() : down_unit(unit, own))) {
+            if (!(unit < p.n_dn ? down_unit(unit, own) : (unit == p.n_dn ? finish_state() : route()))) {
                 if (tid == 0) {
                     const int at = atomicAdd(defer, 1);
                     atomicExch(defer + 1 + at, unit + 1);
@@ -779,9 +826,10 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
             }
             own = false;
         }
+        if (then >= 0) { unit = then; then = -1; continue; }
         if (!s_misc[1]) break;                                           // (uniform: written before the first barrier)
         if (left < 0) {
-            if (tid == 0) { __threadfence(); s_misc[2] = min(ld_relaxed_gpu(defer), p.n_dn + 1); }
+            if (tid == 0) { __threadfence(); s_misc[2] = min(ld_relaxed_gpu(defer), p.n_dn + 2); }
             __syncthreads();
             left = s_misc[2];
             __syncthreads();
@@ -810,14 +858,16 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
             __syncthreads();
             for (int i = tid; i < p.E; i += TThreads) st_relaxed_gpu_u32(slot + i, kNotYet);
         }
-        if (cta == 0) pdl_wait_prior_grid();
+        // No CTA leaves before the kernel before this one has: the CTAs of the next one but one take over from that kernel, one on
+        // every SM, before an SM can offer them two places.
+        pdl_wait_prior_grid();
     }
 }
 
 StepSmem step_smem(const edg_layer_desc& d, int Kt, int rmax) {
     StepSmem S;
     const uint32_t NCK = d.H / 512, TG = d.I / 256, NT = 2 * TG, RG = 16 * TG, sets = (d.n_adapters == 1 ? 1 : d.K) + 1;
-    const uint32_t gpw = NCK * 32 / d.group > 0 ? NCK * 32 / d.group : 1, hw = Kt * d.I, items = Kt * 4;
+    const uint32_t hw = Kt * d.I, items = Kt * 4;
     auto up16 = [](uint32_t v) { return (v + 15) / 16 * 16; };
     S.h = 0;
     S.hb = up16(hw / 32 * 36 * 4);                                       // (blocks of 32 or more values, four words of padding each)
@@ -826,15 +876,14 @@ StepSmem step_smem(const edg_layer_desc& d, int Kt, int rmax) {
     S.part = up16(S.hbias + hw / 32 * 4);
     S.udi = up16(S.part + items * 17 * 4);
     uint32_t un = up16(S.udi + items * (rmax + 1) * 4);
-    S.codes_warp = NT * NCK * 256;
     auto at_least = [&](uint32_t v) { if (un < v) un = up16(v); };
-    at_least(TW * S.codes_warp);
+    at_least(NT * NCK * TW * 256);
     if (d.pre_dtype == EDG_F16) at_least(16u * (d.H * 2 + 16));          // a tile of the head
     at_least((uint32_t)d.E * 4 + 256);
     S.un = 0;
     uint32_t o = un;
-    S.sz_warp = NT * gpw * 64;
-    S.sz = o;        o += TW * S.sz_warp;
+    S.sz_tile = d.H / d.group * 64;
+    S.sz = o;        o += NT * S.sz_tile;
     S.xb = o;        o += d.H * 2;
     S.x = o;         o += d.H * 2;
     S.xsum = o;      o += d.H / 32 * 4;
@@ -847,6 +896,7 @@ StepSmem step_smem(const edg_layer_desc& d, int Kt, int rmax) {
     S.hl = o;        o += 32 * 4;
     S.sel = o;       o += 64 * 4;
     S.red = o;       o += 64 * 4;
+    S.bar = o;       o += 16;
     S.total = o;
     return S;
 }
@@ -894,10 +944,10 @@ bool step_supported(const edg_layer_desc& d, bool shared) {
 }
 
 size_t step_exchange_words(const edg_layer_desc& d) {
-    const size_t sets = (d.n_adapters == 1 ? 1 : d.K) + 1;               // h, A_down h, A x
-    return ((size_t)(d.K + 1) * d.I + (size_t)16 * (d.K + 1) * d.rank + sets * 8 * d.rank + 63) / 64 * 64;
+    const size_t sets = (d.n_adapters == 1 ? 1 : d.K) + 1;               // h, A_down h, A x, logits
+    return ((size_t)(d.K + 1) * d.I + (size_t)16 * (d.K + 1) * d.rank + sets * 8 * d.rank + d.E + 63) / 64 * 64;
 }
-size_t step_region_words(const edg_layer_desc& d) { return kStepBufs * step_exchange_words(d) + (size_t)kStepStates * d.H; }
+size_t step_region_words(const edg_layer_desc& d) { return kStepBufs * step_exchange_words(d) + (size_t)kStepStates * kStateCopies * d.H; }
 
 int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* slots, const int32_t* table, const int32_t* experts,
                  const float* gates, const void* x, const edg_lora* lora, void* y, const void* W_pre, int32_t* inds_next, float* gates_next,
@@ -932,6 +982,7 @@ int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* 
     p.hx_words = (uint32_t)step_exchange_words(*d);
     p.ud_off = (uint32_t)(d->K + 1) * d->I;
     p.ux_off = p.ud_off + 16u * (d->K + 1) * d->rank;
+    p.lx_off = p.ux_off + ((d->n_adapters == 1 ? 1u : (uint32_t)d->K) + 1u) * 8u * d->rank;
     p.vx = p.hx + (size_t)kStepBufs * p.hx_words;
     p.I = d->I; p.E = d->E; p.group = d->group;
     while ((1 << p.gshift) < d->group) ++p.gshift;
@@ -946,7 +997,9 @@ int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* 
     const int n_sm = sm_count(), spare = n_sm - p.n_exp;
     p.n_headc = spare > 0 && p.n_head > spare ? spare : p.n_head;
     const int extra = max(p.n_headc, p.x_next != nullptr ? 1 : 0);       // (somebody has to write x_next)
-    const int grid = max(n_sm, p.n_exp + extra);
+    const int grid = max(n_sm, p.n_exp + extra), idle = p.n_exp + p.n_headc;
+    p.cta_route = W_pre == nullptr ? -1 : (idle < grid ? idle : idle - 1);
+    p.cta_state = p.x_next == nullptr ? -1 : (W_pre == nullptr ? p.n_exp : (idle + 1 < grid ? idle + 1 : p.n_exp));
     p.flag_in = flag_in; p.flag_out = W_pre != nullptr ? flag_out : -1; p.stale = stale;
     p.dep = flag_in >= 0 && ex.dep_wait >= 0;
     p.S = step_smem(*d, p.Kt, p.rmax);
