@@ -16,20 +16,59 @@ __device__ __forceinline__ void trace_stamp(const P& p, int m) {
     }
 }
 
-static __device__ __noinline__ void topk_large(float* work, int E, int K, int lane, int32_t* inds, float* gates) {
+static __device__ __noinline__ void topk_any(float* work, int E, int K, int lane, int32_t* inds, float* gates) {
     warp_softmax_topk(work, E, K, lane, inds, gates);
+}
+
+// The usual case of warp_softmax_topk_reg, E <= 256: a logit for every choice and no two of the chosen equal.  False: it is
+// not this case, nothing useful has been written.  A round takes the largest key of the warp and strikes it from the lane that
+// held it -- no sorted lists, nothing to shuffle in between.
+__device__ __forceinline__ bool topk_distinct(const float* work, int E, int K, int lane, int32_t* inds, float* gates) {
+    const unsigned full = 0xFFFFFFFFu;
+    uint32_t key[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int e = u * 32 + lane;
+        const float v = e < E ? work[e] : __int_as_float(0x7fffffff);
+        key[u] = (v == v) ? float_key(v) : 0u;
+    }
+    float myv = 0.f;
+    bool fine = true;
+#pragma unroll 1
+    for (int j = 0; j < K; ++j) {
+        const uint32_t best = __reduce_max_sync(full, max(max(max(key[0], key[1]), max(key[2], key[3])), max(max(key[4], key[5]), max(key[6], key[7]))));
+        int hits = 0, at = 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (key[u] == best) { ++hits; at = u; key[u] = 0u; }
+        const unsigned who = __ballot_sync(full, hits > 0);
+        fine = fine && best != 0u && hits <= 1 && (who & (who - 1)) == 0u;
+        if (hits) inds[j] = at * 32 + lane;
+        if (lane == j) myv = key_float(best);
+    }
+    if (!__all_sync(full, fine)) return false;
+    __syncwarp();
+    const int myi = lane < K ? inds[lane] : 0x7FFFFFFF;
+    const float m = __shfl_sync(full, myv, 0);
+    const float ex = lane < K ? expf(myv - m) : 0.f;
+    const float sum = warp_sum(ex);
+    int rank = 0;
+#pragma unroll 8
+    for (int i = 0; i < K; ++i) rank += __shfl_sync(full, myi, i) < myi ? 1 : 0;
+    __syncwarp();
+    if (lane < K) { inds[rank] = myi; gates[rank] = ex / sum; }
+    return true;
 }
 
 // The top-k of the logits in `work` by one warp, into the caller's inds_next / gates_next and, first, as one (expert, gate) word per
 // choice into `pair` (this lane's word of the ring slot, or null), where a chained next step picks them up.  FENCE: what the
 // publishers of the logits had observed travels on with them.  `work`: E floats and 256 bytes for the winners.
 template <bool FENCE, typename P>
-__device__ __noinline__ void emit_routing(const P& p, float* work, int lane, unsigned long long* pair) {
+__device__ __forceinline__ void emit_routing(const P& p, float* work, int lane, unsigned long long* pair) {
     __syncwarp();
     int32_t* s_i = reinterpret_cast<int32_t*>(work) + p.E;        // [K] winners, then [K] gates
     float* s_g = reinterpret_cast<float*>(s_i + 32);
-    if (p.E <= 256) warp_softmax_topk_reg<8>(work, p.E, p.K, lane, s_i, s_g);
-    else topk_large(work, p.E, p.K, lane, s_i, s_g);
+    if (p.E > 256 || !topk_distinct(work, p.E, p.K, lane, s_i, s_g)) topk_any(work, p.E, p.K, lane, s_i, s_g);
     __syncwarp();
     if (lane == 0) trace_stamp(p, 25);
     if (lane < p.K) {

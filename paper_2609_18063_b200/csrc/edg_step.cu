@@ -3,23 +3,29 @@
 //
 // What bounds it is not the 15 MB it streams (2.4 us) but the chain of trips -- routing -> table -> weights -> h -> other
 // CTAs -> y -- and the instructions between them.  So everything that does not depend on a trip is under way before it: a CTA
-// issues all its gate/up weights at once (72 KB, 16-byte asynchronous copies into shared memory by the lanes of the warp that
-// will use them), announces its down weights to the L2, and loads its adapter rows; sixteen warps share the arithmetic.
+// issues all its gate/up weights at once (72 KB in eight bulk copies, by the warp that learns the routing; as 16-byte copies of
+// all warps the issue alone took 2 us), announces its down weights to the L2, and loads its adapter rows; sixteen warps share
+// the arithmetic.
 //   * Gate/up: expert CTA 16 k + 4 c + j computes rows c I/4 + j I/16 .. of gate and up of routed expert k over all of
 //     K = H.  Warp w multiplies H/512 chunks (32 codes each) of every row tile on mma.sync fragments.
 //   * h, and the partial A_down h, go to all CTAs through global memory, in band: a word that does not hold the
 //     "not yet" pattern (a NaN no arithmetic produces) is valid by itself, so the exchange costs one store and
-//     one load on the way, and no barrier.  The rank-r projections A x are shared by all CTAs of the grid in the same way.
+//     one load on the way, and no barrier.  Four copies: 128 readers of the same lines queue at their slice of the L2.  The
+//     rank-r projections A x are shared by all CTAs of the grid in the same way, those without expert work first; so are the
+//     head's logits, which one warp turns into the next routing (a counter of arrivals with its fences took 10 us from x to
+//     the routing, most of a step; now 7 us).
 //   * Down: CTA d computes output rows 16 d .. 16 d + 15 over the h of ALL experts, so y needs no second pass over partials
 //     (the throughput form writes 32 partial rows per output, counts arrivals and lets four CTAs sum them).
 //   * Head rows have CTAs of their own, among those that the experts leave of one per SM.
 //   * A dependent chain hands x + y on, unnormalised, in band as well: every CTA of the next step, resident and
-//     with its weights in shared memory by then, polls it, forms the norm and its bf16 state by itself.  A CTA without expert
-//     work writes the caller's x_next meanwhile.
+//     with its weights in shared memory by then, polls it, forms the norm and its bf16 state by itself.  Eight copies: 148
+//     pollers of the same lines held the writes up by 2-4 us.  A CTA without expert work writes the caller's x_next meanwhile.
 // Two launches of this form fit an SM side by side (64 registers x 512 threads, under 113 KB of shared memory).
 //
 // Measured (H 2048, I 512, E 256, K 8, groups of 64, rank 16; the four-CTA clusters per expert quarter it replaces first): a link of
-// a chain 20.4 -> 14.9 us, a step alone 24 -> 15 us (12 layers of K = 4 through the resident stack, host loop included: 295 -> 177 us).
+// a chain 20.4 -> 11.8 us, a step alone 24 -> 13 us (12 layers of K = 4 through the resident stack, host loop included: 295 -> 155 us).
+// Of the 11.8 us the two exchanges take 5.5 (a store, a poll under way, a poll that sees it, the slowest of 128), the
+// arithmetic of gate/up 1.7, of down 1.5.
 //
 // Waiting is safe without a cooperative launch: a CTA may wait for the h of others only when all CTAs of its grid have
 // started (a counter says so; it is also the epoch that names the exchange buffers).  One that finds
@@ -40,7 +46,7 @@ constexpr int kStepMaxK = 16;
 constexpr int kStepMaxRank = 64;
 constexpr uint32_t kEpochStarts = 8192;       // what one grid adds to the start counter in total
 constexpr uint32_t kWaitStarted = 256;        // polls before a CTA whose grid is not fully resident gives its rows away
-constexpr int kStepBufs = 4, kStateCopies = 8;
+constexpr int kStepBufs = 4, kStateCopies = 8, kHCopies = 4;
 
 // byte offsets in shared memory; h .. udi lie inside the union, used once the gate/up weights are
 struct StepSmem {
@@ -66,13 +72,13 @@ struct StepParams {
     uint16_t* x_next;
     unsigned long long* trace;                // (this form is not traced: null)
     uint32_t* starts;                         // the start counter
-    float* hx;                                // [kStepBufs][hx_words]: h; the A_down h partials of every expert CTA; the A x partials; head logits
+    float* hx;                                // [kStepBufs][hx_words]: kHCopies of (h; the A_down h partials of every expert CTA); the A x partials; head logits
     float* vx;                                // [kStepStates][kStateCopies][H]: x + y of a dependent chain
     int32_t* defer;                           // [kStepStates][H/16 + 4]: number, then (unit + 1) of those left to the last starter
-    uint32_t hx_words, ud_off, ux_off, lx_off;
+    uint32_t hx_words, hc_words, ud_off, ux_off, lx_off;
     int I, E, K, Kt, group, gshift, rank, rank_shared, rmax, n_adapters, n_slots, pre_dtype, out_dtype;
     int cta_route, cta_state;                 // CTAs that compute the routing for the next step and the caller's x_next, or -1
-    int n_gu, n_dn, n_exp, n_head, n_headc;   // CTAs with gate/up, with down work, the larger of both; tiles of 16 head rows, CTAs for them
+    int n_gu, n_dn, n_exp, n_head, n_headc;   // CTAs with gate/up, with down work, the larger of both; tiles of the head, CTAs for them
     int flag_in, flag_out, stale, dep;        // dep: x arrives in band from the step before
     float sigma, eps;
     RecordLayout L;
@@ -88,6 +94,9 @@ __device__ __forceinline__ uint4 ld_relaxed16(const void* p) {
     uint4 v;
     asm volatile("ld.relaxed.gpu.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
     return v;
+}
+__device__ __forceinline__ void st_relaxed16(void* p, uint4 v) {
+    asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 __device__ __forceinline__ bool there(uint4 v) { return v.x != kNotYet && v.y != kNotYet && v.z != kNotYet && v.w != kNotYet; }
 __device__ __forceinline__ float round_as(float v, int out_dtype) {      // a value as it reads back from the output type
@@ -135,6 +144,28 @@ __device__ __forceinline__ float inv_rms(float* s_red, float4 v, bool on, int H,
         all += tot;
     }
     return rsqrtf(all / (float)H + eps);
+}
+
+// 16 head rows (in shared memory, row by row with 16 bytes of padding) as the M of the MMA, the state as column 0, a quarter of K
+// per warp of four; part [16] receives this warp's sums.
+template <int H>
+__device__ __forceinline__ void head_rows(const uint8_t* rows, const uint16_t* x, float* part, int warp, int lane) {
+    const int g8 = lane >> 2, t4 = lane & 3;
+    float c[4] = {0.f, 0.f, 0.f, 0.f};
+    const uint8_t* wr = rows + g8 * (H * 2 + 16) + warp * (H / 2) + t4 * 16;
+#pragma unroll 8
+    for (int j = 0; j < H / 128; ++j) {
+        const uint4 a = *reinterpret_cast<const uint4*>(wr + j * 64), b = *reinterpret_cast<const uint4*>(wr + 8 * (H * 2 + 16) + j * 64);
+        uint4 xb = make_uint4(0, 0, 0, 0);
+        if (g8 == 0) {
+            const uint4 v = *reinterpret_cast<const uint4*>(x + warp * (H / 4) + j * 32 + t4 * 8);
+            xb = make_uint4(h2_as_u32(__floats2half2_rn(bf16_lo(v.x), bf16_hi(v.x))), h2_as_u32(__floats2half2_rn(bf16_lo(v.y), bf16_hi(v.y))),
+                            h2_as_u32(__floats2half2_rn(bf16_lo(v.z), bf16_hi(v.z))), h2_as_u32(__floats2half2_rn(bf16_lo(v.w), bf16_hi(v.w))));
+        }
+        mma16816(c, a.x, b.x, a.y, b.y, xb.x, xb.y);
+        mma16816(c, a.z, b.z, a.w, b.w, xb.z, xb.w);
+    }
+    if (t4 == 0) { part[g8] = c[0]; part[8 + g8] = c[2]; }
 }
 
 // NCK = H / 512: chunks of 32 codes per warp; DCH = I / 128: chunks of a quarter of I; CPB: chunks per scaled block; EX: code arithmetic.
@@ -210,12 +241,12 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         take_x(i, v);
     }
     const bool head_mma = p.pre_dtype == EDG_F16 && p.E % 16 == 0;
-    auto load_head = [&](int tile) {                                     // row by row, padded by 16 bytes against bank conflicts
+    auto load_head = [&](int tile, int threads) {                        // row by row, padded by 16 bytes against bank conflicts
         const uint8_t* src = static_cast<const uint8_t*>(p.W_pre) + (size_t)tile * 16 * H * 2;
 #pragma unroll 4
-        for (int i = tid; i < 16 * (H / 8); i += TThreads) cp16(un + (i / (H / 8)) * (H * 2 + 16) + (i % (H / 8)) * 16, src + (size_t)i * 16);
+        for (int i = tid; i < 16 * (H / 8); i += threads) cp16(un + (i / (H / 8)) * (H * 2 + 16) + (i % (H / 8)) * 16, src + (size_t)i * 16);
     };
-    if (has_head && head_mma) load_head(cta - p.n_exp);
+    if (has_head && head_mma) load_head(cta - p.n_exp, TThreads);
     if (p.stale >= 0 && cta == 0)
         for (int i = tid; i < p.E + kPairWords; i += TThreads) st_relaxed_gpu_u32(&p.logits_ws[(size_t)p.stale * (p.E + kPairWords) + i], kNotYet);
 
@@ -346,8 +377,8 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         __syncthreads();
     }
     if (p.dep && tid < H / 8) take_x(tid, *reinterpret_cast<const uint4*>(s_x + tid * 8));
-    if (p.dep) __syncthreads();
-    float* hx = p.hx + (size_t)(epoch % kStepBufs) * p.hx_words;
+    if (has_head) cp_wait<0>();
+    if (p.dep || has_head) __syncthreads();
     auto all_started = [&]() {
         uint32_t c;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(p.starts) : "memory");
@@ -358,6 +389,66 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         if ((it % kWaitStarted) == kWaitStarted - 1 && !all_started()) give_up = true;
         if (it >= kSpinLimit) { atomicExch(p.status, EDG_E_TIMEOUT); got = true; }
     };
+    float* hx = p.hx + (size_t)(epoch % kStepBufs) * p.hx_words;
+    // ---- the head's rows.  Four warps take tiles of 16 through the tensor cores; any other head goes in tiles of four, a row in four tasks
+    if (has_head && head_mma && warp < 4) {
+#pragma unroll 1
+        for (int tile = cta - p.n_exp; tile < p.n_head; tile += p.n_headc) {
+            if (tile >= p.n_headc) {                                     // (the first tile has been on its way since the start)
+                load_head(tile, 128);
+                cp_commit();
+                cp_wait<0>();
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+            }
+            head_rows<H>(un, s_x, s_red + warp * 16, warp, lane);
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            if (tid < 16) {
+                float lg = s_red[tid];
+                for (int w = 1; w < 4; ++w) lg += s_red[w * 16 + tid];   // fixed order
+                st_relaxed_gpu_u32(hx + p.lx_off + tile * 16 + tid, __float_as_uint(lg));
+            }
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+        }
+    } else if (has_head && !head_mma) {
+#pragma unroll 1
+        for (int tile = cta - p.n_exp; tile < p.n_head; tile += p.n_headc) {
+            const int e = tile * 4 + (warp >> 2), part = (warp & 3) * 32 + lane;
+            float acc = 0.f;
+            if (e < p.E && p.pre_dtype == EDG_F16) {
+                const __half* wr = static_cast<const __half*>(p.W_pre) + (size_t)e * H;
+                for (int c = part * 8; c < H; c += 1024) {
+                    const uint4 w = ld_keep16(wr + c);
+                    const uint4 xv = *reinterpret_cast<const uint4*>(s_x + c);
+                    const float2 a = __half22float2(u32_as_h2(w.x)), b = __half22float2(u32_as_h2(w.y));
+                    const float2 d = __half22float2(u32_as_h2(w.z)), f = __half22float2(u32_as_h2(w.w));
+                    acc = fmaf(a.x, bf16_lo(xv.x), acc); acc = fmaf(a.y, bf16_hi(xv.x), acc);
+                    acc = fmaf(b.x, bf16_lo(xv.y), acc); acc = fmaf(b.y, bf16_hi(xv.y), acc);
+                    acc = fmaf(d.x, bf16_lo(xv.z), acc); acc = fmaf(d.y, bf16_hi(xv.z), acc);
+                    acc = fmaf(f.x, bf16_lo(xv.w), acc); acc = fmaf(f.y, bf16_hi(xv.w), acc);
+                }
+            } else if (e < p.E) {
+                const float* wr = static_cast<const float*>(p.W_pre) + (size_t)e * H + part * 4;
+                uint4 w[NCK];
+#pragma unroll
+                for (int j = 0; j < NCK; ++j) w[j] = ld_keep16(wr + j * 512);
+#pragma unroll
+                for (int j = 0; j < NCK; ++j) {
+                    const uint2 xv = *reinterpret_cast<const uint2*>(s_x + part * 4 + j * 512);
+                    acc = fmaf(__uint_as_float(w[j].x), bf16_lo(xv.x), acc); acc = fmaf(__uint_as_float(w[j].y), bf16_hi(xv.x), acc);
+                    acc = fmaf(__uint_as_float(w[j].z), bf16_lo(xv.y), acc); acc = fmaf(__uint_as_float(w[j].w), bf16_hi(xv.y), acc);
+                }
+            }
+            acc = warp_sum(acc);
+            __syncthreads();                                             // (the sums of the tile before have been read)
+            if (lane == 0) s_red[warp] = acc;
+            __syncthreads();
+            if (tid < 4 && tile * 4 + tid < p.E) {
+                float lg = 0.f;
+                for (int w = 0; w < 4; ++w) lg += s_red[tid * 4 + w];
+                st_relaxed_gpu_u32(hx + p.lx_off + tile * 4 + tid, __float_as_uint(lg));
+            }
+        }
+    }
     // ---- this warp's share of A x
     auto a_dot = [&](int set, int q, bool first) {
         float v = 0.f;
@@ -472,12 +563,13 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
                 v = fmaf(p.sigma, b_dot(reinterpret_cast<const uint16_t*>(smem + S.bgu) + (m * RG + i) * r, s_uf + m * r, r), v);
             const float up = __shfl_down_sync(0xFFFFFFFFu, v, 4);
             if ((tid & 7) == 0) {
-                const float h = valid ? silu_f(v) * up : 0.f;
-                s_hl[i] = h;
-                st_relaxed_gpu_u32(hx + (size_t)kpos * p.I + n0 + i, __float_as_uint(h));
+                s_hl[i] = valid ? silu_f(v) * up : 0.f;
             }
         }
         __syncthreads();
+        if (warp == TW - 1)                                              // h goes out, 16 bytes and a copy per lane
+            for (int i = lane; i < kHCopies * RG / 4; i += 32)
+                st_relaxed16(hx + (size_t)(i / (RG / 4)) * p.hc_words + (size_t)kpos * p.I + n0 + i % (RG / 4) * 4, reinterpret_cast<const uint4*>(s_hl)[i % (RG / 4)]);
         if (r > 0 && warp * 8 < r) {                                     // partial of A_down h over this CTA's rows, four lanes per rank
             const uint16_t* A = reinterpret_cast<const uint16_t*>(smem + S.ad);
             const int j = tid >> 2, part = tid & 3;                      // (TThreads / 4 ranks in one go: kStepMaxRank and more)
@@ -485,7 +577,8 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
             if (j < r && valid)
                 for (int n = part; n < RG; n += 4) u = fmaf(bf16_bits_to_float(A[j * RG + n]), s_hl[n], u);
             u = group_sum<4>(u);
-            if (j < r && part == 0) st_relaxed_gpu_u32(hx + p.ud_off + (size_t)cta * p.rmax + j, __float_as_uint(u));
+            static_assert(kHCopies == 4, "a copy per lane of the group");
+            if (j < r) st_relaxed_gpu_u32(hx + (size_t)part * p.hc_words + p.ud_off + (size_t)cta * p.rmax + j, __float_as_uint(u));
         }
     }
 
@@ -512,93 +605,21 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         for (int u = 0; u < kPre; ++u) load_item(cta, warp + u * TW, dw[u], dz[u]);
     }
 
-    // (every CTA of the step before has used its exchange buffers up: they are cleared for the step three epochs on)
-    {
+    constexpr int kHPad = 32 * CPB + 4;                                  // (a block of h, padded against bank conflicts)
+    // Every CTA of the step before has used its exchange buffers up: they are cleared for the step three epochs on, which cannot start
+    // before this kernel has ended (two CTAs fit an SM, a grid has one for every SM at least, and none leaves before the kernel
+    // before its own).  By the CTAs without expert work, if there are any.
+    if (cta >= p.n_exp || (int)gridDim.x == p.n_exp) {
         float* hc = p.hx + (size_t)((epoch + kStepBufs - 1) % kStepBufs) * p.hx_words;
         float* vc = p.vx + (size_t)((epoch + kStepStates / 2) % kStepStates) * kStateCopies * H;
-        const uint32_t all = gridDim.x * TThreads;
-        for (uint32_t i = tid * gridDim.x + cta; i < p.hx_words; i += all) st_relaxed_gpu_u32(hc + i, kNotYet);
-        for (uint32_t i = tid * gridDim.x + cta; i < (uint32_t)H * kStateCopies; i += all) st_relaxed_gpu_u32(vc + i, kNotYet);
-        if (cta == 0 && tid == 0) st_relaxed_gpu(p.defer + (size_t)((epoch + kStepStates / 2) % kStepStates) * (p.n_dn + 4), 0);
-    }
-    // ---- the head's rows, in tiles of 16
-    if (has_head) {
-#pragma unroll 1
-        for (int tile = cta - p.n_exp; tile < p.n_head; tile += p.n_headc) {
-            const int e0 = tile * 16;
-            const bool own = warp == 0 && lane < 16 && e0 + lane < p.E;
-            float lg = 0.f;
-            if (tile >= p.n_headc) {                                     // (the first tile has been on its way since the start)
-                __syncthreads();
-                if (head_mma) { load_head(tile); cp_commit(); cp_wait<0>(); }
-                __syncthreads();
-            }
-            if (head_mma) {
-                // 16 rows as the M of the MMA, x as column 0, four warps with a quarter of K each
-                if (warp < 4) {
-                    float c[4] = {0.f, 0.f, 0.f, 0.f};
-                    const uint8_t* wr = un + g8 * (H * 2 + 16) + warp * (H / 2) + t4 * 16;
-#pragma unroll 4
-                    for (int j = 0; j < H / 128; ++j) {
-                        const uint4 a = *reinterpret_cast<const uint4*>(wr + j * 64), b = *reinterpret_cast<const uint4*>(wr + 8 * (H * 2 + 16) + j * 64);
-                        uint4 xb = make_uint4(0, 0, 0, 0);
-                        if (g8 == 0) {
-                            const uint4 v = *reinterpret_cast<const uint4*>(s_x + warp * (H / 4) + j * 32 + t4 * 8);
-                            xb = make_uint4(h2_as_u32(__floats2half2_rn(bf16_lo(v.x), bf16_hi(v.x))), h2_as_u32(__floats2half2_rn(bf16_lo(v.y), bf16_hi(v.y))),
-                                            h2_as_u32(__floats2half2_rn(bf16_lo(v.z), bf16_hi(v.z))), h2_as_u32(__floats2half2_rn(bf16_lo(v.w), bf16_hi(v.w))));
-                        }
-                        mma16816(c, a.x, b.x, a.y, b.y, xb.x, xb.y);
-                        mma16816(c, a.z, b.z, a.w, b.w, xb.z, xb.w);
-                    }
-                    if (t4 == 0) { s_red[warp * 16 + g8] = c[0]; s_red[warp * 16 + 8 + g8] = c[2]; }
-                }
-                __syncthreads();
-                if (own) {
-                    lg = s_red[lane];
-                    for (int w = 1; w < 4; ++w) lg += s_red[w * 16 + lane];      // fixed order
-                }
-            } else {
-                // any other head: a row in four tasks
-#pragma unroll 1
-                for (int task = warp; task < 64; task += TW) {
-                    const int e = e0 + (task >> 2);
-                    float acc = 0.f;
-                    if (e < p.E && p.pre_dtype == EDG_F16) {
-                        const __half* wr = static_cast<const __half*>(p.W_pre) + (size_t)e * H;
-                        for (int c = ((task & 3) * 32 + lane) * 8; c < H; c += 1024) {
-                            const uint4 w = ld_keep16(wr + c);
-                            const uint4 xv = *reinterpret_cast<const uint4*>(s_x + c);
-                            const float2 a = __half22float2(u32_as_h2(w.x)), b = __half22float2(u32_as_h2(w.y));
-                            const float2 d = __half22float2(u32_as_h2(w.z)), f = __half22float2(u32_as_h2(w.w));
-                            acc = fmaf(a.x, bf16_lo(xv.x), acc); acc = fmaf(a.y, bf16_hi(xv.x), acc);
-                            acc = fmaf(b.x, bf16_lo(xv.y), acc); acc = fmaf(b.y, bf16_hi(xv.y), acc);
-                            acc = fmaf(d.x, bf16_lo(xv.z), acc); acc = fmaf(d.y, bf16_hi(xv.z), acc);
-                            acc = fmaf(f.x, bf16_lo(xv.w), acc); acc = fmaf(f.y, bf16_hi(xv.w), acc);
-                        }
-                    } else if (e < p.E) {
-                        const float* wr = static_cast<const float*>(p.W_pre) + (size_t)e * H + ((task & 3) * 32 + lane) * 4;
-                        uint4 w[NCK];
-#pragma unroll
-                        for (int j = 0; j < NCK; ++j) w[j] = ld_keep16(wr + j * 512);
-#pragma unroll
-                        for (int j = 0; j < NCK; ++j) {
-                            const uint2 xv = *reinterpret_cast<const uint2*>(s_x + ((task & 3) * 32 + lane) * 4 + j * 512);
-                            acc = fmaf(__uint_as_float(w[j].x), bf16_lo(xv.x), acc); acc = fmaf(__uint_as_float(w[j].y), bf16_hi(xv.x), acc);
-                            acc = fmaf(__uint_as_float(w[j].z), bf16_lo(xv.y), acc); acc = fmaf(__uint_as_float(w[j].w), bf16_hi(xv.y), acc);
-                        }
-                    }
-                    acc = warp_sum(acc);
-                    if (lane == 0) s_red[task] = acc;
-                }
-                __syncthreads();
-                if (warp == 0 && lane < 16)
-                    for (int w = 0; w < 4; ++w) lg += s_red[lane * 4 + w];
-            }
-            if (own) st_relaxed_gpu_u32(hx + p.lx_off + e0 + lane, __float_as_uint(lg));
-        }
+        const int from = (int)gridDim.x == p.n_exp ? 0 : p.n_exp;
+        const uint32_t t0 = (cta - from) * TThreads + tid, all = (gridDim.x - from) * TThreads;
+        const uint4 none = make_uint4(kNotYet, kNotYet, kNotYet, kNotYet);
+        for (uint32_t i = t0; i < p.hx_words / 4; i += all) st_relaxed16(hc + i * 4, none);
+        for (uint32_t i = t0; i < (uint32_t)H * kStateCopies / 4; i += all) st_relaxed16(vc + i * 4, none);
+        if (t0 == 0) st_relaxed_gpu(p.defer + (size_t)((epoch + kStepStates / 2) % kStepStates) * (p.n_dn + 4), 0);
     }
 
-    constexpr int kHPad = 32 * CPB + 4;                                  // (a block of h, padded against bank conflicts)
     // ---- down: output rows 16 d .. 16 d + 15 over the h of all experts.  False: the h did not come while the grid was not fully resident.
     float* s_h = reinterpret_cast<float*>(un + S.h);
     uint4* s_hb = reinterpret_cast<uint4*>(un + S.hb);
@@ -609,15 +630,16 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
     auto down_unit = [&](int d, bool own) -> bool {
         bool give_up = false;
         const int n8 = p.Kt * p.I / 8;
+        const float* hr = hx + (size_t)(cta % kHCopies) * p.hc_words;
 #pragma unroll 1
         for (int i0 = 0, m = 0; i0 < n8 || m * udn < n_items; i0 += TThreads, ++m) {
             const int i = i0 + tid, item = m * udn + udq;
             const bool on = i < n8, ud = udq < udn && item < n_items && p.rmax > 0 && (item >= 4 * p.K ? p.rank_shared : p.rank) > 0;
             uint4 a = make_uint4(0, 0, 0, 0), b = a, u = a;
-            const float* up = hx + p.ud_off + (size_t)item * 4 * p.rmax + udj;
+            const float* up = hr + p.ud_off + (size_t)item * 4 * p.rmax + udj;
             bool got = !on && !ud;
             for (uint32_t it = 0; !got && !give_up; ++it) {
-                if (on) { a = ld_relaxed16(hx + i * 8); b = ld_relaxed16(hx + i * 8 + 4); }
+                if (on) { a = ld_relaxed16(hr + i * 8); b = ld_relaxed16(hr + i * 8 + 4); }
                 if (ud) {
                     u.x = ld_relaxed_gpu_u32(up); u.y = ld_relaxed_gpu_u32(up + p.rmax);
                     u.z = ld_relaxed_gpu_u32(up + 2 * p.rmax); u.w = ld_relaxed_gpu_u32(up + 3 * p.rmax);
@@ -718,14 +740,21 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
 #pragma unroll 8
             for (int i = 0; i < n; ++i) yv += __shfl_sync(0xFFFFFFFFu, o, i);
         }
-        const int row = d * 16 + warp;
-        if (p.x_next != nullptr && lane < kStateCopies)
-            st_relaxed_gpu_u32(p.vx + (size_t)(epoch % kStepStates * kStateCopies + lane) * H + row,
-                               __float_as_uint(bf16_bits_to_float(s_x[row]) + round_as(yv, p.out_dtype)));
         if (lane == 0) {
-            if (p.out_dtype == EDG_F32) store_out<float>(static_cast<float*>(p.y), row, yv);
-            else if (p.out_dtype == EDG_F16) store_out<__half>(static_cast<__half*>(p.y), row, yv);
-            else store_out<bf16_t>(static_cast<bf16_t*>(p.y), row, yv);
+            s_red[warp] = yv;
+            s_red[16 + warp] = bf16_bits_to_float(s_x[d * 16 + warp]) + round_as(yv, p.out_dtype);
+        }
+        __syncthreads();
+        static_assert(kStateCopies == 8, "a copy per four lanes");
+        if (warp == 0) {
+            if (p.x_next != nullptr)
+                st_relaxed16(p.vx + (size_t)(epoch % kStepStates * kStateCopies + lane / 4) * H + d * 16 + lane % 4 * 4, reinterpret_cast<const uint4*>(s_red + 16)[lane % 4]);
+        } else if (warp == 1 && lane < 16) {
+            const float v = s_red[lane];
+            const int row = d * 16 + lane;
+            if (p.out_dtype == EDG_F32) store_out<float>(static_cast<float*>(p.y), row, v);
+            else if (p.out_dtype == EDG_F16) store_out<__half>(static_cast<__half*>(p.y), row, v);
+            else store_out<bf16_t>(static_cast<bf16_t*>(p.y), row, v);
         }
         __syncthreads();
         return true;
@@ -783,20 +812,20 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
                 for (uint32_t it = 0; was != ~0ull && it < kSpinLimit; ++it) was = ld_relaxed_gpu_u64(pr);
                 if (was != ~0ull) atomicExch(p.status, EDG_E_TIMEOUT);
                 __syncwarp();
-                // (the logits move on into the ring slot, beside the routing made of them)
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int i = i0 + u * 32 + lane;
-                    if (i < p.E) {
-                        work[i] = __uint_as_float(v[u]);
-                        if (p.flag_out >= 0) st_relaxed_gpu_u32(slot + i, v[u]);
-                        st_relaxed_gpu_u32(hx + p.lx_off + i, kNotYet);
-                        if (p.logits_next != nullptr) p.logits_next[i] = __uint_as_float(v[u]);
-                    }
-                }
+                for (int u = 0; u < 8; ++u)
+                    if (i0 + u * 32 + lane < p.E) work[i0 + u * 32 + lane] = __uint_as_float(v[u]);
             }
             if (!give_up) {
                 emit_routing<false>(p, work, lane, p.flag_out >= 0 ? pr : nullptr);
+                // the logits move on into the ring slot, beside the routing made of them
+#pragma unroll 4
+                for (int i = lane; i < p.E; i += 32) {
+                    const uint32_t v = ld_relaxed_gpu_u32(hx + p.lx_off + i);
+                    if (p.flag_out >= 0) st_relaxed_gpu_u32(slot + i, v);
+                    st_relaxed_gpu_u32(hx + p.lx_off + i, kNotYet);
+                    if (p.logits_next != nullptr) p.logits_next[i] = __uint_as_float(v);
+                }
             }
         }
         return !__syncthreads_or(give_up);
@@ -943,9 +972,10 @@ bool step_supported(const edg_layer_desc& d, bool shared) {
     return step_smem(d, d.K + (shared ? 1 : 0), d.rank).total <= kStepSmemLimit;
 }
 
+static size_t step_copy_words(const edg_layer_desc& d) { return ((size_t)(d.K + 1) * d.I + (size_t)16 * (d.K + 1) * d.rank + 63) / 64 * 64; }
 size_t step_exchange_words(const edg_layer_desc& d) {
     const size_t sets = (d.n_adapters == 1 ? 1 : d.K) + 1;               // h, A_down h, A x, logits
-    return ((size_t)(d.K + 1) * d.I + (size_t)16 * (d.K + 1) * d.rank + sets * 8 * d.rank + d.E + 63) / 64 * 64;
+    return kHCopies * step_copy_words(d) + (sets * 8 * d.rank + d.E + 63) / 64 * 64;
 }
 size_t step_region_words(const edg_layer_desc& d) { return kStepBufs * step_exchange_words(d) + (size_t)kStepStates * kStateCopies * d.H; }
 
@@ -981,7 +1011,8 @@ int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* 
     p.hx = reinterpret_cast<float*>(ws + W.step_x);
     p.hx_words = (uint32_t)step_exchange_words(*d);
     p.ud_off = (uint32_t)(d->K + 1) * d->I;
-    p.ux_off = p.ud_off + 16u * (d->K + 1) * d->rank;
+    p.hc_words = (uint32_t)step_copy_words(*d);
+    p.ux_off = kHCopies * p.hc_words;
     p.lx_off = p.ux_off + ((d->n_adapters == 1 ? 1u : (uint32_t)d->K) + 1u) * 8u * d->rank;
     p.vx = p.hx + (size_t)kStepBufs * p.hx_words;
     p.I = d->I; p.E = d->E; p.group = d->group;
@@ -991,11 +1022,12 @@ int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* 
     p.L = record_layout(d->H, d->I, d->group);
     p.n_gu = 16 * p.Kt; p.n_dn = d->H / 16;
     p.n_exp = p.n_gu > p.n_dn ? p.n_gu : p.n_dn;
-    p.n_head = W_pre != nullptr ? (d->E + 15) / 16 : 0;
+    const int head_tile = d->pre_dtype == EDG_F16 && d->E % 16 == 0 ? 16 : 4;
+    p.n_head = W_pre != nullptr ? (d->E + head_tile - 1) / head_tile : 0;
     // One CTA per SM when they suffice: two launches of a chain then sit side by side on every SM, and no SM has two CTAs of the
     // same launch (which held a step up by 5 us of 15).  The head's tiles share the CTAs that the experts leave.
     const int n_sm = sm_count(), spare = n_sm - p.n_exp;
-    p.n_headc = spare > 0 && p.n_head > spare ? spare : p.n_head;
+    p.n_headc = min(p.n_head, spare > 2 ? spare - 2 : 16);               // (two more for the routing and the caller's x_next)
     const int extra = max(p.n_headc, p.x_next != nullptr ? 1 : 0);       // (somebody has to write x_next)
     const int grid = max(n_sm, p.n_exp + extra), idle = p.n_exp + p.n_headc;
     p.cta_route = W_pre == nullptr ? -1 : (idle < grid ? idle : idle - 1);
