@@ -1,4 +1,5 @@
-"""ctypes binding of the C ABI declared in ``include/edg_moe.h``: argument marshalling only.
+"""Binding of the C ABI declared in ``include/edg_moe.h``: argument marshalling only, by ctypes, and for the calls a decoder
+makes per layer and token by a small C extension (``csrc/edg_python.c``).
 
 Every function has the name and argument order of its C counterpart.  Buffers are torch tensors
 (device or pinned), numpy arrays (host) or raw integer addresses; torch is used for memory and
@@ -30,6 +31,10 @@ if not os.path.exists(LIB_PATH):
         f"{LIB_PATH} is missing: build it with `python -m paper_2609_18063_b200.build` "
         "(nvcc, sm_100a). There is no fallback path.")
 _lib = C.CDLL(LIB_PATH)
+try:
+    from . import _edgcall
+except ImportError as e:
+    raise ImportError(f"the C extension is missing or does not load ({e}): build it with `python -m paper_2609_18063_b200.build`") from e
 
 
 class EdgError(RuntimeError):
@@ -160,10 +165,19 @@ def _ptr(buf) -> Optional[int]:
 def _stream(stream) -> Optional[int]:
     if stream is None:
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        current = torch.cuda.current_stream().cuda_stream            # (initialises CUDA on the first call)
+        if hasattr(torch._C, "_cuda_getCurrentRawStream") and hasattr(torch._C, "_cuda_getDevice"):
+            _edgcall.streams(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+        return current
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
+
+
+_edgcall.init({n: C.cast(getattr(_lib, n), C.c_void_p).value for n in (
+    "prerouter_topk", "prerouter_topk_tokens", "softmax_topk_rows", "sigmoid_group_topk_rows", "prerouter_mlp_topk",
+    "moe_expert_ffn_int4_lora", "moe_layer_decode", "moe_layer_decode_dependent", "edg_stack_decode_token", "edg_next_hidden_state")},
+    _ptr, _stream, _check)
 
 
 _DT = {"f32": F32, "f16": F16, "bf16": BF16}
@@ -262,13 +276,11 @@ def set_trace_buffer(dev_buffer) -> None:
 
 
 def prerouter_topk(desc, W_pre, s, n_heads, inds, gates, logits_opt=None, stream=None, inds_host_mirror_opt=None) -> None:
-    _check(_lib.prerouter_topk(C.byref(desc), _ptr(W_pre), _ptr(s), n_heads, _ptr(inds), _ptr(gates),
-                               _ptr(logits_opt), _ptr(inds_host_mirror_opt), _stream(stream)), "prerouter_topk")
+    _edgcall.prerouter_topk(desc, W_pre, s, n_heads, inds, gates, logits_opt, inds_host_mirror_opt, stream)
 
 
 def prerouter_topk_tokens(desc, W_pre, s, T, inds, gates, logits_opt=None, stream=None) -> None:
-    _check(_lib.prerouter_topk_tokens(C.byref(desc), _ptr(W_pre), _ptr(s), T, _ptr(inds), _ptr(gates),
-                                      _ptr(logits_opt), _stream(stream)), "prerouter_topk_tokens")
+    _edgcall.prerouter_topk_tokens(desc, W_pre, s, T, inds, gates, logits_opt, stream)
 
 
 class MlpHead(C.Structure):
@@ -277,29 +289,22 @@ class MlpHead(C.Structure):
 
 def prerouter_mlp_topk(desc, W1, b1, W2, b2, W_res, width, s, cur_inds, prev_inds, n_heads, inds, gates,
                        logits_opt=None, stream=None) -> None:
-    head = MlpHead(_ptr(W1), _ptr(b1), _ptr(W2), _ptr(b2), _ptr(W_res), int(width))
-    _check(_lib.prerouter_mlp_topk(C.byref(desc), C.byref(head), _ptr(s), _ptr(cur_inds), _ptr(prev_inds), n_heads,
-                                   _ptr(inds), _ptr(gates), _ptr(logits_opt), _stream(stream)), "prerouter_mlp_topk")
+    _edgcall.prerouter_mlp_topk(desc, W1, b1, W2, b2, W_res, int(width), s, cur_inds, prev_inds, n_heads, inds, gates, logits_opt,
+                                stream)
 
 
 def sigmoid_group_topk_rows(logits, T, E, K, n_groups, keep_groups, scale, bias, inds, gates, stream=None) -> None:
-    _check(_lib.sigmoid_group_topk_rows(_ptr(logits), T, E, K, n_groups, keep_groups, float(scale), _ptr(bias),
-                                        _ptr(inds), _ptr(gates), _stream(stream)), "sigmoid_group_topk_rows")
+    _edgcall.sigmoid_group_topk_rows(logits, T, E, K, n_groups, keep_groups, scale, bias, inds, gates, stream)
 
 
 def softmax_topk_rows(desc, logits, T, inds, gates, stream=None) -> None:
-    _check(_lib.softmax_topk_rows(C.byref(desc), _ptr(logits), T, _ptr(inds), _ptr(gates), _stream(stream)),
-           "softmax_topk_rows")
+    _edgcall.softmax_topk_rows(desc, logits, T, inds, gates, stream)
 
 
 def moe_expert_ffn_int4_lora(desc, slot_pool, slot_table, T, slots, experts, gates, x, lora, y,
                              workspace, workspace_bytes=None, stream=None) -> None:
-    if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    _check(_lib.moe_expert_ffn_int4_lora(C.byref(desc), _ptr(slot_pool), _ptr(slot_table), T, _ptr(slots),
-                                         _ptr(experts), _ptr(gates), _ptr(x),
-                                         None if lora is None else C.byref(lora), _ptr(y), _ptr(workspace),
-                                         workspace_bytes, _stream(stream)), "moe_expert_ffn_int4_lora")
+    _edgcall.moe_expert_ffn_int4_lora(desc, slot_pool, slot_table, T, slots, experts, gates, x, lora, y, workspace,
+                                      workspace_bytes, stream)
 
 
 def moe_expert_ffn_int4_lora_static(desc, slot_pool, slot_table, slots, experts, gates, x, lora, y, stream=None) -> None:
@@ -423,38 +428,24 @@ def stage_experts_to_slots(store: Store, layer: int, inds_host, n: Optional[int]
 def moe_layer_decode(store: Store, layer, x, inds_cur, gates_cur, W_pre_next, inds_next, gates_next,
                      logits_next_opt, y, workspace, workspace_bytes=None, stream=None,
                      inds_next_host_mirror_opt=None) -> None:
-    if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    _check(_lib.moe_layer_decode(store.handle, layer, _ptr(x), _ptr(inds_cur), _ptr(gates_cur), _ptr(W_pre_next),
-                                 _ptr(inds_next), _ptr(gates_next), _ptr(logits_next_opt),
-                                 _ptr(inds_next_host_mirror_opt), _ptr(y),
-                                 _ptr(workspace), workspace_bytes, _stream(stream)), "moe_layer_decode")
+    _edgcall.moe_layer_decode(store.handle, layer, x, inds_cur, gates_cur, W_pre_next, inds_next, gates_next, logits_next_opt,
+                              inds_next_host_mirror_opt, y, workspace, workspace_bytes, stream)
 
 
 def stack_decode_token(store: Store, x, inds_cur, gates_cur, W_pre, inds_next, gates_next, logits_next_opt,
                        mirror_cur, mirror_next, y, workspace, workspace_bytes=None, stream=None, prefetch=True) -> int:
     """edg_stack_decode_token; returns the number of experts copied for this token."""
-    if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    miss = C.c_int32()
-    _check(_lib.edg_stack_decode_token(store.handle, _ptr(x), _ptr(inds_cur), _ptr(gates_cur), _ptr(W_pre),
-                                       _ptr(inds_next), _ptr(gates_next), _ptr(logits_next_opt), _ptr(mirror_cur),
-                                       _ptr(mirror_next), _ptr(y), _ptr(workspace), workspace_bytes, _stream(stream),
-                                       int(bool(prefetch)), C.byref(miss)), "edg_stack_decode_token")
-    return miss.value
+    return _edgcall.stack_decode_token(store.handle, x, inds_cur, gates_cur, W_pre, inds_next, gates_next, logits_next_opt,
+                                       mirror_cur, mirror_next, y, workspace, workspace_bytes, stream, prefetch)
 
 
 def next_hidden_state(desc, x, y, x_next, eps=1e-6, stream=None) -> None:
-    _check(_lib.edg_next_hidden_state(C.byref(desc), _ptr(x), _ptr(y), _ptr(x_next), float(eps), _stream(stream)),
-           "edg_next_hidden_state")
+    _edgcall.next_hidden_state(desc, x, y, x_next, eps, stream)
 
 
 def moe_layer_decode_dependent(store: Store, layer, x, inds_cur, gates_cur, W_pre_next, inds_next, gates_next,
                                logits_next_opt, y, x_next, workspace, eps=1e-6, workspace_bytes=None, stream=None,
                                inds_next_host_mirror_opt=None) -> None:
-    if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    _check(_lib.moe_layer_decode_dependent(store.handle, layer, _ptr(x), _ptr(inds_cur), _ptr(gates_cur), _ptr(W_pre_next),
-                                           _ptr(inds_next), _ptr(gates_next), _ptr(logits_next_opt),
-                                           _ptr(inds_next_host_mirror_opt), _ptr(y), _ptr(x_next), float(eps),
-                                           _ptr(workspace), workspace_bytes, _stream(stream)), "moe_layer_decode_dependent")
+    _edgcall.moe_layer_decode_dependent(store.handle, layer, x, inds_cur, gates_cur, W_pre_next, inds_next, gates_next,
+                                        logits_next_opt, inds_next_host_mirror_opt, y, x_next, eps, workspace, workspace_bytes,
+                                        stream)
