@@ -10,6 +10,7 @@
 
 #include "edg_common.cuh"
 #include "edg_mma.cuh"
+#include "edg_head.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -321,8 +322,8 @@ __global__ void __launch_bounds__(128) softmax_topk_rows_kernel(const float* log
 // hidden state followed by two K-hot vectors (this layer's experts at this token and at the previous
 // one), so fc1 is a dot product over the hidden state plus a gather of 2K columns.  Phase 1: the D
 // rows of fc1 are dealt to the CTAs of the cluster, a warp per row; every activation is written
-// into the shared memory of all CTAs.  Phase 2: the E rows of fc2 (+ the residual row over the
-// hidden state) likewise; the logits land in the leader, which does softmax + top-k.
+// into the shared memory of all CTAs; then the E residual rows over the hidden state, whose sums stay with the
+// lanes.  Phase 2: the E rows of fc2; the logits land in the leader, which does softmax + top-k.
 struct MlpParams {
     const __half* W1;       // [n_heads][D][H + 2E]
     const __half* b1;       // [n_heads][D] or null
@@ -339,49 +340,21 @@ struct MlpParams {
     int32_t* mirror;        // [n_heads][K] in mapped pinned host memory, or null
 };
 
-// dot product of an fp16 row of n (a multiple of 8) weights with fp32 activations, by one warp
-__device__ __forceinline__ float half_row_dot(const __half* row, const float* sx, int n, int lane) {
-    const uint4* wp = reinterpret_cast<const uint4*>(row);
-    float acc = 0.f;
-#pragma unroll 8
-    for (int c = lane; c < n / 8; c += 32) {
-        const uint4 w = ld_stream16(wp + c);
-        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&w.x));
-        const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&w.y));
-        const float2 d = __half22float2(*reinterpret_cast<const __half2*>(&w.z));
-        const float2 e = __half22float2(*reinterpret_cast<const __half2*>(&w.w));
-        const float* x = sx + c * 8;
-        acc = fmaf(a.x, x[0], acc); acc = fmaf(a.y, x[1], acc);
-        acc = fmaf(b.x, x[2], acc); acc = fmaf(b.y, x[3], acc);
-        acc = fmaf(d.x, x[4], acc); acc = fmaf(d.y, x[5], acc);
-        acc = fmaf(e.x, x[6], acc); acc = fmaf(e.y, x[7], acc);
-    }
-    return acc;                          // (not yet summed over the lanes)
+static __device__ __forceinline__ void ring_wait(uint64_t* bar, uint32_t parity) {
+    for (uint32_t i = 0; i < kSpinLimit && !mbar_try_wait(bar, parity); ++i) {}
 }
 
-// two rows at once against the same activations: twice the loads in flight, the activations read once
-__device__ __forceinline__ void half_row_dot2(const __half* row0, const __half* row1, const float* sx, int n, int lane,
-                                              float& acc0, float& acc1) {
-    const uint4* wp0 = reinterpret_cast<const uint4*>(row0);
-    const uint4* wp1 = reinterpret_cast<const uint4*>(row1);
-    acc0 = 0.f; acc1 = 0.f;
-#pragma unroll 8
-    for (int c = lane; c < n / 8; c += 32) {
-        const uint4 w0 = ld_stream16(wp0 + c), w1 = ld_stream16(wp1 + c);
-        const float4 x0 = *reinterpret_cast<const float4*>(sx + c * 8), x1 = *reinterpret_cast<const float4*>(sx + c * 8 + 4);
-        float2 a = __half22float2(*reinterpret_cast<const __half2*>(&w0.x)), b = __half22float2(*reinterpret_cast<const __half2*>(&w0.y));
-        float2 d = __half22float2(*reinterpret_cast<const __half2*>(&w0.z)), e = __half22float2(*reinterpret_cast<const __half2*>(&w0.w));
-        acc0 = fmaf(a.x, x0.x, acc0); acc0 = fmaf(a.y, x0.y, acc0); acc0 = fmaf(b.x, x0.z, acc0); acc0 = fmaf(b.y, x0.w, acc0);
-        acc0 = fmaf(d.x, x1.x, acc0); acc0 = fmaf(d.y, x1.y, acc0); acc0 = fmaf(e.x, x1.z, acc0); acc0 = fmaf(e.y, x1.w, acc0);
-        a = __half22float2(*reinterpret_cast<const __half2*>(&w1.x)); b = __half22float2(*reinterpret_cast<const __half2*>(&w1.y));
-        d = __half22float2(*reinterpret_cast<const __half2*>(&w1.z)); e = __half22float2(*reinterpret_cast<const __half2*>(&w1.w));
-        acc1 = fmaf(a.x, x0.x, acc1); acc1 = fmaf(a.y, x0.y, acc1); acc1 = fmaf(b.x, x0.z, acc1); acc1 = fmaf(b.y, x0.w, acc1);
-        acc1 = fmaf(d.x, x1.x, acc1); acc1 = fmaf(d.y, x1.y, acc1); acc1 = fmaf(e.x, x1.z, acc1); acc1 = fmaf(e.y, x1.w, acc1);
-    }
-}
+constexpr int kMlpWarps = 8;            // warps per CTA of the full head
+constexpr int kMlpPieces = 128;          // 16-byte pieces of a row in one slot of a warp's ring
+constexpr int kMlpSlots = 3;
 
-constexpr int kMlpWarps = 8;      // warps per CTA of the full head (16 measured no faster)
-
+// What bounds the full head is its 3.9 MB of weights (H 2048, D 512, E 256): 40 heads take 24 us to stream.  Loads into registers
+// left the memory idle between a warp's rows (reduction, gelu), across the cluster barrier and in front of the residual path: 64.6 us
+// (2.3 TB/s).  Here every warp streams all its rows -- W1, then the residual rows, which need no activations, then W2 -- through a
+// ring of three 2 KB slots of its own, refilled by bulk copies as soon as a slot is read, so the barrier finds the W2 rows in
+// place; three CTAs fit an SM (100 KB in flight): 39.3 us.
+// Per lane the products are summed in the order of the pieces (lane, lane + 32, ..), then over the lanes: results do not depend
+// on the slots.
 template <typename WT>
 __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(MlpParams p) {
     cg::cluster_group cluster = cg::this_cluster();
@@ -389,17 +362,102 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(MlpParams
     const int csize = (int)cluster.num_blocks();
     const int head = blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    extern __shared__ float smem[];
-    float* s_logits = smem;             // [E]   (the leader's copy collects every CTA's rows)
-    float* s_x = smem + p.E;            // [H]   hidden state widened to fp32
-    float* s_a = s_x + p.H;             // [D]   gelu(fc1), complete in every CTA after the first cluster barrier
+    constexpr int kSlotBytes = kMlpPieces * 16;
+    extern __shared__ __align__(128) uint8_t smem8[];
+    uint8_t* ring = smem8 + warp * kMlpSlots * kSlotBytes;                              // this warp's slots
+    float* s_x0 = reinterpret_cast<float*>(smem8 + kMlpWarps * kMlpSlots * kSlotBytes); // [H/2] values 0-3 of every eight of the state,
+    float* s_x1 = s_x0 + p.H / 2;       // [H/2] and values 4-7
+    float* s_a0 = s_x1 + p.H / 2;       // [D/2] gelu(fc1) in the same way, complete in every CTA after the first cluster barrier
+    float* s_a1 = s_a0 + p.D / 2;       // [D/2]
+    const int perD = (p.D + csize - 1) / csize, perE = (p.E + csize - 1) / csize;
+    float* s_part = s_a1 + p.D / 2;     // [perE][32] lanes' sums of the residual path
+    float* s_logits = s_part + perE * 32;   // [E]   (the leader's copy collects every CTA's rows)
+    float* s_win = s_logits + p.E;      // 64 words for the winners
+    __shared__ __align__(8) uint64_t bars[kMlpWarps][kMlpSlots];
+
+    if (lane == 0) {
+        for (int i = 0; i < kMlpSlots; ++i) mbar_init(&bars[warp][i], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    // this warp's items: rows of W1, rows of the residual path, rows of W2, each in pieces of up to a slot
+    const int F = p.H + 2 * p.E;
+    const int r0 = crank * perD + warp, rend = min(p.D, (crank + 1) * perD), e0 = crank * perE + warp, eend = min(p.E, (crank + 1) * perE);
+    const int n1 = r0 < rend ? (rend - r0 + kMlpWarps - 1) / kMlpWarps : 0, n2 = e0 < eend ? (eend - e0 + kMlpWarps - 1) / kMlpWarps : 0;
+    const int p1 = p.H / 8, pr = p.Wres != nullptr ? p.H * (int)sizeof(WT) / 16 : 0, p2 = p.D / 8;       // 16-byte pieces of a row
+    const int c1 = (p1 + kMlpPieces - 1) / kMlpPieces, cr = (pr + kMlpPieces - 1) / kMlpPieces, c2 = (p2 + kMlpPieces - 1) / kMlpPieces;
+    const int total = n1 * c1 + n2 * (cr + c2);
+    // the slot after next: which row and piece the next copy fetches
+    int f_kind = n1 > 0 ? 0 : (cr > 0 ? 1 : 2), f_row = 0, f_chunk = 0, fetched = 0;
+    auto fetch = [&]() {                                                 // lane 0
+        const uint8_t* src;
+        int pieces, chunks, rows;
+        if (f_kind == 0) {
+            src = reinterpret_cast<const uint8_t*>(p.W1 + ((size_t)head * p.D + r0 + f_row * kMlpWarps) * F);
+            pieces = p1; chunks = c1; rows = n1;
+        } else if (f_kind == 1) {
+            src = static_cast<const uint8_t*>(p.Wres) + ((size_t)head * p.E + e0 + f_row * kMlpWarps) * p.H * sizeof(WT);
+            pieces = pr; chunks = cr; rows = n2;
+        } else {
+            src = reinterpret_cast<const uint8_t*>(p.W2 + ((size_t)head * p.E + e0 + f_row * kMlpWarps) * p.D);
+            pieces = p2; chunks = c2; rows = n2;
+        }
+        const int slot = fetched % kMlpSlots, n = min(kMlpPieces, pieces - f_chunk * kMlpPieces);
+        mbar_expect_tx(&bars[warp][slot], n * 16);
+        bulk_g2s(ring + slot * kSlotBytes, src + (size_t)f_chunk * kSlotBytes, n * 16, &bars[warp][slot]);
+        ++fetched;
+        if (++f_chunk == chunks) {
+            f_chunk = 0;
+            if (++f_row == rows) { f_row = 0; f_kind = f_kind == 0 && cr > 0 ? 1 : 2; }
+        }
+    };
+    if (lane == 0)
+        for (int i = 0; i < min(total, kMlpSlots); ++i) fetch();
 
     const uint16_t* sv = p.s + (size_t)head * p.H;
-    for (int i = threadIdx.x; i < p.H; i += blockDim.x) s_x[i] = bf16_bits_to_float(sv[i]);
+    for (int i = threadIdx.x; i < p.H / 8; i += blockDim.x) {
+        const uint4 v = *reinterpret_cast<const uint4*>(sv + i * 8);
+        *reinterpret_cast<float4*>(s_x0 + i * 4) = make_float4(bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y));
+        *reinterpret_cast<float4*>(s_x1 + i * 4) = make_float4(bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w));
+    }
     __syncthreads();
 
-    const int F = p.H + 2 * p.E;
-    const int perD = (p.D + csize - 1) / csize;
+    int used = 0;
+    // acc + this lane's share of a row (n pieces, in c chunks) times v; the row's slots go back to the ring
+    auto row_dot = [&](int n, int chunks, auto piece) {
+        float acc = 0.f;
+        for (int ch = 0; ch < chunks; ++ch, ++used) {
+            const int slot = used % kMlpSlots;
+            ring_wait(&bars[warp][slot], (used / kMlpSlots) & 1);
+            const uint4* src = reinterpret_cast<const uint4*>(ring + slot * kSlotBytes);
+            uint4 w[kMlpPieces / 32];
+#pragma unroll
+            for (int j = 0; j < kMlpPieces / 32; ++j)
+                w[j] = ch * kMlpPieces + j * 32 + lane < n ? src[j * 32 + lane] : make_uint4(0, 0, 0, 0);
+            __syncwarp();
+            if (lane == 0 && fetched < total) fetch();
+#pragma unroll
+            for (int j = 0; j < kMlpPieces / 32; ++j)
+                if (ch * kMlpPieces + j * 32 + lane < n) acc = piece(w[j], ch * kMlpPieces + j * 32 + lane, acc);
+        }
+        return acc;
+    };
+    auto halves = [](const uint4& w, const float* v0, const float* v1, int c, float acc) {       // eight fp16 weights
+        const float4 x0 = *reinterpret_cast<const float4*>(v0 + c * 4), x1 = *reinterpret_cast<const float4*>(v1 + c * 4);
+        const float2 a = __half22float2(u32_as_h2(w.x)), b = __half22float2(u32_as_h2(w.y)), d = __half22float2(u32_as_h2(w.z)), e = __half22float2(u32_as_h2(w.w));
+        acc = fmaf(a.x, x0.x, acc); acc = fmaf(a.y, x0.y, acc); acc = fmaf(b.x, x0.z, acc); acc = fmaf(b.y, x0.w, acc);
+        acc = fmaf(d.x, x1.x, acc); acc = fmaf(d.y, x1.y, acc); acc = fmaf(e.x, x1.z, acc); acc = fmaf(e.y, x1.w, acc);
+        return acc;
+    };
+    auto by_state = [&](const uint4& w, int c, float acc) { return halves(w, s_x0, s_x1, c, acc); };
+    auto by_gelu = [&](const uint4& w, int c, float acc) { return halves(w, s_a0, s_a1, c, acc); };
+    auto by_state32 = [&](const uint4& w, int c, float acc) {            // four fp32 weights
+        const float4 x = *reinterpret_cast<const float4*>((c & 1 ? s_x1 : s_x0) + (c >> 1) * 4);
+        acc = fmaf(__uint_as_float(w.x), x.x, acc); acc = fmaf(__uint_as_float(w.y), x.y, acc);
+        acc = fmaf(__uint_as_float(w.z), x.z, acc); acc = fmaf(__uint_as_float(w.w), x.w, acc);
+        return acc;
+    };
+
     // the K-hot parts of the feature pick columns: lane k < K holds the k-th expert of either list
     int hc = -1, hq = -1;
     if (lane < p.K) {
@@ -408,53 +466,58 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(MlpParams
         if (hc < 0 || hc >= p.E) hc = -1;
         if (hq < 0 || hq >= p.E) hq = -1;
     }
-    const int rend = min(p.D, (crank + 1) * perD);
-    for (int r = crank * perD + warp; r < rend; r += 2 * kMlpWarps) {      // two rows of this warp at a time
-        const int r1 = r + kMlpWarps;
-        const bool two = r1 < rend;
-        const __half* row0 = p.W1 + ((size_t)head * p.D + r) * F;
-        const __half* row1 = two ? row0 + (size_t)kMlpWarps * F : row0;
-        // (the gathered columns are fetched together with the rows, not after them)
-        const __half gc0 = hc >= 0 ? row0[p.H + hc] : __float2half(0.f), gq0 = hq >= 0 ? row0[p.H + p.E + hq] : __float2half(0.f);
-        const __half gc1 = hc >= 0 ? row1[p.H + hc] : __float2half(0.f), gq1 = hq >= 0 ? row1[p.H + p.E + hq] : __float2half(0.f);
-        float z0, z1;
-        half_row_dot2(row0, row1, s_x, p.H, lane, z0, z1);
-        z0 = warp_sum(z0 + __half2float(gc0) + __half2float(gq0));
-        z1 = warp_sum(z1 + __half2float(gc1) + __half2float(gq1));
-        if (p.b1 != nullptr) {
-            z0 += __half2float(p.b1[(size_t)head * p.D + r]);
-            if (two) z1 += __half2float(p.b1[(size_t)head * p.D + r1]);
-        }
-        const float a0 = 0.5f * z0 * (1.f + erff(z0 * 0.70710678118654752f));
-        const float a1 = 0.5f * z1 * (1.f + erff(z1 * 0.70710678118654752f));
-        if (lane < csize) {
-            float* dst = cluster.map_shared_rank(s_a, lane);
-            dst[r] = a0;
-            if (two) dst[r1] = a1;
-        }
+    for (int i = 0; i < n1; ++i) {
+        const int r = r0 + i * kMlpWarps;
+        // (the gathered columns are fetched while the row is on its way)
+        const __half* row = p.W1 + ((size_t)head * p.D + r) * F;
+        const __half gc = hc >= 0 ? row[p.H + hc] : __float2half(0.f), gq = hq >= 0 ? row[p.H + p.E + hq] : __float2half(0.f);
+        const float bias = p.b1 != nullptr ? __half2float(p.b1[(size_t)head * p.D + r]) : 0.f;
+        float z = row_dot(p1, c1, by_state);
+        z = warp_sum(z + __half2float(gc) + __half2float(gq));
+        if (p.b1 != nullptr) z += bias;
+        const float a = 0.5f * z * (1.f + erff(z * 0.70710678118654752f));
+        if (lane < csize) *cluster.map_shared_rank(((r & 4) ? s_a1 : s_a0) + (r >> 3) * 4 + (r & 3), lane) = a;
     }
+    if (cr > 0)
+        for (int i = 0; i < n2; ++i) {
+            float v;
+            if constexpr (sizeof(WT) == 2) v = row_dot(pr, cr, by_state);
+            else v = row_dot(pr, cr, by_state32);
+            s_part[(warp + i * kMlpWarps) * 32 + lane] = v;
+        }
     cluster.sync();                     // every CTA holds all D activations
 
     float* leader = cluster.map_shared_rank(s_logits, 0);
-    const int perE = (p.E + csize - 1) / csize;
-    for (int e = crank * perE + warp; e < min(p.E, (crank + 1) * perE); e += kMlpWarps) {
-        // (both dot products' loads are issued before either sum is reduced)
-        float l = half_row_dot(p.W2 + ((size_t)head * p.E + e) * p.D, s_a, p.D, lane);
-        if (p.Wres != nullptr) l += RowDot<WT>::partial(p.Wres, (size_t)head * p.E + e, s_x, p.H, lane);
+    for (int i = 0; i < n2; ++i) {
+        const int e = e0 + i * kMlpWarps;
+        const float bias = p.b2 != nullptr ? __half2float(p.b2[(size_t)head * p.E + e]) : 0.f;
+        float l = row_dot(p2, c2, by_gelu);
+        if (cr > 0) l += s_part[(warp + i * kMlpWarps) * 32 + lane];
         l = warp_sum(l);
-        if (p.b2 != nullptr) l += __half2float(p.b2[(size_t)head * p.E + e]);
+        if (p.b2 != nullptr) l += bias;
         if (lane == 0) leader[e] = l;
     }
     cluster.sync();                     // every CTA's logits have landed in the leader
     if (crank != 0) return;
 
-    if (p.logits != nullptr)
-        for (int e = threadIdx.x; e < p.E; e += blockDim.x) p.logits[(size_t)head * p.E + e] = s_logits[e];
-    __syncthreads();
     if (warp == 0) {
-        warp_softmax_topk(s_logits, p.E, p.K, lane, p.inds + (size_t)head * p.K, p.gates + (size_t)head * p.K);
-        mirror_inds(p.mirror != nullptr ? p.mirror + (size_t)head * p.K : nullptr, p.inds + (size_t)head * p.K, p.K, lane);
-    }
+        int32_t* s_i = reinterpret_cast<int32_t*>(s_win);
+        int32_t* inds = p.inds + (size_t)head * p.K;
+        float* gates = p.gates + (size_t)head * p.K;
+        if (p.E <= 256 && topk_distinct(s_logits, p.E, p.K, lane, s_i, s_win + 32)) {
+            __syncwarp();
+            if (lane < p.K) { inds[lane] = s_i[lane]; gates[lane] = s_win[32 + lane]; }
+            if (p.mirror != nullptr && lane < p.K)
+                asm volatile("st.relaxed.sys.global.s32 [%0], %1;" ::"l"(p.mirror + (size_t)head * p.K + lane), "r"(s_i[lane]) : "memory");
+        } else {
+            if (p.logits != nullptr)                                     // (the general form may overwrite them)
+                for (int e = lane; e < p.E; e += 32) p.logits[(size_t)head * p.E + e] = s_logits[e];
+            __syncwarp();
+            warp_softmax_topk(s_logits, p.E, p.K, lane, inds, gates);
+            mirror_inds(p.mirror != nullptr ? p.mirror + (size_t)head * p.K : nullptr, inds, p.K, lane);
+        }
+    } else if (p.logits != nullptr && p.E <= 256)
+        for (int e = threadIdx.x - 32; e < p.E; e += blockDim.x - 32) p.logits[(size_t)head * p.E + e] = s_logits[e];
 }
 
 // Appendix A, sigmoid-group routing, one warp per row of given logits: sigma = sigmoid(l); a group's
@@ -662,9 +725,16 @@ int32_t edg::run_prerouter_mlp(const edg_layer_desc* desc, const edg_mlp_head* h
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(edg::kPreCluster, n_heads, 1);
     cfg.blockDim = dim3(edg::kMlpWarps * 32, 1, 1);
-    cfg.dynamicSmemBytes = (size_t)(desc->E + desc->H + D) * sizeof(float);
+    if ((size_t)(desc->E + desc->H + D) * sizeof(float) > 48 * 1024) return EDG_E_SHAPE;
+    const int perE = (desc->E + edg::kPreCluster - 1) / edg::kPreCluster;
+    cfg.dynamicSmemBytes = edg::kMlpWarps * edg::kMlpSlots * edg::kMlpPieces * 16 + (size_t)(desc->E + desc->H + D + perE * 32 + 64) * sizeof(float);
     cfg.stream = stream;
-    if (cfg.dynamicSmemBytes > 48 * 1024) return EDG_E_SHAPE;
+    static bool configured = false;
+    if (!configured) {
+        EDG_CUDA_TRY(cudaFuncSetAttribute(edg::prerouter_mlp_kernel<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+        EDG_CUDA_TRY(cudaFuncSetAttribute(edg::prerouter_mlp_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+        configured = true;
+    }
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = edg::kPreCluster;
