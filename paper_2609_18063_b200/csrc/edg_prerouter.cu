@@ -520,6 +520,98 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(MlpParams
         for (int e = threadIdx.x - 32; e < p.E; e += blockDim.x - 32) p.logits[(size_t)head * p.E + e] = s_logits[e];
 }
 
+// Appendix A, sigmoid-group routing when the groups divide the warp and the warp the experts (the 8B tier: 128 experts in 8 groups):
+// lane l holds the V = E / 32 consecutive entries from l V on, so a group is a run of lanes and everything stays in registers;
+// order by (lane, entry) is order by index, so the first lane that holds a round's best key has the winner, ties included.
+// The form over shared memory below spends its time on instructions too, three times as many: 4096 rows 10.3 us, here 7.8
+// (one launch after the other; 6 of them are the host's).
+// Same values in the same order as that form.
+template <int V>
+__global__ void __launch_bounds__(256) sigmoid_group_topk_lanes_kernel(const float* logits, const float* bias, int T, int K, int n, int keep,
+                                                                       float scale, int32_t* inds, float* gates) {
+    constexpr int E = 32 * V;
+    const unsigned full = 0xFFFFFFFFu;
+    __shared__ int s_i[8][32];
+    __shared__ float s_g[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int t = blockIdx.x * 8 + warp;
+    if (t >= T) return;
+    float sg[V], sel[V];
+    constexpr int W = V % 4 == 0 ? 4 : (V % 2 == 0 ? 2 : 1);
+    const float* src = logits + (size_t)t * E + lane * V;
+#pragma unroll
+    for (int u = 0; u < V; u += W) {
+        if constexpr (W == 4) {
+            const float4 v = *reinterpret_cast<const float4*>(src + u);
+            sg[u] = v.x; sg[u + 1] = v.y; sg[u + 2] = v.z; sg[u + 3] = v.w;
+        } else if constexpr (W == 2) {
+            const float2 v = *reinterpret_cast<const float2*>(src + u);
+            sg[u] = v.x; sg[u + 1] = v.y;
+        } else sg[u] = src[u];
+    }
+    float m1 = -CUDART_INF_F, m2 = -CUDART_INF_F;
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+        sg[u] = 1.f / (1.f + expf(-sg[u]));
+        sel[u] = bias != nullptr ? sg[u] + bias[lane * V + u] : sg[u];
+        if (sel[u] > m1) { m2 = m1; m1 = sel[u]; } else if (sel[u] > m2) m2 = sel[u];
+    }
+    // group scores, merged over the 32 / n lanes of a group, and the group's rank
+    const int lpg = 32 / n, grp = lane / lpg;
+    for (int o = 1; o < lpg; o <<= 1) {
+        const float o1 = __shfl_xor_sync(full, m1, o), o2 = __shfl_xor_sync(full, m2, o);
+        const float hi = fmaxf(m1, o1), lo = fminf(m1, o1);
+        m2 = fmaxf(lo, fmaxf(m2, o2));
+        m1 = hi;
+    }
+    const float gs = m1 + m2;
+    int rank = 0;
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+        const float gj = __shfl_sync(full, gs, j * lpg);
+        rank += (gj > gs || (gj == gs && j < grp)) ? 1 : 0;
+    }
+    uint32_t key[V];
+    uint32_t top = 0u;
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+        key[u] = rank < keep && sel[u] == sel[u] ? float_key(sel[u]) : 0u;
+        top = max(top, key[u]);
+    }
+    int got = 0;
+    for (; got < K; ++got) {
+        const uint32_t best = __reduce_max_sync(full, top);
+        if (best == 0u) break;                                   // fewer than K survivors
+        const unsigned who = __ballot_sync(full, top == best);
+        if (lane == __ffs(who) - 1) {
+            int at = 0;
+            float g = 0.f;
+#pragma unroll
+            for (int u = V - 1; u >= 0; --u)
+                if (key[u] == best) { at = u; g = sg[u]; }
+            top = 0u;
+#pragma unroll
+            for (int u = 0; u < V; ++u) {
+                if (u == at) key[u] = 0u;
+                top = max(top, key[u]);
+            }
+            s_i[warp][got] = lane * V + at;
+            s_g[warp][got] = g;
+        }
+    }
+    __syncwarp();
+    const int myi = lane < got ? s_i[warp][lane] : 0x7FFFFFFF;
+    const float myv = lane < got ? s_g[warp][lane] : 0.f;
+    const float sum = warp_sum(myv);
+    int pos = 0;
+#pragma unroll 4
+    for (int i = 0; i < K; ++i) pos += __shfl_sync(full, myi, i) < myi ? 1 : 0;
+    if (lane < got) {
+        inds[(size_t)t * K + pos] = myi;
+        gates[(size_t)t * K + pos] = scale * myv / (sum + 1e-20f);
+    }
+}
+
 // Appendix A, sigmoid-group routing, one warp per row of given logits: sigma = sigmoid(l); a group's
 // score is the sum of its two largest selection scores (sigma, plus a bias when one is given); the
 // best `keep` of the `n` groups survive (ties to the lower group); top-K among the survivors by
@@ -692,8 +784,28 @@ extern "C" int32_t sigmoid_group_topk_rows(const float* logits, int32_t T, int32
     if (!logits || !inds || !gates || T < 1) return EDG_E_INVAL;
     if (E < 2 || E > 1024 || n_groups < 1 || n_groups > 32 || E % n_groups != 0 || E / n_groups < 2) return EDG_E_SHAPE;
     if (keep_groups < 1 || keep_groups > n_groups || K < 1 || K > 32 || K > keep_groups * (E / n_groups)) return EDG_E_SHAPE;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (32 % n_groups == 0 && E % 32 == 0 && edg::aligned(logits, 16)) {       // (E / n_groups is then a multiple of E / 32)
+        void (*k)(const float*, const float*, int, int, int, int, float, int32_t*, float*) = nullptr;
+        switch (E / 32) {
+            case 1: k = edg::sigmoid_group_topk_lanes_kernel<1>; break;
+            case 2: k = edg::sigmoid_group_topk_lanes_kernel<2>; break;
+            case 3: k = edg::sigmoid_group_topk_lanes_kernel<3>; break;
+            case 4: k = edg::sigmoid_group_topk_lanes_kernel<4>; break;
+            case 5: k = edg::sigmoid_group_topk_lanes_kernel<5>; break;
+            case 6: k = edg::sigmoid_group_topk_lanes_kernel<6>; break;
+            case 8: k = edg::sigmoid_group_topk_lanes_kernel<8>; break;
+            case 12: k = edg::sigmoid_group_topk_lanes_kernel<12>; break;
+            case 16: k = edg::sigmoid_group_topk_lanes_kernel<16>; break;
+        }
+        if (k != nullptr) {
+            k<<<(T + 7) / 8, 256, 0, st>>>(logits, bias_opt, T, K, n_groups, keep_groups, scale, inds, gates);
+            EDG_CUDA_TRY(cudaGetLastError());
+            return EDG_OK;
+        }
+    }
     const size_t sm = 4 * 2 * (size_t)E * sizeof(float);
-    edg::sigmoid_group_topk_rows_kernel<<<(T + 3) / 4, 128, sm, static_cast<cudaStream_t>(stream)>>>(
+    edg::sigmoid_group_topk_rows_kernel<<<(T + 3) / 4, 128, sm, st>>>(
         logits, bias_opt, T, E, K, n_groups, keep_groups, scale, inds, gates);
     EDG_CUDA_TRY(cudaGetLastError());
     return EDG_OK;
