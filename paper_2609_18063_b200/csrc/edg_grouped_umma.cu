@@ -18,10 +18,9 @@
 // The 8 k values of a core row are kept in the order (k0,k4,k1,k5,k2,k6,k3,k7) in which the int4 codes
 // come out of a 32-bit word -- for A and B alike, so the dot product is unchanged.
 //
-// Warps 0-7 (two threads per weight row and per token, each covering half of a stage's k) dequantise /
-// convert into a ring of two (gate/up) or three (down) stages, with the loads of the next chunk in flight while the current one is
-// processed, and later run the epilogue (each warp its 32 lanes of tensor memory, half of the token
-// columns); warp 8 allocates the tensor memory and its lane 0 issues the MMAs.
+// Warps 0-7 dequantise the weights into a ring of two stages, with the codes of the next four chunks in flight in registers, and
+// later run the epilogue (each warp its 32 lanes of tensor memory, half of the token columns); warp 8 allocates the tensor memory
+// and its lane 0 issues the MMAs; lane 0 of warp 9 fetches the activations into a ring of their own.
 // Every wait is bounded: a wait that gives up raises the status word and the kernel still frees its
 // tensor memory and returns.
 #include "edg_grouped.cuh"
@@ -31,13 +30,15 @@ namespace {
 
 constexpr int U_TN = kUmmaTokens;            // token columns per tile
 constexpr int U_KC = 32;                     // k per stage
-constexpr int U_STAGES_MAX = 3;
+constexpr int U_STAGES = 2;                  // of weights: four operand tiles each
+constexpr int U_ACT_MAX = 4;                 // slots of activations
+constexpr int U_AHEAD = 4;                   // chunks of codes in flight per thread
 constexpr uint32_t U_TILE = 128 * U_KC * 2;  // bytes of a [128 x 32] fp16 operand tile
 constexpr uint32_t U_LBO = 16 * 128;         // between k cores
 constexpr uint32_t U_SBO = 128;              // between row groups
 constexpr uint32_t U_SPIN = 1u << 22;
 constexpr int U_PROD_WARPS = 8;
-constexpr int U_THREADS = (U_PROD_WARPS + 1) * 32;
+constexpr int U_THREADS = (U_PROD_WARPS + 2) * 32;
 
 __device__ __forceinline__ uint32_t s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void bar_init(uint64_t* b, uint32_t count) {
@@ -122,33 +123,41 @@ __device__ __forceinline__ uint4 f32x8_to_f16(const float* src, int n, float sig
 }
 
 struct UmmaSmem {
-    uint8_t* stage[U_STAGES_MAX];
-    uint64_t* full;     // [stages] operands written (one arrival per producer warp)
+    uint8_t* stage;     // [U_STAGES][4 tiles]
+    uint8_t* act;       // [slots of activations]
+    uint64_t* full;     // [stages] weights written (one arrival per producer warp)
     uint64_t* empty;    // [stages] MMAs that read the stage have completed
+    uint64_t* afull;    // [slots] activations arrived
+    uint64_t* aempty;   // [slots] MMAs that read the slot have completed
     uint64_t* done;     // all MMAs of the tile have completed
     uint32_t* tptr;
     int* pair;          // [U_TN]
 };
-__device__ __forceinline__ UmmaSmem carve(uint8_t* smem, int tiles_per_stage, int stages) {
+__device__ __forceinline__ UmmaSmem carve(uint8_t* smem, uint32_t act_bytes) {
     UmmaSmem S;
-    for (int s = 0; s < U_STAGES_MAX; ++s) S.stage[s] = smem + (size_t)(s < stages ? s : 0) * tiles_per_stage * U_TILE;
-    uint8_t* o = smem + (size_t)stages * tiles_per_stage * U_TILE;
-    S.full = reinterpret_cast<uint64_t*>(o);
-    S.empty = S.full + U_STAGES_MAX;
-    S.done = S.empty + U_STAGES_MAX;
+    S.stage = smem;
+    S.act = smem + U_STAGES * 4 * U_TILE;
+    S.full = reinterpret_cast<uint64_t*>(S.act + act_bytes);
+    S.empty = S.full + U_STAGES;
+    S.afull = S.empty + U_STAGES;
+    S.aempty = S.afull + U_ACT_MAX;
+    S.done = S.aempty + U_ACT_MAX;
     S.tptr = reinterpret_cast<uint32_t*>(S.done + 1);
     S.pair = reinterpret_cast<int*>(S.tptr + 2);
     return S;
 }
-constexpr size_t umma_smem_bytes(int tiles_per_stage, int stages) { return (size_t)stages * tiles_per_stage * U_TILE + 128 + U_TN * 4; }
-constexpr int U_STAGES_GU = 2, U_STAGES_D = 2;
+// gate/up: x, 8 KB a chunk, four slots; down: h and its residual, 16 KB a chunk, three slots.  Two CTAs fit an SM either way.
+constexpr int U_ACT_GU = 4, U_ACT_D = 3;
+constexpr uint32_t U_ACT_GU_BYTES = U_ACT_GU * U_TILE, U_ACT_D_BYTES = U_ACT_D * 2 * U_TILE;
+constexpr size_t umma_smem_bytes(uint32_t act_bytes) { return (size_t)U_STAGES * 4 * U_TILE + act_bytes + 128 + U_TN * 4; }
 
 // common prologue: pair list, barriers, tensor memory
-__device__ __forceinline__ uint32_t umma_begin(const GroupedParams& p, const UmmaSmem& S, int slot, int first, int cnt, int cols, int full_count) {
+__device__ __forceinline__ uint32_t umma_begin(const GroupedParams& p, const UmmaSmem& S, int slot, int first, int cnt, int cols) {
     const int tid = threadIdx.x, warp = tid >> 5;
     if (tid < U_TN) S.pair[tid] = tid < cnt ? p.lists[(size_t)slot * p.T + first + tid] : -1;
     if (tid == 0) {
-        for (int s = 0; s < U_STAGES_MAX; ++s) { bar_init(&S.full[s], full_count); bar_init(&S.empty[s], 1); }
+        for (int s = 0; s < U_STAGES; ++s) { bar_init(&S.full[s], U_PROD_WARPS); bar_init(&S.empty[s], 1); }
+        for (int s = 0; s < U_ACT_MAX; ++s) { bar_init(&S.afull[s], 1); bar_init(&S.aempty[s], 1); }
         bar_init(S.done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -167,11 +176,60 @@ __device__ __forceinline__ void umma_end(uint32_t tmem, int cols) {
     if ((threadIdx.x >> 5) == U_PROD_WARPS)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
 }
+// lane 0 of the copy warp: the activations of every chunk, as slots become free
+__device__ __forceinline__ void fetch_activations(const UmmaSmem& S, const uint8_t* src, int n_chunks, int slots, uint32_t bytes, int32_t* status) {
+    for (int c = 0; c < n_chunks; ++c) {
+        const int sl = c % slots;
+        bar_wait(&S.aempty[sl], ((uint32_t)(c / slots) & 1) ^ 1, status);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s32(&S.afull[sl])), "r"(bytes) : "memory");
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(s32(S.act + sl * bytes)), "l"(src + (size_t)c * bytes), "r"(bytes), "r"(s32(&S.afull[sl])) : "memory");
+    }
+}
 // a producer warp has written its part of a stage
 __device__ __forceinline__ void stage_written(uint64_t* full) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes -> visible to the tensor core
     __syncwarp();
     if ((threadIdx.x & 31) == 0) bar_arrive(full);
+}
+
+// A producer thread: row r of the two operand tiles at `tile` of every stage, from 32 codes a chunk.  The loads run four chunks
+// ahead: with one, a chunk took as long as a load from memory.
+template <typename LC, typename LZ>
+__device__ __forceinline__ void produce(const UmmaSmem& S, int n_chunks, int gshift, int tile, int r, LC codes, LZ sz, int32_t* status) {
+    uint4 cw[U_AHEAD];
+    uint32_t nz[U_AHEAD];
+    auto starts = [&](int c) { return ((c * U_KC) & ((1 << gshift) - 1)) == 0; };      // a group of k begins with chunk c
+#pragma unroll
+    for (int j = 0; j < U_AHEAD; ++j) {                                  // (the chunks are a multiple of four)
+        cw[j] = codes(j);
+        nz[j] = starts(j) ? sz((j * U_KC) >> gshift) : 0u;
+    }
+    __half2 sc = __float2half2_rn(0.f), zr = sc;
+    for (int c0 = 0; c0 < n_chunks; c0 += U_AHEAD)
+#pragma unroll
+        for (int j = 0; j < U_AHEAD; ++j) {
+            const int c = c0 + j, st = c % U_STAGES;
+            const uint32_t w[4] = {cw[j].x, cw[j].y, cw[j].z, cw[j].w};
+            if (starts(c)) {
+                const __half2 a = u32_as_h2(nz[j]);
+                sc = __low2half2(a); zr = __high2half2(a);
+            }
+            if (c + U_AHEAD < n_chunks) {
+                cw[j] = codes(c + U_AHEAD);
+                if (starts(c + U_AHEAD)) nz[j] = sz(((c + U_AHEAD) * U_KC) >> gshift);
+            }
+            bar_wait(&S.empty[st], ((uint32_t)(c / U_STAGES) & 1) ^ 1, status);        // the MMAs that read this stage are done
+            uint8_t* sb = S.stage + (st * 4 + tile) * U_TILE;
+#pragma unroll
+            for (int kc = 0; kc < 4; ++kc) {
+                uint4 hi, lo;
+                dequant_hi_lo(w[kc], sc, zr, hi, lo);
+                *reinterpret_cast<uint4*>(sb + core_off(r, kc)) = hi;
+                *reinterpret_cast<uint4*>(sb + U_TILE + core_off(r, kc)) = lo;
+            }
+            stage_written(&S.full[st]);
+        }
 }
 
 // ---------------------------------------------------------------- token states as operand tiles
@@ -201,19 +259,19 @@ __global__ void __launch_bounds__(256) umma_gather_x_kernel(GroupedParams p) {
 }
 
 // ---------------------------------------------------------------- gate/up
-// stage = [gate hi][gate lo][up hi][up lo][x] (x by one bulk copy per chunk); tensor memory: gate in
+// stage = [gate hi][gate lo][up hi][up lo], x in slots of its own (one bulk copy per chunk); tensor memory: gate in
 // columns 0..127, up in 128..255.  Thread t dequantises row t % 128 of gate (t < 128) or up.
 __global__ void __launch_bounds__(U_THREADS, 2) umma_gate_up_kernel(GroupedParams p) {
     const int tile = blockIdx.y;             // row blocks of a tile are neighbours in the grid: they share its activations in L2
     if (tile >= *p.n_tiles) return;
     extern __shared__ __align__(128) uint8_t smem[];
-    const UmmaSmem S = carve(smem, 5, U_STAGES_GU);
+    const UmmaSmem S = carve(smem, U_ACT_GU_BYTES);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int slot = p.tiles[2 * tile], first = p.tiles[2 * tile + 1];
     const int cnt = min(U_TN, p.counts[slot] - first);
     const int row0 = blockIdx.x * 128;
     const uint8_t* rec = p.pool + (size_t)slot * p.L.bytes;
-    const uint32_t tmem = umma_begin(p, S, slot, first, cnt, 2 * U_TN, U_PROD_WARPS + 1);
+    const uint32_t tmem = umma_begin(p, S, slot, first, cnt, 2 * U_TN);
     const int n_chunks = p.H / U_KC;
     const int r_chunks = p.rank > 0 ? (p.rank + 31) / 32 : 0;          // adapter: chunks of up to 32 ranks
     const int gshift = 31 - __clz(p.group);
@@ -221,43 +279,12 @@ __global__ void __launch_bounds__(U_THREADS, 2) umma_gate_up_kernel(GroupedParam
     if (warp < U_PROD_WARPS) {
         const int r = tid & 127, half = tid >> 7;                    // weight row; matrix (0 gate, 1 up) and, in the epilogue, half of the columns
         const int pair = S.pair[r];
-        const uint8_t* xq = p.xq + (size_t)tile * (p.H / 32) * U_TILE;
         const uint8_t* cp = rec + (half ? p.L.codes_up : p.L.codes_gate);
         const uint8_t* zp = rec + (half ? p.L.sz_up : p.L.sz_gate);
-        uint4 cw = ld_stream16(cp + code_off(p.H, row0 + r, 0));
-        const int n_groups = p.H >> gshift;
-        uint32_t nsz = ld_stream4(zp + sz_off(p.H, p.group, row0 + r, 0));      // (scale, zero) one group ahead
-        __half2 sc = __float2half2_rn(0.f), zr = sc;
-        for (int c = 0; c < n_chunks; ++c) {
-            const int st = c % U_STAGES_GU;
-            const uint32_t use = (uint32_t)(c / U_STAGES_GU);
-            uint4 nw = cw;
-            if (c + 1 < n_chunks) nw = ld_stream16(cp + code_off(p.H, row0 + r, c + 1));   // in flight during this chunk
-            if (((c * U_KC) & (p.group - 1)) == 0) {                 // a new group: its (scale, zero), and the load of the next
-                const __half2 a = u32_as_h2(nsz);
-                sc = __low2half2(a); zr = __high2half2(a);
-                nsz = ld_stream4(zp + sz_off(p.H, p.group, row0 + r, min(((c * U_KC) >> gshift) + 1, n_groups - 1)));
-            }
-            bar_wait(&S.empty[st], (use & 1) ^ 1, p.status);          // the MMAs that read this stage are done
-            uint8_t* sb = S.stage[st];
-            if (tid == 0) {
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s32(&S.full[st])), "r"(U_TILE) : "memory");
-                asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                             ::"r"(s32(sb + 4 * U_TILE)), "l"(xq + (size_t)c * U_TILE), "r"(U_TILE), "r"(s32(&S.full[st])) : "memory");
-            }
-            const uint32_t w[4] = {cw.x, cw.y, cw.z, cw.w};
-#pragma unroll
-            for (int kc = 0; kc < 4; ++kc) {
-                uint4 hi, lo;
-                dequant_hi_lo(w[kc], sc, zr, hi, lo);
-                *reinterpret_cast<uint4*>(sb + (2 * half) * U_TILE + core_off(r, kc)) = hi;
-                *reinterpret_cast<uint4*>(sb + (2 * half + 1) * U_TILE + core_off(r, kc)) = lo;
-            }
-            stage_written(&S.full[st]);
-            cw = nw;
-        }
+        produce(S, n_chunks, gshift, 2 * half, r, [&](int c) { return ld_stream16(cp + code_off(p.H, row0 + r, c)); },
+                [&](int g) { return ld_stream4(zp + sz_off(p.H, p.group, row0 + r, g)); }, p.status);
         // the adapter as extra k: A = B_gate / B_up rows (fp16 of bf16), B = sigma * (A_gate x) / sigma * (A_up x);
-        // the threads of matrix m write its A rows and its B rows (gate's B in slot 4, up's in slot 1)
+        // the threads of matrix m write its A rows and its B rows (gate's B in tile 3, up's in tile 1)
         if (r_chunks > 0) {
             const int first_pair = S.pair[0];
             const int ad = first_pair >= 0 ? p.pair_ad[first_pair] : 0;
@@ -266,19 +293,18 @@ __global__ void __launch_bounds__(U_THREADS, 2) umma_gate_up_kernel(GroupedParam
             if (pair >= 0) um = p.u_gu + (((size_t)(pair / p.K) * n_sets + (p.n_adapters == 1 ? 0 : pair % p.K)) * 2 + half) * p.rank;
             const uint16_t* Bm = reinterpret_cast<const uint16_t*>(half ? p.lora.B_up : p.lora.B_gate) + ((size_t)ad * p.I + row0 + r) * p.rank;
             for (int rc = 0; rc < r_chunks; ++rc) {
-                const int c = n_chunks + rc, st = c % U_STAGES_GU;
-                const uint32_t use = (uint32_t)(c / U_STAGES_GU);
+                const int c = n_chunks + rc, st = c % U_STAGES;
+                const uint32_t use = (uint32_t)(c / U_STAGES);
                 bar_wait(&S.empty[st], (use & 1) ^ 1, p.status);
-                uint8_t* sb = S.stage[st];
+                uint8_t* sb = S.stage + st * 4 * U_TILE;
 #pragma unroll
                 for (int kc = 0; kc < 4; ++kc) {
                     const int j0 = rc * 32 + kc * 8, n = p.rank - j0;          // rank is a multiple of 8
                     uint4 a = make_uint4(0, 0, 0, 0);
                     if (n > 0) a = bf16x8_to_f16(*reinterpret_cast<const uint4*>(Bm + j0));
                     *reinterpret_cast<uint4*>(sb + (2 * half) * U_TILE + core_off(r, kc)) = a;
-                    *reinterpret_cast<uint4*>(sb + (half ? 1 : 4) * U_TILE + core_off(r, kc)) = f32x8_to_f16(um != nullptr ? um + j0 : nullptr, n, p.sigma);
+                    *reinterpret_cast<uint4*>(sb + (half ? 1 : 3) * U_TILE + core_off(r, kc)) = f32x8_to_f16(um != nullptr ? um + j0 : nullptr, n, p.sigma);
                 }
-                if (tid == 0) bar_arrive(&S.full[st]);               // stands in for the bulk copy's arrival
                 stage_written(&S.full[st]);
             }
         }
@@ -311,36 +337,40 @@ __global__ void __launch_bounds__(U_THREADS, 2) umma_gate_up_kernel(GroupedParam
                 }
             }
         }
+    } else if (warp == U_PROD_WARPS + 1) {
+        if (lane == 0) fetch_activations(S, p.xq + (size_t)tile * (p.H / 32) * U_TILE, n_chunks, U_ACT_GU, U_TILE, p.status);
     } else if (lane == 0) {
         // ---- the MMA issuer.  Descriptors differ only in their address field: base + offset >> 4.
         const uint32_t idesc = umma_idesc((cnt + 15) & ~15);
-        const uint64_t d0 = umma_desc(s32(S.stage[0]));
-        constexpr uint64_t kTile = U_TILE >> 4, kStep = (2 * U_LBO) >> 4, kStage = (5 * U_TILE) >> 4;
+        const uint64_t d0 = umma_desc(s32(S.stage)), a0 = umma_desc(s32(S.act));
+        constexpr uint64_t kTile = U_TILE >> 4, kStep = (2 * U_LBO) >> 4, kStage = (4 * U_TILE) >> 4;
         const uint32_t tg = tmem, tu = tmem + U_TN;
         for (int c = 0; c < n_chunks; ++c) {
-            const int st = c % U_STAGES_GU;
-            bar_wait(&S.full[st], (uint32_t)(c / U_STAGES_GU) & 1, p.status);
+            const int st = c % U_STAGES, sl = c % U_ACT_GU;
+            bar_wait(&S.full[st], (uint32_t)(c / U_STAGES) & 1, p.status);
+            bar_wait(&S.afull[sl], (uint32_t)(c / U_ACT_GU) & 1, p.status);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t ds = d0 + st * kStage;
+            const uint64_t ds = d0 + st * kStage, as = a0 + sl * kTile;
 #pragma unroll
             for (int ks = 0; ks < U_KC / 16; ++ks) {
-                const uint64_t dk = ds + ks * kStep, db = dk + 4 * kTile;
+                const uint64_t dk = ds + ks * kStep, db = as + ks * kStep;
                 umma(tg, dk, db, idesc, c > 0 || ks > 0);
                 umma(tg, dk + kTile, db, idesc, true);
                 umma(tu, dk + 2 * kTile, db, idesc, c > 0 || ks > 0);
                 umma(tu, dk + 3 * kTile, db, idesc, true);
             }
             umma_commit(&S.empty[st]);
+            umma_commit(&S.aempty[sl]);
         }
         for (int rc = 0; rc < r_chunks; ++rc) {
-            const int c = n_chunks + rc, st = c % U_STAGES_GU;
-            bar_wait(&S.full[st], (uint32_t)(c / U_STAGES_GU) & 1, p.status);
+            const int c = n_chunks + rc, st = c % U_STAGES;
+            bar_wait(&S.full[st], (uint32_t)(c / U_STAGES) & 1, p.status);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint64_t ds = d0 + st * kStage;
             const int ksteps = min(2, (p.rank - rc * 32 + 15) / 16);
             for (int ks = 0; ks < ksteps; ++ks) {
                 const uint64_t dk = ds + ks * kStep;
-                umma(tg, dk, dk + 4 * kTile, idesc, true);
+                umma(tg, dk, dk + 3 * kTile, idesc, true);
                 umma(tu, dk + 2 * kTile, dk + kTile, idesc, true);
             }
             umma_commit(&S.empty[st]);
@@ -352,60 +382,30 @@ __global__ void __launch_bounds__(U_THREADS, 2) umma_gate_up_kernel(GroupedParam
 
 // ---------------------------------------------------------------- down
 // A CTA covers 256 output rows (two accumulators of 128 columns in tensor memory) for the tile's tokens:
-// stage = [W0 hi][W0 lo][W1 hi][W1 lo][h hi][h lo], the h tiles arriving by one bulk copy per chunk
-// (written in operand order by the gate/up kernel), thread t dequantising row t of the 256.
+// stage = [W0 hi][W0 lo][W1 hi][W1 lo], thread t dequantising row t of the 256; [h hi][h lo] in slots of their own, one bulk copy
+// per chunk (written in operand order by the gate/up kernel).
 // o = gate weight * (W h + sigma B (A h))
 __global__ void __launch_bounds__(U_THREADS, 2) umma_down_kernel(GroupedParams p) {
     const int tile = blockIdx.y;             // row blocks of a tile are neighbours in the grid: they share its activations in L2
     if (tile >= *p.n_tiles) return;
     extern __shared__ __align__(128) uint8_t smem[];
-    const UmmaSmem S = carve(smem, 6, U_STAGES_D);
+    const UmmaSmem S = carve(smem, U_ACT_D_BYTES);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int slot = p.tiles[2 * tile], first = p.tiles[2 * tile + 1];
     const int cnt = min(U_TN, p.counts[slot] - first);
     const int row0 = blockIdx.x * 256;
     const uint8_t* rec = p.pool + (size_t)slot * p.L.bytes;
-    const uint32_t tmem = umma_begin(p, S, slot, first, cnt, 2 * U_TN, U_PROD_WARPS + 1);
+    const uint32_t tmem = umma_begin(p, S, slot, first, cnt, 2 * U_TN);
     const int n_chunks = p.I / U_KC;
     const int r_chunks = p.rank > 0 ? (p.rank + 31) / 32 : 0;
     const int gshift = 31 - __clz(p.group);
 
     if (warp < U_PROD_WARPS) {
         const int r = tid & 127, m = tid >> 7;                       // row r of half m: output row row0 + tid
-        const uint8_t* hq = p.hq + (size_t)tile * (p.I / 32) * 2 * U_TILE;
         const uint8_t* cdp = rec + p.L.codes_down;
-        uint4 cd = ld_stream16(cdp + down_code_off(p.H, p.I, row0 + tid, 0));
-        const int n_groups = p.I >> gshift;
-        uint32_t nsz = ld_stream4(rec + p.L.sz_down + down_sz_off(p.H, p.I, p.group, row0 + tid, 0));
-        __half2 sd = __float2half2_rn(0.f), zd = sd;
-        for (int c = 0; c < n_chunks; ++c) {
-            const int st = c % U_STAGES_D;
-            const uint32_t use = (uint32_t)(c / U_STAGES_D);
-            uint4 nd = cd;
-            if (c + 1 < n_chunks) nd = ld_stream16(cdp + down_code_off(p.H, p.I, row0 + tid, c + 1));
-            if (((c * U_KC) & (p.group - 1)) == 0) {
-                const __half2 a = u32_as_h2(nsz);
-                sd = __low2half2(a); zd = __high2half2(a);
-                nsz = ld_stream4(rec + p.L.sz_down + down_sz_off(p.H, p.I, p.group, row0 + tid, min(((c * U_KC) >> gshift) + 1, n_groups - 1)));
-            }
-            bar_wait(&S.empty[st], (use & 1) ^ 1, p.status);
-            uint8_t* sb = S.stage[st];
-            if (tid == 0) {
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s32(&S.full[st])), "r"(2 * U_TILE) : "memory");
-                asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                             ::"r"(s32(sb + 4 * U_TILE)), "l"(hq + (size_t)c * 2 * U_TILE), "r"(2 * U_TILE), "r"(s32(&S.full[st])) : "memory");
-            }
-            const uint32_t wd[4] = {cd.x, cd.y, cd.z, cd.w};
-#pragma unroll
-            for (int kc = 0; kc < 4; ++kc) {
-                uint4 hi, lo;
-                dequant_hi_lo(wd[kc], sd, zd, hi, lo);
-                *reinterpret_cast<uint4*>(sb + (2 * m) * U_TILE + core_off(r, kc)) = hi;
-                *reinterpret_cast<uint4*>(sb + (2 * m + 1) * U_TILE + core_off(r, kc)) = lo;
-            }
-            stage_written(&S.full[st]);
-            cd = nd;
-        }
+        const float my_gate = m == 0 && S.pair[r] >= 0 ? p.gates[S.pair[r]] : 0.f;
+        produce(S, n_chunks, gshift, 2 * m, r, [&](int c) { return ld_stream16(cdp + down_code_off(p.H, p.I, row0 + tid, c)); },
+                [&](int g) { return ld_stream4(rec + p.L.sz_down + down_sz_off(p.H, p.I, p.group, row0 + tid, g)); }, p.status);
         if (r_chunks > 0) {
             const int first_pair = S.pair[0];
             const int ad = first_pair >= 0 ? p.pair_ad[first_pair] : 0;
@@ -413,25 +413,27 @@ __global__ void __launch_bounds__(U_THREADS, 2) umma_down_kernel(GroupedParams p
             const float* ud = (m == 0 && pair >= 0) ? p.u_d + (size_t)pair * p.rank : nullptr;
             const uint16_t* Bd = reinterpret_cast<const uint16_t*>(p.lora.B_down) + ((size_t)ad * p.H + row0 + tid) * p.rank;
             for (int rc = 0; rc < r_chunks; ++rc) {
-                const int c = n_chunks + rc, st = c % U_STAGES_D;
-                const uint32_t use = (uint32_t)(c / U_STAGES_D);
+                const int c = n_chunks + rc, st = c % U_STAGES;
+                const uint32_t use = (uint32_t)(c / U_STAGES);
                 bar_wait(&S.empty[st], (use & 1) ^ 1, p.status);
-                uint8_t* sb = S.stage[st];
+                uint8_t* sb = S.stage + st * 4 * U_TILE;
 #pragma unroll
                 for (int kc = 0; kc < 4; ++kc) {
                     const int j0 = rc * 32 + kc * 8, n = p.rank - j0;
                     uint4 a = make_uint4(0, 0, 0, 0);
                     if (n > 0) a = bf16x8_to_f16(*reinterpret_cast<const uint4*>(Bd + j0));
                     *reinterpret_cast<uint4*>(sb + (2 * m) * U_TILE + core_off(r, kc)) = a;
-                    if (m == 0) *reinterpret_cast<uint4*>(sb + 4 * U_TILE + core_off(r, kc)) = f32x8_to_f16(ud != nullptr ? ud + j0 : nullptr, n, p.sigma);
+                    if (m == 0) *reinterpret_cast<uint4*>(sb + U_TILE + core_off(r, kc)) = f32x8_to_f16(ud != nullptr ? ud + j0 : nullptr, n, p.sigma);
                 }
-                if (tid == 0) bar_arrive(&S.full[st]);               // stands in for the bulk copy's arrival
                 stage_written(&S.full[st]);
             }
         }
         // ---- epilogue: o[pair][row] = gate weight * acc; thread t = row t, accumulator t / 128
         bar_wait(S.done, 0, p.status);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        float* gate = reinterpret_cast<float*>(S.act);               // (the activations have been used)
+        if (m == 0) gate[r] = my_gate;
+        asm volatile("bar.sync 1, %0;" ::"n"(U_PROD_WARPS * 32) : "memory");
         const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + m * U_TN;
         for (int c0 = 0; c0 < cnt; c0 += 32) {
             uint32_t v[32];
@@ -440,21 +442,24 @@ __global__ void __launch_bounds__(U_THREADS, 2) umma_down_kernel(GroupedParams p
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
                 const int pr = (c0 + j) < cnt ? S.pair[c0 + j] : -1;
-                if (pr >= 0) p.o[(size_t)pr * p.H + row0 + tid] = p.gates[pr] * __uint_as_float(v[j]);
+                if (pr >= 0) p.o[(size_t)pr * p.H + row0 + tid] = gate[c0 + j] * __uint_as_float(v[j]);
             }
         }
+    } else if (warp == U_PROD_WARPS + 1) {
+        if (lane == 0) fetch_activations(S, p.hq + (size_t)tile * (p.I / 32) * 2 * U_TILE, n_chunks, U_ACT_D, 2 * U_TILE, p.status);
     } else if (lane == 0) {
         const uint32_t idesc = umma_idesc((cnt + 15) & ~15);
-        const uint64_t d0 = umma_desc(s32(S.stage[0]));
-        constexpr uint64_t kTile = U_TILE >> 4, kStep = (2 * U_LBO) >> 4, kStage = (6 * U_TILE) >> 4;
+        const uint64_t d0 = umma_desc(s32(S.stage)), a0 = umma_desc(s32(S.act));
+        constexpr uint64_t kTile = U_TILE >> 4, kStep = (2 * U_LBO) >> 4, kStage = (4 * U_TILE) >> 4;
         for (int c = 0; c < n_chunks; ++c) {
-            const int st = c % U_STAGES_D;
-            bar_wait(&S.full[st], (uint32_t)(c / U_STAGES_D) & 1, p.status);
+            const int st = c % U_STAGES, sl = c % U_ACT_D;
+            bar_wait(&S.full[st], (uint32_t)(c / U_STAGES) & 1, p.status);
+            bar_wait(&S.afull[sl], (uint32_t)(c / U_ACT_D) & 1, p.status);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t ds = d0 + st * kStage;
+            const uint64_t ds = d0 + st * kStage, as = a0 + sl * 2 * kTile;
 #pragma unroll
             for (int ks = 0; ks < U_KC / 16; ++ks) {
-                const uint64_t w0 = ds + ks * kStep, hhi = w0 + 4 * kTile;
+                const uint64_t w0 = ds + ks * kStep, hhi = as + ks * kStep;
 #pragma unroll
                 for (int m = 0; m < 2; ++m) {
                     const uint64_t whi = w0 + 2 * m * kTile;
@@ -464,17 +469,18 @@ __global__ void __launch_bounds__(U_THREADS, 2) umma_down_kernel(GroupedParams p
                 }
             }
             umma_commit(&S.empty[st]);
+            umma_commit(&S.aempty[sl]);
         }
         for (int rc = 0; rc < r_chunks; ++rc) {
-            const int c = n_chunks + rc, st = c % U_STAGES_D;
-            bar_wait(&S.full[st], (uint32_t)(c / U_STAGES_D) & 1, p.status);
+            const int c = n_chunks + rc, st = c % U_STAGES;
+            bar_wait(&S.full[st], (uint32_t)(c / U_STAGES) & 1, p.status);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint64_t ds = d0 + st * kStage;
             const int ksteps = min(2, (p.rank - rc * 32 + 15) / 16);
             for (int ks = 0; ks < ksteps; ++ks) {
                 const uint64_t w0 = ds + ks * kStep;
-                umma(tmem, w0, w0 + 4 * kTile, idesc, true);
-                umma(tmem + U_TN, w0 + 2 * kTile, w0 + 4 * kTile, idesc, true);
+                umma(tmem, w0, w0 + kTile, idesc, true);
+                umma(tmem + U_TN, w0 + 2 * kTile, w0 + kTile, idesc, true);
             }
             umma_commit(&S.empty[st]);
         }
@@ -492,23 +498,23 @@ bool umma_grouped_supported(const edg_layer_desc& d) {
 cudaError_t launch_umma_gate_up(const GroupedParams& p, int max_tiles, cudaStream_t st) {
     static bool configured = false;
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(umma_gate_up_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umma_smem_bytes(5, U_STAGES_GU));
+        cudaError_t e = cudaFuncSetAttribute(umma_gate_up_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umma_smem_bytes(U_ACT_GU_BYTES));
         if (e != cudaSuccess) return e;
         configured = true;
     }
     umma_gather_x_kernel<<<dim3(8, max_tiles), 256, 0, st>>>(p);
-    umma_gate_up_kernel<<<dim3(p.I / 128, max_tiles), U_THREADS, umma_smem_bytes(5, U_STAGES_GU), st>>>(p);
+    umma_gate_up_kernel<<<dim3(p.I / 128, max_tiles), U_THREADS, umma_smem_bytes(U_ACT_GU_BYTES), st>>>(p);
     return cudaGetLastError();
 }
 
 cudaError_t launch_umma_down(const GroupedParams& p, int max_tiles, cudaStream_t st) {
     static bool configured = false;
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(umma_down_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umma_smem_bytes(6, U_STAGES_D));
+        cudaError_t e = cudaFuncSetAttribute(umma_down_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umma_smem_bytes(U_ACT_D_BYTES));
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    umma_down_kernel<<<dim3(p.H / 256, max_tiles), U_THREADS, umma_smem_bytes(6, U_STAGES_D), st>>>(p);
+    umma_down_kernel<<<dim3(p.H / 256, max_tiles), U_THREADS, umma_smem_bytes(U_ACT_D_BYTES), st>>>(p);
     return cudaGetLastError();
 }
 
