@@ -63,7 +63,7 @@ struct StepParams {
     const uint8_t* shared_rec;
     void* y;
     int32_t* status;
-    int32_t *pre_counter, *done;              // the ring's counters in the control block
+    int32_t* done;                            // readers of a ring slot, in the control block
     float* logits_ws;                         // [ring][E + kPairWords]
     const void* W_pre;
     int32_t* inds_next;
@@ -1000,7 +1000,6 @@ int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* 
     const WorkspaceLayout W = workspace_layout(*d, 1);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     p.status = reinterpret_cast<int32_t*>(ws + W.ctrl);
-    p.pre_counter = reinterpret_cast<int32_t*>(ws + W.ctrl + kCtrlHead);
     p.done = reinterpret_cast<int32_t*>(ws + W.ctrl + kCtrlDone);
     p.logits_ws = reinterpret_cast<float*>(ws + W.logits);
     p.W_pre = W_pre; p.inds_next = inds_next; p.gates_next = gates_next; p.logits_next = logits_next; p.inds_mirror = ex.inds_mirror;
