@@ -76,16 +76,21 @@ __host__ __device__ inline RecordLayout record_layout(int H, int I, int group) {
 // Workspace layout for T tokens (floats unless noted).  The first kCtrlBytes bytes are a control
 // block that must start out zero: its first int32 is the device-side status word, the rest are the
 // counters of the ring that chained batch-1 layer-steps share (arrivals of the reduce, head rows
-// delivered, reducers finished -- one set per ring slot).
+// delivered, reducers finished -- one set per ring slot), and what the latency form of the step counts.  It is all that a
+// call takes over from the calls before it, whatever their shape and T; what the links of a chain hand to one another
+// lies in front of everything that depends on T.
 constexpr int kPairWords = 64;         // words behind the logits of a ring slot: 32 (expert, gate) pairs, the routing itself
 constexpr int kHandoffRing = 128;      // ring slots shared by chained batch-1 layer-steps in flight
-constexpr int kDepWords = 16;           // words per ring slot of the dependent chain: 4 sums of squares, 4 "rows written" flags, a counter
+constexpr int kDepWords = 16;           // words per ring slot of the dependent chain: 4 sums of squares, 4 "rows written" flags
 constexpr size_t kCtrlBytes = 4096;    // control block: status word at 0, then the ring's counters
 constexpr size_t kCtrlCounters = 64;                               // [ring][4] arrivals per block of output rows
 constexpr size_t kCtrlHead = kCtrlCounters + kHandoffRing * 16;    // [ring] head rows delivered
 constexpr size_t kCtrlDone = kCtrlHead + kHandoffRing * 4;         // [ring] reducers finished
 constexpr size_t kCtrlNorm = kCtrlDone + kHandoffRing * 4;         // [ring] reducers that have delivered their sum of squares (dependent chain)
-static_assert(kCtrlNorm + kHandoffRing * 4 <= kCtrlBytes, "control block too small");
+constexpr size_t kCtrlStarts = kCtrlNorm + kHandoffRing * 4 + 64;  // start counter of the latency form, on a line of its own
+constexpr int kStepBufs = 4, kStepDeferWords = 8;                  // links of a dependent chain in flight (and one to spare); units, one bit each
+constexpr size_t kCtrlDefer = kCtrlStarts + 128;                   // [kStepBufs][kStepDeferWords] units left to the CTA that starts last
+static_assert(kCtrlStarts % 128 == 0 && kCtrlDefer + kStepBufs * kStepDeferWords * 4 <= kCtrlBytes, "control block too small");
 
 struct WorkspaceLayout {
     size_t ctrl;      // kCtrlBytes control block
@@ -115,13 +120,10 @@ struct WorkspaceLayout {
     size_t g_xq;      // [tiles][cap * H] fp16      : token states in operand order
     size_t g_hq;      // [tiles][2 * cap * I] fp16  : h, value and residual, in operand order
     // the form of the batch-1 step that runs alone or as a link of a dependent chain (edg_step.cu):
-    size_t step;      // kStepCtrlBytes: start counter at 0, lists of deferred units from kStepDeferOff (starts as zeros)
-    size_t step_x;    // exchange buffers: h and A_down h partials (4 of them), x + y (16); a word not written holds 0xFFFFFFFF
+    size_t step_x;    // [kStepBufs] exchange buffers: h and A_down h partials, A x, logits; then [kStepBufs] of x + y
     size_t bytes;
 };
 
-constexpr int kStepStates = 16;
-constexpr size_t kStepDeferOff = 256, kStepCtrlBytes = kStepDeferOff + kStepStates * (2048 / 16 + 4) * 4;
 int sm_count();
 size_t step_region_words(const edg_layer_desc& d);
 size_t step_exchange_words(const edg_layer_desc& d);
@@ -142,17 +144,16 @@ inline WorkspaceLayout workspace_layout(const edg_layer_desc& d, int T) {
     const size_t n_sets = d.n_adapters == 1 ? 1 : (size_t)d.K;
     const size_t r = d.rank > 0 ? (size_t)d.rank : 1;
     W.ctrl = 0;
-    W.u_gu = kCtrlBytes;
-    W.h = round_up(W.u_gu + (size_t)T * n_sets * 2 * r * sizeof(float), 256);
-    W.u_d = round_up(W.h + (size_t)T * d.K * d.I * sizeof(float), 256);
-    W.logits = round_up(W.u_d + (size_t)T * d.K * r * sizeof(float), 256);
+    W.logits = kCtrlBytes;
     W.dep = round_up(W.logits + (size_t)kHandoffRing * (d.E + kPairWords) * sizeof(float), 256);
     W.partial = round_up(W.dep + (size_t)kHandoffRing * kDepWords * sizeof(float), 256);
     const size_t one_set = (size_t)kDownSlices * (d.K + 1) * d.H * sizeof(float);   // K routed experts and the shared expert
     W.lone_bytes = W.partial + one_set;
-    size_t end = round_up(W.partial + (size_t)kHandoffRing * one_set, 256);
-    W.step = end;     end = round_up(W.step + kStepCtrlBytes, 256);
-    W.step_x = end;   end = round_up(W.step_x + step_region_words(d) * sizeof(float), 256);
+    W.step_x = round_up(W.partial + (size_t)kHandoffRing * one_set, 256);
+    W.u_gu = round_up(W.step_x + step_region_words(d) * sizeof(float), 256);
+    W.h = round_up(W.u_gu + (size_t)T * n_sets * 2 * r * sizeof(float), 256);
+    W.u_d = round_up(W.h + (size_t)T * d.K * d.I * sizeof(float), 256);
+    size_t end = round_up(W.u_d + (size_t)T * d.K * r * sizeof(float), 256);
     W.o = W.pair_slot = W.pair_ad = W.counts = W.n_tiles = W.tiles = W.lists = W.hq = W.xq = end;
     W.g_tiles = W.g_done = W.g_order = W.g_cnt = W.g_u = W.g_xq = W.g_hq = end;
     if (T > 1) {
@@ -202,7 +203,7 @@ unsigned long long* trace_buffer();      // set by edg_set_trace_buffer, or null
 bool step_supported(const edg_layer_desc& d, bool shared);
 int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* slots, const int32_t* table, const int32_t* experts,
                  const float* gates, const void* x, const edg_lora* lora, void* y, const void* W_pre, int32_t* inds_next, float* gates_next,
-                 float* logits_next, void* workspace, int flag_in, int flag_out, int stale, cudaStream_t st, const FusedExtras& extras);
+                 float* logits_next, void* workspace, int flag_in, int flag_out, int pos, cudaStream_t st, const FusedExtras& extras);
 // One fused launch for a batch-1 layer-step (edg_decode_fused.cu).  W_pre may be null (no prediction).
 int32_t run_fused_layer(const edg_layer_desc* d, const void* slot_pool, const int32_t* slots, const int32_t* table,
                         const int32_t* experts, const float* gates, const void* x, const edg_lora* lora, void* y,

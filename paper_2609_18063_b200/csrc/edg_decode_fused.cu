@@ -149,7 +149,7 @@ struct FusedParams {
     int stale;                    // -1, or a ring slot whose unread logits this (unchained) call clears
     int32_t* inds_mirror;         // [K] copy of inds_next in mapped pinned host memory, or null
     uint16_t* x_next;             // [H] bf16 or null: bf16(rmsnorm(x + y)), the next layer-step's hidden state in a dependent chain
-    float* dep_ws;                // [kRing][kDepWords]: per ring slot, kC partial sums of squares, (words 4..7) the reducers' "my rows of x_next are written" flags, (word 8) a counter
+    float* dep_ws;                // [kRing][kDepWords]: per ring slot, kC partial sums of squares, (words 4..7) the reducers' "my rows of x_next are written" flags
     int32_t* norm_cnt;            // [kRing] reducers that have delivered their sum of squares
     float eps;
     int head_extra;               // CTAs behind those of the experts that evaluate the head and nothing else (0: the first CTAs of the grid do)
@@ -1176,7 +1176,6 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
             //      sums are there -- the reducers are running CTAs that publish before they wait --, adds
             //      them in a fixed order and normalises the rows it still holds in registers.  The last one
             //      to have written its rows raises the flag the next step waits for.
-            int32_t* norm_done = reinterpret_cast<int32_t*>(p.dep_ws + p.ring * kDepWords + 8);
             ss = warp_sum(ss);
             if (lane == 0) s_red[warp] = ss;
             __syncthreads();
@@ -1186,11 +1185,11 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                 st_relaxed_gpu_u32(p.dep_ws + p.ring * kDepWords + crank, __float_as_uint(tot));
                 int seen = atom_add_acq_rel_gpu(&p.norm_cnt[p.ring], 1) + 1;
                 uint32_t it = 0;
-                while (seen < kC && ++it < kSpinLimit) {
+                while ((seen & 0xFF) < kC && ++it < kSpinLimit) {
                     __nanosleep(20);
                     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(p.norm_cnt + p.ring) : "memory");
                 }
-                if (seen < kC) atomicExch(p.status, EDG_E_TIMEOUT);
+                if ((seen & 0xFF) < kC) atomicExch(p.status, EDG_E_TIMEOUT);
                 float all = 0.f;
                 for (int c = 0; c < kC; ++c) all += __uint_as_float(ld_relaxed_gpu_u32(p.dep_ws + p.ring * kDepWords + c));
                 s_red[kFW] = rsqrtf(all / (float)p.H + p.eps);
@@ -1209,11 +1208,9 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                 // (the release covers the rows every thread of this CTA wrote before the barrier)
                 asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.dep_ws + p.ring * kDepWords + 4 + crank), "r"(1u) : "memory");
                 trace_stamp(p, 21);
-                // off the critical path: the last reducer past the exchange of sums resets its counters
-                if (atom_add_acq_rel_gpu(norm_done, 1) == kC - 1) {
-                    st_relaxed_gpu(p.norm_cnt + p.ring, 0);
-                    st_relaxed_gpu(norm_done, 0);
-                }
+                // off the critical path: the last reducer past the exchange of sums resets the counter (arrivals in its low byte,
+                // reducers past the exchange above it)
+                if (atom_add_acq_rel_gpu(&p.norm_cnt[p.ring], 256) >> 8 == kC - 1) st_relaxed_gpu(p.norm_cnt + p.ring, 0);
             }
         }
         if (p.flag_in >= 0) {

@@ -27,13 +27,18 @@
 // Of the 11.8 us the two exchanges take 5.5 (a store, a poll under way, a poll that sees it, the slowest of 128), the
 // arithmetic of gate/up 1.7, of down 1.5.
 //
-// Waiting is safe without a cooperative launch: a CTA may wait for the h of others only when all CTAs of its grid have
-// started (a counter says so; it is also the epoch that names the exchange buffers).  One that finds
-// its grid not fully resident for a while -- other grids hold the SMs -- leaves its down rows to the CTA that starts last.
+// Waiting is safe without a cooperative launch: a CTA reads the words of others only when all CTAs of its grid have
+// started and cleared what they will publish (a counter in the control block says so).  One that finds its grid not fully resident for a while -- other grids hold the
+// SMs -- leaves its down rows to the CTA that starts last.
+// Nothing in the exchange buffers is taken over from a launch before: ahead of counting itself in, a CTA sets the words that it
+// will publish to "not yet", a store or two per lane while the routing is on its way.  So it does not matter what the workspace
+// held -- a prompt's scratch, the buffers of another layer shape, zeros --; the control block is all that has to last.
 //
 // The order of every sum is that of the throughput form of the layer kernel with four clusters per expert: per row four
 // chains over K, per (expert, quarter of I) one partial with its adapter delta, partials summed in order.  A chain of
 // dependent steps (EX = false: biased codes, edg_mma.cuh) therefore reproduces the results of earlier versions bit for bit.
+#include <type_traits>
+
 #include "edg_mma.cuh"
 #include "edg_head.cuh"
 
@@ -46,7 +51,7 @@ constexpr int kStepMaxK = 16;
 constexpr int kStepMaxRank = 64;
 constexpr uint32_t kEpochStarts = 8192;       // what one grid adds to the start counter in total
 constexpr uint32_t kWaitStarted = 256;        // polls before a CTA whose grid is not fully resident gives its rows away
-constexpr int kStepBufs = 4, kStateCopies = 8, kHCopies = 4;
+constexpr int kStateCopies = 8, kHCopies = 4;
 
 // byte offsets in shared memory; h .. udi lie inside the union, used once the gate/up weights are
 struct StepSmem {
@@ -70,21 +75,22 @@ struct StepParams {
     float *gates_next, *logits_next;
     int32_t* inds_mirror;
     uint16_t* x_next;
-    unsigned long long* trace;                // (this form is not traced: null)
-    uint32_t* starts;                         // the start counter
-    float* hx;                                // [kStepBufs][hx_words]: kHCopies of (h; the A_down h partials of every expert CTA); the A x partials; head logits
-    float* vx;                                // [kStepStates][kStateCopies][H]: x + y of a dependent chain
-    int32_t* defer;                           // [kStepStates][H/16 + 4]: number, then (unit + 1) of those left to the last starter
-    uint32_t hx_words, hc_words, ud_off, ux_off, lx_off;
+    uint32_t *starts, *ready;                 // CTAs that have started; that have cleared their words
+    float* hx;                                // this link's exchange buffer: kHCopies of (h; the A_down h partials of every expert CTA); the A x partials; head logits
+    float *vx, *vx_in;                        // [kStateCopies][H]: x + y of a dependent chain, of this link and of the one before it
+    uint32_t* defer;                          // [kStepDeferWords]: units left to the CTA that starts last, a bit each
+    uint32_t hc_words, ud_off, ux_off, lx_off;
     int I, E, K, Kt, group, gshift, rank, rank_shared, rmax, n_adapters, n_slots, pre_dtype, out_dtype;
     int cta_route, cta_state;                 // CTAs that compute the routing for the next step and the caller's x_next, or -1
     int n_gu, n_dn, n_exp, n_head, n_headc;   // CTAs with gate/up, with down work, the larger of both; tiles of the head, CTAs for them
-    int flag_in, flag_out, stale, dep;        // dep: x arrives in band from the step before
+    int head_tile;                            // rows of a tile of the head
+    int flag_in, flag_out, dep;               // dep: x arrives in band from the step before
     float sigma, eps;
     RecordLayout L;
     StepSmem S;
 };
 
+__device__ __forceinline__ void trace_stamp(const StepParams&, int) {}                   // (this form is not traced)
 __device__ __forceinline__ void cp16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
@@ -199,12 +205,26 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
     constexpr int MP = CPB == 2 ? 2 : 1, VP = MP;                        // row tiles, and items of the down projection, at once
     constexpr int CT = NCK * TW * 256;                                   // bytes of a row tile's codes
 
-    // ---- start: count this CTA in, let the next kernel come
     if (tid == 0) {
         mbar_init(bar_w, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // rows of A_gate, A_up of every set: four tasks (the four warps of the throughput form) per row, all CTAs share them, those without
+    // expert work first, then the last warps of the others
+    const int sets = p.n_adapters == 1 ? 1 : p.K;
+    const int set_tasks = 8 * p.rank, n_task = sets * set_tasks + 8 * p.rank_shared, spare = (int)gridDim.x - p.n_exp;
+    auto task_set = [&](int task) { return task >= sets * set_tasks ? sets : (sets == 1 ? 0 : task / set_tasks); };
+    auto first_task = [&](int w) { return cta >= p.n_exp ? (TW - 1 - w) * spare + cta - p.n_exp : TW * spare + (TW - 1 - w) * p.n_exp + cta; };
+    float* hx = p.hx;
+    auto ux_word = [&](int task) {
+        const int set = task_set(task), q = task - set * set_tasks;
+        return hx + p.ux_off + (size_t)set * 8 * p.rmax + (q & 3) * 2 * p.rmax + (q >> 2);
+    };
+    // ---- start (warp 1): count this CTA in, let the next kernel come; "not yet" into every word this CTA will publish, and say so
+    const bool links = p.flag_in >= 0 || p.flag_out >= 0;                // the next kernel may be a link that does not wait for this one's end
+    if (tid == 32) {
         uint32_t old;
-        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(p.starts) : "memory");
+        asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(p.starts) : "memory");
         const bool last = old % kEpochStarts == gridDim.x - 1;
         if (last) {                                                      // (returns before the next kernel, which counts on, may come)
             uint32_t sum;
@@ -214,9 +234,35 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         }
         s_misc[0] = (int)(old / kEpochStarts);
         s_misc[1] = last ? 1 : 0;
-        pdl_launch_dependents();
+        if (!links) pdl_launch_dependents();
     }
     if (p.flag_in < 0) pdl_wait_prior_grid();                            // a step on its own: everything queued before it has happened
+    if (warp == 1) {
+        const uint4 none = make_uint4(kNotYet, kNotYet, kNotYet, kNotYet);
+        if (has_gu) {
+            for (int i = lane; i < kHCopies * RG / 4; i += 32)
+                st_relaxed16(hx + (size_t)(i / (RG / 4)) * p.hc_words + (size_t)kpos * p.I + n0 + i % (RG / 4) * 4, none);
+            for (int i = lane; i < r; i += 32)
+                for (int c = 0; c < kHCopies; ++c) st_relaxed_gpu_u32(hx + (size_t)c * p.hc_words + p.ud_off + (size_t)cta * p.rmax + i, kNotYet);
+        }
+        if (lane < TW)
+            for (int task = first_task(lane); task < n_task; task += TW * gridDim.x) st_relaxed_gpu_u32(ux_word(task), kNotYet);
+        if (has_head && lane < p.head_tile)
+            for (int e = (cta - p.n_exp) * p.head_tile + lane; e < p.E; e += p.n_headc * p.head_tile) st_relaxed_gpu_u32(hx + p.lx_off + e, kNotYet);
+        if (has_dn && p.x_next != nullptr)
+            for (int i = lane; i < kStateCopies * 4; i += 32) st_relaxed16(p.vx + (size_t)(i / 4) * H + cta * 16 + i % 4 * 4, none);
+        if (p.flag_in < 0 && p.flag_out >= 0)                            // a chain starts: so does its hand-off ring
+            for (int i = cta * 32 + lane; i < kHandoffRing * (p.E + kPairWords) / 4; i += gridDim.x * 32) st_relaxed16(p.logits_ws + (size_t)i * 4, none);
+        __syncwarp();
+        if (lane == 0) {
+            // every grid adds kEpochStarts in total
+            asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p.ready), "r"(cta == 0 ? kEpochStarts - gridDim.x + 1 : 1u) : "memory");
+            if (links) {                                                 // (a link finds its words and its predecessor's cleared)
+                __threadfence();
+                pdl_launch_dependents();
+            }
+        }
+    }
     // eight values of the state (value i of them): the B words of the MMAs, the block sums
     auto take_x = [&](int i, uint4 v) {
         const float f[8] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y), bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w)};
@@ -247,8 +293,6 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         for (int i = tid; i < 16 * (H / 8); i += threads) cp16(un + (i / (H / 8)) * (H * 2 + 16) + (i % (H / 8)) * 16, src + (size_t)i * 16);
     };
     if (has_head && head_mma) load_head(cta - p.n_exp, TThreads);
-    if (p.stale >= 0 && cta == 0)
-        for (int i = tid; i < p.E + kPairWords; i += TThreads) st_relaxed_gpu_u32(&p.logits_ws[(size_t)p.stale * (p.E + kPairWords) + i], kNotYet);
 
     // ---- the routing (warp 0): from memory, or from the hand-off ring for a link of a chain
     if (warp == 0) {
@@ -309,7 +353,6 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         for (int i = tid; i < r * cpr; i += TThreads)
             cp16(smem + S.ad + i * 16, static_cast<const uint16_t*>(lo.A_down) + ((size_t)ad_k * r + i / cpr) * p.I + n0 + (i % cpr) * 8);
     }
-    const int sets = p.n_adapters == 1 ? 1 : p.K;
     auto load_bd = [&](int d) {                                          // [set][16][rank]: one set, or one per expert; the shared expert's behind them
         for (int s = warp; s <= sets; s += TW) {
             const int rk = s == sets ? p.rank_shared : p.rank;
@@ -329,18 +372,13 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
                 bulk_prefetch_l2(rec + p.L.codes_down + (size_t)(i & 3) * ((size_t)H * sw / 2) + code_off(sw, cta * 16, 0), DCH * 256);
                 bulk_prefetch_l2(rec + p.L.sz_down + down_sz_off(H, p.I, p.group, cta * 16, (i & 3) * (sw >> gsh)), (sw >> gsh) * 64);
             }
-    // ---- rows of A_gate, A_up of every set: four tasks (the four warps of the throughput form) per row, all CTAs share them
-    const int set_tasks = 8 * p.rank, n_task = sets * set_tasks + 8 * p.rank_shared;
     auto a_row = [&](int set, int q) {                                   // lane's first values of task q of a set
         const edg_lora& l = set == sets ? p.shared_lora : p.lora;
         const int rk = set == sets ? p.rank_shared : p.rank, up = (q >> 2) >= rk ? 1 : 0;
         const size_t row = (size_t)(set == sets || p.n_adapters == 1 ? 0 : s_ad[set]) * rk + ((q >> 2) - up * rk);
         return static_cast<const uint16_t*>(up ? l.A_up : l.A_gate) + row * H + ((q & 3) * 32 + lane) * 8;
     };
-    auto task_set = [&](int task) { return task >= sets * set_tasks ? sets : (sets == 1 ? 0 : task / set_tasks); };
-    // (the CTAs without expert work first, then the last warps of the others)
-    const int spare = (int)gridDim.x - p.n_exp;
-    const int task0 = cta >= p.n_exp ? (TW - 1 - warp) * spare + cta - p.n_exp : TW * spare + (TW - 1 - warp) * p.n_exp + cta;
+    const int task0 = first_task(warp);
     uint4 pa[NCK / 2];
     if (task0 < n_task) {
         const int set = task_set(task0);
@@ -348,12 +386,21 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
 #pragma unroll
         for (int sweep = 0; sweep < NCK / 2; ++sweep) pa[sweep] = ld_keep16(a + sweep * 1024);
     }
+    // Have all CTAs of this grid started, and cleared their words?  (Asked by the warps that read A x, by one at least, while they wait
+    // for something else; ahead of the products it would hold them up.)
+    auto all_ready = [&]() {
+        uint32_t c;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(p.ready) : "memory");
+        return c / kEpochStarts != epoch;
+    };
+    const bool asks = warp >= 8 && (warp == 8 || tid - 256 < 2 * r);
+    bool open = asks && all_ready();
     // A_down h partials this thread adds up (tid -> (expert and quarter, rank))
     const int udq = p.rmax > 0 ? tid / p.rmax : 0, udj = tid - udq * p.rmax, udn = p.rmax > 0 ? TThreads / p.rmax : 1;
     // ---- the hidden state
     if (p.dep) {
         const bool on = tid * 4 < H;
-        const float* src = p.vx + (size_t)((epoch + kStepStates - 1) % kStepStates * kStateCopies + cta % kStateCopies) * H + 4 * tid;
+        const float* src = p.vx_in + (size_t)(cta % kStateCopies) * H + 4 * tid;
         uint4 w = make_uint4(0, 0, 0, 0);
         bool got = !on;
         for (uint32_t it = 0; !got && it < kSpinLimit; ++it) {
@@ -379,17 +426,12 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
     if (p.dep && tid < H / 8) take_x(tid, *reinterpret_cast<const uint4*>(s_x + tid * 8));
     if (has_head) cp_wait<0>();
     if (p.dep || has_head) __syncthreads();
-    auto all_started = [&]() {
-        uint32_t c;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(p.starts) : "memory");
-        return c / kEpochStarts != epoch;
+    // a word of another CTA that does not come: the result is flagged at the very end
+    auto late = [&](uint32_t it) {
+        if (it < kSpinLimit) return false;
+        atomicExch(p.status, EDG_E_TIMEOUT);
+        return true;
     };
-    // after `it` polls without success: give up when the grid is not fully resident, go on with a flagged result at the very end
-    auto tired = [&](uint32_t it, bool& give_up, bool& got) {
-        if ((it % kWaitStarted) == kWaitStarted - 1 && !all_started()) give_up = true;
-        if (it >= kSpinLimit) { atomicExch(p.status, EDG_E_TIMEOUT); got = true; }
-    };
-    float* hx = p.hx + (size_t)(epoch % kStepBufs) * p.hx_words;
     // ---- the head's rows.  Four warps take tiles of 16 through the tensor cores; any other head goes in tiles of four, a row in four tasks
     if (has_head && head_mma && warp < 4) {
 #pragma unroll 1
@@ -462,7 +504,7 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
     for (int task = task0; task < n_task; task += TW * gridDim.x) {
         const int set = task_set(task), q = task - set * set_tasks;
         const float v = a_dot(set, q, task == task0);
-        if (lane == 0) st_relaxed_gpu_u32(hx + p.ux_off + (size_t)set * 8 * p.rmax + (q & 3) * 2 * p.rmax + (q >> 2), __float_as_uint(v));
+        if (lane == 0) st_relaxed_gpu_u32(ux_word(task), __float_as_uint(v));
     }
     if (valid) {
         // ---- gate/up on the tensor cores, a gate tile and its up tile at once where the registers allow it; per (row, scaled block)
@@ -510,21 +552,22 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         }
     }
     // A x of this expert: the four tasks of a row, from whoever has computed them
-    bool miss = false;
-    if (valid && tid >= 256 && tid - 256 < 2 * r) {
+    if (asks)
+        for (uint32_t it = 0; !open && (it < kWaitStarted || (s_misc[1] && it < kSpinLimit)); ++it) open = all_ready();
+    if (open && valid && tid - 256 < 2 * r) {
         const float* ux = hx + p.ux_off + (size_t)(is_shared ? sets : (p.n_adapters == 1 ? 0 : kpos)) * 8 * p.rmax + (tid - 256);
         uint32_t u[4];
         bool got = false;
-        for (uint32_t it = 0; !got && !miss; ++it) {
+        for (uint32_t it = 0; !got; ++it) {
 #pragma unroll
             for (int w = 0; w < 4; ++w) u[w] = ld_relaxed_gpu_u32(ux + w * 2 * p.rmax);
-            got = u[0] != kNotYet && u[1] != kNotYet && u[2] != kNotYet && u[3] != kNotYet;
-            if (!got) tired(it, miss, got);
+            got = (u[0] != kNotYet && u[1] != kNotYet && u[2] != kNotYet && u[3] != kNotYet) || late(it);
         }
         s_uf[tid - 256] = ((__uint_as_float(u[0]) + __uint_as_float(u[1])) + __uint_as_float(u[2])) + __uint_as_float(u[3]);
     }
     cp_wait<0>();
-    if (__syncthreads_or(miss)) {                                    // not all of this grid is resident: all of them here
+    open = !__syncthreads_or(asks && !open);
+    if (!open) {                                                         // not all of this grid is resident: all of them here
         const int set = is_shared ? sets : (p.n_adapters == 1 ? 0 : kpos);
 #pragma unroll 1
         for (int q = warp; q < 8 * r; q += TW) {
@@ -606,29 +649,16 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
     }
 
     constexpr int kHPad = 32 * CPB + 4;                                  // (a block of h, padded against bank conflicts)
-    // Every CTA of the step before has used its exchange buffers up: they are cleared for the step three epochs on, which cannot start
-    // before this kernel has ended (two CTAs fit an SM, a grid has one for every SM at least, and none leaves before the kernel
-    // before its own).  By the CTAs without expert work, if there are any.
-    if (cta >= p.n_exp || (int)gridDim.x == p.n_exp) {
-        float* hc = p.hx + (size_t)((epoch + kStepBufs - 1) % kStepBufs) * p.hx_words;
-        float* vc = p.vx + (size_t)((epoch + kStepStates / 2) % kStepStates) * kStateCopies * H;
-        const int from = (int)gridDim.x == p.n_exp ? 0 : p.n_exp;
-        const uint32_t t0 = (cta - from) * TThreads + tid, all = (gridDim.x - from) * TThreads;
-        const uint4 none = make_uint4(kNotYet, kNotYet, kNotYet, kNotYet);
-        for (uint32_t i = t0; i < p.hx_words / 4; i += all) st_relaxed16(hc + i * 4, none);
-        for (uint32_t i = t0; i < (uint32_t)H * kStateCopies / 4; i += all) st_relaxed16(vc + i * 4, none);
-        if (t0 == 0) st_relaxed_gpu(p.defer + (size_t)((epoch + kStepStates / 2) % kStepStates) * (p.n_dn + 4), 0);
-    }
 
-    // ---- down: output rows 16 d .. 16 d + 15 over the h of all experts.  False: the h did not come while the grid was not fully resident.
+    // ---- down: output rows 16 d .. 16 d + 15 over the h of all experts
     float* s_h = reinterpret_cast<float*>(un + S.h);
     uint4* s_hb = reinterpret_cast<uint4*>(un + S.hb);
     float* s_hsum = reinterpret_cast<float*>(un + S.hsum);
     float* s_hbias = reinterpret_cast<float*>(un + S.hbias);
     float* s_part = reinterpret_cast<float*>(un + S.part);               // [items][17]
     float* s_udi = reinterpret_cast<float*>(un + S.udi);                 // [items][rmax + 1]
-    auto down_unit = [&](int d, bool own) -> bool {
-        bool give_up = false;
+    auto down_unit = [&](int d, auto is_own) {
+        constexpr bool own = decltype(is_own)::value;
         const int n8 = p.Kt * p.I / 8;
         const float* hr = hx + (size_t)(cta % kHCopies) * p.hc_words;
 #pragma unroll 1
@@ -638,14 +668,13 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
             uint4 a = make_uint4(0, 0, 0, 0), b = a, u = a;
             const float* up = hr + p.ud_off + (size_t)item * 4 * p.rmax + udj;
             bool got = !on && !ud;
-            for (uint32_t it = 0; !got && !give_up; ++it) {
+            for (uint32_t it = 0; !got; ++it) {
                 if (on) { a = ld_relaxed16(hr + i * 8); b = ld_relaxed16(hr + i * 8 + 4); }
                 if (ud) {
                     u.x = ld_relaxed_gpu_u32(up); u.y = ld_relaxed_gpu_u32(up + p.rmax);
                     u.z = ld_relaxed_gpu_u32(up + 2 * p.rmax); u.w = ld_relaxed_gpu_u32(up + 3 * p.rmax);
                 }
-                got = there(a) && there(b) && there(u);
-                if (!got) tired(it, give_up, got);
+                got = (there(a) && there(b) && there(u)) || late(it);
             }
             if (ud)                                                      // A_down h of an (expert, quarter): its four CTAs in order
                 s_udi[item * (p.rmax + 1) + udj] = ((__uint_as_float(u.x) + __uint_as_float(u.y)) + __uint_as_float(u.z)) + __uint_as_float(u.w);
@@ -665,8 +694,8 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
                 *reinterpret_cast<uint4*>(q + 4) = b;
             }
         }
-        if (!own) { load_bd(d); cp_commit(); cp_wait<0>(); }
-        if (__syncthreads_or(give_up)) return false;
+        if constexpr (!own) { load_bd(d); cp_commit(); cp_wait<0>(); }
+        __syncthreads();
         if (!EX) {                                                       // block sums in the order of the throughput form
             for (int blk = tid; blk < p.Kt * p.I / (32 * CPB); blk += TThreads) {
                 const float4* hq = reinterpret_cast<const float4*>(s_h + blk * kHPad);
@@ -748,7 +777,7 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         static_assert(kStateCopies == 8, "a copy per four lanes");
         if (warp == 0) {
             if (p.x_next != nullptr)
-                st_relaxed16(p.vx + (size_t)(epoch % kStepStates * kStateCopies + lane / 4) * H + d * 16 + lane % 4 * 4, reinterpret_cast<const uint4*>(s_red + 16)[lane % 4]);
+                st_relaxed16(p.vx + (size_t)(lane / 4) * H + d * 16 + lane % 4 * 4, reinterpret_cast<const uint4*>(s_red + 16)[lane % 4]);
         } else if (warp == 1 && lane < 16) {
             const float v = s_red[lane];
             const int row = d * 16 + lane;
@@ -757,20 +786,19 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
             else store_out<bf16_t>(static_cast<bf16_t*>(p.y), row, v);
         }
         __syncthreads();
-        return true;
     };
     // the caller's x_next (one CTA without expert work; the next link of the chain does not wait for it)
-    auto finish_state = [&]() -> bool {
+    auto finish_state = [&]() {
         const bool on = tid * 4 < H;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        bool give_up = false, got = !on;
-        for (uint32_t it = 0; !got && !give_up; ++it) {
-            const uint4 w = ld_relaxed16(p.vx + (size_t)(epoch % kStepStates * kStateCopies + cta % kStateCopies) * H + 4 * tid);
-            got = there(w);
+        bool got = !on;
+        for (uint32_t it = 0; !got; ++it) {
+            const uint4 w = ld_relaxed16(p.vx + (size_t)(cta % kStateCopies) * H + 4 * tid);
+            got = there(w) || late(it);
             v = make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
-            if (!got) { __nanosleep(32); tired(it, give_up, got); }
+            if (!got) __nanosleep(32);
         }
-        if (__syncthreads_or(give_up)) return false;
+        __syncthreads();
         const float inv = inv_rms(s_red, v, on, H, p.eps);
         if (on) {
             bf16_t* xn = reinterpret_cast<bf16_t*>(p.x_next) + 4 * tid;
@@ -778,11 +806,9 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
             store_out<bf16_t>(xn, 2, v.z * inv); store_out<bf16_t>(xn, 3, v.w * inv);
         }
         __syncthreads();
-        return true;
     };
     // the routing of the next step, by one warp, as soon as all logits are there
-    auto route = [&]() -> bool {
-        bool give_up = false;
+    auto route = [&]() {
         if (warp == 0) {
             float* work = reinterpret_cast<float*>(un);
             float* slot = p.logits_ws + (size_t)max(p.flag_out, 0) * (p.E + kPairWords);
@@ -790,10 +816,10 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
             unsigned long long was = ~0ull;
             if (p.flag_out >= 0 && lane < p.K) was = ld_relaxed_gpu_u64(pr);
 #pragma unroll 1
-            for (int i0 = 0; i0 < p.E && !give_up; i0 += 256) {          // 8 independent loads per lane and pass
+            for (int i0 = 0; i0 < p.E; i0 += 256) {          // 8 independent loads per lane and pass
                 uint32_t v[8];
                 bool got = false;
-                for (uint32_t it = 0; !got && !give_up; ++it) {
+                for (uint32_t it = 0; !got; ++it) {
                     bool all = true;
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
@@ -802,12 +828,8 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
                     }
 #pragma unroll
                     for (int u = 0; u < 8; ++u) all = all && v[u] != kNotYet;
-                    got = __all_sync(0xFFFFFFFFu, all);
-                    if (!got) tired(it, give_up, got);
-                    give_up = __any_sync(0xFFFFFFFFu, give_up);
-                    got = __all_sync(0xFFFFFFFFu, got);
+                    got = __all_sync(0xFFFFFFFFu, all) || late(it);
                 }
-                if (give_up) break;
                 // the step that last read this slot of the ring has reset it
                 for (uint32_t it = 0; was != ~0ull && it < kSpinLimit; ++it) was = ld_relaxed_gpu_u64(pr);
                 if (was != ~0ull) atomicExch(p.status, EDG_E_TIMEOUT);
@@ -816,59 +838,63 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
                 for (int u = 0; u < 8; ++u)
                     if (i0 + u * 32 + lane < p.E) work[i0 + u * 32 + lane] = __uint_as_float(v[u]);
             }
-            if (!give_up) {
-                emit_routing<false>(p, work, lane, p.flag_out >= 0 ? pr : nullptr);
-                // the logits move on into the ring slot, beside the routing made of them
+            emit_routing<false>(p, work, lane, p.flag_out >= 0 ? pr : nullptr);
+            // the logits move on into the ring slot, beside the routing made of them
 #pragma unroll 4
-                for (int i = lane; i < p.E; i += 32) {
-                    const uint32_t v = ld_relaxed_gpu_u32(hx + p.lx_off + i);
-                    if (p.flag_out >= 0) st_relaxed_gpu_u32(slot + i, v);
-                    st_relaxed_gpu_u32(hx + p.lx_off + i, kNotYet);
-                    if (p.logits_next != nullptr) p.logits_next[i] = __uint_as_float(v);
-                }
+            for (int i = lane; i < p.E; i += 32) {
+                const uint32_t v = ld_relaxed_gpu_u32(hx + p.lx_off + i);
+                if (p.flag_out >= 0) st_relaxed_gpu_u32(slot + i, v);
+                st_relaxed_gpu_u32(hx + p.lx_off + i, kNotYet);
+                if (p.logits_next != nullptr) p.logits_next[i] = __uint_as_float(v);
             }
         }
-        return !__syncthreads_or(give_up);
+        __syncthreads();
     };
-    // A CTA's own units (its rows, or the routing: n_dn + 1, and the caller's x_next: n_dn); then, if it is the one that started last, what others have left to
-    // it.  An entry of the list is claimed by an atomic: by the last starter, or by the one that left it, if it finds
+    // A CTA's own units (its rows, or the routing: n_dn + 1, and the caller's x_next: n_dn); then, if it is the one that started last,
+    // what others have left to it.  A bit is claimed by an atomic: by the last starter, or by the one that left it, if it finds
     // afterwards that the last one has started -- then nothing stands in the way of waiting any more.
-    int32_t* defer = p.defer + (size_t)(epoch % kStepStates) * (p.n_dn + 4);
-    int unit = has_dn ? cta : (cta == p.cta_route ? p.n_dn + 1 : (cta == p.cta_state ? p.n_dn : -1)), left = -1, next = 0;
+    int unit = has_dn ? cta : (cta == p.cta_route ? p.n_dn + 1 : (cta == p.cta_state ? p.n_dn : -1));
     int then = cta == p.cta_route && cta == p.cta_state ? p.n_dn : -1;
-    bool own = true;
+    if (has_dn && open) {                                                // (by far the usual case; the loop is code that is hardly ever fetched)
+        down_unit(cta, std::true_type{});
+        unit = -1;
+    }
 #pragma unroll 1
     for (;;) {
-        if (unit >= 0) {
-            if (!(unit < p.n_dn ? down_unit(unit, own) : (unit == p.n_dn ? finish_state() : route()))) {
-                if (tid == 0) {
-                    const int at = atomicAdd(defer, 1);
-                    atomicExch(defer + 1 + at, unit + 1);
-                    __threadfence();
-                    s_misc[2] = all_started() && atomicCAS(defer + 1 + at, unit + 1, 0) == unit + 1 ? 1 : 0;
-                }
-                __syncthreads();
-                if (!s_misc[2]) unit = -1;
-                own = false;
-                __syncthreads();
-                continue;
+        if (unit >= 0 && !open) {
+            if (tid == 0) {
+                const uint32_t bit = 1u << (unit & 31);
+                atomicOr(p.defer + (unit >> 5), bit);
+                __threadfence();
+                s_misc[3] = all_ready() ? 1 : 0;
+                s_misc[2] = s_misc[3] && (atomicAnd(p.defer + (unit >> 5), ~bit) & bit) ? 1 : 0;
             }
-            own = false;
+            __syncthreads();
+            if (!s_misc[2]) unit = -1;
+            open = s_misc[3] != 0;
+            __syncthreads();
+        }
+        if (unit >= 0) {
+            if (unit < p.n_dn) down_unit(unit, std::false_type{});
+            else if (unit == p.n_dn) finish_state();
+            else route();
         }
         if (then >= 0) { unit = then; then = -1; continue; }
         if (!s_misc[1]) break;                                           // (uniform: written before the first barrier)
-        if (left < 0) {
-            if (tid == 0) { __threadfence(); s_misc[2] = min(ld_relaxed_gpu(defer), p.n_dn + 2); }
-            __syncthreads();
-            left = s_misc[2];
-            __syncthreads();
+        if (tid == 0) {
+            int next = -1;
+            __threadfence();
+            for (int w = 0; w < kStepDeferWords && next < 0; ++w)
+                for (uint32_t left; next < 0 && (left = ld_relaxed_gpu_u32(p.defer + w)) != 0;) {
+                    const uint32_t bit = left & (0u - left);
+                    if (atomicAnd(p.defer + w, ~bit) & bit) next = w * 32 + __ffs(bit) - 1;
+                }
+            s_misc[2] = next;
         }
-        if (next >= left) break;
-        if (tid == 0) s_misc[2] = atomicExch(defer + 1 + next, 0) - 1;
         __syncthreads();
         unit = s_misc[2];
         __syncthreads();
-        ++next;
+        if (unit < 0) break;
     }
     // ---- a link of a chain: the last CTA to have read the routing resets its ring slot; kernels of a chain complete in order
     if (p.flag_in >= 0) {
@@ -978,11 +1004,11 @@ size_t step_exchange_words(const edg_layer_desc& d) {
     const size_t sets = (d.n_adapters == 1 ? 1 : d.K) + 1;               // h, A_down h, A x, logits
     return kHCopies * step_copy_words(d) + (sets * 8 * d.rank + d.E + 63) / 64 * 64;
 }
-size_t step_region_words(const edg_layer_desc& d) { return kStepBufs * step_exchange_words(d) + (size_t)kStepStates * kStateCopies * d.H; }
+size_t step_region_words(const edg_layer_desc& d) { return kStepBufs * (step_exchange_words(d) + (size_t)kStateCopies * d.H); }
 
 int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* slots, const int32_t* table, const int32_t* experts,
                  const float* gates, const void* x, const edg_lora* lora, void* y, const void* W_pre, int32_t* inds_next, float* gates_next,
-                 float* logits_next, void* workspace, int flag_in, int flag_out, int stale, cudaStream_t st, const FusedExtras& ex) {
+                 float* logits_next, void* workspace, int flag_in, int flag_out, int pos, cudaStream_t st, const FusedExtras& ex) {
     StepParams p{};
     p.pool = static_cast<const uint8_t*>(slot_pool);
     p.slots = slots; p.table = table; p.experts = experts; p.gates = gates;
@@ -1006,15 +1032,19 @@ int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* 
     p.W_pre = W_pre; p.inds_next = inds_next; p.gates_next = gates_next; p.logits_next = logits_next; p.inds_mirror = ex.inds_mirror;
     p.x_next = static_cast<uint16_t*>(ex.x_next);
     p.eps = ex.eps;
-    p.starts = reinterpret_cast<uint32_t*>(ws + W.step);
-    p.defer = reinterpret_cast<int32_t*>(ws + W.step + kStepDeferOff);
-    p.hx = reinterpret_cast<float*>(ws + W.step_x);
-    p.hx_words = (uint32_t)step_exchange_words(*d);
+    const int buf = pos % kStepBufs, before = (pos + kStepBufs - 1) % kStepBufs;
+    const size_t hx_words = step_exchange_words(*d);
+    p.starts = reinterpret_cast<uint32_t*>(ws + W.ctrl + kCtrlStarts);
+    p.ready = p.starts + 16;
+    p.defer = reinterpret_cast<uint32_t*>(ws + W.ctrl + kCtrlDefer) + buf * kStepDeferWords;
+    float* region = reinterpret_cast<float*>(ws + W.step_x);
+    p.hx = region + buf * hx_words;
+    p.vx = region + kStepBufs * hx_words + (size_t)buf * kStateCopies * d->H;
+    p.vx_in = region + kStepBufs * hx_words + (size_t)before * kStateCopies * d->H;
     p.ud_off = (uint32_t)(d->K + 1) * d->I;
     p.hc_words = (uint32_t)step_copy_words(*d);
     p.ux_off = kHCopies * p.hc_words;
     p.lx_off = p.ux_off + ((d->n_adapters == 1 ? 1u : (uint32_t)d->K) + 1u) * 8u * d->rank;
-    p.vx = p.hx + (size_t)kStepBufs * p.hx_words;
     p.I = d->I; p.E = d->E; p.group = d->group;
     while ((1 << p.gshift) < d->group) ++p.gshift;
     p.n_adapters = d->n_adapters; p.n_slots = d->n_slots; p.pre_dtype = d->pre_dtype; p.out_dtype = d->out_dtype;
@@ -1022,8 +1052,8 @@ int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* 
     p.L = record_layout(d->H, d->I, d->group);
     p.n_gu = 16 * p.Kt; p.n_dn = d->H / 16;
     p.n_exp = p.n_gu > p.n_dn ? p.n_gu : p.n_dn;
-    const int head_tile = d->pre_dtype == EDG_F16 && d->E % 16 == 0 ? 16 : 4;
-    p.n_head = W_pre != nullptr ? (d->E + head_tile - 1) / head_tile : 0;
+    p.head_tile = d->pre_dtype == EDG_F16 && d->E % 16 == 0 ? 16 : 4;
+    p.n_head = W_pre != nullptr ? (d->E + p.head_tile - 1) / p.head_tile : 0;
     // One CTA per SM when they suffice: two launches of a chain then sit side by side on every SM, and no SM has two CTAs of the
     // same launch (which held a step up by 5 us of 15).  The head's tiles share the CTAs that the experts leave.
     const int n_sm = sm_count(), spare = n_sm - p.n_exp;
@@ -1032,7 +1062,7 @@ int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* 
     const int grid = max(n_sm, p.n_exp + extra), idle = p.n_exp + p.n_headc;
     p.cta_route = W_pre == nullptr ? -1 : (idle < grid ? idle : idle - 1);
     p.cta_state = p.x_next == nullptr ? -1 : (W_pre == nullptr ? p.n_exp : (idle + 1 < grid ? idle + 1 : p.n_exp));
-    p.flag_in = flag_in; p.flag_out = W_pre != nullptr ? flag_out : -1; p.stale = stale;
+    p.flag_in = flag_in; p.flag_out = W_pre != nullptr ? flag_out : -1;
     p.dep = flag_in >= 0 && ex.dep_wait >= 0;
     p.S = step_smem(*d, p.Kt, p.rmax);
     const cudaError_t e = d->H == 2048 ? (d->I == 512 ? launch_shape<4, 4>(p, grid, st) : launch_shape<4, 2>(p, grid, st))

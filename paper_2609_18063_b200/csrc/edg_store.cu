@@ -140,7 +140,8 @@ struct edg_store {
     // chaining of consecutive batch-1 layer-steps: when a call consumes the routing that the
     // previous call on the same stream and workspace produced, its kernel is launched as a
     // programmatic dependent of that one and waits on a device flag instead of the kernel's end
-    bool chain_latency = false;            // that step ran in the latency form
+    bool chain_latency = false;            // that step ran in the latency form,
+    int chain_pos = 0;                     // as the link of this number of its chain
     const void* chain_x_next = nullptr;    // the hidden state the last batch-1 layer-step produces for its successor, or null
     const void* chain_inds = nullptr;
     const void* chain_ws = nullptr;
@@ -612,7 +613,7 @@ static int32_t layer_decode(edg_store* s, int32_t layer, const void* x,
         if (!workspace || !edg::aligned(workspace, 256) || workspace_bytes < edg::workspace_layout(s->d, 1).bytes)
             return EDG_E_WORKSPACE;
         if (!edg::aligned(x, 16) || !edg::aligned(y, 16) || (W_pre_next && !edg::aligned(W_pre_next, 16))) return EDG_E_INVAL;
-        bool chained = s->chaining && !s->hot && s->chain_inds != nullptr && s->chain_inds == inds_cur &&
+        bool chained = s->chaining && !s->hot && s->chain_inds != nullptr && s->chain_inds == inds_cur && s->chain_flag >= 0 &&
                        s->chain_ws == workspace && s->chain_stream == stream;
         // Chaining pays when steps queue up on the device: a chained step runs as a few long-lived
         // CTAs that share the GPU with dozens of other steps.  A step that finds the GPU idle -- the
@@ -624,30 +625,29 @@ static int32_t layer_decode(edg_store* s, int32_t layer, const void* x,
         if (chained && s->chaining == 1 && capturing == cudaStreamCaptureStatusNone && s->step_done_valid &&
             cudaEventQuery(s->step_done) == cudaSuccess)
             chained = false;
-        // A workspace seen for the first time gets its ring cleared: counters to zero, logits to
-        // "not yet written".  After that the ring looks after itself: a chained step resets the
-        // slot it has read, and a step that starts over clears the slot the last head left unread.
-        bool fresh = s->ring_ws != workspace;
-        if (fresh) {
+        const bool shared = !s->shared_rec.empty() && s->shared_rec[layer] != nullptr;
+        const bool latency_ok = edg::step_supported(s->d, shared) && edg::trace_buffer() == nullptr;     // (only the other form is traced)
+        bool chain = chained;
+        // The hand-off ring starts out cleared: counters zero, logits "not yet written".  A step in the latency form that
+        // starts a chain does that itself; where the throughput form starts one, it is done for the first chain in a
+        // workspace.  After that the ring looks after itself: a chained step resets the slot it has read, and a step that
+        // starts over clears the slot the last head left unread.  Without chaining nobody reads the ring, and nothing is
+        // written to it.
+        if (s->chaining && !latency_ok && s->ring_ws != workspace) {
             uint8_t* w8 = static_cast<uint8_t*>(workspace);
             const edg::WorkspaceLayout W = edg::workspace_layout(s->d, 1);
             EDG_CUDA_TRY(cudaMemsetAsync(w8 + edg::kCtrlCounters, 0, edg::kCtrlBytes - edg::kCtrlCounters, st));
             EDG_CUDA_TRY(cudaMemsetAsync(w8 + W.logits, 0xFF, (size_t)edg::kHandoffRing * (s->d.E + edg::kPairWords) * sizeof(float), st));
-            EDG_CUDA_TRY(cudaMemsetAsync(w8 + W.step, 0, edg::kStepCtrlBytes, st));
-            EDG_CUDA_TRY(cudaMemsetAsync(w8 + W.step_x, 0xFF, edg::step_region_words(s->d) * sizeof(float), st));
-            EDG_CUDA_TRY(cudaMemsetAsync(w8 + W.dep, 0, (size_t)edg::kHandoffRing * edg::kDepWords * sizeof(float), st));
             s->ring_ws = workspace;
             s->ring_next = 0;
             s->pub_slot = -1;
+            chain = false;
         }
-        bool chain = chained && !fresh;
         // a chained step whose x is the state the previous step is still producing waits for it on the device
         bool dep_chain = chain && s->chain_x_next != nullptr && s->chain_x_next == x;
         // A step that shares the GPU with dozens of others, chained through the routing alone, runs in the throughput form; one
         // that is alone, or a link of a dependent chain, in the latency form.  (A step that writes the next hidden state while
         // its own is at hand already starts a dependent chain: it is launched alone, its successors wait for it.)
-        const bool shared = !s->shared_rec.empty() && s->shared_rec[layer] != nullptr;
-        const bool latency_ok = edg::step_supported(s->d, shared) && edg::trace_buffer() == nullptr;     // (only the other form is traced)
         if (dep_chain && latency_ok != s->chain_latency) chain = dep_chain = false;                      // the forms hand x on in ways of their own
         if (latency_ok && chain && !dep_chain && x_next != nullptr) chain = false;
         const bool latency = latency_ok && (!chain || dep_chain);
@@ -656,7 +656,8 @@ static int32_t layer_decode(edg_store* s, int32_t layer, const void* x,
         if (!chain && s->pub_slot >= 0) stale = s->pub_slot;         // nobody will read that head's logits
         s->pub_slot = -1;
         const int ring = s->ring_next;                               // ring slot of this step's scratch and of the head it evaluates
-        const int flag_out = W_pre_next != nullptr ? ring : -1;
+        const int flag_out = W_pre_next != nullptr && s->chaining && !s->hot ? ring : -1;
+        const int pos = latency && dep_chain ? s->chain_pos + 1 : 0;
         s->ring_next = (ring + 1) % edg::kHandoffRing;
         edg::FusedExtras extras;
         extras.inds_mirror = W_pre_next != nullptr ? inds_next_host_mirror_opt : nullptr;
@@ -669,11 +670,11 @@ static int32_t layer_decode(edg_store* s, int32_t layer, const void* x,
         }
         if (latency)
             rc = edg::run_step(&s->d, pool, slot_arg, table, expert_arg, gates_cur, x, (lora && s->d.rank > 0) ? lora : nullptr, y,
-                               W_pre_next, inds_next, gates_next, logits_next_opt, workspace, flag_in, flag_out, stale, st, extras);
+                               W_pre_next, inds_next, gates_next, logits_next_opt, workspace, flag_in, flag_out, pos, st, extras);
         else rc = edg::run_fused_layer(&s->d, pool, slot_arg, table, expert_arg, gates_cur, x,
                                   (lora && s->d.rank > 0) ? lora : nullptr, y, W_pre_next, inds_next, gates_next,
                                   logits_next_opt, workspace, flag_in, flag_out, ring, stale, st, &extras);
-        if (W_pre_next != nullptr) s->pub_slot = flag_out;
+        s->pub_slot = flag_out;
         if (rc != EDG_OK) return rc;
         s->step_done_valid = false;
         if (capturing == cudaStreamCaptureStatusNone && s->chaining == 1) {
@@ -683,6 +684,7 @@ static int32_t layer_decode(edg_store* s, int32_t layer, const void* x,
         }
         s->chain_x_next = x_next;
         s->chain_latency = latency;
+        s->chain_pos = pos;
         s->chain_inds = W_pre_next != nullptr ? inds_next : nullptr;
         s->chain_ws = workspace;
         s->chain_stream = stream;
@@ -783,6 +785,8 @@ extern "C" int32_t edg_stack_decode_token(edg_store* s, const void* x, const int
 
 extern "C" int32_t edg_store_set_chaining(edg_store* s, int32_t enable) {
     if (!store_ok(s)) return EDG_E_INVAL;
+    const int was = s->chaining;
     s->chaining = enable < 0 ? 0 : (enable > 2 ? 2 : enable);
+    if (was == 0) s->ring_ws = nullptr;                    // (whatever has used the workspace in between)
     return EDG_OK;
 }
