@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
     const bool asks = warp >= 8 && (warp == 8 || tid - 256 < 2 * r);
     bool open = asks && all_ready();
     // A_down h partials this thread adds up (tid -> (expert and quarter, rank))
-    const int udq = p.rmax > 0 ? tid / p.rmax : 0, udj = tid - udq * p.rmax, udn = p.rmax > 0 ? TThreads / p.rmax : 1;
+    const int udq = p.rmax > 0 ? tid / p.rmax : 0, udj = tid - udq * p.rmax, udn = p.rmax > 0 ? TThreads / p.rmax : TThreads;   // (none: no rounds beyond those of h)
     // ---- the hidden state
     if (p.dep) {
         const bool on = tid * 4 < H;
