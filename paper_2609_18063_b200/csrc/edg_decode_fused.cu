@@ -154,6 +154,7 @@ struct FusedParams {
     float eps;
     int head_extra;               // CTAs behind those of the experts that evaluate the head and nothing else (0: the first CTAs of the grid do)
     int dep_wait;                 // -1, or the ring slot whose flag says that this step's x has been written
+    int slot_until_end;           // the step before may write to this step's ring slot until it ends
     const uint8_t* shared_rec;    // record of the layer's always-on shared expert (one more expert with gate 1), or null
     edg_lora shared_lora;         // its own adapter, leading dimension 1 (null pointers with rank_shared == 0)
     int n_shared;                 // 0 or 1
@@ -1217,6 +1218,7 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
             // The last of the kC reducers resets the ring slot this step has taken its logits from.
             // By then every CTA has read them and the reduce scratch of this ring slot is free
             // again; the step that reuses either gets its own routing only after this.
+            if (p.slot_until_end) pdl_wait_prior_grid();
             __threadfence();
             __syncthreads();
             if (tid == 0) s_flag[3] = (atomicAdd(&p.done[p.flag_in], 1) == kC - 1) ? 1 : 0;
@@ -1341,6 +1343,7 @@ int32_t run_fused_layer(const edg_layer_desc* d, const void* slot_pool, const in
         p.x_next = static_cast<uint16_t*>(extras->x_next);
         p.eps = extras->eps;
         p.dep_wait = flag_in >= 0 ? extras->dep_wait : -1;
+        p.slot_until_end = extras->slot_until_end ? 1 : 0;
     }
     p.dep_ws = reinterpret_cast<float*>(ws + W.dep);
     p.norm_cnt = reinterpret_cast<int32_t*>(ws + W.ctrl + kCtrlNorm);

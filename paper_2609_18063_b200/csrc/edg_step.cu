@@ -810,7 +810,8 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
     // the routing of the next step, by one warp, as soon as all logits are there
     auto route = [&]() {
         if (warp == 0) {
-            float* work = reinterpret_cast<float*>(un);
+            float* work = reinterpret_cast<float*>(un);                  // [E], and 256 bytes for the winners
+            float* kept = work + p.E + 64;                               // [E] (selecting may overwrite the others)
             float* slot = p.logits_ws + (size_t)max(p.flag_out, 0) * (p.E + kPairWords);
             unsigned long long* pr = reinterpret_cast<unsigned long long*>(slot + p.E) + lane;
             unsigned long long was = ~0ull;
@@ -836,16 +837,16 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
                 __syncwarp();
 #pragma unroll
                 for (int u = 0; u < 8; ++u)
-                    if (i0 + u * 32 + lane < p.E) work[i0 + u * 32 + lane] = __uint_as_float(v[u]);
+                    if (i0 + u * 32 + lane < p.E) work[i0 + u * 32 + lane] = kept[i0 + u * 32 + lane] = __uint_as_float(v[u]);
             }
             emit_routing<false>(p, work, lane, p.flag_out >= 0 ? pr : nullptr);
-            // the logits move on into the ring slot, beside the routing made of them
+            // The logits move on into the ring slot and to the caller.  The next step may be under way with that routing by now: it
+            // resets the slot only when this kernel has ended.
 #pragma unroll 4
             for (int i = lane; i < p.E; i += 32) {
-                const uint32_t v = ld_relaxed_gpu_u32(hx + p.lx_off + i);
-                if (p.flag_out >= 0) st_relaxed_gpu_u32(slot + i, v);
+                if (p.flag_out >= 0) st_relaxed_gpu_u32(slot + i, __float_as_uint(kept[i]));
                 st_relaxed_gpu_u32(hx + p.lx_off + i, kNotYet);
-                if (p.logits_next != nullptr) p.logits_next[i] = __uint_as_float(v);
+                if (p.logits_next != nullptr) p.logits_next[i] = kept[i];
             }
         }
         __syncthreads();
@@ -898,6 +899,9 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
     }
     // ---- a link of a chain: the last CTA to have read the routing resets its ring slot; kernels of a chain complete in order
     if (p.flag_in >= 0) {
+        // No CTA leaves before the kernel before this one has: the CTAs of the next one but one take over from that kernel, one on
+        // every SM, before an SM can offer them two places.  What that kernel still had to write into the slot is there, too.
+        pdl_wait_prior_grid();
         __syncthreads();
         if (tid == 0) {
             __threadfence();
@@ -913,9 +917,6 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
             __syncthreads();
             for (int i = tid; i < p.E; i += TThreads) st_relaxed_gpu_u32(slot + i, kNotYet);
         }
-        // No CTA leaves before the kernel before this one has: the CTAs of the next one but one take over from that kernel, one on
-        // every SM, before an SM can offer them two places.
-        pdl_wait_prior_grid();
     }
 }
 
@@ -934,7 +935,7 @@ StepSmem step_smem(const edg_layer_desc& d, int Kt, int rmax) {
     auto at_least = [&](uint32_t v) { if (un < v) un = up16(v); };
     at_least(NT * NCK * TW * 256);
     if (d.pre_dtype == EDG_F16) at_least(16u * (d.H * 2 + 16));          // a tile of the head
-    at_least((uint32_t)d.E * 4 + 256);
+    at_least((uint32_t)d.E * 8 + 256);                                   // the logits, for the routing
     S.un = 0;
     uint32_t o = un;
     S.sz_tile = d.H / d.group * 64;

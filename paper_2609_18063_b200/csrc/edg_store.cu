@@ -664,6 +664,7 @@ static int32_t layer_decode(edg_store* s, int32_t layer, const void* x,
         extras.x_next = x_next;
         extras.eps = eps;
         extras.dep_wait = dep_chain ? flag_in : -1;
+        extras.slot_until_end = chain && s->chain_latency;
         if (shared) {
             extras.shared_rec = s->shared_rec[layer];
             extras.shared_lora = s->shared_has_lora[layer] ? &s->shared_lora[layer] : nullptr;

@@ -132,3 +132,38 @@ def test_chains_on_streams_of_their_own():
                 assert torch.equal(a, b)
     for c in chains:
         c.store.close()
+
+
+@pytest.mark.parametrize("E,then", [(256, "dependent"), (1024, "dependent"), (256, "throughput"), (1024, "throughput")])
+def test_the_logits_a_link_hands_on(E, then):
+    """150 chained links -- the hand-off ring wraps -- of a layer with the most experts there can be: the logits every link leaves, with the
+    next one under way on the routing made of them; and steps chained through the routing alone behind one that runs by itself."""
+    cfg, steps, n = dataclasses.replace(_cfg(1024, 256, 64, E, 8, 8, 1), pre_dtype="f16"), 150, 8
+    d = edg.make_desc(cfg, n_slots=E)
+    some = torch.from_numpy(np.stack([edg.pack_expert(d, synth.expert_tensors(cfg, 0, e)) for e in range(n)]))
+    host = some[torch.arange(E) % n].contiguous().pin_memory()
+    pool, tables = torch.empty((1, E, host.shape[1]), dtype=torch.uint8, device="cuda"), torch.empty((1, E), dtype=torch.int32, device="cuda")
+    lora, keep = layer_io.lora_to_device(d, [synth.lora_tensors(cfg, 0, 0)])
+    store = edg.Store(d, [host], pool, tables, [lora], torch.cuda.Stream())
+    store.load_whole_layer(0)
+    W_np = synth.prerouter_weights(cfg)
+    W, ws = torch.from_numpy(W_np).cuda(), layer_io.new_workspace(d)
+    X = synth.hidden_states(cfg, steps + 1, stream=83)
+    xs = x_dev(X)
+    inds, gates = torch.zeros((steps + 1, 8), dtype=torch.int32, device="cuda"), torch.zeros((steps + 1, 8), device="cuda")
+    logits, y = torch.full((steps + 1, E), float("nan"), device="cuda"), torch.zeros((steps, cfg.H), device="cuda")
+    edg.prerouter_topk(d, W, xs[steps], 1, inds[0], gates[0], logits[0])
+    store.set_chaining(2)
+    for t in range(steps):
+        if then == "dependent":
+            edg.moe_layer_decode_dependent(store, 0, xs[t], inds[t], gates[t], W, inds[t + 1], gates[t + 1], logits[t + 1], y[t], xs[t + 1], ws)
+        else:
+            edg.moe_layer_decode(store, 0, xs[t], inds[t], gates[t], W, inds[t + 1], gates[t + 1], logits[t + 1], y[t], ws)
+    assert edg.workspace_status(ws) == 0
+    bits, lh, ih, gh = xs.view(torch.int16).cpu().numpy().view(np.uint16), logits.cpu().numpy(), inds.cpu().numpy(), gates.cpu().numpy()
+    for t in range(steps):
+        _check_routing(lh[t + 1], ih[t + 1], gh[t + 1], W_np.astype(np.float32), bits[t], 8)
+    for t in range(0, steps, 29):
+        _assert_close(y[t].cpu().numpy(), orc.moe_ffn(bits[t], ih[t], gh[t].astype(np.float64), lambda e: synth.expert_tensors(cfg, 0, e % n),
+                                                      lambda e: synth.lora_tensors(cfg, 0, 0), cfg.lora_scale, cfg.group))
+    store.close()
