@@ -247,6 +247,13 @@ __device__ __forceinline__ float group_sum(float v) {
     return v;
 }
 
+template <int LPR>
+__device__ __forceinline__ uint32_t group_max(uint32_t v) {
+#pragma unroll
+    for (int o = LPR / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    return v;
+}
+
 // ---- int4 -> fp32 without conversion instructions.
 //
 // A float whose exponent field is 0 or 1 has the value (bit pattern) * 2^-149, so masking one

@@ -437,30 +437,45 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
     if (p.table != nullptr && warp == 0)      // (warp 0 alone: it resolves the routing before the CTA's first barrier)
         for (int i = lane; i < p.E; i += 32) s_table[i] = __ldcg(&p.table[i]);
     auto convert_x = [&]() {
-    for (int t0 = 0; t0 * 8 < p.H; t0 += kFW * 32) {
-        const int t = t0 + tid;
-        const bool on = t * 8 < p.H;
-        float sum = 0.f, sodd = 0.f;
-        if (on) {
-            const uint4 v = *reinterpret_cast<const uint4*>(p.x + t * 8);
-            const float f[8] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y),
-                                bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w)};
-            s_xb[t] = EX ? permute8_s(f) : permute8(f);
-            // fp16 is exact for bf16 inputs in the normal range; sum what the MMA will see
+    constexpr int kRounds = NCW / 4;                              // eight activations a thread and round
+    uint4 v[kRounds];
+    uint32_t m = 0;
 #pragma unroll
-            for (int e = 0; e < 8; e += 2) {
-                sum += __half2float(__float2half_rn(f[e]));
-                sodd += __half2float(__float2half_rn(f[e + 1]));
-            }
+    for (int q = 0; q < kRounds; ++q) {
+        v[q] = *reinterpret_cast<const uint4*>(p.x + (q * kFW * 32 + tid) * 8);
+        const uint32_t w = max(max(max(v[q].x & 0x7FFFu, v[q].y & 0x7FFFu), max(v[q].z & 0x7FFFu, v[q].w & 0x7FFFu)) << 16,
+                               max(max(v[q].x & 0x7FFF0000u, v[q].y & 0x7FFF0000u), max(v[q].z & 0x7FFF0000u, v[q].w & 0x7FFF0000u)));
+        m = max(m, w);
+    }
+    float scale = 1.f;
+    if (EX) {                                                     // the largest magnitude of the state
+        m = __reduce_max_sync(0xFFFFFFFFu, m);
+        if (lane == 0) s_flag[warp] = (int)m;
+        __syncthreads();
+        scale = vector_scale(max(max((uint32_t)s_flag[0], (uint32_t)s_flag[1]), max((uint32_t)s_flag[2], (uint32_t)s_flag[3])));
+        if (tid == 0) s_xbias[0] = kUnscaleS * vector_unscale(scale);
+    }
+#pragma unroll
+    for (int q = 0; q < kRounds; ++q) {
+        const int t = q * kFW * 32 + tid;
+        float sum = 0.f, sodd = 0.f;
+        const float f[8] = {bf16_lo(v[q].x), bf16_hi(v[q].x), bf16_lo(v[q].y), bf16_hi(v[q].y),
+                            bf16_lo(v[q].z), bf16_hi(v[q].z), bf16_lo(v[q].w), bf16_hi(v[q].w)};
+        s_xb[t] = EX ? permute8_s(f, scale) : permute8(f);
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) {          // of what the MMA will see (without a scale fp16 is exact in its normal range only)
+            sum += EX ? f[e] : __half2float(__float2half_rn(f[e]));
+            sodd += EX ? f[e + 1] : __half2float(__float2half_rn(f[e + 1]));
         }
         sum = group_sum<4 * CPB>(sum);
         sodd = group_sum<4 * CPB>(sodd);
-        if (on && (t % (4 * CPB)) == 0) {
-            s_xsum[t / (4 * CPB)] = EX ? (sum + sodd) * kScaleS : sum + sodd;
+        if ((t % (4 * CPB)) == 0) {
+            s_xsum[t / (4 * CPB)] = EX ? (sum + sodd) * (kScaleS * scale) : sum + sodd;
             if (!EX) s_xbias[t / (4 * CPB)] = fmaf(1024.f, sum, 64.f * sodd);
         }
     }
     };
+    static_assert(kFW == 4, "a word of s_flag per warp");
     if (p.dep_wait < 0) convert_x();          // (a step that waits for its hidden state converts it once it is there)
     if (tid < kMaxRank) s_ud[tid] = 0.f;
 
@@ -673,11 +688,11 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                     for (int j = 0; j < 8; ++j) {
                         uint4 xb = make_uint4(0, 0, 0, 0);
                         if (g8 == 0) {
-                            xb = xbp[j * 4];
-                            if (EX) {                          // undo the 2^-4 of the odd positions
-                                xb.y = h2_as_u32(__hmul2(u32_as_h2(xb.y), __float2half2_rn(16.f)));
-                                xb.w = h2_as_u32(__hmul2(u32_as_h2(xb.w), __float2half2_rn(16.f)));
-                            }
+                            if (EX) {                          // (s_xb holds scaled blocks)
+                                const uint4 v = *reinterpret_cast<const uint4*>(p.x + mk0 + b * 256 + j * 32 + t4 * 8);
+                                const float f[8] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y), bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w)};
+                                xb = permute8(f);
+                            } else xb = xbp[j * 4];
                         }
                         mma16816(c, lw[j].x, lw2[j].x, lw[j].y, lw2[j].y, __byte_perm(xb.x, xb.y, 0x5410), __byte_perm(xb.z, xb.w, 0x5410));
                         mma16816(c, lw[j].z, lw2[j].z, lw[j].w, lw2[j].w, __byte_perm(xb.x, xb.y, 0x7632), __byte_perm(xb.z, xb.w, 0x7632));
@@ -944,10 +959,11 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                     }
                 }
                 if (t4 == 0) {
+                    const float un = EX ? s_xbias[0] : 1.f;
 #pragma unroll
                     for (int mt = 0; mt < NT; ++mt) {
-                        s_part[warp * 2 * rows_gu + mt * 16 + g8] = EX ? a_lo[mt] * kUnscaleS : a_lo[mt];
-                        s_part[warp * 2 * rows_gu + mt * 16 + 8 + g8] = EX ? a_hi[mt] * kUnscaleS : a_hi[mt];
+                        s_part[warp * 2 * rows_gu + mt * 16 + g8] = EX ? a_lo[mt] * un : a_lo[mt];
+                        s_part[warp * 2 * rows_gu + mt * 16 + 8 + g8] = EX ? a_hi[mt] * un : a_hi[mt];
                     }
                 }
             }
@@ -1025,7 +1041,12 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                 const float4 a = *reinterpret_cast<const float4*>(hq + i * 32 + q * 8);
                 const float4 b = *reinterpret_cast<const float4*>(hq + i * 32 + q * 8 + 4);
                 const float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-                s_hb[tid] = EX ? (lo ? permute8_lo_s(f) : permute8_s(f)) : (lo ? permute8_lo(f) : permute8(f));
+                if (EX) {
+                    constexpr unsigned mask = DCH * 8 == 32 ? 0xFFFFFFFFu : (1u << (DCH * 8)) - 1;
+                    const float scale = vector_scale(__reduce_max_sync(mask, abs_max8(f)));
+                    s_hb[tid] = lo ? permute8_lo_s(f, scale) : permute8_s(f, scale);
+                    if (tid == 0) s_hbias[0] = scale;
+                } else s_hb[tid] = lo ? permute8_lo(f) : permute8(f);
             } else if (tid >= 64 && tid < 64 + DCH / CPB) {
                 const int j = tid - 64;
                 float v = 0.f, vo = 0.f;
@@ -1033,7 +1054,7 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                     v += hq[j * 32 * CPB + e];
                     vo += hq[j * 32 * CPB + e + 1];
                 }
-                s_hsum[j] = EX ? (v + vo) * kScaleS : v + vo;
+                s_hsum[j] = EX ? (v + vo) * kScaleS : v + vo;                  // (EX: without the quarter's power of two)
                 if (!EX) s_hbias[j] = fmaf(1024.f, v, 64.f * vo);
             }
             __syncthreads();
@@ -1043,6 +1064,7 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
             {
                 const uint8_t* dbase = smem + S.d_codes + g8 * 16 + t4 * 4;
                 const uint8_t* dsz = smem + S.d_sz;
+                const float hscale = EX ? s_hbias[0] : 1.f, hun = EX ? kUnscaleS * vector_unscale(hscale) : 1.f;
                 // a warp's row tiles in two passes of TD tiles (the registers of one pass); the sums
                 // over the quarters of an expert are kept in s_o, every row by the lane that owns it
 #pragma unroll 1
@@ -1071,7 +1093,7 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                             }
                         }
                         const int gi = (ib * CPB * 32) >> p.gshift;
-                        const float hs = s_hsum[ib], hbias = EX ? 0.f : s_hbias[ib];
+                        const float hs = EX ? s_hsum[ib] * hscale : s_hsum[ib], hbias = EX ? 0.f : s_hbias[ib];
 #pragma unroll
                         for (int tt = 0; tt < TD; ++tt) {
                             const int ti = warp + kFW * (ps * TD + tt);
@@ -1087,7 +1109,7 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
                         for (int tt = 0; tt < TD; ++tt) {
                             const int ti = warp + kFW * (ps * TD + tt);
                             // (the first quarter of an expert starts the sums)
-                            const float vl = EX ? acc_lo[tt] * kUnscaleS : acc_lo[tt], vh = EX ? acc_hi[tt] * kUnscaleS : acc_hi[tt];
+                            const float vl = EX ? acc_lo[tt] * hun : acc_lo[tt], vh = EX ? acc_hi[tt] * hun : acc_hi[tt];
                             s_o[ti * 16 + g8] = it ? s_o[ti * 16 + g8] + vl : vl;
                             s_o[ti * 16 + 8 + g8] = it ? s_o[ti * 16 + 8 + g8] + vh : vh;
                         }

@@ -74,7 +74,10 @@ __device__ __forceinline__ uint4 permute8(const float (&v)[8]) {
 // 5, 7 (their nibble sits four bits higher) q * 2^-20 -- five instructions a word and nothing to remove: the tensor cores take
 // subnormal operands exactly.  The activations at odd positions carry the missing 2^-4 (permute8_s), sums of products come
 // out as 2^-24 of the dot product with the codes, in which unit the caller removes the zero point
-// (fma(-z, 2^-24 * sum of the activations, c)); kUnscaleS brings the end result back.  1e-6 relative on a layer's output.
+// (fma(-z, 2^-24 * sum of the activations, c)); kUnscaleS brings the end result back.
+// fp16 would round small activations to multiples of 2^-25, and those at odd positions to 2^-21.  So a vector of them (the state, a
+// quarter of an expert's h) is brought to a largest magnitude of 2^13 .. 2^14 first, by a power of two whose inverse goes into the
+// factor of the end result: what is lost is 2^-34 of the largest, whatever the magnitude.
 constexpr float kScaleS = 5.9604644775390625e-8f;      // 2^-24
 constexpr float kUnscaleS = 16777216.f;                // 2^24
 __device__ __forceinline__ void dequant_word_s(uint32_t w, uint32_t (&out)[4]) {
@@ -84,13 +87,22 @@ __device__ __forceinline__ void dequant_word_s(uint32_t w, uint32_t (&out)[4]) {
     out[2] = w2 & 0x000F000Fu;
     out[3] = w2 & 0x00F000F0u;
 }
-// permute8 and permute8_lo with the activations at odd positions scaled by 2^-4
-__device__ __forceinline__ uint4 permute8_s(const float (&v)[8]) {
-    const float f[8] = {v[0], v[1] * 0.0625f, v[2], v[3] * 0.0625f, v[4], v[5] * 0.0625f, v[6], v[7] * 0.0625f};
+// the power of two for a vector whose largest magnitude has the bits m (2^126 at most; infinities stay what they are), and its inverse
+__device__ __forceinline__ float vector_scale(uint32_t m) { return __uint_as_float(min(267u - (m >> 23), 253u) << 23); }
+__device__ __forceinline__ float vector_unscale(float s) { return __uint_as_float((254u << 23) - __float_as_uint(s)); }
+__device__ __forceinline__ uint32_t abs_max8(const float (&v)[8]) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) m = max(m, __float_as_uint(v[i]) & 0x7FFFFFFFu);
+    return m;
+}
+// permute8 and permute8_lo of the activations times the vector's power of two, those at odd positions times 2^-4 more
+__device__ __forceinline__ uint4 permute8_s(const float (&v)[8], float s) {
+    const float o = s * 0.0625f, f[8] = {v[0] * s, v[1] * o, v[2] * s, v[3] * o, v[4] * s, v[5] * o, v[6] * s, v[7] * o};
     return permute8(f);
 }
-__device__ __forceinline__ uint4 permute8_lo_s(const float (&v)[8]) {
-    const float f[8] = {v[0], v[1] * 0.0625f, v[2], v[3] * 0.0625f, v[4], v[5] * 0.0625f, v[6], v[7] * 0.0625f};
+__device__ __forceinline__ uint4 permute8_lo_s(const float (&v)[8], float s) {
+    const float o = s * 0.0625f, f[8] = {v[0] * s, v[1] * o, v[2] * s, v[3] * o, v[4] * s, v[5] * o, v[6] * s, v[7] * o};
     return permute8_lo(f);
 }
 // The biased form: codes 0, 2, 4, 6 of a word as 1024 + q, codes 1, 3, 5, 7 as 64 + q, five instructions a word too.  The dot

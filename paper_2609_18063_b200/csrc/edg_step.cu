@@ -266,17 +266,29 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
     // eight values of the state (value i of them): the B words of the MMAs, the block sums
     auto take_x = [&](int i, uint4 v) {
         const float f[8] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y), bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w)};
-        s_xb[i] = EX ? permute8_s(f) : permute8(f);
+        float scale = 1.f;
+        if (EX) {                                                        // the largest magnitude of the state, over the warps that hold it
+            uint32_t* s_max = reinterpret_cast<uint32_t*>(s_red) + 32;
+            const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, abs_max8(f));
+            if (lane == 0) s_max[i / 32] = m;
+            asm volatile("bar.sync 2, %0;" ::"n"(H / 8) : "memory");
+            uint32_t all = 0;
+#pragma unroll
+            for (int w = 0; w < H / 256; ++w) all = max(all, s_max[w]);
+            scale = vector_scale(all);
+            if (i == 0) s_xbias[0] = kUnscaleS * vector_unscale(scale);
+        }
+        s_xb[i] = EX ? permute8_s(f, scale) : permute8(f);
         float sum = 0.f, sodd = 0.f;
 #pragma unroll
-        for (int e = 0; e < 8; e += 2) {
-            sum += __half2float(__float2half_rn(f[e]));
-            sodd += __half2float(__float2half_rn(f[e + 1]));
+        for (int e = 0; e < 8; e += 2) {                                 // of what the MMA sees
+            sum += EX ? f[e] : __half2float(__float2half_rn(f[e]));
+            sodd += EX ? f[e + 1] : __half2float(__float2half_rn(f[e + 1]));
         }
         sum = group_sum<4 * CPB>(sum);
         sodd = group_sum<4 * CPB>(sodd);
         if (i % (4 * CPB) == 0) {
-            s_xsum[i / (4 * CPB)] = EX ? (sum + sodd) * kScaleS : sum + sodd;
+            s_xsum[i / (4 * CPB)] = EX ? (sum + sodd) * (kScaleS * scale) : sum + sodd;
             if (!EX) s_xbias[i / (4 * CPB)] = fmaf(1024.f, sum, 64.f * sodd);
         }
     };
@@ -598,7 +610,7 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
                         const float2 st = reinterpret_cast<const float2*>(un + mt * CT + (blk / NBW) * NCK * 256)[(blk % NBW) * 16 + ((row + 4 * w) & 15)];
                         v = fmaf(st.x, st.y, v);
                     }
-                if (EX) v *= kUnscaleS;
+                if (EX) v *= s_xbias[0];
             }
             const float p1 = __shfl_down_sync(0xFFFFFFFFu, v, 1), p2 = __shfl_down_sync(0xFFFFFFFFu, v, 2), p3 = __shfl_down_sync(0xFFFFFFFFu, v, 3);
             v = ((v + p1) + p2) + p3;
@@ -680,14 +692,16 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
                 s_udi[item * (p.rmax + 1) + udj] = ((__uint_as_float(u.x) + __uint_as_float(u.y)) + __uint_as_float(u.z)) + __uint_as_float(u.w);
             const float f[8] = {__uint_as_float(a.x), __uint_as_float(a.y), __uint_as_float(a.z), __uint_as_float(a.w),
                                 __uint_as_float(b.x), __uint_as_float(b.y), __uint_as_float(b.z), __uint_as_float(b.w)};
+            const float scale = EX ? vector_scale(group_max<4 * DCH>(abs_max8(f))) : 1.f;      // of an (expert, quarter)
             if (on) {                                                    // [chunk][value, residual][4]
-                s_hb[(i >> 2) * 8 + (i & 3)] = EX ? permute8_s(f) : permute8(f);
-                s_hb[(i >> 2) * 8 + 4 + (i & 3)] = EX ? permute8_lo_s(f) : permute8_lo(f);
+                s_hb[(i >> 2) * 8 + (i & 3)] = EX ? permute8_s(f, scale) : permute8(f);
+                s_hb[(i >> 2) * 8 + 4 + (i & 3)] = EX ? permute8_lo_s(f, scale) : permute8_lo(f);
             }
             if (EX) {
                 float s = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]));
                 s = group_sum<4 * CPB>(s);
-                if (on && i % (4 * CPB) == 0) s_hsum[i / (4 * CPB)] = s * kScaleS;
+                if (on && i % (4 * CPB) == 0) s_hsum[i / (4 * CPB)] = s * (kScaleS * scale);
+                if (on && i % (4 * DCH) == 0) s_hbias[i / (4 * DCH)] = kUnscaleS * vector_unscale(scale);
             } else if (on) {
                 float* q = s_h + (i / (4 * CPB)) * kHPad + (i % (4 * CPB)) * 8;
                 *reinterpret_cast<uint4*>(q) = a;
@@ -752,8 +766,8 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
                             acc_lo = fmaf(__low2float(z0), fmaf(-__high2float(z0), hs, EX ? c[v][b][0] + c[v][b][1] : c[v][b][0] + c[v][b][1] - hbias), acc_lo);
                             acc_hi = fmaf(__low2float(z1), fmaf(-__high2float(z1), hs, EX ? c[v][b][2] + c[v][b][3] : c[v][b][2] + c[v][b][3] - hbias), acc_hi);
                         }
-                        s_part[item * 17 + g8] = EX ? acc_lo * kUnscaleS : acc_lo;
-                        s_part[item * 17 + 8 + g8] = EX ? acc_hi * kUnscaleS : acc_hi;
+                        s_part[item * 17 + g8] = EX ? acc_lo * s_hbias[item] : acc_lo;
+                        s_part[item * 17 + 8 + g8] = EX ? acc_hi * s_hbias[item] : acc_hi;
                     }
                 }
             }
