@@ -6,6 +6,8 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <atomic>
+
 #include "../../include/edg_moe.h"
 
 namespace edg {
@@ -18,6 +20,29 @@ void set_cuda_error(cudaError_t e);            // records the error for edg_last
         cudaError_t _e = (expr);                                             \
         if (_e != cudaSuccess) { ::edg::set_cuda_error(_e); return EDG_E_CUDA; } \
     } while (0)
+
+// A kernel's attributes are those of the device that is current when they are set: what has to be set once is set once per device.
+class OncePerDevice {
+    std::atomic<uint64_t> done_{0};
+public:
+    template <typename F>
+    cudaError_t operator()(F set) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        const uint64_t bit = dev < 64 ? 1ull << dev : 0;
+        if ((done_.load(std::memory_order_acquire) & bit) != 0) return cudaSuccess;
+        e = set();                                                       // (setting them twice does no harm)
+        if (e == cudaSuccess) done_.fetch_or(bit, std::memory_order_release);
+        return e;
+    }
+};
+template <typename... Kernels>
+cudaError_t allow_smem(size_t bytes, Kernels... kernels) {
+    cudaError_t e = cudaSuccess;
+    ((e = e == cudaSuccess ? cudaFuncSetAttribute(kernels, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) : e), ...);
+    return e;
+}
 
 inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 

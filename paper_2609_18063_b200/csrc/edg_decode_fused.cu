@@ -1286,15 +1286,13 @@ bool fused_supported(const edg_layer_desc& d) {
 template <int NCW, int DCH, int TG, int TD, int CPB, bool EX>
 static cudaError_t launch_form(const FusedParams& p, size_t smem, bool pdl, cudaStream_t st) {
     auto kern = fused_layer_kernel<NCW, DCH, TG, TD, CPB, EX>;
-    static bool configured = false;       // per-process, per-instantiation one-time attributes
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmemLimit);
-        if (e != cudaSuccess) return e;
+    static OncePerDevice once;
+    const cudaError_t e = once([&] {
+        const cudaError_t s = allow_smem(kFusedSmemLimit, kern);
         // four CTAs per SM: more clusters resident at once
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+        return s != cudaSuccess ? s : cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    });
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((p.K / p.epc + p.n_shared) * (kDownSlices / p.qpc) * kC + p.head_extra, 1, 1);
     cfg.blockDim = dim3(kFW * 32, 1, 1);

@@ -886,15 +886,11 @@ int32_t run_grouped_ffn(const edg_layer_desc* d, const GroupedParams& g, const W
                           {kc_el / g.group * 8, 2 * GW, (uint32_t)p.sp, 1, 1});
     if (!ok) { set_cuda_error(cudaErrorInvalidValue); return EDG_E_CUDA; }
 
-    static bool configured = false;
-    if (!configured) {
-        EDG_CUDA_TRY(cudaFuncSetAttribute(grouped_ffn_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GSmemLimit));
-        EDG_CUDA_TRY(cudaFuncSetAttribute(grouped_ffn_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GSmemLimit));
-        EDG_CUDA_TRY(cudaFuncSetAttribute(grouped_ffn_kernel<1, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GSmemLimit));
-        EDG_CUDA_TRY(cudaFuncSetAttribute(grouped_ffn_kernel<2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GSmemLimit));
-        EDG_CUDA_TRY(cudaFuncSetAttribute(group_pairs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024));
-        configured = true;
-    }
+    static OncePerDevice once;
+    EDG_CUDA_TRY(once([] {
+        const cudaError_t e = allow_smem(GSmemLimit, grouped_ffn_kernel<1, 1>, grouped_ffn_kernel<2, 1>, grouped_ffn_kernel<1, 4>, grouped_ffn_kernel<2, 4>);
+        return e != cudaSuccess ? e : allow_smem(210 * 1024, group_pairs_kernel);
+    }));
     GroupArgs ga{};
     ga.slots = g.slots; ga.table = g.table; ga.experts = g.experts;
     ga.pair_slot = g.pair_slot; ga.order = order; ga.n_tiles = n_tiles; ga.ticket = p.ticket;

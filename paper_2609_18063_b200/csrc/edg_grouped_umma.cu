@@ -501,24 +501,18 @@ bool umma_grouped_supported(const edg_layer_desc& d) {
 }
 
 cudaError_t launch_umma_gate_up(const GroupedParams& p, int max_tiles, cudaStream_t st) {
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(umma_gate_up_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umma_smem_bytes(U_ACT_GU_BYTES));
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static OncePerDevice once;
+    const cudaError_t e = once([] { return allow_smem(umma_smem_bytes(U_ACT_GU_BYTES), umma_gate_up_kernel); });
+    if (e != cudaSuccess) return e;
     umma_gather_x_kernel<<<dim3(8, max_tiles), 256, 0, st>>>(p);
     umma_gate_up_kernel<<<dim3(p.I / 128, max_tiles), U_THREADS, umma_smem_bytes(U_ACT_GU_BYTES), st>>>(p);
     return cudaGetLastError();
 }
 
 cudaError_t launch_umma_down(const GroupedParams& p, int max_tiles, cudaStream_t st) {
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(umma_down_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umma_smem_bytes(U_ACT_D_BYTES));
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static OncePerDevice once;
+    const cudaError_t e = once([] { return allow_smem(umma_smem_bytes(U_ACT_D_BYTES), umma_down_kernel); });
+    if (e != cudaSuccess) return e;
     umma_down_kernel<<<dim3(p.H / 256, max_tiles), U_THREADS, umma_smem_bytes(U_ACT_D_BYTES), st>>>(p);
     return cudaGetLastError();
 }

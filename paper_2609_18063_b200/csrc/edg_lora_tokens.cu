@@ -208,8 +208,8 @@ bool launch_lora_ax_tokens(const edg_layer_desc* d, const void* x, const edg_lor
     const uint16_t* xx = static_cast<const uint16_t*>(x);
 #define EDG_LAX(TI, KB_)                                                                                         \
     do {                                                                                                         \
-        static bool conf = false;                                                                                \
-        if (!conf) { cudaFuncSetAttribute(lora_ax_tokens_kernel<TI, KB_>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024); conf = true; } \
+        static OncePerDevice once;                                                                               \
+        once([] { return allow_smem(64 * 1024, lora_ax_tokens_kernel<TI, KB_>); });                              \
         lora_ax_tokens_kernel<TI, KB_><<<grid, 256, sm, st>>>(xx, Ag, Au, u_gu, T, H, r);                        \
     } while (0)
     if (H == 2048) { if (tiles == 1) EDG_LAX(1, 8); else EDG_LAX(2, 8); }

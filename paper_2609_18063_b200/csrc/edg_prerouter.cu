@@ -729,13 +729,8 @@ int32_t run_prerouter(const edg_layer_desc* d, const void* W_pre, const void* s,
     cfg.attrs = at;
     cfg.numAttrs = 1;
     if (batched) {
-        static bool configured = false;
-        if (!configured) {
-            EDG_CUDA_TRY(cudaFuncSetAttribute(prerouter_tokens_kernel<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-            EDG_CUDA_TRY(cudaFuncSetAttribute(prerouter_tokens_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-            EDG_CUDA_TRY(cudaFuncSetAttribute(prerouter_tokens_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-            configured = true;
-        }
+        static OncePerDevice once;
+        EDG_CUDA_TRY(once([] { return allow_smem(200 * 1024, prerouter_tokens_kernel<__half>, prerouter_tokens_kernel<float>, prerouter_tokens_mma_kernel); }));
         if (cfg.dynamicSmemBytes > 200 * 1024) return EDG_E_SHAPE;
         // an fp16 head whose rows and columns split into whole MMA tiles goes to the tensor cores
         if (d->pre_dtype == EDG_F16 && d->E % (16 * kPreCluster) == 0 && d->H % (32 * kPreWarps) == 0) {
@@ -841,12 +836,8 @@ int32_t edg::run_prerouter_mlp(const edg_layer_desc* desc, const edg_mlp_head* h
     const int perE = (desc->E + edg::kPreCluster - 1) / edg::kPreCluster;
     cfg.dynamicSmemBytes = edg::kMlpWarps * edg::kMlpSlots * edg::kMlpPieces * 16 + (size_t)(desc->E + desc->H + D + perE * 32 + 64) * sizeof(float);
     cfg.stream = stream;
-    static bool configured = false;
-    if (!configured) {
-        EDG_CUDA_TRY(cudaFuncSetAttribute(edg::prerouter_mlp_kernel<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-        EDG_CUDA_TRY(cudaFuncSetAttribute(edg::prerouter_mlp_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-        configured = true;
-    }
+    static edg::OncePerDevice once;
+    EDG_CUDA_TRY(once([] { return edg::allow_smem(200 * 1024, edg::prerouter_mlp_kernel<__half>, edg::prerouter_mlp_kernel<float>); }));
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = edg::kPreCluster;

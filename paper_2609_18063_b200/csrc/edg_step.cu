@@ -976,14 +976,12 @@ constexpr size_t kStepSmemLimit = 112 * 1024, kStepSmemLone = 120 * 1024;      /
 template <int NCK, int DCH, int CPB, bool EX>
 cudaError_t launch_step(const StepParams& p, int grid, cudaStream_t st) {
     auto kern = step_kernel<NCK, DCH, CPB, EX>;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStepSmemLone);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static OncePerDevice once;
+    const cudaError_t e = once([&] {
+        const cudaError_t s = allow_smem(kStepSmemLone, kern);
+        return s != cudaSuccess ? s : cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    });
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, 1, 1);
     cfg.blockDim = dim3(TThreads, 1, 1);
