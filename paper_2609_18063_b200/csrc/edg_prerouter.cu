@@ -3,7 +3,7 @@
 //
 // One thread-block cluster per head: the E rows of the head are split over the CTAs of the
 // cluster, every CTA writes its logits straight into the leader CTA's shared memory
-// (distributed shared memory), and after one cluster barrier a single warp of the leader does
+// (distributed shared memory; a first arrival says that they all run), and after one cluster barrier a single warp of the leader does
 // softmax + top-k with warp shuffles.  No global scratch, no atomics, one launch.
 #include <cooperative_groups.h>
 #include <math_constants.h>
@@ -78,6 +78,7 @@ template <> struct RowDot<float> {
 
 template <typename WT>
 __global__ void __launch_bounds__(kPreWarps * 32) prerouter_kernel(PreParams p) {
+    cluster_arrive_relaxed();
     cg::cluster_group cluster = cg::this_cluster();
     const int crank = (int)cluster.block_rank();
     const int csize = (int)cluster.num_blocks();
@@ -90,6 +91,7 @@ __global__ void __launch_bounds__(kPreWarps * 32) prerouter_kernel(PreParams p) 
     const uint16_t* sv = p.s + (size_t)head * p.H;
     for (int i = threadIdx.x; i < p.H; i += blockDim.x) s_x[i] = bf16_bits_to_float(sv[i]);
     __syncthreads();
+    cluster_wait();                     // every CTA of the cluster runs: the leader's shared memory may be written
 
     float* leader = cluster.map_shared_rank(s_logits, 0);
     const int per = (p.E + csize - 1) / csize;
@@ -120,6 +122,7 @@ constexpr int kTokBlock = 8;
 
 template <typename WT>
 __global__ void __launch_bounds__(kPreWarps * 32) prerouter_tokens_kernel(PreParams p, int T) {
+    cluster_arrive_relaxed();
     cg::cluster_group cluster = cg::this_cluster();
     const int crank = (int)cluster.block_rank();
     const int csize = (int)cluster.num_blocks();
@@ -134,6 +137,7 @@ __global__ void __launch_bounds__(kPreWarps * 32) prerouter_tokens_kernel(PrePar
             s_x[tt * p.H + i] = t < T ? bf16_bits_to_float(p.s[(size_t)t * p.H + i]) : 0.f;
     }
     __syncthreads();
+    cluster_wait();                     // every CTA of the cluster runs: the leader's shared memory may be written
 
     float* leader = cluster.map_shared_rank(s_logits, 0);
     const int per = (p.E + csize - 1) / csize;
@@ -213,6 +217,7 @@ __global__ void __launch_bounds__(kPreWarps * 32) prerouter_tokens_kernel(PrePar
 // in fp32.
 constexpr int kMmaHeadKs = 256;        // k per warp and pass: 8 blocks of 32
 __global__ void __launch_bounds__(kPreWarps * 32) prerouter_tokens_mma_kernel(PreParams p, int T) {
+    cluster_arrive_relaxed();
     cg::cluster_group cluster = cg::this_cluster();
     const int crank = (int)cluster.block_rank();
     const int csize = (int)cluster.num_blocks();
@@ -256,6 +261,7 @@ __global__ void __launch_bounds__(kPreWarps * 32) prerouter_tokens_mma_kernel(Pr
         *reinterpret_cast<uint4*>(s_xh + tt * xs + c * 16) = o;
     }
     __syncthreads();
+    cluster_wait();                     // every CTA of the cluster runs: the leader's shared memory may be written
 
     float* leader = cluster.map_shared_rank(s_logits, 0);
     for (int r0 = r_first; r0 < (crank + 1) * per; r0 += 32) {
@@ -357,6 +363,7 @@ constexpr int kMlpSlots = 3;
 // on the slots.
 template <typename WT>
 __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(MlpParams p) {
+    cluster_arrive_relaxed();
     cg::cluster_group cluster = cg::this_cluster();
     const int crank = (int)cluster.block_rank();
     const int csize = (int)cluster.num_blocks();
@@ -421,6 +428,7 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(MlpParams
         *reinterpret_cast<float4*>(s_x1 + i * 4) = make_float4(bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w));
     }
     __syncthreads();
+    cluster_wait();                     // every CTA of the cluster runs: its shared memory may be written
 
     int used = 0;
     // acc + this lane's share of a row (n pieces, in c chunks) times v; the row's slots go back to the ring
