@@ -346,8 +346,34 @@ struct MlpParams {
     int32_t* mirror;        // [n_heads][K] in mapped pinned host memory, or null
 };
 
-static __device__ __forceinline__ void ring_wait(uint64_t* bar, uint32_t parity) {
-    for (uint32_t i = 0; i < kSpinLimit && !mbar_try_wait(bar, parity); ++i) {}
+#ifndef EDG_MLP_RING_POLLS
+#define EDG_MLP_RING_POLLS kSpinLimit
+#endif
+static __device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, uint32_t polls) {
+    for (uint32_t i = 0; i < polls; ++i)
+        if (mbar_try_wait(bar, parity)) return true;
+    return false;
+}
+
+// piece c of a row of weights times v, whose values 0-3 of every eight are in v0 and 4-7 in v1: eight fp16 weights, or four fp32
+static __device__ __forceinline__ float mul_halves(const uint4& w, const float* v0, const float* v1, int c, float acc) {
+    const float4 x0 = *reinterpret_cast<const float4*>(v0 + c * 4), x1 = *reinterpret_cast<const float4*>(v1 + c * 4);
+    const float2 a = __half22float2(u32_as_h2(w.x)), b = __half22float2(u32_as_h2(w.y)), d = __half22float2(u32_as_h2(w.z)), e = __half22float2(u32_as_h2(w.w));
+    acc = fmaf(a.x, x0.x, acc); acc = fmaf(a.y, x0.y, acc); acc = fmaf(b.x, x0.z, acc); acc = fmaf(b.y, x0.w, acc);
+    acc = fmaf(d.x, x1.x, acc); acc = fmaf(d.y, x1.y, acc); acc = fmaf(e.x, x1.z, acc); acc = fmaf(e.y, x1.w, acc);
+    return acc;
+}
+static __device__ __forceinline__ float mul_floats(const uint4& w, const float* v0, const float* v1, int c, float acc) {
+    const float4 x = *reinterpret_cast<const float4*>((c & 1 ? v1 : v0) + (c >> 1) * 4);
+    acc = fmaf(__uint_as_float(w.x), x.x, acc); acc = fmaf(__uint_as_float(w.y), x.y, acc);
+    acc = fmaf(__uint_as_float(w.z), x.z, acc); acc = fmaf(__uint_as_float(w.w), x.w, acc);
+    return acc;
+}
+// fc1 with its gathered columns and bias, gelu
+static __device__ __forceinline__ float gelu_row(float z, __half gc, __half gq, bool biased, float bias) {
+    z = warp_sum(z + __half2float(gc) + __half2float(gq));
+    if (biased) z += bias;
+    return 0.5f * z * (1.f + erff(z * 0.70710678118654752f));
 }
 
 constexpr int kMlpWarps = 8;            // warps per CTA of the full head
@@ -361,8 +387,43 @@ constexpr int kMlpSlots = 3;
 // place; three CTAs fit an SM (100 KB in flight): 39.3 us.
 // Per lane the products are summed in the order of the pieces (lane, lane + 32, ..), then over the lanes: results do not depend
 // on the slots.
+// There is no status word to raise when a copy does not come.  A warp that has polled for one in vain (EDG_MLP_RING_POLLS times) issues no
+// more of them, and in the end the leader evaluates the head once more by itself, with plain loads in the same order.
 template <typename WT>
-__global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(MlpParams p) {
+static __device__ __noinline__ void head_with_plain_loads(const MlpParams& p, int head, const float* s_x0, const float* s_x1, float* s_a0, float* s_a1,
+                                                          float* s_logits) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int hc = lane < p.K ? p.cur[(size_t)head * p.K + lane] : -1, hq = lane < p.K ? p.prev[(size_t)head * p.K + lane] : -1;
+    if (hc >= p.E) hc = -1;
+    if (hq >= p.E) hq = -1;
+    for (int r = warp; r < p.D; r += kMlpWarps) {
+        const __half* row = p.W1 + ((size_t)head * p.D + r) * (p.H + 2 * p.E);
+        const __half gc = hc >= 0 ? row[p.H + hc] : __float2half(0.f), gq = hq >= 0 ? row[p.H + p.E + hq] : __float2half(0.f);
+        float z = 0.f;
+        for (int c = lane; c < p.H / 8; c += 32) z = mul_halves(reinterpret_cast<const uint4*>(row)[c], s_x0, s_x1, c, z);
+        z = gelu_row(z, gc, gq, p.b1 != nullptr, p.b1 != nullptr ? __half2float(p.b1[(size_t)head * p.D + r]) : 0.f);
+        if (lane == 0) ((r & 4) ? s_a1 : s_a0)[(r >> 3) * 4 + (r & 3)] = z;
+    }
+    __syncthreads();
+    for (int e = warp; e < p.E; e += kMlpWarps) {
+        float l = 0.f, v = 0.f;
+        const uint4* row = reinterpret_cast<const uint4*>(p.W2 + ((size_t)head * p.E + e) * p.D);
+        for (int c = lane; c < p.D / 8; c += 32) l = mul_halves(row[c], s_a0, s_a1, c, l);
+        if (p.Wres != nullptr) {
+            row = reinterpret_cast<const uint4*>(static_cast<const WT*>(p.Wres) + ((size_t)head * p.E + e) * p.H);
+            for (int c = lane; c < p.H * (int)sizeof(WT) / 16; c += 32)
+                v = sizeof(WT) == 2 ? mul_halves(row[c], s_x0, s_x1, c, v) : mul_floats(row[c], s_x0, s_x1, c, v);
+            l += v;
+        }
+        l = warp_sum(l);
+        if (p.b2 != nullptr) l += __half2float(p.b2[(size_t)head * p.E + e]);
+        if (lane == 0) s_logits[e] = l;
+    }
+    __syncthreads();
+}
+
+template <typename WT>
+__global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(const __grid_constant__ MlpParams p) {
     cluster_arrive_relaxed();
     cg::cluster_group cluster = cg::this_cluster();
     const int crank = (int)cluster.block_rank();
@@ -381,8 +442,11 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(MlpParams
     float* s_logits = s_part + perE * 32;   // [E]   (the leader's copy collects every CTA's rows)
     float* s_win = s_logits + p.E;      // 64 words for the winners
     __shared__ __align__(8) uint64_t bars[kMlpWarps][kMlpSlots];
+    __shared__ int s_lost[kMlpWarps + 1];   // per warp the first item whose copy did not come, or -1; whether there is one at all (the leader's)
 
     if (lane == 0) {
+        s_lost[warp] = -1;
+        s_lost[kMlpWarps] = 0;
         for (int i = 0; i < kMlpSlots; ++i) mbar_init(&bars[warp][i], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -393,7 +457,8 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(MlpParams
     const int n1 = r0 < rend ? (rend - r0 + kMlpWarps - 1) / kMlpWarps : 0, n2 = e0 < eend ? (eend - e0 + kMlpWarps - 1) / kMlpWarps : 0;
     const int p1 = p.H / 8, pr = p.Wres != nullptr ? p.H * (int)sizeof(WT) / 16 : 0, p2 = p.D / 8;       // 16-byte pieces of a row
     const int c1 = (p1 + kMlpPieces - 1) / kMlpPieces, cr = (pr + kMlpPieces - 1) / kMlpPieces, c2 = (p2 + kMlpPieces - 1) / kMlpPieces;
-    const int total = n1 * c1 + n2 * (cr + c2);
+    int total = n1 * c1 + n2 * (cr + c2);
+    uint32_t polls = EDG_MLP_RING_POLLS;                                 // 0 once a copy has not come
     // the slot after next: which row and piece the next copy fetches
     int f_kind = n1 > 0 ? 0 : (cr > 0 ? 1 : 2), f_row = 0, f_chunk = 0, fetched = 0;
     auto fetch = [&]() {                                                 // lane 0
@@ -436,7 +501,10 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(MlpParams
         float acc = 0.f;
         for (int ch = 0; ch < chunks; ++ch, ++used) {
             const int slot = used % kMlpSlots;
-            ring_wait(&bars[warp][slot], (used / kMlpSlots) & 1);
+            if (!ring_wait(&bars[warp][slot], (used / kMlpSlots) & 1, polls)) {
+                if (lane == 0 && s_lost[warp] < 0) { s_lost[warp] = used; total = fetched; }
+                polls = 0;
+            }
             const uint4* src = reinterpret_cast<const uint4*>(ring + slot * kSlotBytes);
             uint4 w[kMlpPieces / 32];
 #pragma unroll
@@ -450,22 +518,9 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(MlpParams
         }
         return acc;
     };
-    auto halves = [](const uint4& w, const float* v0, const float* v1, int c, float acc) {       // eight fp16 weights
-        const float4 x0 = *reinterpret_cast<const float4*>(v0 + c * 4), x1 = *reinterpret_cast<const float4*>(v1 + c * 4);
-        const float2 a = __half22float2(u32_as_h2(w.x)), b = __half22float2(u32_as_h2(w.y)), d = __half22float2(u32_as_h2(w.z)), e = __half22float2(u32_as_h2(w.w));
-        acc = fmaf(a.x, x0.x, acc); acc = fmaf(a.y, x0.y, acc); acc = fmaf(b.x, x0.z, acc); acc = fmaf(b.y, x0.w, acc);
-        acc = fmaf(d.x, x1.x, acc); acc = fmaf(d.y, x1.y, acc); acc = fmaf(e.x, x1.z, acc); acc = fmaf(e.y, x1.w, acc);
-        return acc;
-    };
-    auto by_state = [&](const uint4& w, int c, float acc) { return halves(w, s_x0, s_x1, c, acc); };
-    auto by_gelu = [&](const uint4& w, int c, float acc) { return halves(w, s_a0, s_a1, c, acc); };
-    auto by_state32 = [&](const uint4& w, int c, float acc) {            // four fp32 weights
-        const float4 x = *reinterpret_cast<const float4*>((c & 1 ? s_x1 : s_x0) + (c >> 1) * 4);
-        acc = fmaf(__uint_as_float(w.x), x.x, acc); acc = fmaf(__uint_as_float(w.y), x.y, acc);
-        acc = fmaf(__uint_as_float(w.z), x.z, acc); acc = fmaf(__uint_as_float(w.w), x.w, acc);
-        return acc;
-    };
-
+    auto by_state = [&](const uint4& w, int c, float acc) { return mul_halves(w, s_x0, s_x1, c, acc); };
+    auto by_state32 = [&](const uint4& w, int c, float acc) { return mul_floats(w, s_x0, s_x1, c, acc); };
+    auto by_gelu = [&](const uint4& w, int c, float acc) { return mul_halves(w, s_a0, s_a1, c, acc); };
     // the K-hot parts of the feature pick columns: lane k < K holds the k-th expert of either list
     int hc = -1, hq = -1;
     if (lane < p.K) {
@@ -480,10 +535,7 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(MlpParams
         const __half* row = p.W1 + ((size_t)head * p.D + r) * F;
         const __half gc = hc >= 0 ? row[p.H + hc] : __float2half(0.f), gq = hq >= 0 ? row[p.H + p.E + hq] : __float2half(0.f);
         const float bias = p.b1 != nullptr ? __half2float(p.b1[(size_t)head * p.D + r]) : 0.f;
-        float z = row_dot(p1, c1, by_state);
-        z = warp_sum(z + __half2float(gc) + __half2float(gq));
-        if (p.b1 != nullptr) z += bias;
-        const float a = 0.5f * z * (1.f + erff(z * 0.70710678118654752f));
+        const float a = gelu_row(row_dot(p1, c1, by_state), gc, gq, p.b1 != nullptr, bias);
         if (lane < csize) *cluster.map_shared_rank(((r & 4) ? s_a1 : s_a0) + (r >> 3) * 4 + (r & 3), lane) = a;
     }
     if (cr > 0)
@@ -505,8 +557,12 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(MlpParams
         if (p.b2 != nullptr) l += bias;
         if (lane == 0) leader[e] = l;
     }
+    if (polls == 0) *cluster.map_shared_rank(s_lost + kMlpWarps, 0) = 1;
+    if (lane == 0 && s_lost[warp] >= 0) // (copies still on their way land before this CTA ends)
+        for (int i = s_lost[warp]; i < fetched; ++i) ring_wait(&bars[warp][i % kMlpSlots], (i / kMlpSlots) & 1, kSpinLimit);
     cluster.sync();                     // every CTA's logits have landed in the leader
     if (crank != 0) return;
+    if (s_lost[kMlpWarps] != 0) head_with_plain_loads<WT>(p, head, s_x0, s_x1, s_a0, s_a1, s_logits);
 
     if (warp == 0) {
         int32_t* s_i = reinterpret_cast<int32_t*>(s_win);

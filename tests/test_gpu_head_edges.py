@@ -1,7 +1,11 @@
 """The full head's streaming rings and the register form of the sigmoid-group gate at the sizes where they can go wrong: rows of half a
 slot, of one, of several and of a broken one, warps and CTAs without rows, fp32 residual rows; every number of entries
 per lane, one expert group per lane, ties and NaN.  The checks are those of test_gpu_routing."""
+import ctypes as C
 import dataclasses
+import os
+import shutil
+import subprocess
 
 import numpy as np
 import pytest
@@ -14,6 +18,8 @@ from workloads import synth
 import test_gpu_routing as routing
 
 pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.mark.parametrize("H,E,K,pre,width,n_heads,variant", [
@@ -50,3 +56,35 @@ def test_group_gate_ties_and_nans():
     want_i, want_w = orc.sigmoid_group_topk(l[1], 4, 8, 4, 2.5)
     assert got[1] == want_i.tolist() == [5, 6, 70, 71]
     assert np.allclose(gates.cpu().numpy()[1], want_w, rtol=2e-6)
+
+
+@pytest.mark.parametrize("pre,variant", [("f16", "full"), ("f32", "full"), ("f16", "no_residual")])
+def test_full_head_whose_copies_do_not_come_in_time(tmp_path, pre, variant):
+    """The library's heads built with no polls at all: every wait for a copy runs out at once, the rows come straight from memory, and the
+    results are those of the rings, bit for bit."""
+    so = str(tmp_path / "late.so")
+    csrc = os.path.join(ROOT, "paper_2609_18063_b200", "csrc")
+    subprocess.run([shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-shared", "-Xcompiler",
+                    "-fPIC", "-Xlinker", "-Bsymbolic", "-DEDG_MLP_RING_POLLS=0", "-I", os.path.join(ROOT, "include"), "-o", so,
+                    os.path.join(csrc, "edg_prerouter.cu"), os.path.join(csrc, "edg_pack.cu")], check=True)
+    late = C.CDLL(so, mode=os.RTLD_LAZY)
+    n, H, E, K, D = 3, 1024, 40, 4, 520
+    d = edg.make_desc(None, H=H, I=256, E=E, K=K, group=32, rank=0, n_adapters=1, n_slots=E, pre_dtype=pre)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(4)
+
+    def rnd(*shape):
+        return (torch.randn(shape, generator=gen, device="cuda") * 0.03).half()
+    W1, b1, W2, b2, Wr, x = rnd(n, D, H + 2 * E), rnd(n, D), rnd(n, E, D), rnd(n, E), rnd(n, E, H), torch.randn((n, H), generator=gen, device="cuda").bfloat16()
+    Wr = (Wr.float() if pre == "f32" else Wr) if variant == "full" else None
+    cur = torch.arange(n * K, dtype=torch.int32, device="cuda").view(n, K)
+    out = [(torch.zeros((n, K), dtype=torch.int32, device="cuda"), torch.zeros((n, K), device="cuda"), torch.zeros((n, E), device="cuda")) for _ in range(2)]
+    edg.prerouter_mlp_topk(d, W1, b1, W2, b2, Wr, D, x, cur, cur, n, *out[0])
+    ptr = lambda t: None if t is None else C.c_void_p(t.data_ptr())
+    head = edg.binding.MlpHead(*[None if t is None else t.data_ptr() for t in (W1, b1, W2, b2, Wr)], D)
+    torch.cuda.synchronize()
+    assert late.prerouter_mlp_topk(C.byref(d), C.byref(head), ptr(x), ptr(cur), ptr(cur), n, *[ptr(t) for t in out[1]], None) == 0
+    torch.cuda.synchronize()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
+    assert out[0][2].abs().max() > 0
