@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(const __g
     extern __shared__ __align__(128) uint8_t smem8[];
     uint8_t* ring = smem8 + warp * kMlpSlots * kSlotBytes;                              // this warp's slots
     float* s_x0 = reinterpret_cast<float*>(smem8 + kMlpWarps * kMlpSlots * kSlotBytes); // [H/2] values 0-3 of every eight of the state,
-    float* s_x1 = s_x0 + p.H / 2;       // [H/2] and values 4-7
+    float* s_x1 = s_x0 + p.H / 2 + 16;  // [H/2] and values 4-7 (in other banks: fp32 rows read both at once)
     float* s_a0 = s_x1 + p.H / 2;       // [D/2] gelu(fc1) in the same way, complete in every CTA after the first cluster barrier
     float* s_a1 = s_a0 + p.D / 2;       // [D/2]
     const int perD = (p.D + csize - 1) / csize, perE = (p.E + csize - 1) / csize;
@@ -898,7 +898,7 @@ int32_t edg::run_prerouter_mlp(const edg_layer_desc* desc, const edg_mlp_head* h
     cfg.blockDim = dim3(edg::kMlpWarps * 32, 1, 1);
     if ((size_t)(desc->E + desc->H + D) * sizeof(float) > 48 * 1024) return EDG_E_SHAPE;
     const int perE = (desc->E + edg::kPreCluster - 1) / edg::kPreCluster;
-    cfg.dynamicSmemBytes = edg::kMlpWarps * edg::kMlpSlots * edg::kMlpPieces * 16 + (size_t)(desc->E + desc->H + D + perE * 32 + 64) * sizeof(float);
+    cfg.dynamicSmemBytes = edg::kMlpWarps * edg::kMlpSlots * edg::kMlpPieces * 16 + (size_t)(desc->E + desc->H + 16 + D + perE * 32 + 64) * sizeof(float);
     cfg.stream = stream;
     static edg::OncePerDevice once;
     EDG_CUDA_TRY(once([] { return edg::allow_smem(200 * 1024, edg::prerouter_mlp_kernel<__half>, edg::prerouter_mlp_kernel<float>); }));
