@@ -177,7 +177,7 @@ def _stream(stream) -> Optional[int]:
 _edgcall.init({n: C.cast(getattr(_lib, n), C.c_void_p).value for n in (
     "prerouter_topk", "prerouter_topk_tokens", "softmax_topk_rows", "sigmoid_group_topk_rows", "prerouter_mlp_topk",
     "moe_expert_ffn_int4_lora", "moe_layer_decode", "moe_layer_decode_dependent", "edg_stack_decode_token", "edg_next_hidden_state")},
-    _ptr, _stream, _check)
+    _ptr, _stream, _check, LayerDesc, Lora, C.c_int32, C.c_size_t)
 
 
 _DT = {"f32": F32, "f16": F16, "bf16": BF16}

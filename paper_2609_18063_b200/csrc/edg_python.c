@@ -26,6 +26,7 @@ static struct {
     __typeof__(&edg_next_hidden_state) edg_next_hidden_state;
 } F;
 static PyObject *py_ptr, *py_stream, *py_check;               /* binding._ptr, binding._stream, binding._check */
+static PyObject *t_desc, *t_lora, *t_int, *t_size;            /* binding.LayerDesc, binding.Lora, ctypes.c_int32, ctypes.c_size_t */
 static PyObject *raw_stream, *raw_device;                     /* torch's current raw stream of a device, current device; or NULL */
 static PyObject *s_data_ptr, *s_is_contiguous, *s_cuda_stream, *s_value, *s_numel, *s_element_size;
 
@@ -87,26 +88,43 @@ static int as_stream(PyObject* o, void** p) {
     return 0;
 }
 
-static int as_int(PyObject* o, int32_t* p) {
-    PyObject* i = PyNumber_Index(o);
+/* what ctypes takes for an integer argument: anything with an index, cut to the type's bits, or an instance of the type itself */
+static int as_bits(PyObject* o, PyObject* type, uint64_t* v) {
+    PyObject* i;
+    if (!PyLong_Check(o) && PyObject_TypeCheck(o, (PyTypeObject*)type)) i = PyObject_GetAttr(o, s_value);
+    else i = PyNumber_Index(o);
     if (i == NULL) return -1;
-    *p = (int32_t)PyLong_AsUnsignedLongMask(i);
+    *v = PyLong_AsUnsignedLongLongMask(i);
     Py_DECREF(i);
-    return PyErr_Occurred() ? -1 : 0;
+    return *v == (uint64_t)-1 && PyErr_Occurred() ? -1 : 0;
+}
+
+static int as_int(PyObject* o, int32_t* p) {
+    uint64_t v = 0;
+    const int rc = as_bits(o, t_int, &v);
+    *p = (int32_t)(uint32_t)v;
+    return rc;
 }
 
 static int as_float(PyObject* o, float* p) {
-    *p = (float)PyFloat_AsDouble(o);
+    PyObject* f = PyNumber_Float(o);
+    if (f == NULL) return -1;
+    *p = (float)PyFloat_AsDouble(f);
+    Py_DECREF(f);
     return PyErr_Occurred() ? -1 : 0;
 }
 
-/* a ctypes structure by value (or, for `opt`, None) */
-static int as_struct(PyObject* o, void* dst, size_t bytes, int opt, int* present) {
+/* a ctypes structure of the given type (or, for `opt`, None), by value */
+static int as_struct(PyObject* o, PyObject* type, void* dst, size_t bytes, int opt, int* present) {
     if (present != NULL) *present = o != Py_None;
     if (opt && o == Py_None) return 0;
+    if (!PyObject_TypeCheck(o, (PyTypeObject*)type)) {
+        PyErr_Format(PyExc_TypeError, "%s expected instead of %s", ((PyTypeObject*)type)->tp_name, Py_TYPE(o)->tp_name);
+        return -1;
+    }
     Py_buffer b;
     if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) return -1;
-    const int ok = (size_t)b.len == bytes;
+    const int ok = (size_t)b.len >= bytes;                    /* (more for a subclass with fields of its own) */
     if (ok) memcpy(dst, b.buf, bytes);
     PyBuffer_Release(&b);
     if (!ok) PyErr_SetString(PyExc_TypeError, "not the expected structure");
@@ -125,11 +143,12 @@ static int as_handle(PyObject* o, void** p) {
 
 /* workspace_bytes, or None: all of the workspace */
 static int as_bytes(PyObject* o, PyObject* workspace, size_t* n) {
-    if (o != Py_None) {
-        *n = PyLong_AsSize_t(o);
-        return PyErr_Occurred() ? -1 : 0;
-    }
     uint64_t a, b;
+    if (o != Py_None) {
+        if (as_bits(o, t_size, &a) != 0) return -1;
+        *n = (size_t)a;
+        return 0;
+    }
     if (take_u64(PyObject_CallMethodNoArgs(workspace, s_numel), &a) != 0 ||
         take_u64(PyObject_CallMethodNoArgs(workspace, s_element_size), &b) != 0)
         return -1;
@@ -151,7 +170,7 @@ static PyObject* py_prerouter_topk(PyObject* self, PyObject* const* a, Py_ssize_
     edg_layer_desc d;
     void *W, *s, *inds, *gates, *logits, *mirror, *st;
     int32_t n, rc;
-    if (as_struct(a[0], &d, sizeof d, 0, NULL) || as_ptr(a[1], &W) || as_ptr(a[2], &s) || as_int(a[3], &n) || as_ptr(a[4], &inds) ||
+    if (as_struct(a[0], t_desc, &d, sizeof d, 0, NULL) || as_ptr(a[1], &W) || as_ptr(a[2], &s) || as_int(a[3], &n) || as_ptr(a[4], &inds) ||
         as_ptr(a[5], &gates) || as_ptr(a[6], &logits) || as_ptr(a[7], &mirror) || as_stream(a[8], &st))
         return NULL;
     CALL(F.prerouter_topk(&d, W, s, n, inds, gates, logits, mirror, st))
@@ -163,7 +182,7 @@ static PyObject* py_prerouter_topk_tokens(PyObject* self, PyObject* const* a, Py
     edg_layer_desc d;
     void *W, *s, *inds, *gates, *logits, *st;
     int32_t T, rc;
-    if (as_struct(a[0], &d, sizeof d, 0, NULL) || as_ptr(a[1], &W) || as_ptr(a[2], &s) || as_int(a[3], &T) || as_ptr(a[4], &inds) ||
+    if (as_struct(a[0], t_desc, &d, sizeof d, 0, NULL) || as_ptr(a[1], &W) || as_ptr(a[2], &s) || as_int(a[3], &T) || as_ptr(a[4], &inds) ||
         as_ptr(a[5], &gates) || as_ptr(a[6], &logits) || as_stream(a[7], &st))
         return NULL;
     CALL(F.prerouter_topk_tokens(&d, W, s, T, inds, gates, logits, st))
@@ -175,7 +194,7 @@ static PyObject* py_softmax_topk_rows(PyObject* self, PyObject* const* a, Py_ssi
     edg_layer_desc d;
     void *logits, *inds, *gates, *st;
     int32_t T, rc;
-    if (as_struct(a[0], &d, sizeof d, 0, NULL) || as_ptr(a[1], &logits) || as_int(a[2], &T) || as_ptr(a[3], &inds) || as_ptr(a[4], &gates) ||
+    if (as_struct(a[0], t_desc, &d, sizeof d, 0, NULL) || as_ptr(a[1], &logits) || as_int(a[2], &T) || as_ptr(a[3], &inds) || as_ptr(a[4], &gates) ||
         as_stream(a[5], &st))
         return NULL;
     CALL(F.softmax_topk_rows(&d, logits, T, inds, gates, st))
@@ -200,7 +219,7 @@ static PyObject* py_prerouter_mlp_topk(PyObject* self, PyObject* const* a, Py_ss
     edg_mlp_head h;
     void *W1, *b1, *W2, *b2, *Wr, *s, *cur, *prev, *inds, *gates, *logits, *st;
     int32_t width, n, rc;
-    if (as_struct(a[0], &d, sizeof d, 0, NULL) || as_ptr(a[1], &W1) || as_ptr(a[2], &b1) || as_ptr(a[3], &W2) || as_ptr(a[4], &b2) ||
+    if (as_struct(a[0], t_desc, &d, sizeof d, 0, NULL) || as_ptr(a[1], &W1) || as_ptr(a[2], &b1) || as_ptr(a[3], &W2) || as_ptr(a[4], &b2) ||
         as_ptr(a[5], &Wr) || as_int(a[6], &width) || as_ptr(a[7], &s) || as_ptr(a[8], &cur) || as_ptr(a[9], &prev) || as_int(a[10], &n) ||
         as_ptr(a[11], &inds) || as_ptr(a[12], &gates) || as_ptr(a[13], &logits) || as_stream(a[14], &st))
         return NULL;
@@ -218,8 +237,8 @@ static PyObject* py_moe_expert_ffn(PyObject* self, PyObject* const* a, Py_ssize_
     size_t bytes;
     int32_t T, rc;
     int has;
-    if (as_struct(a[0], &d, sizeof d, 0, NULL) || as_ptr(a[1], &pool) || as_ptr(a[2], &table) || as_int(a[3], &T) || as_ptr(a[4], &slots) ||
-        as_ptr(a[5], &experts) || as_ptr(a[6], &gates) || as_ptr(a[7], &x) || as_struct(a[8], &lo, sizeof lo, 1, &has) || as_ptr(a[9], &y) ||
+    if (as_struct(a[0], t_desc, &d, sizeof d, 0, NULL) || as_ptr(a[1], &pool) || as_ptr(a[2], &table) || as_int(a[3], &T) || as_ptr(a[4], &slots) ||
+        as_ptr(a[5], &experts) || as_ptr(a[6], &gates) || as_ptr(a[7], &x) || as_struct(a[8], t_lora, &lo, sizeof lo, 1, &has) || as_ptr(a[9], &y) ||
         as_ptr(a[10], &ws) || as_bytes(a[11], a[10], &bytes) || as_stream(a[12], &st))
         return NULL;
     CALL(F.moe_expert_ffn_int4_lora(&d, pool, table, T, slots, experts, gates, x, has ? &lo : NULL, y, ws, bytes, st))
@@ -274,16 +293,16 @@ static PyObject* py_next_hidden_state(PyObject* self, PyObject* const* a, Py_ssi
     void *x, *y, *xn, *st;
     float eps;
     int32_t rc;
-    if (as_struct(a[0], &d, sizeof d, 0, NULL) || as_ptr(a[1], &x) || as_ptr(a[2], &y) || as_ptr(a[3], &xn) || as_float(a[4], &eps) ||
+    if (as_struct(a[0], t_desc, &d, sizeof d, 0, NULL) || as_ptr(a[1], &x) || as_ptr(a[2], &y) || as_ptr(a[3], &xn) || as_float(a[4], &eps) ||
         as_stream(a[5], &st))
         return NULL;
     CALL(F.edg_next_hidden_state(&d, x, y, xn, eps, st))
     return done(rc, "edg_next_hidden_state");
 }
 
-/* init(addresses: dict name -> int, _ptr, _stream, _check) */
+/* init(addresses: dict name -> int, _ptr, _stream, _check, LayerDesc, Lora, c_int32, c_size_t) */
 static PyObject* py_init(PyObject* self, PyObject* const* a, Py_ssize_t nargs) {
-    ARGS("init", 4);
+    ARGS("init", 8);
 #define TAKE(name)                                                                                        \
     do {                                                                                                  \
         PyObject* v = PyDict_GetItemString(a[0], #name);                                                  \
@@ -297,6 +316,12 @@ static PyObject* py_init(PyObject* self, PyObject* const* a, Py_ssize_t nargs) {
     py_ptr = Py_NewRef(a[1]);
     py_stream = Py_NewRef(a[2]);
     py_check = Py_NewRef(a[3]);
+    for (int i = 4; i < 8; ++i)
+        if (!PyType_Check(a[i])) return PyErr_Format(PyExc_TypeError, "init: argument %d is no type", i);
+    t_desc = Py_NewRef(a[4]);
+    t_lora = Py_NewRef(a[5]);
+    t_int = Py_NewRef(a[6]);
+    t_size = Py_NewRef(a[7]);
     Py_RETURN_NONE;
 }
 
