@@ -23,9 +23,9 @@
 // Two launches of this form fit an SM side by side (64 registers x 512 threads, under 113 KB of shared memory).
 //
 // Measured (H 2048, I 512, E 256, K 8, groups of 64, rank 16; the four-CTA clusters per expert quarter it replaces first): a link of
-// a chain 20.4 -> 11.8 us, a step alone 24 -> 13 us (12 layers of K = 4 through the resident stack, host loop included: 295 -> 155 us).
-// Of the 11.8 us the two exchanges take 5.5 (a store, a poll under way, a poll that sees it, the slowest of 128), the
-// arithmetic of gate/up 1.7, of down 1.5.
+// a chain 20.4 -> 12.1 us, a step alone 24 -> 14.1 us (12 layers of K = 4 through the resident stack, host loop included: 295 -> 154 us).
+// Of the 12.1 us the two exchanges take 5.5 (a store, a poll under way, a poll that sees it, the slowest of 128), the
+// arithmetic of gate/up 1.7, of down 1.6.
 //
 // Waiting is safe without a cooperative launch: a CTA reads the words of others only when all CTAs of its grid have
 // started and cleared what they will publish (a counter in the control block says so).  One that finds its grid not fully resident for a while -- other grids hold the
@@ -896,15 +896,19 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         }
         if (then >= 0) { unit = then; then = -1; continue; }
         if (!s_misc[1]) break;                                           // (uniform: written before the first barrier)
-        if (tid == 0) {
-            int next = -1;
+        if (warp == 0) {                                                 // the words at once: a trip each would hold the end of the step up
             __threadfence();
-            for (int w = 0; w < kStepDeferWords && next < 0; ++w)
-                for (uint32_t left; next < 0 && (left = ld_relaxed_gpu_u32(p.defer + w)) != 0;) {
-                    const uint32_t bit = left & (0u - left);
-                    if (atomicAnd(p.defer + w, ~bit) & bit) next = w * 32 + __ffs(bit) - 1;
-                }
-            s_misc[2] = next;
+            int next = -1;
+            for (;;) {
+                const uint32_t left = lane < kStepDeferWords ? ld_relaxed_gpu_u32(p.defer + lane) : 0u;
+                const unsigned any = __ballot_sync(0xFFFFFFFFu, left != 0);
+                if (any == 0) break;
+                const uint32_t bit = left & (0u - left);
+                if (lane == __ffs(any) - 1 && (atomicAnd(p.defer + lane, ~bit) & bit)) next = lane * 32 + __ffs(bit) - 1;
+                next = __shfl_sync(0xFFFFFFFFu, next, __ffs(any) - 1);
+                if (next >= 0) break;
+            }
+            if (lane == 0) s_misc[2] = next;
         }
         __syncthreads();
         unit = s_misc[2];

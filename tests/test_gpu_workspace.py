@@ -171,3 +171,29 @@ def test_a_layer_with_a_full_head_around_a_prompt(layers):
         L.check(y, L.X[t], L.inds[t].cpu().numpy(), L.gates[t].cpu().numpy())
         L.prompt(ws, T)
     L.store.set_mlp_head(0)
+
+
+@pytest.mark.parametrize("cfg", [SMALL, WIDE, MANY], ids=lambda c: c.name)
+def test_captured_steps_replayed_without_chaining(layers, cfg):
+    """Steps with a head of their own in a CUDA graph, chaining off: a replay starts on what the replay before it left in the workspace."""
+    L, K = layers(cfg), cfg.K
+    ws = layer_io.new_workspace(L.d)
+    y = torch.zeros((3, cfg.H), device="cuda")
+    inds, gates, logits = torch.zeros((3, K), dtype=torch.int32, device="cuda"), torch.zeros((3, K), device="cuda"), torch.zeros((3, cfg.E), device="cuda")
+
+    def steps():
+        for t in range(3):
+            edg.moe_layer_decode(L.store, 0, L.xd[t], L.inds[t], L.gates[t], L.W, inds[t], gates[t], logits[t], y[t], ws)
+    steps()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        steps()
+    for _ in range(3):
+        for a in (y, inds, gates, logits):
+            a.zero_()
+        g.replay()
+        assert edg.workspace_status(ws) == 0
+        for t in range(3):
+            L.check(y[t], L.X[t], L.inds[t].cpu().numpy(), L.gates[t].cpu().numpy())
+            _check_routing(logits[t].cpu().numpy(), inds[t].cpu().numpy(), gates[t].cpu().numpy(), L.W_np.astype(np.float32), L.X[t], K)
