@@ -376,8 +376,9 @@ int32_t edg_store_mark_computed(edg_store* store, int32_t layer, void* stream);
  *               block (sticky status word, see edg_workspace_status, and arrival counters) that
  *               the caller zeroes once before first use; the rest needs no initialisation, and
  *               between calls it may be used for anything else (between the calls of a chain, see
- *               moe_layer_decode, for calls with T > 1 only).  Calls that share a workspace must be
- *               ordered on the device; they may differ in T, in shape and in the store they use.
+ *               moe_layer_decode, only for calls with T > 1 of the same shape).  Calls that share a
+ *               workspace must be ordered on the device; they may differ in T, in shape and in the
+ *               store they use.
  * An index outside its range makes the kernels skip that expert and raise the status word; no
  * out-of-range address is ever formed.
  * T = 1 is batch-1 decode (fused dequant GEMV kernels).  T > 1 is batched decode / prefill. */

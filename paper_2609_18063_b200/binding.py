@@ -271,7 +271,7 @@ def workspace_status(workspace, stream=None) -> int:
 
 
 def set_trace_buffer(dev_buffer) -> None:
-    """Phase timestamps of the batch-1 layer kernel into `dev_buffer` (uint64 [CTAs][16]); None = off."""
+    """Phase timestamps of the batch-1 layer kernel into `dev_buffer` (uint64 [CTAs][32]); None = off."""
     _check(_lib.edg_set_trace_buffer(_ptr(dev_buffer)), "edg_set_trace_buffer")
 
 

@@ -36,8 +36,9 @@ struct GroupedParams {
 
 // tcgen05 path for large groups (prefill): tiles of 128 tokens
 constexpr int kUmmaTokens = 128;
-// Where the 128-token tiles overtake the streaming form (us, streaming against tcgen05): 256 experts, 87 pairs per slot 920 : 947,
-// 128 1297 : 1166; 64 experts, 62 361 : 384, 125 667 : 675, 256 1286 : 1203; H 1024, I 256, 250 85 : 131, 1024 243 : 218.
+// Where the 128-token tiles overtake the streaming form, by the layer of 256 experts (us, streaming against tcgen05): 87 pairs per slot
+// 920 : 947, 128 1297 : 1166.  Smaller layers would cross later, and lose what lies between: 64 experts, 62 361 : 384, 125 667 : 675,
+// 256 1286 : 1203; H 1024, I 256, 250 85 : 131, 1024 243 : 218.  (A line by the layer's size and the units per SM is not worked out.)
 constexpr int kUmmaPairsPerSlot = 96;
 bool umma_grouped_supported(const edg_layer_desc& d);
 cudaError_t launch_umma_gate_up(const GroupedParams& p, int max_tiles, cudaStream_t st);

@@ -17,10 +17,10 @@
 // themselves and the weights of the first down units are on their way while the last gate/up units are computed:
 //   gate/up unit: 8 row tiles (16 rows each) of gate and of up, one per warp, over all of K = H;
 //   down unit:    16 row tiles of the output, two per warp, over all of K = I.
-// A stage is 128 k for every warp: its codes are ONE tensor copy of 32 KB (the record's tile-major sections seen as
-// an array of runs, row tiles, matrices or column slices, and slots), the (scale, zero) pairs one more, the tokens'
-// words one bulk copy: three issues per 38 KB, because arming a barrier or issuing a copy holds its lane for 50 to
-// 100 ns whatever its size.
+// A stage is 128 k for every warp of a group: its codes are ONE tensor copy of 16 KB (the record's tile-major sections seen
+// as an array of runs, row tiles, matrices or column slices, and slots), the (scale, zero) pairs one more (2 KB at groups
+// of 64), the tokens' words one bulk copy (2 or 4 KB per 8 tokens): three issues per 20 to 34 KB, because arming a barrier or
+// issuing a copy holds its lane for 50 to 100 ns whatever its size.
 // No CTA-wide barrier after the start: a warp owns whole rows, so nothing is exchanged between warps but h, which
 // goes through global memory in operand order; a counter per tile says when all of a tile's rows are there.  Units are handed
 // out in order, so whoever waits waits for units that are already running; every wait is bounded all the same.

@@ -584,11 +584,12 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(const __g
         for (int e = threadIdx.x - 32; e < p.E; e += blockDim.x - 32) p.logits[(size_t)head * p.E + e] = s_logits[e];
 }
 
-// Appendix A, sigmoid-group routing when the groups divide the warp and the warp the experts (the 8B tier: 128 experts in 8 groups):
+// Appendix A, sigmoid-group routing when the groups divide the warp and the experts are 32 times one of the V below (the 8B tier: 128
+// experts in 8 groups; the other multiples of 32 up to 1024 have no instantiation and take the form over shared memory):
 // lane l holds the V = E / 32 consecutive entries from l V on, so a group is a run of lanes and everything stays in registers;
 // order by (lane, entry) is order by index, so the first lane that holds a round's best key has the winner, ties included.
-// The form over shared memory below spends its time on instructions too, three times as many: 4096 rows 10.3 us, here 7.8
-// (one launch after the other; 6 of them are the host's).
+// The form over shared memory below spends its time on instructions too, three times as many: a call on 4096 rows of 128, one after
+// the other, 11.1 us, here 8.2 (6 of them are the host's).
 // Same values in the same order as that form.
 template <int V>
 __global__ void __launch_bounds__(256) sigmoid_group_topk_lanes_kernel(const float* logits, const float* bias, int T, int K, int n, int keep,

@@ -167,3 +167,38 @@ def test_the_logits_a_link_hands_on(E, then):
         _assert_close(y[t].cpu().numpy(), orc.moe_ffn(bits[t], ih[t], gh[t].astype(np.float64), lambda e: synth.expert_tensors(cfg, 0, e % n),
                                                       lambda e: synth.lora_tensors(cfg, 0, 0), cfg.lora_scale, cfg.group))
     store.close()
+
+
+def test_traced_steps_run_in_the_throughput_form():
+    """With a trace buffer set, lone steps (head CTAs of their own behind those of the experts) and dependent chains (norm and state handed on
+    by the reducers) of shapes that otherwise take the latency form: right results, and a stamp of every expert CTA's end."""
+    cfg, steps = _cfg(2048, 512, 64, 64, 8, 16, 1), 4
+    cfg = dataclasses.replace(cfg, pre_dtype="f16")
+    c = _Chain(cfg, steps, False, 91)
+    n_ctas = 16 * (cfg.K + 1) + cfg.E // 16 + 3
+    trace = torch.zeros((n_ctas, 32), dtype=torch.int64, device="cuda")
+    alone = torch.zeros_like(c.y)
+    edg.set_trace_buffer(trace)
+    try:
+        for t in range(steps):
+            c.run(t)
+        torch.cuda.synchronize()
+        ends = int((trace[:, 9] > 0).sum())
+        xs, inds, gates, logits, y = [a.cpu().numpy() if a.dtype != torch.bfloat16 else a.view(torch.int16).cpu().numpy().view(np.uint16)
+                                      for a in c.result()]
+        c.store.set_chaining(0)
+        for t in range(steps):
+            edg.moe_layer_decode(c.store, 0, c.xs[t], c.inds[t], c.gates[t], c.W, torch.zeros_like(c.inds[0]), torch.zeros_like(c.gates[0]), None,
+                                 alone[t], c.ws)
+        torch.cuda.synchronize()
+    finally:
+        edg.set_trace_buffer(None)
+    assert ends >= 16 * cfg.K and edg.workspace_status(c.ws) == 0
+    experts = {}
+    for t in range(steps):
+        ref = orc.moe_ffn(xs[t], inds[t], gates[t].astype(np.float64), lambda e: experts.setdefault(e, synth.expert_tensors(cfg, 0, e)),
+                          lambda e: synth.lora_tensors(cfg, 0, 0), cfg.lora_scale, cfg.group)
+        _assert_close(y[t], ref)
+        _assert_close(alone[t].cpu().numpy(), ref)
+        _check_routing(logits[t + 1], inds[t + 1], gates[t + 1], c.W_np.astype(np.float32), xs[t], cfg.K)
+    c.store.close()
