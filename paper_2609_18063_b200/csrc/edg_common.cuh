@@ -234,7 +234,7 @@ int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* 
 int32_t run_fused_layer(const edg_layer_desc* d, const void* slot_pool, const int32_t* slots, const int32_t* table,
                         const int32_t* experts, const float* gates, const void* x, const edg_lora* lora, void* y,
                         const void* W_pre, int32_t* inds_next, float* gates_next, float* logits_next,
-                        void* workspace, int flag_in, int flag_out, int ring, int stale, cudaStream_t st,
+                        void* workspace, int flag_in, int flag_out, int ring, cudaStream_t st,
                         const FusedExtras* extras = nullptr);
 // a4-a6 for T tokens on whatever kernels fit the shape (edg_ffn.cu)
 int32_t run_ffn(const edg_layer_desc* d, const void* slot_pool, int32_t T, const int32_t* slots,

@@ -146,7 +146,6 @@ struct FusedParams {
     int gshift;                   // log2(group)
     int qpc;                      // quarters of the intermediate dimension per cluster: 4 (one cluster per expert), 2 or 1
     int epc;                      // experts per cluster, one after the other: 1, or 2 or 4 (only with qpc = 4)
-    int stale;                    // -1, or a ring slot whose unread logits this (unchained) call clears
     int32_t* inds_mirror;         // [K] copy of inds_next in mapped pinned host memory, or null
     uint16_t* x_next;             // [H] bf16 or null: bf16(rmsnorm(x + y)), the next layer-step's hidden state in a dependent chain
     float* dep_ws;                // [kRing][kDepWords]: per ring slot, kC partial sums of squares, (words 4..7) the reducers' "my rows of x_next are written" flags
@@ -336,11 +335,6 @@ __global__ void __launch_bounds__(kFW * 32, 4) fused_layer_kernel(const __grid_c
         __threadfence();
     }
     if (tid == 0) pdl_launch_dependents();
-    // A call that does not continue a chain runs alone on its workspace: it clears what the last
-    // head left unread in the ring.
-    if (p.stale >= 0 && blockIdx.x == 0) {
-        for (int i = tid; i < p.E + kPairWords; i += kFW * 32) st_relaxed_gpu_u32(&p.logits_ws[(size_t)p.stale * (p.E + kPairWords) + i], kNotYet);
-    }
 
     // ---- a1 for the next step, first of all: the loads of the head rows depend on nothing but x,
     //      and the routing they lead to is what the next layer-step waits for.  The rows are dealt
@@ -1322,7 +1316,7 @@ static cudaError_t launch_fused(const FusedParams& p, size_t smem, bool pdl, cud
 int32_t run_fused_layer(const edg_layer_desc* d, const void* slot_pool, const int32_t* slots, const int32_t* table,
                         const int32_t* experts, const float* gates, const void* x, const edg_lora* lora, void* y,
                         const void* W_pre, int32_t* inds_next, float* gates_next, float* logits_next,
-                        void* workspace, int flag_in, int flag_out, int ring, int stale, cudaStream_t st,
+                        void* workspace, int flag_in, int flag_out, int ring, cudaStream_t st,
                         const FusedExtras* extras) {
     const bool has_lora = lora != nullptr && d->rank > 0;
     FusedParams p{};
@@ -1356,7 +1350,6 @@ int32_t run_fused_layer(const edg_layer_desc* d, const void* slot_pool, const in
     p.trace = g_trace;
     p.done = reinterpret_cast<int32_t*>(ws + W.ctrl + kCtrlDone);
     p.ring = ring;
-    p.stale = stale;
     p.dep_wait = -1;
     if (extras != nullptr) {
         p.inds_mirror = extras->inds_mirror;

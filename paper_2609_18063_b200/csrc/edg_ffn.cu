@@ -322,7 +322,7 @@ int32_t run_ffn(const edg_layer_desc* d, const void* slot_pool, int32_t T, const
     // batch-1 decode on the shapes the fused kernel covers: one launch for the whole FFN
     if (T == 1 && fused_supported(*d))
         return run_fused_layer(d, slot_pool, slots, table, experts, gates, x, has_lora ? lora : nullptr, y,
-                               nullptr, nullptr, nullptr, nullptr, workspace, -1, -1, 0, -1, st);
+                               nullptr, nullptr, nullptr, nullptr, workspace, -1, -1, 0, st);
 
     // several tokens: group the (token, choice) pairs per expert and run the tensor-core path
     if (T > 1) return run_grouped(d, slot_pool, T, slots, table, experts, gates, x, has_lora ? lora : nullptr, y, workspace, st);

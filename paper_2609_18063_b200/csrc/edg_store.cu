@@ -147,9 +147,8 @@ struct edg_store {
     const void* chain_ws = nullptr;
     void* chain_stream = nullptr;
     int chain_flag = 0;
-    const void* ring_ws = nullptr;         // workspace whose hand-off ring this store has initialised
+    const void* ring_ws = nullptr;         // workspace whose ring counters this store has initialised
     int ring_next = 0;                     // ring slot of the next batch-1 layer-step
-    int pub_slot = -1;                     // ring slot holding logits no step has read yet, or -1
     int chaining = 0;                      // 0 off (default), 1 when the previous step is still in flight (or under capture), 2 always
     cudaEvent_t step_done = nullptr;       // recorded behind every batch-1 layer-step launched outside a capture
     bool step_done_valid = false;
@@ -628,19 +627,10 @@ static int32_t layer_decode(edg_store* s, int32_t layer, const void* x,
         const bool shared = !s->shared_rec.empty() && s->shared_rec[layer] != nullptr;
         const bool latency_ok = edg::step_supported(s->d, shared) && edg::trace_buffer() == nullptr;     // (only the other form is traced)
         bool chain = chained;
-        // The hand-off ring starts out cleared: counters zero, logits "not yet written".  A step in the latency form that
-        // starts a chain does that itself; where the throughput form starts one, it is done for the first chain in a
-        // workspace.  After that the ring looks after itself: a chained step resets the slot it has read, and a step that
-        // starts over clears the slot the last head left unread.  Without chaining nobody reads the ring, and nothing is
-        // written to it.
         if (s->chaining && !latency_ok && s->ring_ws != workspace) {
-            uint8_t* w8 = static_cast<uint8_t*>(workspace);
-            const edg::WorkspaceLayout W = edg::workspace_layout(s->d, 1);
-            EDG_CUDA_TRY(cudaMemsetAsync(w8 + edg::kCtrlCounters, 0, edg::kCtrlBytes - edg::kCtrlCounters, st));
-            EDG_CUDA_TRY(cudaMemsetAsync(w8 + W.logits, 0xFF, (size_t)edg::kHandoffRing * (s->d.E + edg::kPairWords) * sizeof(float), st));
+            EDG_CUDA_TRY(cudaMemsetAsync(static_cast<uint8_t*>(workspace) + edg::kCtrlCounters, 0, edg::kCtrlBytes - edg::kCtrlCounters, st));
             s->ring_ws = workspace;
             s->ring_next = 0;
-            s->pub_slot = -1;
             chain = false;
         }
         // a chained step whose x is the state the previous step is still producing waits for it on the device
@@ -652,13 +642,15 @@ static int32_t layer_decode(edg_store* s, int32_t layer, const void* x,
         if (latency_ok && chain && !dep_chain && x_next != nullptr) chain = false;
         const bool latency = latency_ok && (!chain || dep_chain);
         const int flag_in = chain ? s->chain_flag : -1;              // ring slot this step's logits arrive in
-        int stale = -1;
-        if (!chain && s->pub_slot >= 0) stale = s->pub_slot;         // nobody will read that head's logits
-        s->pub_slot = -1;
         const int ring = s->ring_next;                               // ring slot of this step's scratch and of the head it evaluates
         const int flag_out = W_pre_next != nullptr && s->chaining && !s->hot ? ring : -1;
         const int pos = latency && dep_chain ? s->chain_pos + 1 : 0;
         s->ring_next = (ring + 1) % edg::kHandoffRing;
+        // The hand-off ring is cleared (logits "not yet written") where a chain starts, since anything may have used the workspace
+        // before: by a step in the latency form itself, ahead of one in the throughput form.  Its links reset the slot they have read.
+        if (!chain && !latency && flag_out >= 0)
+            EDG_CUDA_TRY(cudaMemsetAsync(static_cast<uint8_t*>(workspace) + edg::workspace_layout(s->d, 1).logits, 0xFF,
+                                         (size_t)edg::kHandoffRing * (s->d.E + edg::kPairWords) * sizeof(float), st));
         edg::FusedExtras extras;
         extras.inds_mirror = W_pre_next != nullptr ? inds_next_host_mirror_opt : nullptr;
         extras.x_next = x_next;
@@ -674,8 +666,7 @@ static int32_t layer_decode(edg_store* s, int32_t layer, const void* x,
                                W_pre_next, inds_next, gates_next, logits_next_opt, workspace, flag_in, flag_out, pos, st, extras);
         else rc = edg::run_fused_layer(&s->d, pool, slot_arg, table, expert_arg, gates_cur, x,
                                   (lora && s->d.rank > 0) ? lora : nullptr, y, W_pre_next, inds_next, gates_next,
-                                  logits_next_opt, workspace, flag_in, flag_out, ring, stale, st, &extras);
-        s->pub_slot = flag_out;
+                                  logits_next_opt, workspace, flag_in, flag_out, ring, st, &extras);
         if (rc != EDG_OK) return rc;
         s->step_done_valid = false;
         if (capturing == cudaStreamCaptureStatusNone && s->chaining == 1) {

@@ -66,7 +66,7 @@ class _Layer:
             want = orc.bf16_to_f64(orc.next_hidden_state(self.X[t], y.cpu().numpy().astype(np.float64), 1e-6))
             assert np.abs(xn.float().cpu().numpy() - want).max() <= 2.0 ** -7 * np.abs(want).max()      # a bf16 step at the largest value
 
-    def chain(self, ws, n=5):
+    def chain(self, ws, n=5, leave_on=False):
         """n dependent steps, chained; each checked on the state the GPU handed on"""
         K = self.cfg.K
         xs = torch.zeros((n + 1, self.cfg.H), dtype=torch.bfloat16, device="cuda")
@@ -78,7 +78,8 @@ class _Layer:
         for t in range(n):
             edg.moe_layer_decode_dependent(self.store, 0, xs[t], inds[t], gates[t], self.W, inds[t + 1], gates[t + 1], logits[t + 1], y[t], xs[t + 1], ws)
         assert edg.workspace_status(ws) == 0
-        self.store.set_chaining(0)
+        if not leave_on:
+            self.store.set_chaining(0)
         bits = xs.view(torch.int16).cpu().numpy().view(np.uint16)
         for t in range(n):
             self.check(y[t], bits[t], inds[t].cpu().numpy(), gates[t].cpu().numpy())
@@ -143,6 +144,22 @@ def test_a_workspace_that_changes_hands_at_the_same_address(layers, cfg):
         L.step(ws)
         L.step(ws, dependent=True)
         L.chain(ws)
+
+
+@pytest.mark.parametrize("cfg", [SMALL, WIDE, MANY], ids=lambda c: c.name)
+def test_chains_with_anything_else_in_the_workspace_between_them(layers, cfg):
+    """Chaining stays on: what a chain before it left in the hand-off ring, or another use of the workspace, is nothing to the next one."""
+    L = layers(cfg)
+    ws = layer_io.new_workspace(L.d)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(4)
+    L.chain(ws, leave_on=True)
+    for _ in range(2):
+        ws[4096:].view(torch.int32).random_(-2 ** 31, 2 ** 31 - 1, generator=gen)
+        L.chain(ws, leave_on=True)
+    for head in (True, False, True):            # steps whose routing nobody takes from the ring
+        L.step(ws, head)
+    L.chain(ws)
 
 
 def test_two_stores_of_different_shapes_in_one_workspace(layers):
