@@ -120,7 +120,7 @@ static_assert(kCtrlStarts % 128 == 0 && kCtrlDefer + kStepBufs * kStepDeferWords
 struct WorkspaceLayout {
     size_t ctrl;      // kCtrlBytes control block
     size_t u_gu;      // [T][n_sets][2][rank] float : A_gate x and A_up x
-    size_t h;         // [T][K][I] float            : silu(gate) * up
+    size_t h;         // [K][I] float               : silu(gate) * up (T = 1)
     size_t u_d;       // [T][K][rank] float         : A_down h
     size_t logits;    // [ring][E + 64] float     : next-step head logits, then the (expert, gate) pairs chosen from them, handed to the chained next step; one set per ring slot
     size_t partial;   // [ring][4(K+1)][H] float  : gate-weighted partial expert outputs of the fused batch-1 kernel, one set per ring slot
@@ -129,13 +129,11 @@ struct WorkspaceLayout {
     // grouped path (T > 1) only:
     size_t o;         // [T*K][H] float             : gate-weighted output of every (token, choice) pair
     size_t pair_slot; // [T*K] int32                : resolved slot of every pair (-1: skipped)
-    size_t pair_ad;   // [T*K] int32                : adapter of every pair
-    size_t counts;    // [n_slots] int32            : pairs per slot
     size_t n_tiles;   // int32
-    size_t tiles;     // [T*K/128 + n_slots][2] int32 : (slot, first position) of every tile of 128 pairs
-    size_t lists;     // [n_slots][T] int32         : pairs of every slot, ascending
-    size_t hq;        // [T*K/128 + n_slots][I/32][2][128 x 32] fp16: h of every 128-token tile as tensor-core operand tiles (value, residual)
-    size_t xq;        // [T*K/128 + n_slots][H/32][128 x 32] fp16: the gathered token states of every tile as operand tiles
+    size_t tiles;     // {slot, first position, pairs, adapter} of every tile of 128 pairs
+    size_t order;     // [T*K] int32                : pairs sorted by slot
+    size_t hq;        // [tiles][I/32][2][4][pairs, up to 128][8] fp16: h of every tile as tensor-core operand tiles (value, residual)
+    size_t xq;        // [tiles][H/64][8][pairs, up to 128][8] fp16: the gathered token states of every tile as operand tiles
     // streaming form of the grouped path (run_grouped_ffn):
     size_t g_tiles;   // [tiles] {slot, first position, pairs, adapter}
     size_t g_done;    // [tiles] int32              : finished row tiles of every tile's h
@@ -159,6 +157,10 @@ inline size_t grouped_max_tiles(const edg_layer_desc& d, int T) {
     const size_t P = (size_t)T * d.K, cap = (size_t)grouped_tile_cap(d, T);
     return P / cap + 1 + (P < (size_t)d.n_slots ? P : (size_t)d.n_slots);
 }
+inline size_t umma_max_tiles(const edg_layer_desc& d, int T) {
+    const size_t P = (size_t)T * d.K;
+    return P / 128 + (P < (size_t)d.n_slots ? P : (size_t)d.n_slots);
+}
 // Whether T tokens go through the tcgen05 tiles (umma_*) or through the streaming form.
 bool grouped_use_umma(const edg_layer_desc& d, int T);
 
@@ -177,9 +179,9 @@ inline WorkspaceLayout workspace_layout(const edg_layer_desc& d, int T) {
     W.step_x = round_up(W.partial + (size_t)kHandoffRing * one_set, 256);
     W.u_gu = round_up(W.step_x + step_region_words(d) * sizeof(float), 256);
     W.h = round_up(W.u_gu + (size_t)T * n_sets * 2 * r * sizeof(float), 256);
-    W.u_d = round_up(W.h + (size_t)T * d.K * d.I * sizeof(float), 256);
+    W.u_d = round_up(W.h + (T > 1 ? 0 : (size_t)d.K * d.I * sizeof(float)), 256);
     size_t end = round_up(W.u_d + (size_t)T * d.K * r * sizeof(float), 256);
-    W.o = W.pair_slot = W.pair_ad = W.counts = W.n_tiles = W.tiles = W.lists = W.hq = W.xq = end;
+    W.o = W.pair_slot = W.n_tiles = W.tiles = W.order = W.hq = W.xq = end;
     W.g_tiles = W.g_done = W.g_order = W.g_cnt = W.g_u = W.g_xq = W.g_hq = end;
     if (T > 1) {
         const size_t P = (size_t)T * d.K;
@@ -187,12 +189,11 @@ inline WorkspaceLayout workspace_layout(const edg_layer_desc& d, int T) {
         W.pair_slot = end;         end = round_up(W.pair_slot + P * 4, 256);
         W.n_tiles = end;           end += 256;
         if (grouped_use_umma(d, T)) {
-            W.pair_ad = end;       end = round_up(W.pair_ad + P * 4, 256);
-            W.counts = end;        end = round_up(W.counts + (size_t)d.n_slots * 4, 256);
-            W.tiles = end;         end = round_up(W.tiles + (P / 128 + 1 + d.n_slots) * 8, 256);
-            W.lists = end;         end = round_up(W.lists + (size_t)d.n_slots * T * 4, 256);
-            W.hq = end;            end = round_up(W.hq + ((P + 127) / 128 + d.n_slots) * (size_t)(d.I / 32) * 2 * 8192, 256);
-            W.xq = end;            end = round_up(W.xq + ((P + 127) / 128 + d.n_slots) * (size_t)(d.H / 32) * 8192, 256);
+            const size_t tiles = umma_max_tiles(d, T);
+            W.tiles = end;         end = round_up(W.tiles + tiles * 16, 256);
+            W.order = end;         end = round_up(W.order + P * 4, 256);
+            W.hq = end;            end = round_up(W.hq + tiles * d.I * 512, 256);
+            W.xq = end;            end = round_up(W.xq + tiles * d.H * 256, 256);
         } else {
             const size_t tiles = grouped_max_tiles(d, T), cap = (size_t)grouped_tile_cap(d, T), r16 = (r + 15) / 16 * 16;
             W.g_tiles = end;       end = round_up(W.g_tiles + tiles * 16, 256);

@@ -359,23 +359,6 @@ int32_t run_ffn(const edg_layer_desc* d, const void* slot_pool, int32_t T, const
     return EDG_OK;
 }
 
-// rank-r projections for the grouped path: phase 0 = A_gate/A_up . x, phase 1 = A_down . h
-void launch_lora_a(const edg_layer_desc* d, const void* slots, const void* table, const void* experts, const void* x,
-                   const edg_lora* lora, float* u_gu, float* h, float* u_d, int32_t* status, int T, int phase, cudaStream_t st) {
-    FfnParams p{};
-    p.slots = static_cast<const int32_t*>(slots); p.table = static_cast<const int32_t*>(table);
-    p.experts = static_cast<const int32_t*>(experts);
-    p.x = static_cast<const uint16_t*>(x);
-    p.lora = *lora;
-    p.status = status; p.u_gu = u_gu; p.h = h; p.u_d = u_d;
-    p.H = d->H; p.I = d->I; p.E = d->E; p.K = d->K; p.group = d->group; p.rank = d->rank;
-    p.n_adapters = d->n_adapters; p.n_slots = d->n_slots;
-    const int n_sets = d->n_adapters == 1 ? 1 : d->K;
-    const int g8 = (p.rank + 7) / 8;
-    const int warps = phase == 0 ? n_sets * 2 * g8 : p.K * g8;
-    lora_a_kernel<<<dim3((warps + 7) / 8, T), 256, 0, st>>>(p, phase, n_sets);
-}
-
 }  // namespace edg
 
 extern "C" int32_t edg_ffn_workspace_bytes(const edg_layer_desc* desc, int32_t T, size_t* bytes) {

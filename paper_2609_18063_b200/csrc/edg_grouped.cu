@@ -7,81 +7,95 @@
 // gate-weighted output goes to a [T*K][H] scratch and is reduced per token in the order of its K choices, so y does not
 // depend on how the groups were scheduled.
 #include "edg_grouped.cuh"
+#include "edg_ptx.cuh"
 
 namespace edg {
 
-__global__ void resolve_pairs_kernel(GroupedParams p) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= p.T * p.K) return;
-    int s = p.slots[i];
-    const int e = p.table != nullptr ? s : (p.experts != nullptr ? p.experts[i] : 0);
-    if (p.table != nullptr) s = (s >= 0 && s < p.E) ? p.table[s] : -1;
-    int ad = 0;
-    if (p.rank > 0 && p.n_adapters != 1) ad = (e >= 0 && e < p.E) ? e : -1;
-    if (s < 0 || s >= p.n_slots || ad < 0) { s = -1; atomicExch(p.status, EDG_E_RANGE); }
-    p.pair_slot[i] = s;
-    p.pair_ad[i] = ad;
+// The slot of every (token, choice) pair.
+__global__ void __launch_bounds__(256) umma_prepare_kernel(GroupedParams p) {
+    pdl_launch_dependents();
+    pdl_wait_prior_grid();
+    const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+    if (i == 0) *p.n_tiles = 0;
+    if (i < (size_t)p.T * p.K) {
+        int s = p.slots[i];
+        const int e = p.table != nullptr ? s : (p.experts != nullptr ? p.experts[i] : 0);
+        if (p.table != nullptr) s = (s >= 0 && s < p.E) ? p.table[s] : -1;
+        if (s < 0 || s >= p.n_slots || (p.rank > 0 && p.n_adapters != 1 && (e < 0 || e >= p.E))) { s = -1; atomicExch(p.status, EDG_E_RANGE); }
+        p.pair_slot[i] = s;
+    }
 }
 
-// One CTA per slot: the slot's pairs in ascending pair index (deterministic, no atomics).  Each
-// warp owns a contiguous range of pairs; a first pass counts, a second pass writes at the offsets.
-constexpr int kListWarps = 16;
+// One CTA per slot: the slot's pairs in ascending pair index (deterministic, no atomics), behind those of the slots before it, and the
+// slot's tiles.  Each warp owns a contiguous range of pairs; a first pass counts, a second pass writes at the offsets.  (Which number
+// a tile gets is decided by a counter: nothing that is computed depends on it.)
+constexpr int kListWarps = 32;
 __global__ void __launch_bounds__(kListWarps * 32) build_lists_kernel(GroupedParams p) {
     const int s = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __shared__ int s_cnt[kListWarps];
+    __shared__ int s_cnt[kListWarps], s_less[kListWarps], s_first, s_tile0;
+    pdl_launch_dependents();
+    pdl_wait_prior_grid();
     const int P = p.T * p.K;
-    const int per = ((P + kListWarps - 1) / kListWarps + 31) / 32 * 32;      // pairs per warp, a multiple of 32
-    const int lo = warp * per, hi = min(P, lo + per);
-    int cnt = 0;
-    for (int base = lo; base < hi; base += 32) {
-        const int i = base + lane;
-        cnt += __popc(__ballot_sync(0xFFFFFFFFu, i < hi && p.pair_slot[i] == s));
+    const int per = ((P + kListWarps - 1) / kListWarps + 127) / 128 * 128;   // pairs per warp, a multiple of 128: four per lane at a time
+    const int lo = min(P, warp * per), hi = min(P, lo + per);
+    auto four = [&](int base) {                                          // (pair_slot is 256-byte aligned, base a multiple of 128)
+        const int i = base + 4 * lane;
+        if (i + 3 < hi) return __ldcg(reinterpret_cast<const int4*>(p.pair_slot + i));
+        return make_int4(i < hi ? p.pair_slot[i] : -1, i + 1 < hi ? p.pair_slot[i + 1] : -1, i + 2 < hi ? p.pair_slot[i + 2] : -1, -1);
+    };
+    int cnt = 0, less = 0;
+#pragma unroll 4
+    for (int base = lo; base < hi; base += 128) {
+        const int4 v = four(base);
+        cnt += (v.x == s) + (v.y == s) + (v.z == s) + (v.w == s);
+        less += ((unsigned)v.x < (unsigned)s) + ((unsigned)v.y < (unsigned)s) + ((unsigned)v.z < (unsigned)s) + ((unsigned)v.w < (unsigned)s);
     }
-    if (lane == 0) s_cnt[warp] = cnt;
+    cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
+    less = __reduce_add_sync(0xFFFFFFFFu, less);
+    if (lane == 0) { s_cnt[warp] = cnt; s_less[warp] = less; }
     __syncthreads();
-    int off = 0, total = 0;
-    for (int w = 0; w < kListWarps; ++w) { if (w < warp) off += s_cnt[w]; total += s_cnt[w]; }
-    for (int base = lo; base < hi; base += 32) {
-        const int i = base + lane;
-        const bool m = i < hi && p.pair_slot[i] == s;
-        const unsigned bal = __ballot_sync(0xFFFFFFFFu, m);
-        if (m) p.lists[(size_t)s * p.T + off + __popc(bal & ((1u << lane) - 1))] = i;
-        off += __popc(bal);
+    int off = 0, total = s_cnt[lane], start = s_less[lane];
+    off = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? total : 0);
+    total = __reduce_add_sync(0xFFFFFFFFu, total);
+    start = __reduce_add_sync(0xFFFFFFFFu, start);
+    if (total == 0) return;
+    const int n_tiles = (total + kUmmaTokens - 1) / kUmmaTokens;
+    if (threadIdx.x == 0) s_tile0 = atomicAdd(p.n_tiles, n_tiles);
+    if (cnt > 0) {
+        off += start;
+#pragma unroll 4
+        for (int base = lo; base < hi; base += 128) {
+            const int4 v = four(base);
+            const int mine = (v.x == s) + (v.y == s) + (v.z == s) + (v.w == s);
+            if (!__any_sync(0xFFFFFFFFu, mine)) continue;
+            int at = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(0xFFFFFFFFu, at, o);
+                if (lane >= o) at += x;
+            }
+            const int all = __shfl_sync(0xFFFFFFFFu, at, 31);
+            at += off - mine;
+            const int i = base + 4 * lane;
+            if (mine > 0 && at == start) s_first = v.x == s ? i : (v.y == s ? i + 1 : (v.z == s ? i + 2 : i + 3));
+            if (v.x == s) p.order[at++] = i;
+            if (v.y == s) p.order[at++] = i + 1;
+            if (v.z == s) p.order[at++] = i + 2;
+            if (v.w == s) p.order[at++] = i + 3;
+            off += all;
+        }
     }
-    if (threadIdx.x == 0) p.counts[s] = total;
-}
-
-// Tile table: slot s contributes ceil(count / ntok) tiles; an exclusive scan over the slots gives
-// each its first tile.  One CTA, slots strided over the threads, scan through shared memory.
-__global__ void __launch_bounds__(1024) build_tiles_kernel(GroupedParams p) {
-    __shared__ int s_n[1024];
-    const int tid = threadIdx.x;
-    // n_slots can exceed the block: each thread owns a contiguous run of slots
-    const int per = (p.n_slots + 1023) / 1024;
-    const int s0 = tid * per, s1 = min(p.n_slots, s0 + per);
-    int mine = 0;
-    for (int s = s0; s < s1; ++s) mine += (p.counts[s] + p.ntok - 1) / p.ntok;
-    s_n[tid] = mine;
     __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {          // inclusive scan
-        const int v = tid >= o ? s_n[tid - o] : 0;
-        __syncthreads();
-        s_n[tid] += v;
-        __syncthreads();
-    }
-    int n = s_n[tid] - mine;                       // exclusive prefix
-    for (int s = s0; s < s1; ++s)
-        for (int first = 0; first < p.counts[s]; first += p.ntok) { p.tiles[2 * n] = s; p.tiles[2 * n + 1] = first; ++n; }
-    if (tid == 1023) *p.n_tiles = s_n[1023];
+    int ad = 0;
+    if (p.rank > 0 && p.n_adapters != 1) ad = p.table != nullptr ? p.slots[s_first] : p.experts[s_first];
+    for (int t = threadIdx.x; t < n_tiles; t += kListWarps * 32)
+        p.tiles[s_tile0 + t] = make_int4(s, start + t * kUmmaTokens, min(kUmmaTokens, total - t * kUmmaTokens), ad);
 }
 
 // ---------------------------------------------------------------- host
 
-void launch_lora_a(const edg_layer_desc* d, const void* slots, const void* table, const void* experts, const void* x,
-                   const edg_lora* lora, float* u_gu, float* h, float* u_d, int32_t* status, int T, int phase, cudaStream_t st);
-
 bool grouped_use_umma(const edg_layer_desc& d, int T) {
-    return (int64_t)T * d.K > (int64_t)kUmmaPairsPerSlot * d.n_slots && umma_grouped_supported(d);
+    return (int64_t)T * d.K > (int64_t)(d.group >= 64 ? kUmmaPairsPerSlot : kUmmaPairsPerSlot32) * d.n_slots && umma_grouped_supported(d);
 }
 
 int32_t run_grouped(const edg_layer_desc* d, const void* slot_pool, int32_t T, const int32_t* slots, const int32_t* table,
@@ -98,36 +112,31 @@ int32_t run_grouped(const edg_layer_desc* d, const void* slot_pool, int32_t T, c
     if (has_lora) p.lora = *lora;
     p.y = y;
     p.status = reinterpret_cast<int32_t*>(ws + W.ctrl);
-    p.u_gu = reinterpret_cast<float*>(ws + W.u_gu);
-    p.h = reinterpret_cast<float*>(ws + W.h);
-    p.u_d = reinterpret_cast<float*>(ws + W.u_d);
+    p.u_gu = reinterpret_cast<__half*>(ws + W.u_gu);
+    p.u_d = reinterpret_cast<__half*>(ws + W.u_d);
     p.o = reinterpret_cast<float*>(ws + W.o);
     p.pair_slot = reinterpret_cast<int32_t*>(ws + W.pair_slot);
     p.T = T; p.H = d->H; p.I = d->I; p.E = d->E; p.K = d->K; p.group = d->group;
+    while ((1 << p.gshift) < d->group) ++p.gshift;
     p.rank = has_lora ? d->rank : 0;
     p.n_adapters = d->n_adapters; p.n_slots = d->n_slots; p.out_dtype = d->out_dtype;
     p.sigma = d->lora_scale;
     p.L = record_layout(d->H, d->I, d->group);
     if (!grouped_use_umma(*d, T)) return run_grouped_ffn(d, p, W, ws, st);
 
-    p.pair_ad = reinterpret_cast<int32_t*>(ws + W.pair_ad);
-    p.counts = reinterpret_cast<int32_t*>(ws + W.counts);
     p.n_tiles = reinterpret_cast<int32_t*>(ws + W.n_tiles);
-    p.tiles = reinterpret_cast<int32_t*>(ws + W.tiles);
-    p.lists = reinterpret_cast<int32_t*>(ws + W.lists);
+    p.tiles = reinterpret_cast<int4*>(ws + W.tiles);
+    p.order = reinterpret_cast<int32_t*>(ws + W.order);
     p.hq = ws + W.hq;
     p.xq = ws + W.xq;
-    p.ntok = kUmmaTokens;
-    const int P = T * d->K, max_tiles = (P + p.ntok - 1) / p.ntok + d->n_slots;
-    resolve_pairs_kernel<<<(P + 255) / 256, 256, 0, st>>>(p);
-    build_lists_kernel<<<d->n_slots, kListWarps * 32, 0, st>>>(p);
-    build_tiles_kernel<<<1, 1024, 0, st>>>(p);
-    if (has_lora && !launch_lora_ax_tokens(d, x, lora, p.u_gu, T, st))
-        launch_lora_a(d, slots, table, experts, x, lora, p.u_gu, p.h, p.u_d, p.status, T, 0, st);
-    EDG_CUDA_TRY(launch_umma_gate_up(p, max_tiles, st));
-    if (has_lora && !launch_lora_adh_pairs(d, lora, p.h, p.u_d, P, st))
-        launch_lora_a(d, slots, table, experts, x, lora, p.u_gu, p.h, p.u_d, p.status, T, 1, st);
-    EDG_CUDA_TRY(launch_umma_down(p, max_tiles, st));
+    const size_t P = (size_t)T * d->K;
+    const int max_tiles = (int)umma_max_tiles(*d, T);
+    EDG_CUDA_TRY(launch_pdl(umma_prepare_kernel, dim3((unsigned)((P + 255) / 256)), 256, 0, st, p));
+    EDG_CUDA_TRY(launch_pdl(build_lists_kernel, dim3(d->n_slots), kListWarps * 32, 0, st, p));
+    if (has_lora) EDG_CUDA_TRY(launch_lora_ax(p, max_tiles, st));
+    EDG_CUDA_TRY(launch_umma(p, false, max_tiles, st));
+    if (has_lora) EDG_CUDA_TRY(launch_lora_adh(p, max_tiles, st));
+    EDG_CUDA_TRY(launch_umma(p, true, max_tiles, st));
     EDG_CUDA_TRY(launch_sum_choices(p, st));
     return EDG_OK;
 }

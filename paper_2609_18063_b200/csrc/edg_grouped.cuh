@@ -16,40 +16,52 @@ struct GroupedParams {
     edg_lora lora;
     void* y;
     int32_t* status;
-    float* u_gu;              // [T][n_sets][2][rank]
-    float* h;                 // [T*K][I]
-    float* u_d;               // [T*K][rank]
+    __half* u_gu;             // [T, or T*K with an adapter per expert][2][rank]  sigma (A_gate x), sigma (A_up x)
+    __half* u_d;              // [T*K][rank]                                      sigma (A_down h)
     float* o;                 // [T*K][H]
     int32_t* pair_slot;       // [T*K]
-    int32_t* pair_ad;         // [T*K]
-    int32_t* counts;          // [n_slots]
-    int32_t* lists;           // [n_slots][T]
-    int32_t* tiles;           // [max tiles][2] = (slot, first position in the slot's list)
+    int32_t* order;           // [T*K] pairs sorted by slot
+    int4* tiles;              // {slot, first position in order, pairs, adapter} of every tile of 128 pairs
     int32_t* n_tiles;
-    uint8_t* hq;              // h of every 128-token tile as fp16 operand tiles (tcgen05 path)
-    uint8_t* xq;              // the gathered token states of every tile as fp16 operand tiles (tcgen05 path)
-    int T, H, I, E, K, group, rank, n_adapters, n_slots, out_dtype;
-    int ntok;                 // tokens per tile of the tcgen05 engine (128)
+    uint8_t* hq;              // h of every tile as fp16 operand tiles, value and residual
+    uint8_t* xq;              // the gathered token states of every tile as fp16 operand tiles
+    int T, H, I, E, K, group, gshift, rank, n_adapters, n_slots, out_dtype;
     float sigma;
     RecordLayout L;
 };
 
 // tcgen05 path for large groups (prefill): tiles of 128 tokens
 constexpr int kUmmaTokens = 128;
-// Where the 128-token tiles overtake the streaming form, by the layer of 256 experts (us, streaming against tcgen05): 87 pairs per slot
-// 920 : 947, 128 1297 : 1166.  Smaller layers would cross later, and lose what lies between: 64 experts, 62 361 : 384, 125 667 : 675,
-// 256 1286 : 1203; H 1024, I 256, 250 85 : 131, 1024 243 : 218.  (A line by the layer's size and the units per SM is not worked out.)
-constexpr int kUmmaPairsPerSlot = 96;
+// Where the 128-token tiles overtake the streaming form, in pairs per slot (us, streaming : tcgen05; H 2048, I 512, groups of 64 where
+// nothing else is said).  256 experts, top 8: 32 422 : 452, 64 706 : 561; 64 experts: 42 161 : 145, 80 238 : 197; groups of 128: 21
+// 185 : 220, 40 263 : 249; H 1024, I 256, 16 experts: 42 59.4 : 60.2, 128 92 : 66.  With groups of 32 the sums leave tensor memory twice
+// as often: 64 214 : 230, 128 322 : 296.
+constexpr int kUmmaPairsPerSlot = 40, kUmmaPairsPerSlot32 = 96;
 bool umma_grouped_supported(const edg_layer_desc& d);
-cudaError_t launch_umma_gate_up(const GroupedParams& p, int max_tiles, cudaStream_t st);
-cudaError_t launch_umma_down(const GroupedParams& p, int max_tiles, cudaStream_t st);
+cudaError_t launch_umma(const GroupedParams& p, bool down, int max_tiles, cudaStream_t st);
 
 // streaming form for small and middling groups (edg_grouped_ffn.cu)
 int32_t run_grouped_ffn(const edg_layer_desc* d, const GroupedParams& p, const WorkspaceLayout& W, uint8_t* ws, cudaStream_t st);
 cudaError_t launch_sum_choices(const GroupedParams& p, cudaStream_t st);
 
-// adapter projections for many tokens / pairs on the tensor cores (one shared adapter); false = shape not covered
-bool launch_lora_ax_tokens(const edg_layer_desc* d, const void* x, const edg_lora* lora, float* u_gu, int T, cudaStream_t st);
-bool launch_lora_adh_pairs(const edg_layer_desc* d, const edg_lora* lora, const float* h, float* u_d, int P, cudaStream_t st);
+// adapter projections of the tcgen05 path (edg_lora_tokens.cu): A_gate x and A_up x; A_down h from the tiles' h
+cudaError_t launch_lora_ax(const GroupedParams& p, int max_tiles, cudaStream_t st);
+cudaError_t launch_lora_adh(const GroupedParams& p, int max_tiles, cudaStream_t st);
+
+// a launch that may begin while the kernel before it runs (it waits for its end by itself)
+template <typename... Params, typename... Args>
+cudaError_t launch_pdl(void (*kern)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
 
 }  // namespace edg

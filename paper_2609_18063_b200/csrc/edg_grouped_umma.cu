@@ -1,103 +1,117 @@
-// a4'-a6' grouped form for large token groups (prefill) on the 5th-generation tensor cores.
+// a4'-a6' grouped form for many tokens (prompts, chunks of them) on the 5th-generation tensor cores.
 //
-// A CTA computes a tile [128 weight rows] x [up to 128 tokens of one expert]: the expert's weights are
-// the A operand (M = 128), the gathered token states the B operand (N = tokens), both K-major in shared
-// memory; tcgen05.mma accumulates in tensor memory (fp32), one elected thread issues, completion is
-// tracked by tcgen05.commit on mbarriers, and the epilogue reads the accumulators with tcgen05.ld.
+// A CTA computes [128 weight rows] x [up to 128 pairs of one expert]: the expert's weights are the A operand (M = 128), the
+// activations of the tile's (token, choice) pairs the B operand (N = pairs), both K-major in shared memory; one elected thread
+// issues tcgen05.mma into tensor memory, tcgen05.commit on mbarriers tracks completion.
 //
-// Exact weights from fp16 operands.  w = s * (q - z) has up to 16 significant bits (11 of the fp16
-// scale, 5 of the integer), one fp16 cannot hold it, and rounding it costs more than the parity bar
-// allows.  So every weight is fed as two fp16 values: hi = fp16(s (q - z)) and the residual
-// lo = s (q - z) - hi, which is exact (an fma computes it without rounding); the tile is multiplied
-// twice into the same accumulator.  The bf16 activations convert to fp16 exactly; the fp32 h of the
-// down projection is fed as an fp16 value plus an fp16 residual (hi.hi + lo.hi + hi.lo).
+// Exact weights from ONE fp16 operand.  w = s (q - z) has up to 16 significant bits, but q - z alone has at most eleven: the MMA
+// sees (q - z) * 2^-9, exactly, and its sums over one group of k (one scale per row) are multiplied by the scale in fp32 where
+// they leave tensor memory, row = lane.  The running sums live in registers (a thread holds one row of the tile, 128 columns), the
+// accumulator is double-buffered, so the tensor core works on the next group meanwhile.  What bounds these kernels is operand
+// traffic through shared memory (128 B a clock): with the weights as value + residual (two operand tiles, multiplied twice) it was
+// twice as much, with h as value + residual on top 1.5 times.  The fp32 h of the down projection is fed as value + residual.
 //
-// Operand layout in shared memory (no swizzle): core matrices of 8 rows x 16 bytes, a [128 x 32] fp16
-// tile being [k core 0..3][row group 0..15][8 rows][16 B]; the descriptor's leading byte offset is the
-// distance between k cores (2048), its stride byte offset the distance between row groups (128).
-// The 8 k values of a core row are kept in the order (k0,k4,k1,k5,k2,k6,k3,k7) in which the int4 codes
-// come out of a 32-bit word -- for A and B alike, so the dot product is unchanged.
+// Operand layout in shared memory (no swizzle): core matrices of 8 rows x 16 bytes; the descriptor's leading byte offset is the
+// distance between k cores, its stride byte offset the distance between row groups (128).  The 8 k values of a core row are
+// kept in the order (k0,k4,k1,k5,k2,k6,k3,k7) in which the int4 codes come out of a 32-bit word -- for A and B alike.
 //
-// Warps 0-7 dequantise the weights into a ring of two stages, with the codes of the next four chunks in flight in registers, and
-// later run the epilogue (each warp its 32 lanes of tensor memory, half of the token columns); warp 8 allocates the tensor memory
-// and its lane 0 issues the MMAs; lane 0 of warp 9 fetches the activations into a ring of their own.
-// Every wait is bounded: a wait that gives up raises the status word and the kernel still frees its
-// tensor memory and returns.
+// Warps 0-3 (48 registers) dequantise: a thread is a weight row, the codes of the next stages in flight in registers.  Warps 4-7 (168
+// registers) take the groups' sums out of tensor memory, 32 columns at a time, and run the epilogue.  Warp 8 issues the MMAs, warp 9 brings the
+// activations, one bulk copy a stage.  Two CTAs share an SM: one's prologue and epilogue run beside the other's main loop.  Every wait
+// is bounded: a wait that gives up raises the status word and the kernel still frees its tensor memory and returns.
+//
+// Measured (4096 tokens, top 8 of 256 by Zipf(1.1), H 2048, I 512, groups of 64, rank 16): gate/up 413 -> 368 us, down 323 -> 302, the
+// whole call with its routing 904 -> 795; with an adapter per expert 1190 -> 839; 2048 tokens (streaming form before) 706 -> 561.
+// Tensor pipe 13 and 23 % active: the limiter is the rate at which lone warps run their instructions (a stage of gate/up takes a
+// CTA 2000 cycles; without the trips to tensor memory it would be 333 us, the operand traffic alone 110).  Found on the way: MMAs issued by one of
+// the warps that take sums out, in between: 1020 us for gate/up; sums out 16 columns at a time: 577; states gathered by 16-byte copies
+// of this kernel, without a pass that gathers them: 554, the copies' bursts hold up every other access to shared memory; four row
+// blocks per CTA one after the other: down 302 -> 400.
 #include "edg_grouped.cuh"
+#include "edg_ptx.cuh"
 
 namespace edg {
 namespace {
 
-constexpr int U_TN = kUmmaTokens;            // token columns per tile
-constexpr int U_KC = 32;                     // k per stage
-constexpr int U_STAGES = 2;                  // of weights: four operand tiles each
-constexpr int U_ACT_MAX = 4;                 // slots of activations
-constexpr int U_AHEAD = 4;                   // chunks of codes in flight per thread
-constexpr uint32_t U_TILE = 128 * U_KC * 2;  // bytes of a [128 x 32] fp16 operand tile
-constexpr uint32_t U_LBO = 16 * 128;         // between k cores
-constexpr uint32_t U_SBO = 128;              // between row groups
-constexpr uint32_t U_SPIN = 1u << 22;
-constexpr int U_PROD_WARPS = 8;
-constexpr int U_THREADS = (U_PROD_WARPS + 2) * 32;
+constexpr int U_TN = kUmmaTokens;            // columns of a tile: pairs
+constexpr uint32_t U_LBO = 16 * 128;         // between k cores of a full tile
+constexpr int U_THREADS = 12 * 32;
+constexpr int U_HQ = 32;                     // columns that the epilogue of gate/up exchanges at a time
+constexpr int U_HS = 68;                     // floats of an h row in shared memory: 64 and padding against bank conflicts
 
-__device__ __forceinline__ uint32_t s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void bar_init(uint64_t* b, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s32(b)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void bar_arrive(uint64_t* b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s32(b)) : "memory");
-}
+// A stage of the ring: gate/up 64 k of weights and of states (16 KB each), three of them; down 32 k of weights (8 KB), of h and its
+// residual (16 KB), four.
+template <bool DOWN> struct Stage {
+    static constexpr int k = DOWN ? 32 : 64, chunks = k / 32, n = DOWN ? 4 : 3;
+    static constexpr uint32_t a_bytes = 128 * k * 2, bytes = a_bytes + 16384;
+    static constexpr int ahead = DOWN ? 4 : 2;           // stages of codes in flight per thread of warps 0-3
+};
+constexpr uint32_t U_BARS = 96 * 1024, U_SMEM = U_BARS + 12 * 8 + 16 + U_TN * 4;
+static_assert(Stage<false>::bytes * Stage<false>::n <= U_BARS && Stage<true>::bytes * Stage<true>::n <= U_BARS, "stages");
+static_assert(2 * (U_SMEM + 1024) <= 228 * 1024, "two CTAs share an SM");
+
 __device__ __forceinline__ void bar_wait(uint64_t* b, uint32_t parity, int32_t* status) {
-    uint32_t ok = 0, it = 0;
-    while (!ok && ++it < U_SPIN)
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(ok) : "r"(s32(b)), "r"(parity) : "memory");
-    if (!ok) atomicExch(status, EDG_E_TIMEOUT);
+    uint32_t it = 0;
+    while (!mbar_try_wait(b, parity))
+        if (++it >= kSpinLimit) { atomicExch(status, EDG_E_TIMEOUT); break; }
 }
-// shared-memory matrix descriptor: K-major, no swizzle
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr) {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((U_LBO >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((U_SBO >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
-}
+// Shared-memory matrix descriptor: K-major, no swizzle.  Its lower word holds the address and the distance between k cores, the upper
+// one is the same for all: row groups 128 bytes apart, descriptor version 1.
+__device__ __forceinline__ uint32_t umma_desc(uint32_t saddr, uint32_t lbo) { return ((saddr >> 4) & 0x3FFF) | (((lbo >> 4) & 0x3FFF) << 16); }
+constexpr uint32_t U_DESC_HI = (128 >> 4) | (1u << 14);
 // instruction descriptor: fp32 accumulator, fp16 A and B, both K-major, M = 128, N = n
 __device__ __forceinline__ uint32_t umma_idesc(int n) {
     return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
-__device__ __forceinline__ void umma(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, bool accumulate) {
-    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate ? 1u : 0u) : "memory");
+__device__ __forceinline__ void umma(uint32_t tmem_d, uint32_t da, uint32_t db, uint32_t idesc, bool accumulate) {
+    asm volatile("{\n.reg .pred p;\n.reg .b64 a, b;\nsetp.ne.b32 p, %4, 0;\nmov.b64 a, {%1, %5};\nmov.b64 b, {%2, %5};\n"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n}"
+                 ::"r"(tmem_d), "r"(da), "r"(db), "r"(idesc), "r"(accumulate ? 1u : 0u), "r"(U_DESC_HI) : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint64_t* b) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(b)) : "memory");
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(b)) : "memory");
 }
+// (load and wait in one statement: nothing that uses the values may move between them)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                 "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-                   "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-                   "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-                 : "r"(taddr));
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+                 "tcgen05.wait::ld.sync.aligned;"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+                 : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xFFFFFFFF;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+    return p != 0;
+}
+__device__ __forceinline__ void fence_to_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// offset of (row r, k core kc) inside an operand tile
-__device__ __forceinline__ uint32_t core_off(int r, int kc) { return (uint32_t)(((kc * 16 + (r >> 3)) * 8 + (r & 7)) * 16); }
-
-// One 32-bit word = 8 codes of a row -> the core row of s (q - z): fp16 value and exact fp16 residual.
-__device__ __forceinline__ void dequant_hi_lo(uint32_t w, __half2 s2, __half2 z2, uint4& hi, uint4& lo) {
-    uint32_t q[4];
-    dequant_word(w, z2, q);                              // (q - z): (k0,k4) (k1,k5) (k2,k6) (k3,k7)
-    uint32_t h[4], l[4];
+// The states of a tile's pairs as the gate/up kernel's B operand, [stage of 64 k][8 k cores][pairs rounded to 16][8 k]: a stage is one bulk
+// copy then.  (Gathered by 16-byte copies of the tiles' own CTAs, the bursts held up every other access to shared memory.)
+// Consecutive threads take consecutive pairs of four k cores: their 16-byte pieces are adjacent in the tile; the reads are 64 bytes
+// of as many rows.
+__global__ void __launch_bounds__(256) umma_gather_x_kernel(const __grid_constant__ GroupedParams p) {
+    pdl_launch_dependents();
+    pdl_wait_prior_grid();
+    const int tile = blockIdx.y;
+    if (tile >= *p.n_tiles) return;
+    const int4 ti = p.tiles[tile];
+    const int n16 = (ti.z + 15) & ~15;
+    uint8_t* out = p.xq + (size_t)tile * p.H * 256;
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n16 * (p.H / 32); i += gridDim.x * 256) {
+        const int tok = i % n16, c = i / n16;
+        uint4 raw[4] = {};
+        if (tok < ti.z) {
+            const uint4* src = reinterpret_cast<const uint4*>(p.x + (size_t)(p.order[ti.y + tok] / p.K) * p.H + c * 32);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const __half2 qz = u32_as_h2(q[i]);
-        const __half2 a = __hmul2(s2, qz);
-        h[i] = h2_as_u32(a);
-        l[i] = h2_as_u32(__hfma2(s2, qz, __hneg2(a)));
+            for (int j = 0; j < 4; ++j) raw[j] = __ldg(src + j);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float f[8] = {bf16_lo(raw[j].x), bf16_hi(raw[j].x), bf16_lo(raw[j].y), bf16_hi(raw[j].y),
+                                bf16_lo(raw[j].z), bf16_hi(raw[j].z), bf16_lo(raw[j].w), bf16_hi(raw[j].w)};
+            *reinterpret_cast<uint4*>(out + ((size_t)(c * 4 + j) * n16 + tok) * 16) = permute8(f);
+        }
     }
-    hi = make_uint4(h[0], h[1], h[2], h[3]);
-    lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
 // 8 bf16 -> 8 fp16 in natural order (adapter matrices)
@@ -109,389 +123,327 @@ __device__ __forceinline__ uint4 bf16x8_to_f16(uint4 v) {
     o.w = h2_as_u32(__floats2half2_rn(bf16_lo(v.w), bf16_hi(v.w)));
     return o;
 }
-// 8 fp32 * sigma -> 8 fp16 in natural order; missing entries (j >= n) are zero
-__device__ __forceinline__ uint4 f32x8_to_f16(const float* src, int n, float sigma) {
-    float f[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) f[j] = (src != nullptr && j < n) ? sigma * src[j] : 0.f;
-    uint4 o;
-    o.x = h2_as_u32(__floats2half2_rn(f[0], f[1]));
-    o.y = h2_as_u32(__floats2half2_rn(f[2], f[3]));
-    o.z = h2_as_u32(__floats2half2_rn(f[4], f[5]));
-    o.w = h2_as_u32(__floats2half2_rn(f[6], f[7]));
-    return o;
-}
 
-struct UmmaSmem {
-    uint8_t* stage;     // [U_STAGES][4 tiles]
-    uint8_t* act;       // [slots of activations]
-    uint64_t* full;     // [stages] weights written (one arrival per producer warp)
-    uint64_t* empty;    // [stages] MMAs that read the stage have completed
-    uint64_t* afull;    // [slots] activations arrived
-    uint64_t* aempty;   // [slots] MMAs that read the slot have completed
-    uint64_t* done;     // all MMAs of the tile have completed
-    uint32_t* tptr;
-    int* pair;          // [U_TN]
-};
-__device__ __forceinline__ UmmaSmem carve(uint8_t* smem, uint32_t act_bytes) {
-    UmmaSmem S;
-    S.stage = smem;
-    S.act = smem + U_STAGES * 4 * U_TILE;
-    S.full = reinterpret_cast<uint64_t*>(S.act + act_bytes);
-    S.empty = S.full + U_STAGES;
-    S.afull = S.empty + U_STAGES;
-    S.aempty = S.afull + U_ACT_MAX;
-    S.done = S.aempty + U_ACT_MAX;
-    S.tptr = reinterpret_cast<uint32_t*>(S.done + 1);
-    S.pair = reinterpret_cast<int*>(S.tptr + 2);
-    return S;
-}
-// gate/up: x, 8 KB a chunk, four slots; down: h and its residual, 16 KB a chunk, three slots.  Two CTAs fit an SM either way.
-constexpr int U_ACT_GU = 4, U_ACT_D = 3;
-constexpr uint32_t U_ACT_GU_BYTES = U_ACT_GU * U_TILE, U_ACT_D_BYTES = U_ACT_D * 2 * U_TILE;
-constexpr size_t umma_smem_bytes(uint32_t act_bytes) { return (size_t)U_STAGES * 4 * U_TILE + act_bytes + 128 + U_TN * 4; }
-
-// common prologue: pair list, barriers, tensor memory
-__device__ __forceinline__ uint32_t umma_begin(const GroupedParams& p, const UmmaSmem& S, int slot, int first, int cnt, int cols) {
-    const int tid = threadIdx.x, warp = tid >> 5;
-    if (tid < U_TN) S.pair[tid] = tid < cnt ? p.lists[(size_t)slot * p.T + first + tid] : -1;
+// One tile: DOWN = false: h = silu(gate) up for 64 rows of the intermediate dimension (rows 0..63 of the tile are gate rows, 64..127
+// the up rows of the same indices), written as the down kernel's B operand; DOWN = true: o[pair][row] = gate weight * (W h) for 128
+// output rows.  The adapter comes first, as stages of its own with scale 1: A = B_lora rows, B = sigma (A_lora x), for gate/up
+// with the ranks of both projections side by side (a gate row is zero in the up ranks and the other way round).
+template <bool DOWN>
+__global__ void __launch_bounds__(U_THREADS, 2) umma_tile_kernel(const __grid_constant__ GroupedParams p) {
+    using St = Stage<DOWN>;
+    extern __shared__ __align__(128) uint8_t smem[];
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + U_BARS);         // [stages] weights and activations are there
+    uint64_t* empty = full + 4;                                          // [stages] the MMAs that read the stage have completed
+    uint64_t* accfull = empty + 4;                                       // [2] a group's sums are complete
+    uint64_t* accempty = accfull + 2;                                    // [2] and have been taken out
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(accempty + 2);
+    int* s_pair = reinterpret_cast<int*>(s_tmem + 4);                    // [U_TN]
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    pdl_launch_dependents();
+    pdl_wait_prior_grid();
+    const int tile = blockIdx.y;                 // row blocks of a tile are neighbours in the grid: they share its activations in L2
+    if (tile >= *p.n_tiles) return;
+    const int4 ti = p.tiles[tile];               // {slot, first position in order, pairs, adapter}
+    const int cnt = ti.z, n16 = (cnt + 15) & ~15;
+    const uint8_t* rec = p.pool + (size_t)ti.x * p.L.bytes;
+    const int K = DOWN ? p.I : p.H, NS = K / St::k, gshift = p.gshift;
+    const int RK = DOWN ? p.rank : 2 * p.rank, RS = (RK + St::k - 1) / St::k;      // ranks, stages of them (ahead of the others)
+    const uint32_t xlbo = (uint32_t)n16 * 16;                            // (tiles of activations are stored without gaps)
+    if (tid < U_TN) s_pair[tid] = tid < cnt ? p.order[ti.y + tid] : -1;
     if (tid == 0) {
-        for (int s = 0; s < U_STAGES; ++s) { bar_init(&S.full[s], U_PROD_WARPS); bar_init(&S.empty[s], 1); }
-        for (int s = 0; s < U_ACT_MAX; ++s) { bar_init(&S.afull[s], 1); bar_init(&S.aempty[s], 1); }
-        bar_init(S.done, 1);
+        for (int s = 0; s < St::n; ++s) { mbar_init(&full[s], 5); mbar_init(&empty[s], 1); }       // (four warps, and who brings the activations)
+        for (int s = 0; s < 2; ++s) { mbar_init(&accfull[s], 1); mbar_init(&accempty[s], 4); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == U_PROD_WARPS) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s32(S.tptr)), "r"(cols) : "memory");
+    if (warp == 8) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(2 * U_TN) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    return *S.tptr;
-}
-__device__ __forceinline__ void umma_end(uint32_t tmem, int cols) {
+    const uint32_t tmem = *s_tmem;
+
+    struct Ring {                                                        // position in the ring of stages
+        int st = 0;
+        uint32_t phase = 0;
+        __device__ __forceinline__ void next() { if (++st == St::n) { st = 0; phase ^= 1u; } }
+    } rp;
+
+    if (warp < 4) {
+        // ================================================= weights into shared memory
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        const int r = tid;
+        const int n = DOWN ? (int)blockIdx.x * 128 + r : (int)blockIdx.x * 64 + (r & 63);
+        const uint8_t *cp, *zp;                  // this row's first chunk of codes and its first (scale, zero) pair
+        if (DOWN) {
+            cp = rec + p.L.codes_down + down_code_off(p.H, p.I, n, 0);
+            zp = rec + p.L.sz_down + down_sz_off(p.H, p.I, p.group, n, 0);
+        } else {
+            cp = rec + (r < 64 ? p.L.codes_gate : p.L.codes_up) + code_off(p.H, n, 0);
+            zp = rec + (r < 64 ? p.L.sz_gate : p.L.sz_up) + sz_off(p.H, p.group, n, 0);
+        }
+        const int cps = p.I / kDownSlices / 32;                          // (a power of two, as is the group)
+        const int cps_sh = 31 - __clz(cps), gps_sh = 31 - __clz(p.I / kDownSlices) - gshift;
+        const uint32_t cslice = (uint32_t)p.H * (p.I / kDownSlices) / 2, zslice = ((uint32_t)p.H << gps_sh) * 4;
+        auto codes = [&](int c) {
+            return ld_stream16(DOWN ? cp + (size_t)(c >> cps_sh) * cslice + (c & (cps - 1)) * 256 : cp + c * 256);
+        };
+        auto pair_of = [&](int c) {                                      // (scale, zero) of the group that holds chunk c
+            const int g = (c * 32) >> gshift;
+            return ld_stream4(DOWN ? zp + (size_t)(g >> gps_sh) * zslice + (g & ((1 << gps_sh) - 1)) * 64 : zp + g * 64);
+        };
+        uint4 cw[St::ahead][St::chunks];
+        uint32_t zz[St::ahead][St::chunks];
+        auto load = [&](int j, int s) {                                  // (no copies of values that are on their way: a copy waits)
+#pragma unroll
+            for (int h = 0; h < St::chunks; ++h) cw[j][h] = codes(s * St::chunks + h);
+            zz[j][0] = pair_of(s * St::chunks);
+            if (!DOWN && gshift == 5) zz[j][St::chunks - 1] = pair_of(s * St::chunks + 1);
+        };
+#pragma unroll
+        for (int j = 0; j < St::ahead; ++j)
+            if (j < NS) load(j, j);
+        auto written = [&]() {
+            fence_to_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&full[rp.st]);
+            rp.next();
+        };
+        // ---- the adapter's rows
+        for (int rs = 0; rs < RS; ++rs) {
+            const uint16_t* B = static_cast<const uint16_t*>(DOWN ? p.lora.B_down : (r < 64 ? p.lora.B_gate : p.lora.B_up)) +
+                                ((size_t)ti.w * (DOWN ? p.H : p.I) + n) * p.rank;
+            const int k0 = DOWN || r < 64 ? 0 : p.rank;
+#pragma unroll 4
+            for (int kc = 0; kc < St::k / 8; ++kc) {
+                const int k = rs * St::k + kc * 8 - k0;
+                uint4 a = make_uint4(0, 0, 0, 0);
+                if (k >= 0 && k < p.rank) a = bf16x8_to_f16(__ldg(reinterpret_cast<const uint4*>(B + k)));
+                *reinterpret_cast<uint4*>(smem + rp.st * St::bytes + kc * U_LBO + r * 16) = a;
+            }
+            written();
+        }
+#pragma unroll 1
+        for (int s0 = 0; s0 < NS; s0 += St::ahead)
+#pragma unroll
+            for (int j = 0; j < St::ahead; ++j) {
+                const int s = s0 + j;
+                if (s >= NS) break;
+                bar_wait(&empty[rp.st], rp.phase ^ 1, p.status);
+                uint8_t* sb = smem + rp.st * St::bytes + r * 16;
+#pragma unroll
+                for (int h = 0; h < St::chunks; ++h) {
+                    const __half2 mz = neg_zero_x(u32_as_h2(!DOWN && gshift == 5 ? zz[j][h] : zz[j][0]));
+                    const uint32_t w[4] = {cw[j][h].x, cw[j][h].y, cw[j][h].z, cw[j][h].w};
+#pragma unroll
+                    for (int kc = 0; kc < 4; ++kc) {
+                        uint32_t q[4];
+                        dequant_word_x(w[kc], mz, q);
+                        *reinterpret_cast<uint4*>(sb + (h * 4 + kc) * U_LBO) = make_uint4(q[0], q[1], q[2], q[3]);
+                    }
+                }
+                if (s + St::ahead < NS) load(j, s + St::ahead);
+                written();
+            }
+    } else if (warp < 8) {
+        // ================================================= groups' sums out of tensor memory, epilogue
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
+        const int r = tid - 128;
+        const int n = DOWN ? (int)blockIdx.x * 128 + r : (int)blockIdx.x * 64 + (r & 63);
+        const uint8_t* zp = rec + (DOWN ? p.L.sz_down + down_sz_off(p.H, p.I, p.group, n, 0) : (r < 64 ? p.L.sz_gate : p.L.sz_up) + sz_off(p.H, p.group, n, 0));
+        const int gps_sh = 31 - __clz(p.I / kDownSlices) - gshift;
+        const uint32_t zslice = ((uint32_t)p.H << gps_sh) * 4;
+        const int ad = RS > 0 ? 1 : 0, NG = (K >> gshift) + ad;
+        auto scale = [&](int g) {                                        // (scale, zero) of group g, g counted with the adapter's
+            if (g < ad || g >= NG) return 0x00001800u;                   // (2^-9, what undoes the unscaling below: the adapter's factor is 1)
+            g -= ad;
+            return ld_stream4(DOWN ? zp + (size_t)(g >> gps_sh) * zslice + (g & ((1 << gps_sh) - 1)) * 64 : zp + g * 64);
+        };
+        float acc[U_TN];
+#pragma unroll
+        for (int j = 0; j < U_TN; ++j) acc[j] = 0.f;
+        const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        uint32_t z0 = scale(0), z1 = scale(1);
+        auto take = [&](int g, int buf, uint32_t& z) {
+            const float s = kUnscaleX * __low2float(u32_as_h2(z));
+            z = scale(g + 2);                                            // (no copies between z0 and z1: a copy waits for the load)
+            bar_wait(&accfull[buf], (uint32_t)(g >> 1) & 1, p.status);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+            for (int b = 0; b < U_TN / 32; ++b)
+                if (b * 32 < n16) {
+                    uint32_t v[32];
+                    tmem_ld32(lane_addr + buf * U_TN + b * 32, v);
+#pragma unroll
+                    for (int j = 0; j < 32; j += 2) fma2(acc[b * 32 + j], acc[b * 32 + j + 1], s, __uint_as_float(v[j]), __uint_as_float(v[j + 1]));
+                }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&accempty[buf]);
+        };
+#pragma unroll 1
+        for (int g = 0; g < NG; g += 2) {
+            take(g, 0, z0);
+            if (g + 1 < NG) take(g + 1, 1, z1);
+        }
+        if (DOWN) {
+            float2* s_pg = reinterpret_cast<float2*>(smem);              // {pair, its weight} (the stages have been used)
+            s_pg[r] = make_float2(__int_as_float(s_pair[r]), r < cnt ? p.gates[s_pair[r]] : 0.f);
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            float* o = p.o + n;
+#pragma unroll
+            for (int b = 0; b < U_TN; b += 8)
+                if (b < cnt) {
+                    float2 pg[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) pg[j] = s_pg[b + j];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (b + j < cnt) o[(size_t)__float_as_int(pg[j].x) * p.H] = pg[j].y * acc[b + j];
+                }
+        } else {
+            // 32 columns at a time: the threads of the gate rows finish the first half of them, those of the up rows the second, and each
+            // hands the other half over; then eight rows of h of a pair go out as one core row of value and one of residual
+            float* s_h = reinterpret_cast<float*>(smem);       // [column][U_HS] (the stages have been used)
+            float* hs = s_h + (r & 63);
+            const bool is_gate = r < 64;
+            constexpr int half = U_HQ / 2;
+            const int give = is_gate ? half : 0, keep = half - give;
+#pragma unroll
+            for (int c0 = 0; c0 < U_TN; c0 += U_HQ) {
+                if (c0 < n16) {
+#pragma unroll
+                    for (int j = 0; j < half; ++j) hs[(give + j) * U_HS] = is_gate ? acc[c0 + half + j] : acc[c0 + j];
+                    asm volatile("bar.sync 1, 128;" ::: "memory");
+                    float* q = hs + keep * U_HS;
+                    float o[half];
+#pragma unroll
+                    for (int j = 0; j < half; ++j) o[j] = q[j * U_HS];
+#pragma unroll
+                    for (int j = 0; j < half; ++j) {
+                        const float mine = is_gate ? acc[c0 + j] : acc[c0 + half + j], gv = is_gate ? mine : o[j];
+                        q[j * U_HS] = __fdividef(gv, 1.f + __expf(-gv)) * (is_gate ? o[j] : mine);
+                    }
+                    asm volatile("bar.sync 1, 128;" ::: "memory");
+#pragma unroll
+                    for (int i = 0; i < U_HQ * 8 / 128; ++i) {
+                        const int piece = i * 128 + r, tok = piece % U_HQ, core = piece / U_HQ, k = (int)blockIdx.x * 64 + core * 8;
+                        const float4 a = *reinterpret_cast<const float4*>(s_h + tok * U_HS + core * 8), b = *reinterpret_cast<const float4*>(s_h + tok * U_HS + core * 8 + 4);
+                        float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+                        if (c0 + tok >= cnt) {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) f[e] = 0.f;
+                        }
+                        if (c0 + tok < n16) {
+                            uint8_t* w = p.hq + (size_t)tile * p.I * 512 + ((size_t)(k >> 5) * 8 + ((k & 31) >> 3)) * n16 * 16 + (c0 + tok) * 16;
+                            *reinterpret_cast<uint4*>(w) = permute8(f);
+                            *reinterpret_cast<uint4*>(w + (size_t)n16 * 64) = permute8_lo(f);
+                        }
+                    }
+                    asm volatile("bar.sync 1, 128;" ::: "memory");
+                }
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");
+        if (warp == 8) {
+            // ============================================= the MMAs.  Descriptors differ only in their address field.  The whole warp walks the
+            // loop and one lane of it issues: what is the same for all lanes then stays in uniform registers, where the MMA wants it.
+            const uint32_t idesc = umma_idesc(n16);
+            const uint32_t a0 = umma_desc(smem_u32(smem), U_LBO), x0 = umma_desc(smem_u32(smem + St::a_bytes), xlbo);
+            constexpr uint32_t kStage = St::bytes >> 4, kStepA = (2 * U_LBO) >> 4;
+            const uint32_t kStepX = (2 * xlbo) >> 4;
+            int g = 0;
+            auto stage_there = [&]() {
+                bar_wait(&full[rp.st], rp.phase, p.status);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            };
+            for (int i = 0; i < RS; ++i) {
+                stage_there();
+                const uint32_t as = a0 + rp.st * kStage, xs = x0 + rp.st * kStage;
+                const int ksteps = min(St::k / 16, (RK - i * St::k + 15) / 16);
+                if (elect_one()) {
+                    for (int ks = 0; ks < ksteps; ++ks) umma(tmem, as + ks * kStepA, xs + ks * kStepX, idesc, i > 0 || ks > 0);
+                    umma_commit(&empty[rp.st]);
+                    if (i == RS - 1) umma_commit(&accfull[0]);
+                }
+                __syncwarp();
+                rp.next();
+            }
+            if (RS > 0) g = 1;
+            const int gmask = (p.group >> 5) - 1;                        // a group is 1, 2 or 4 chunks of 32 k
+#pragma unroll 1
+            for (int s = 0; s < NS; ++s) {
+                stage_there();
+                const uint32_t as = a0 + rp.st * kStage, xs = x0 + rp.st * kStage;
+#pragma unroll
+                for (int h = 0; h < St::chunks; ++h) {
+                    const int c = s * St::chunks + h;
+                    const bool first = (c & gmask) == 0, last = (c & gmask) == gmask;
+                    if (first) {
+                        bar_wait(&accempty[g & 1], ((uint32_t)(g >> 1) & 1) ^ 1, p.status);
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    }
+                    const uint32_t d = tmem + (g & 1) * U_TN;
+                    if (elect_one()) {
+#pragma unroll
+                        for (int ks = 0; ks < 2; ++ks) {
+                            umma(d, as + (2 * h + ks) * kStepA, xs + (2 * h + ks) * kStepX, idesc, !first || ks > 0);
+                            if (DOWN) umma(d, as + ks * kStepA, xs + (2 + ks) * kStepX, idesc, true);    // (values, then residuals)
+                        }
+                        if (last) umma_commit(&accfull[g & 1]);
+                        if (h == St::chunks - 1) umma_commit(&empty[rp.st]);
+                    }
+                    __syncwarp();
+                    if (last) ++g;
+                }
+                rp.next();
+            }
+        } else if (warp == 9) {
+            // ============================================= activations.  Eight rows of a tile (pairs) and four k cores per copy of a warp
+            for (int rs = 0; rs < RS; ++rs) {                            // A_lora x (or h) times sigma, fp16, per token or pair
+                const uint8_t* src = reinterpret_cast<const uint8_t*>(DOWN ? p.u_d : p.u_gu);
+                const uint32_t dst = smem_u32(smem + rs * St::bytes + St::a_bytes) + (lane >> 3) * xlbo + (lane & 7) * 16;
+                for (int rg = 0; rg * 8 < n16; ++rg) {
+                    const int pr = s_pair[rg * 8 + (lane & 7)];
+                    const uint8_t* row = src + (size_t)(pr < 0 ? 0 : (DOWN || p.n_adapters != 1 ? pr : pr / p.K)) * RK * 2;
+#pragma unroll
+                    for (int h = 0; h < St::chunks; ++h) {
+                        const int core = rs * (St::k / 8) + h * 4 + (lane >> 3);
+                        const bool in = pr >= 0 && core < RK / 8;        // (zeros beyond the ranks, and for no pair)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                                     ::"r"(dst + h * 4 * xlbo + rg * 128), "l"(row + (in ? core : 0) * 16), "r"(in ? 16 : 0) : "memory");
+                    }
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+                rp.next();
+            }
+            // (the main stages behind them are asked for first)
+            const uint32_t bytes = (uint32_t)n16 * 128;                  // of 64 k of states, or 32 k of h and its residual
+            const uint8_t* src = DOWN ? p.hq + (size_t)tile * p.I * 512 : p.xq + (size_t)tile * p.H * 256;
+            for (int s = 0; s < NS; ++s) {
+                if (RS > 0 && s == min(St::n - RS, NS - 1)) {            // (before the first wait for a stage that they free)
+                    asm volatile("cp.async.wait_group 0;" ::: "memory");
+                    fence_to_async();
+                    __syncwarp();
+                    if (lane == 0)
+                        for (int rs = 0; rs < RS; ++rs) mbar_arrive(&full[rs]);
+                }
+                if (lane == 0) {
+                    bar_wait(&empty[rp.st], rp.phase ^ 1, p.status);
+                    mbar_expect_tx(&full[rp.st], bytes);
+                    bulk_g2s(smem + rp.st * St::bytes + St::a_bytes, src + (size_t)s * bytes, bytes, &full[rp.st]);
+                }
+                __syncwarp();
+                rp.next();
+            }
+        }
+    }
+    __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if ((threadIdx.x >> 5) == U_PROD_WARPS)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
-}
-// lane 0 of the copy warp: the activations of every chunk, as slots become free
-__device__ __forceinline__ void fetch_activations(const UmmaSmem& S, const uint8_t* src, int n_chunks, int slots, uint32_t bytes, int32_t* status) {
-    for (int c = 0; c < n_chunks; ++c) {
-        const int sl = c % slots;
-        bar_wait(&S.aempty[sl], ((uint32_t)(c / slots) & 1) ^ 1, status);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s32(&S.afull[sl])), "r"(bytes) : "memory");
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(s32(S.act + sl * bytes)), "l"(src + (size_t)c * bytes), "r"(bytes), "r"(s32(&S.afull[sl])) : "memory");
-    }
-}
-// a producer warp has written its part of a stage
-__device__ __forceinline__ void stage_written(uint64_t* full) {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes -> visible to the tensor core
-    __syncwarp();
-    if ((threadIdx.x & 31) == 0) bar_arrive(full);
-}
-
-// A producer thread: row r of the two operand tiles at `tile` of every stage, from 32 codes a chunk.  The loads run four chunks
-// ahead: with one, a chunk took as long as a load from memory.
-template <typename LC, typename LZ>
-__device__ __forceinline__ void produce(const UmmaSmem& S, int n_chunks, int gshift, int tile, int r, LC codes, LZ sz, int32_t* status) {
-    uint4 cw[U_AHEAD];
-    uint32_t nz[U_AHEAD];
-    auto starts = [&](int c) { return ((c * U_KC) & ((1 << gshift) - 1)) == 0; };      // a group of k begins with chunk c
-#pragma unroll
-    for (int j = 0; j < U_AHEAD; ++j) {                                  // (the chunks are a multiple of four)
-        cw[j] = codes(j);
-        nz[j] = starts(j) ? sz((j * U_KC) >> gshift) : 0u;
-    }
-    __half2 sc = __float2half2_rn(0.f), zr = sc;
-    for (int c0 = 0; c0 < n_chunks; c0 += U_AHEAD)
-#pragma unroll
-        for (int j = 0; j < U_AHEAD; ++j) {
-            const int c = c0 + j, st = c % U_STAGES;
-            const uint32_t w[4] = {cw[j].x, cw[j].y, cw[j].z, cw[j].w};
-            if (starts(c)) {
-                const __half2 a = u32_as_h2(nz[j]);
-                sc = __low2half2(a); zr = __high2half2(a);
-            }
-            if (c + U_AHEAD < n_chunks) {
-                cw[j] = codes(c + U_AHEAD);
-                if (starts(c + U_AHEAD)) nz[j] = sz(((c + U_AHEAD) * U_KC) >> gshift);
-            }
-            bar_wait(&S.empty[st], ((uint32_t)(c / U_STAGES) & 1) ^ 1, status);        // the MMAs that read this stage are done
-            uint8_t* sb = S.stage + (st * 4 + tile) * U_TILE;
-#pragma unroll
-            for (int kc = 0; kc < 4; ++kc) {
-                uint4 hi, lo;
-                dequant_hi_lo(w[kc], sc, zr, hi, lo);
-                *reinterpret_cast<uint4*>(sb + core_off(r, kc)) = hi;
-                *reinterpret_cast<uint4*>(sb + U_TILE + core_off(r, kc)) = lo;
-            }
-            stage_written(&S.full[st]);
-        }
-}
-
-// ---------------------------------------------------------------- token states as operand tiles
-// xq[tile][chunk of 32 k][128 tokens x 32 k]: thread = (token of the tile, k core); the four row blocks
-// of a tile then fetch every chunk with one bulk copy instead of gathering it again.
-__global__ void __launch_bounds__(256) umma_gather_x_kernel(GroupedParams p) {
-    const int tile = blockIdx.y;
-    if (tile >= *p.n_tiles) return;
-    const int slot = p.tiles[2 * tile], first = p.tiles[2 * tile + 1];
-    const int cnt = min(U_TN, p.counts[slot] - first);
-    const int cores = p.H / 8;                                   // 16-byte pieces per token
-    uint8_t* out = p.xq + (size_t)tile * (p.H / 32) * U_TILE;
-    // consecutive threads take consecutive tokens of four k cores: their 16-byte pieces are adjacent in the operand tile (coalesced
-    // writes); the reads are 64 bytes from 128 different rows (one k core at a time, half of every 32-byte sector came in vain:
-    // 64 us for 4096 tokens of 8 choices, now 55)
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < U_TN * (cores / 4); i += gridDim.x * blockDim.x) {
-        const int tok = i % U_TN, c = i / U_TN;
-        uint4 raw[4] = {};
-        if (tok < cnt) {
-            const int pair = p.lists[(size_t)slot * p.T + first + tok];
-            const uint4* src = reinterpret_cast<const uint4*>(p.x + (size_t)(pair / p.K) * p.H + c * 32);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) raw[j] = src[j];
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float f[8] = {bf16_lo(raw[j].x), bf16_hi(raw[j].x), bf16_lo(raw[j].y), bf16_hi(raw[j].y),
-                                bf16_lo(raw[j].z), bf16_hi(raw[j].z), bf16_lo(raw[j].w), bf16_hi(raw[j].w)};
-            *reinterpret_cast<uint4*>(out + (size_t)c * U_TILE + core_off(tok, j)) = permute8(f);
-        }
-    }
-}
-
-// ---------------------------------------------------------------- gate/up
-// stage = [gate hi][gate lo][up hi][up lo], x in slots of its own (one bulk copy per chunk); tensor memory: gate in
-// columns 0..127, up in 128..255.  Thread t dequantises row t % 128 of gate (t < 128) or up.
-__global__ void __launch_bounds__(U_THREADS, 2) umma_gate_up_kernel(GroupedParams p) {
-    const int tile = blockIdx.y;             // row blocks of a tile are neighbours in the grid: they share its activations in L2
-    if (tile >= *p.n_tiles) return;
-    extern __shared__ __align__(128) uint8_t smem[];
-    const UmmaSmem S = carve(smem, U_ACT_GU_BYTES);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int slot = p.tiles[2 * tile], first = p.tiles[2 * tile + 1];
-    const int cnt = min(U_TN, p.counts[slot] - first);
-    const int row0 = blockIdx.x * 128;
-    const uint8_t* rec = p.pool + (size_t)slot * p.L.bytes;
-    const uint32_t tmem = umma_begin(p, S, slot, first, cnt, 2 * U_TN);
-    const int n_chunks = p.H / U_KC;
-    const int r_chunks = p.rank > 0 ? (p.rank + 31) / 32 : 0;          // adapter: chunks of up to 32 ranks
-    const int gshift = 31 - __clz(p.group);
-
-    if (warp < U_PROD_WARPS) {
-        const int r = tid & 127, half = tid >> 7;                    // weight row; matrix (0 gate, 1 up) and, in the epilogue, half of the columns
-        const int pair = S.pair[r];
-        const uint8_t* cp = rec + (half ? p.L.codes_up : p.L.codes_gate);
-        const uint8_t* zp = rec + (half ? p.L.sz_up : p.L.sz_gate);
-        produce(S, n_chunks, gshift, 2 * half, r, [&](int c) { return ld_stream16(cp + code_off(p.H, row0 + r, c)); },
-                [&](int g) { return ld_stream4(zp + sz_off(p.H, p.group, row0 + r, g)); }, p.status);
-        // the adapter as extra k: A = B_gate / B_up rows (fp16 of bf16), B = sigma * (A_gate x) / sigma * (A_up x);
-        // the threads of matrix m write its A rows and its B rows (gate's B in tile 3, up's in tile 1)
-        if (r_chunks > 0) {
-            const int first_pair = S.pair[0];
-            const int ad = first_pair >= 0 ? p.pair_ad[first_pair] : 0;
-            const int n_sets = p.n_adapters == 1 ? 1 : p.K;
-            const float* um = nullptr;
-            if (pair >= 0) um = p.u_gu + (((size_t)(pair / p.K) * n_sets + (p.n_adapters == 1 ? 0 : pair % p.K)) * 2 + half) * p.rank;
-            const uint16_t* Bm = reinterpret_cast<const uint16_t*>(half ? p.lora.B_up : p.lora.B_gate) + ((size_t)ad * p.I + row0 + r) * p.rank;
-            for (int rc = 0; rc < r_chunks; ++rc) {
-                const int c = n_chunks + rc, st = c % U_STAGES;
-                const uint32_t use = (uint32_t)(c / U_STAGES);
-                bar_wait(&S.empty[st], (use & 1) ^ 1, p.status);
-                uint8_t* sb = S.stage + st * 4 * U_TILE;
-#pragma unroll
-                for (int kc = 0; kc < 4; ++kc) {
-                    const int j0 = rc * 32 + kc * 8, n = p.rank - j0;          // rank is a multiple of 8
-                    uint4 a = make_uint4(0, 0, 0, 0);
-                    if (n > 0) a = bf16x8_to_f16(*reinterpret_cast<const uint4*>(Bm + j0));
-                    *reinterpret_cast<uint4*>(sb + (2 * half) * U_TILE + core_off(r, kc)) = a;
-                    *reinterpret_cast<uint4*>(sb + (half ? 1 : 3) * U_TILE + core_off(r, kc)) = f32x8_to_f16(um != nullptr ? um + j0 : nullptr, n, p.sigma);
-                }
-                stage_written(&S.full[st]);
-            }
-        }
-        // ---- epilogue: h = silu(gate) * up, thread = weight row, 32 token columns at a time
-        bar_wait(S.done, 0, p.status);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        for (int c0 = half * (U_TN / 2); c0 < min(cnt, (half + 1) * (U_TN / 2)); c0 += 32) {
-            uint32_t g[32], u[32];
-            tmem_ld32(lane_addr + c0, g);
-            tmem_ld32(lane_addr + U_TN + c0, u);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            // h goes out twice: fp32 per pair (for the down adapter's projection), and as the down
-            // kernel's B operand: fp16 value and fp16 residual in operand-tile order, this row being k
-            // index i = row0 + r of the tile's chunk i / 32 (k core (i % 32) / 8, slot of i % 8 in the
-            // (k0,k4,k1,k5,k2,k6,k3,k7) order)
-            const int i = row0 + r, e = i & 7;
-            uint8_t* hq = p.hq + ((size_t)tile * (p.I / 32) + (i >> 5)) * 2 * U_TILE + (size_t)((e < 4 ? 2 * e : 2 * (e - 4) + 1) * 2);
-            const int kc = (i & 31) >> 3;
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const int pr = (c0 + j) < cnt ? S.pair[c0 + j] : -1;
-                if (pr >= 0) {
-                    const float hv = silu_f(__uint_as_float(g[j])) * __uint_as_float(u[j]);
-                    p.h[(size_t)pr * p.I + i] = hv;
-                    const __half hh = __float2half_rn(hv);
-                    const __half hl = __float2half_rn(hv - __half2float(hh));
-                    *reinterpret_cast<__half*>(hq + core_off(c0 + j, kc)) = hh;
-                    *reinterpret_cast<__half*>(hq + U_TILE + core_off(c0 + j, kc)) = hl;
-                }
-            }
-        }
-    } else if (warp == U_PROD_WARPS + 1) {
-        if (lane == 0) fetch_activations(S, p.xq + (size_t)tile * (p.H / 32) * U_TILE, n_chunks, U_ACT_GU, U_TILE, p.status);
-    } else if (lane == 0) {
-        // ---- the MMA issuer.  Descriptors differ only in their address field: base + offset >> 4.
-        const uint32_t idesc = umma_idesc((cnt + 15) & ~15);
-        const uint64_t d0 = umma_desc(s32(S.stage)), a0 = umma_desc(s32(S.act));
-        constexpr uint64_t kTile = U_TILE >> 4, kStep = (2 * U_LBO) >> 4, kStage = (4 * U_TILE) >> 4;
-        const uint32_t tg = tmem, tu = tmem + U_TN;
-        for (int c = 0; c < n_chunks; ++c) {
-            const int st = c % U_STAGES, sl = c % U_ACT_GU;
-            bar_wait(&S.full[st], (uint32_t)(c / U_STAGES) & 1, p.status);
-            bar_wait(&S.afull[sl], (uint32_t)(c / U_ACT_GU) & 1, p.status);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t ds = d0 + st * kStage, as = a0 + sl * kTile;
-#pragma unroll
-            for (int ks = 0; ks < U_KC / 16; ++ks) {
-                const uint64_t dk = ds + ks * kStep, db = as + ks * kStep;
-                umma(tg, dk, db, idesc, c > 0 || ks > 0);
-                umma(tg, dk + kTile, db, idesc, true);
-                umma(tu, dk + 2 * kTile, db, idesc, c > 0 || ks > 0);
-                umma(tu, dk + 3 * kTile, db, idesc, true);
-            }
-            umma_commit(&S.empty[st]);
-            umma_commit(&S.aempty[sl]);
-        }
-        for (int rc = 0; rc < r_chunks; ++rc) {
-            const int c = n_chunks + rc, st = c % U_STAGES;
-            bar_wait(&S.full[st], (uint32_t)(c / U_STAGES) & 1, p.status);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t ds = d0 + st * kStage;
-            const int ksteps = min(2, (p.rank - rc * 32 + 15) / 16);
-            for (int ks = 0; ks < ksteps; ++ks) {
-                const uint64_t dk = ds + ks * kStep;
-                umma(tg, dk, dk + 3 * kTile, idesc, true);
-                umma(tu, dk + 2 * kTile, dk + kTile, idesc, true);
-            }
-            umma_commit(&S.empty[st]);
-        }
-        umma_commit(S.done);
-    }
-    umma_end(tmem, 2 * U_TN);
-}
-
-// ---------------------------------------------------------------- down
-// A CTA covers 256 output rows (two accumulators of 128 columns in tensor memory) for the tile's tokens:
-// stage = [W0 hi][W0 lo][W1 hi][W1 lo], thread t dequantising row t of the 256; [h hi][h lo] in slots of their own, one bulk copy
-// per chunk (written in operand order by the gate/up kernel).
-// o = gate weight * (W h + sigma B (A h))
-__global__ void __launch_bounds__(U_THREADS, 2) umma_down_kernel(GroupedParams p) {
-    const int tile = blockIdx.y;             // row blocks of a tile are neighbours in the grid: they share its activations in L2
-    if (tile >= *p.n_tiles) return;
-    extern __shared__ __align__(128) uint8_t smem[];
-    const UmmaSmem S = carve(smem, U_ACT_D_BYTES);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int slot = p.tiles[2 * tile], first = p.tiles[2 * tile + 1];
-    const int cnt = min(U_TN, p.counts[slot] - first);
-    const int row0 = blockIdx.x * 256;
-    const uint8_t* rec = p.pool + (size_t)slot * p.L.bytes;
-    const uint32_t tmem = umma_begin(p, S, slot, first, cnt, 2 * U_TN);
-    const int n_chunks = p.I / U_KC;
-    const int r_chunks = p.rank > 0 ? (p.rank + 31) / 32 : 0;
-    const int gshift = 31 - __clz(p.group);
-
-    if (warp < U_PROD_WARPS) {
-        const int r = tid & 127, m = tid >> 7;                       // row r of half m: output row row0 + tid
-        const uint8_t* cdp = rec + p.L.codes_down;
-        const float my_gate = m == 0 && S.pair[r] >= 0 ? p.gates[S.pair[r]] : 0.f;
-        produce(S, n_chunks, gshift, 2 * m, r, [&](int c) { return ld_stream16(cdp + down_code_off(p.H, p.I, row0 + tid, c)); },
-                [&](int g) { return ld_stream4(rec + p.L.sz_down + down_sz_off(p.H, p.I, p.group, row0 + tid, g)); }, p.status);
-        if (r_chunks > 0) {
-            const int first_pair = S.pair[0];
-            const int ad = first_pair >= 0 ? p.pair_ad[first_pair] : 0;
-            const int pair = S.pair[r];
-            const float* ud = (m == 0 && pair >= 0) ? p.u_d + (size_t)pair * p.rank : nullptr;
-            const uint16_t* Bd = reinterpret_cast<const uint16_t*>(p.lora.B_down) + ((size_t)ad * p.H + row0 + tid) * p.rank;
-            for (int rc = 0; rc < r_chunks; ++rc) {
-                const int c = n_chunks + rc, st = c % U_STAGES;
-                const uint32_t use = (uint32_t)(c / U_STAGES);
-                bar_wait(&S.empty[st], (use & 1) ^ 1, p.status);
-                uint8_t* sb = S.stage + st * 4 * U_TILE;
-#pragma unroll
-                for (int kc = 0; kc < 4; ++kc) {
-                    const int j0 = rc * 32 + kc * 8, n = p.rank - j0;
-                    uint4 a = make_uint4(0, 0, 0, 0);
-                    if (n > 0) a = bf16x8_to_f16(*reinterpret_cast<const uint4*>(Bd + j0));
-                    *reinterpret_cast<uint4*>(sb + (2 * m) * U_TILE + core_off(r, kc)) = a;
-                    if (m == 0) *reinterpret_cast<uint4*>(sb + U_TILE + core_off(r, kc)) = f32x8_to_f16(ud != nullptr ? ud + j0 : nullptr, n, p.sigma);
-                }
-                stage_written(&S.full[st]);
-            }
-        }
-        // ---- epilogue: o[pair][row] = gate weight * acc; thread t = row t, accumulator t / 128
-        bar_wait(S.done, 0, p.status);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        float* gate = reinterpret_cast<float*>(S.act);               // (the activations have been used)
-        if (m == 0) gate[r] = my_gate;
-        asm volatile("bar.sync 1, %0;" ::"n"(U_PROD_WARPS * 32) : "memory");
-        const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + m * U_TN;
-        for (int c0 = 0; c0 < cnt; c0 += 32) {
-            uint32_t v[32];
-            tmem_ld32(lane_addr + c0, v);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const int pr = (c0 + j) < cnt ? S.pair[c0 + j] : -1;
-                if (pr >= 0) p.o[(size_t)pr * p.H + row0 + tid] = gate[c0 + j] * __uint_as_float(v[j]);
-            }
-        }
-    } else if (warp == U_PROD_WARPS + 1) {
-        if (lane == 0) fetch_activations(S, p.hq + (size_t)tile * (p.I / 32) * 2 * U_TILE, n_chunks, U_ACT_D, 2 * U_TILE, p.status);
-    } else if (lane == 0) {
-        const uint32_t idesc = umma_idesc((cnt + 15) & ~15);
-        const uint64_t d0 = umma_desc(s32(S.stage)), a0 = umma_desc(s32(S.act));
-        constexpr uint64_t kTile = U_TILE >> 4, kStep = (2 * U_LBO) >> 4, kStage = (4 * U_TILE) >> 4;
-        for (int c = 0; c < n_chunks; ++c) {
-            const int st = c % U_STAGES, sl = c % U_ACT_D;
-            bar_wait(&S.full[st], (uint32_t)(c / U_STAGES) & 1, p.status);
-            bar_wait(&S.afull[sl], (uint32_t)(c / U_ACT_D) & 1, p.status);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t ds = d0 + st * kStage, as = a0 + sl * 2 * kTile;
-#pragma unroll
-            for (int ks = 0; ks < U_KC / 16; ++ks) {
-                const uint64_t w0 = ds + ks * kStep, hhi = as + ks * kStep;
-#pragma unroll
-                for (int m = 0; m < 2; ++m) {
-                    const uint64_t whi = w0 + 2 * m * kTile;
-                    umma(tmem + m * U_TN, whi, hhi, idesc, c > 0 || ks > 0);
-                    umma(tmem + m * U_TN, whi + kTile, hhi, idesc, true);
-                    umma(tmem + m * U_TN, whi, hhi + kTile, idesc, true);
-                }
-            }
-            umma_commit(&S.empty[st]);
-            umma_commit(&S.aempty[sl]);
-        }
-        for (int rc = 0; rc < r_chunks; ++rc) {
-            const int c = n_chunks + rc, st = c % U_STAGES;
-            bar_wait(&S.full[st], (uint32_t)(c / U_STAGES) & 1, p.status);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t ds = d0 + st * kStage;
-            const int ksteps = min(2, (p.rank - rc * 32 + 15) / 16);
-            for (int ks = 0; ks < ksteps; ++ks) {
-                const uint64_t w0 = ds + ks * kStep;
-                umma(tmem, w0, w0 + kTile, idesc, true);
-                umma(tmem + U_TN, w0 + 2 * kTile, w0 + kTile, idesc, true);
-            }
-            umma_commit(&S.empty[st]);
-        }
-        umma_commit(S.done);
-    }
-    umma_end(tmem, 2 * U_TN);
+    if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * U_TN) : "memory");
 }
 
 }  // namespace
@@ -500,21 +452,16 @@ bool umma_grouped_supported(const edg_layer_desc& d) {
     return d.H % 256 == 0 && d.I % 128 == 0 && (d.group & (d.group - 1)) == 0 && d.group >= 32 && d.rank % 8 == 0;
 }
 
-cudaError_t launch_umma_gate_up(const GroupedParams& p, int max_tiles, cudaStream_t st) {
+cudaError_t launch_umma(const GroupedParams& p, bool down, int max_tiles, cudaStream_t st) {
     static OncePerDevice once;
-    const cudaError_t e = once([] { return allow_smem(umma_smem_bytes(U_ACT_GU_BYTES), umma_gate_up_kernel); });
+    const cudaError_t e = once([] { return allow_smem(U_SMEM, umma_tile_kernel<false>, umma_tile_kernel<true>); });
     if (e != cudaSuccess) return e;
-    umma_gather_x_kernel<<<dim3(8, max_tiles), 256, 0, st>>>(p);
-    umma_gate_up_kernel<<<dim3(p.I / 128, max_tiles), U_THREADS, umma_smem_bytes(U_ACT_GU_BYTES), st>>>(p);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_umma_down(const GroupedParams& p, int max_tiles, cudaStream_t st) {
-    static OncePerDevice once;
-    const cudaError_t e = once([] { return allow_smem(umma_smem_bytes(U_ACT_D_BYTES), umma_down_kernel); });
-    if (e != cudaSuccess) return e;
-    umma_down_kernel<<<dim3(p.H / 256, max_tiles), U_THREADS, umma_smem_bytes(U_ACT_D_BYTES), st>>>(p);
-    return cudaGetLastError();
+    if (!down) {
+        const cudaError_t g = launch_pdl(umma_gather_x_kernel, dim3(8, max_tiles), 256, 0, st, p);
+        if (g != cudaSuccess) return g;
+    }
+    if (down) return launch_pdl(umma_tile_kernel<true>, dim3(p.H / 128, max_tiles), U_THREADS, U_SMEM, st, p);
+    return launch_pdl(umma_tile_kernel<false>, dim3(p.I / 64, max_tiles), U_THREADS, U_SMEM, st, p);
 }
 
 }  // namespace edg

@@ -1,233 +1,145 @@
-// The rank-r projections of the unmerged adapter (Sec. 3.3: delta = sigma * B (A v)) for many tokens at
-// once, on the tensor cores: u = A_gate x and A_up x per token (before gate/up), u_d = A_down h per
-// (token, choice) pair (before down).  With one adapter per layer the A matrices are the same for every
-// token, so 8 tokens (or pairs) become the 8 columns of m16n8k16 tiles whose rows are the adapter's
-// rows: an A row is read once per 8 tokens instead of once per token.  Operands are fetched 16 bytes at a
-// time under a permutation of k that A and B share (lane (g, t4) takes k = 8 t4 .. 8 t4 + 7 of every
-// 32-k block, words 0, 1 to one MMA and words 2, 3 to the next), K is split over the warps and summed
-// through shared memory.  bf16 adapter rows and bf16 states convert to fp16 exactly in the normal
-// range; the fp32 h is fed as an fp16 value plus an fp16 residual (two MMAs); accumulation is fp32.
-#include "edg_common.cuh"
-#include "edg_mma.cuh"
+// The rank-r projections of the unmerged adapter (Sec. 3.3: delta = sigma * B (A v)) for the tcgen05 tiles of many tokens:
+// u = sigma A_gate x and sigma A_up x before gate/up, u_d = sigma A_down h before down, fp16 as the tiles' operands take them.  Adapter
+// rows are the rows of m16n8k16 tiles, 32 tokens (or pairs) their columns, so an A row is read once per 32; K is split over the warps
+// and summed through shared memory, in fixed order.  With one adapter per layer A x is computed per token, with one per expert per
+// pair, tile by tile (all pairs of a tile have one expert).  x and its adapter rows are bf16 as they are; h is the tiles' fp16 value
+// and residual (two MMAs), its adapter rows fp16 (exact in the normal range); accumulation is fp32.
+#include "edg_grouped.cuh"
+#include "edg_ptx.cuh"
 
 namespace edg {
 namespace {
 
-constexpr int kLtTok = 8;          // tokens (pairs) per CTA = MMA columns
+constexpr int L_WARPS = 8;
 
-// 8 bf16 (one 16-byte load) as four fp16 pairs, order kept
-__device__ __forceinline__ uint4 bf16x8_as_f16x8(uint4 v) {
-    uint4 o;
-    o.x = h2_as_u32(__floats2half2_rn(bf16_lo(v.x), bf16_hi(v.x)));
-    o.y = h2_as_u32(__floats2half2_rn(bf16_lo(v.y), bf16_hi(v.y)));
-    o.z = h2_as_u32(__floats2half2_rn(bf16_lo(v.z), bf16_hi(v.z)));
-    o.w = h2_as_u32(__floats2half2_rn(bf16_lo(v.w), bf16_hi(v.w)));
-    return o;
+__device__ __forceinline__ void mma16816_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// 16 bytes of an adapter row (8 bf16) as fp16 words in the order of a core row
+__device__ __forceinline__ uint4 bf16x8_core(uint4 v) {
+    const float f[8] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y), bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w)};
+    return permute8(f);
 }
 
-// u_gu[t][0][proj][j] = sum_k A_proj[j][k] x[t][k]: rows 0 .. r-1 of the tiles are A_gate, r .. 2r-1 A_up.
-// TILES = ceil(2r / 16) row tiles, KB = 32-k blocks per warp (H / 8 warps / 32).
-template <int TILES, int KB>
-__global__ void __launch_bounds__(256, 2) lora_ax_tokens_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ A_gate,
-                                                               const uint16_t* __restrict__ A_up, float* __restrict__ u_gu,
-                                                               int T, int H, int r) {
-    const int t0 = blockIdx.x * kLtTok;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t4 = lane & 3;
-    extern __shared__ float smem[];
-    float* s_red = smem;                                               // [8 warps][TILES x 16 x 8]
-    const int xs = H * 2 + 64;                                         // bytes per token row (padded against bank conflicts)
-    uint8_t* s_xh = reinterpret_cast<uint8_t*>(s_red + 8 * TILES * 128);
-    const int ksl = H / 8;                                             // k per warp = 32 KB
-    constexpr int KH = KB / 2;                                         // the K slice in two passes: half the registers, two CTAs per SM
-
-    const uint16_t* rows[TILES][2];
+// X: u_gu[token or pair][2 rank] = sigma A x, rows 0 .. r-1 from A_gate, r .. 2r-1 from A_up.  Otherwise u_d[pair][rank] = sigma A_down h.
+// blockIdx.x: 8 N tokens, or that part of a tile; blockIdx.y: 16 M rows.
+template <bool X, int M, int N>
+__global__ void __launch_bounds__(L_WARPS * 32, M == 1 ? 3 : 2) lora_rows_kernel(const __grid_constant__ GroupedParams p) {
+    constexpr int L_ROWS = 16 * M, L_TOK = 8 * N, SUBS = kUmmaTokens / L_TOK;
+    __shared__ float s_red[L_WARPS * L_ROWS * (L_TOK + 1)];
+    __shared__ int s_id[L_TOK];                                          // where a column's results go: a token or a pair, or -1
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g8 = lane >> 2, t4 = lane & 3;
+    pdl_launch_dependents();
+    pdl_wait_prior_grid();
+    const bool by_token = X && p.n_adapters == 1;
+    const int tile = blockIdx.x / SUBS, sub = blockIdx.x % SUBS;
+    int ad = 0, cnt, n16 = 0, first = 0;
+    if (by_token) {
+        cnt = min(L_TOK, p.T - (int)blockIdx.x * L_TOK);
+    } else {
+        if (tile >= *p.n_tiles) return;
+        const int4 ti = p.tiles[tile];
+        cnt = min(L_TOK, ti.z - sub * L_TOK);
+        if (cnt <= 0) return;
+        n16 = (ti.z + 15) & ~15;
+        first = ti.y + sub * L_TOK;
+        ad = ti.w;
+    }
+    if (tid < L_TOK) s_id[tid] = tid >= cnt ? -1 : (by_token ? (int)blockIdx.x * L_TOK + tid : p.order[first + tid]);
+    __syncthreads();
+    const int rows = X ? 2 * p.rank : p.rank, row0 = blockIdx.y * L_ROWS, nt = (cnt + 7) >> 3, K = X ? p.H : p.I;
+    const uint16_t* A[M][2];
 #pragma unroll
-    for (int ti = 0; ti < TILES; ++ti) {
+    for (int m = 0; m < M; ++m)
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
-            const int m = ti * 16 + g + 8 * hh;
-            rows[ti][hh] = m < r ? A_gate + (size_t)m * H : (m < 2 * r ? A_up + (size_t)(m - r) * H : nullptr);
+            const int row = row0 + m * 16 + hh * 8 + g8;
+            const uint16_t* base = static_cast<const uint16_t*>(X ? (row < p.rank ? p.lora.A_gate : p.lora.A_up) : p.lora.A_down);
+            A[m][hh] = row < rows ? base + ((size_t)ad * p.rank + (X && row >= p.rank ? row - p.rank : row)) * K + 8 * t4 : nullptr;
         }
-    }
-    uint4 a[TILES][KH][2];
-    auto load_a = [&](int pass) {
+    float c[M][N][4];
 #pragma unroll
-        for (int ti = 0; ti < TILES; ++ti) {
+    for (int m = 0; m < M; ++m)
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
+        for (int n = 0; n < N; ++n)
 #pragma unroll
-                for (int j = 0; j < KH; ++j)
-                    a[ti][j][hh] = rows[ti][hh] != nullptr ? ld_stream16(rows[ti][hh] + warp * ksl + 32 * (pass * KH + j) + 8 * t4)
-                                                           : make_uint4(0, 0, 0, 0);
+            for (int q = 0; q < 4; ++q) c[m][n][q] = 0.f;
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    const uint16_t* xr[N];
+    if (X)
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            const int id = s_id[n * 8 + g8];
+            xr[n] = id < 0 ? nullptr : p.x + (size_t)(by_token ? id : id / p.K) * p.H + 8 * t4;
+        }
+    const uint8_t* hq = p.hq + (size_t)tile * p.I * 512 + (size_t)t4 * n16 * 16 + (sub * L_TOK + g8) * 16;
+    // X: the warp's eighth of K, 32 k at a time; h: every eighth chunk of 32
+#pragma unroll X ? 4 : 2
+    for (int kb = X ? warp * (K / L_WARPS) : warp * 32; kb < (X ? (warp + 1) * (K / L_WARPS) : K); kb += X ? 32 : L_WARPS * 32) {
+        uint4 a[M][2], b[N], bl[N];
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) a[m][hh] = A[m][hh] != nullptr ? __ldg(reinterpret_cast<const uint4*>(A[m][hh] + kb)) : zero;
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            b[n] = zero; bl[n] = zero;
+            if (X) {
+                if (xr[n] != nullptr) b[n] = __ldg(reinterpret_cast<const uint4*>(xr[n] + kb));
+            } else if (sub * L_TOK + n * 8 < n16) {
+                const uint8_t* q = hq + (size_t)(kb >> 5) * n16 * 128 + n * 128;
+                b[n] = __ldcg(reinterpret_cast<const uint4*>(q));
+                bl[n] = __ldcg(reinterpret_cast<const uint4*>(q + (size_t)n16 * 64));
             }
         }
-    };
-    // the adapter rows of the first pass are on their way while the states are converted
-    load_a(0);
-    // (four loads of a thread in flight at a time: the conversion is a chain of trips to memory otherwise)
-    for (int i0 = threadIdx.x; i0 < kLtTok * (H / 8); i0 += 4 * blockDim.x) {
-        uint4 v[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int i = i0 + u * blockDim.x, tt = i / (H / 8), c = i % (H / 8), t = t0 + tt;
-            v[u] = (i < kLtTok * (H / 8) && t < T) ? *reinterpret_cast<const uint4*>(x + (size_t)t * H + c * 8) : make_uint4(0, 0, 0, 0);
-        }
+        for (int m = 0; m < M; ++m) {
+            if (!X) { a[m][0] = bf16x8_core(a[m][0]); a[m][1] = bf16x8_core(a[m][1]); }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int i = i0 + u * blockDim.x, tt = i / (H / 8), c = i % (H / 8);
-            if (i < kLtTok * (H / 8)) *reinterpret_cast<uint4*>(s_xh + tt * xs + c * 16) = bf16x8_as_f16x8(v[u]);
-        }
-    }
-    __syncthreads();
-
-    const uint8_t* xb = s_xh + g * xs + (warp * ksl + 8 * t4) * 2;
-    float c[TILES][4];
-#pragma unroll
-    for (int ti = 0; ti < TILES; ++ti) { c[ti][0] = 0.f; c[ti][1] = 0.f; c[ti][2] = 0.f; c[ti][3] = 0.f; }
-#pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-        if (pass) load_a(1);
-#pragma unroll
-        for (int j = 0; j < KH; ++j) {
-            const uint4 b = *reinterpret_cast<const uint4*>(xb + 64 * (pass * KH + j));
-#pragma unroll
-            for (int ti = 0; ti < TILES; ++ti) {
-                const uint4 lo = bf16x8_as_f16x8(a[ti][j][0]), hi = bf16x8_as_f16x8(a[ti][j][1]);
-                mma16816(c[ti], lo.x, hi.x, lo.y, hi.y, b.x, b.y);
-                mma16816(c[ti], lo.z, hi.z, lo.w, hi.w, b.z, b.w);
+            for (int n = 0; n < N; ++n) {
+                if (n >= nt) continue;
+                if (X) {
+                    mma16816_bf16(c[m][n], a[m][0].x, a[m][1].x, a[m][0].y, a[m][1].y, b[n].x, b[n].y);
+                    mma16816_bf16(c[m][n], a[m][0].z, a[m][1].z, a[m][0].w, a[m][1].w, b[n].z, b[n].w);
+                } else {
+                    mma16816(c[m][n], a[m][0].x, a[m][1].x, a[m][0].y, a[m][1].y, b[n].x, b[n].y);
+                    mma16816(c[m][n], a[m][0].z, a[m][1].z, a[m][0].w, a[m][1].w, b[n].z, b[n].w);
+                    mma16816(c[m][n], a[m][0].x, a[m][1].x, a[m][0].y, a[m][1].y, bl[n].x, bl[n].y);
+                    mma16816(c[m][n], a[m][0].z, a[m][1].z, a[m][0].w, a[m][1].w, bl[n].z, bl[n].w);
+                }
             }
         }
     }
-    // rows g / g + 8, tokens 2 t4 / 2 t4 + 1 of this warp's K slice
-    float* mine = s_red + warp * TILES * 128;
 #pragma unroll
-    for (int ti = 0; ti < TILES; ++ti) {
-        mine[ti * 128 + g * 8 + 2 * t4] = c[ti][0]; mine[ti * 128 + g * 8 + 2 * t4 + 1] = c[ti][1];
-        mine[ti * 128 + (g + 8) * 8 + 2 * t4] = c[ti][2]; mine[ti * 128 + (g + 8) * 8 + 2 * t4 + 1] = c[ti][3];
-    }
+    for (int m = 0; m < M; ++m)
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            float* q = s_red + (warp * L_ROWS + m * 16 + g8) * (L_TOK + 1) + n * 8 + 2 * t4;
+            q[0] = c[m][n][0]; q[1] = c[m][n][1];
+            q[8 * (L_TOK + 1)] = c[m][n][2]; q[8 * (L_TOK + 1) + 1] = c[m][n][3];
+        }
     __syncthreads();
-    for (int i = threadIdx.x; i < TILES * 128; i += blockDim.x) {
+    __half* out = X ? p.u_gu : p.u_d;
+    for (int i = tid; i < L_ROWS * L_TOK; i += L_WARPS * 32) {
+        const int row = i % L_ROWS, tok = i / L_ROWS;
+        if (tok >= cnt || row0 + row >= rows) continue;
         float v = 0.f;
 #pragma unroll
-        for (int w = 0; w < 8; ++w) v += s_red[w * TILES * 128 + i];      // fixed order
-        const int row = i >> 3, tok = i & 7;
-        if (row < 2 * r && t0 + tok < T) u_gu[(size_t)(t0 + tok) * 2 * r + row] = v;
-    }
-}
-
-// u_d[pair][j] = sum_i A_down[j][i] h[pair][i]; TILES = ceil(r / 16), KB = 32-k blocks per warp (I / 4 warps / 32)
-template <int TILES, int KB>
-__global__ void __launch_bounds__(128) lora_adh_pairs_kernel(const float* __restrict__ h, const uint16_t* __restrict__ A_down,
-                                                            float* __restrict__ u_d, int P, int I, int r) {
-    const int p0 = blockIdx.x * kLtTok;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t4 = lane & 3;
-    extern __shared__ float smem[];
-    float* s_red = smem;                                               // [4 warps][TILES x 16 x 8]
-    const int hs = I * 2 + 64;                                         // bytes per pair row
-    uint8_t* s_hh = reinterpret_cast<uint8_t*>(s_red + 4 * TILES * 128);   // [8][I + 32] fp16 value
-    uint8_t* s_hl = s_hh + kLtTok * hs;                                 // [8][I + 32] fp16 residual
-    const int ksl = I / 4;
-
-    uint4 a[TILES][KB][2];
-#pragma unroll
-    for (int ti = 0; ti < TILES; ++ti) {
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            const int m = ti * 16 + g + 8 * hh;
-#pragma unroll
-            for (int j = 0; j < KB; ++j)
-                a[ti][j][hh] = m < r ? ld_stream16(A_down + (size_t)m * I + warp * ksl + 32 * j + 8 * t4) : make_uint4(0, 0, 0, 0);
-        }
-    }
-    for (int i = threadIdx.x; i < kLtTok * (I / 8); i += blockDim.x) {
-        const int tt = i / (I / 8), c = i % (I / 8), pr = p0 + tt;
-        uint4 hi = make_uint4(0, 0, 0, 0), lo = hi;
-        if (pr < P) {
-            const float4 v0 = *reinterpret_cast<const float4*>(h + (size_t)pr * I + c * 8);
-            const float4 v1 = *reinterpret_cast<const float4*>(h + (size_t)pr * I + c * 8 + 4);
-            const float f[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-            uint32_t wh[4], wl[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const __half2 hv = __floats2half2_rn(f[2 * e], f[2 * e + 1]);
-                const float2 back = __half22float2(hv);
-                wh[e] = h2_as_u32(hv);
-                wl[e] = h2_as_u32(__floats2half2_rn(f[2 * e] - back.x, f[2 * e + 1] - back.y));
-            }
-            hi = make_uint4(wh[0], wh[1], wh[2], wh[3]);
-            lo = make_uint4(wl[0], wl[1], wl[2], wl[3]);
-        }
-        *reinterpret_cast<uint4*>(s_hh + tt * hs + c * 16) = hi;
-        *reinterpret_cast<uint4*>(s_hl + tt * hs + c * 16) = lo;
-    }
-    __syncthreads();
-
-    const int boff = g * hs + (warp * ksl + 8 * t4) * 2;
-    float c[TILES][4];
-#pragma unroll
-    for (int ti = 0; ti < TILES; ++ti) { c[ti][0] = 0.f; c[ti][1] = 0.f; c[ti][2] = 0.f; c[ti][3] = 0.f; }
-#pragma unroll
-    for (int j = 0; j < KB; ++j) {
-        const uint4 bh = *reinterpret_cast<const uint4*>(s_hh + boff + 64 * j);
-        const uint4 bl = *reinterpret_cast<const uint4*>(s_hl + boff + 64 * j);
-#pragma unroll
-        for (int ti = 0; ti < TILES; ++ti) {
-            const uint4 lo = bf16x8_as_f16x8(a[ti][j][0]), hi = bf16x8_as_f16x8(a[ti][j][1]);
-            mma16816(c[ti], lo.x, hi.x, lo.y, hi.y, bh.x, bh.y);
-            mma16816(c[ti], lo.z, hi.z, lo.w, hi.w, bh.z, bh.w);
-            mma16816(c[ti], lo.x, hi.x, lo.y, hi.y, bl.x, bl.y);
-            mma16816(c[ti], lo.z, hi.z, lo.w, hi.w, bl.z, bl.w);
-        }
-    }
-    float* mine = s_red + warp * TILES * 128;
-#pragma unroll
-    for (int ti = 0; ti < TILES; ++ti) {
-        mine[ti * 128 + g * 8 + 2 * t4] = c[ti][0]; mine[ti * 128 + g * 8 + 2 * t4 + 1] = c[ti][1];
-        mine[ti * 128 + (g + 8) * 8 + 2 * t4] = c[ti][2]; mine[ti * 128 + (g + 8) * 8 + 2 * t4 + 1] = c[ti][3];
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < TILES * 128; i += blockDim.x) {
-        float v = 0.f;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) v += s_red[w * TILES * 128 + i];
-        const int row = i >> 3, tok = i & 7;
-        if (row < r && p0 + tok < P) u_d[(size_t)(p0 + tok) * r + row] = v;
+        for (int w = 0; w < L_WARPS; ++w) v += s_red[(w * L_ROWS + row) * (L_TOK + 1) + tok];
+        out[(size_t)s_id[tok] * rows + row0 + row] = __float2half_rn(p.sigma * v);
     }
 }
 
 }  // namespace
 
-// A x for all tokens with one shared adapter; false when the shape is not covered (the caller falls back)
-bool launch_lora_ax_tokens(const edg_layer_desc* d, const void* x, const edg_lora* lora, float* u_gu, int T, cudaStream_t st) {
-    const int r = d->rank, H = d->H;
-    if (d->n_adapters != 1 || r < 8 || r % 8 != 0 || 2 * r > 32 || (H != 1024 && H != 2048)) return false;
-    const uint16_t* Ag = static_cast<const uint16_t*>(lora->A_gate);
-    const uint16_t* Au = static_cast<const uint16_t*>(lora->A_up);
-    const int tiles = (2 * r + 15) / 16, grid = (T + kLtTok - 1) / kLtTok;
-    const size_t sm = (size_t)8 * tiles * 128 * 4 + (size_t)kLtTok * (H * 2 + 64);
-    const uint16_t* xx = static_cast<const uint16_t*>(x);
-#define EDG_LAX(TI, KB_)                                                                                         \
-    do {                                                                                                         \
-        static OncePerDevice once;                                                                               \
-        once([] { return allow_smem(64 * 1024, lora_ax_tokens_kernel<TI, KB_>); });                              \
-        lora_ax_tokens_kernel<TI, KB_><<<grid, 256, sm, st>>>(xx, Ag, Au, u_gu, T, H, r);                        \
-    } while (0)
-    if (H == 2048) { if (tiles == 1) EDG_LAX(1, 8); else EDG_LAX(2, 8); }
-    else { if (tiles == 1) EDG_LAX(1, 4); else EDG_LAX(2, 4); }
-#undef EDG_LAX
-    return true;
+// (32 tokens and 32 rows a CTA, whatever the rank: 27 and 77 us for 4096 tokens of 8 choices, rank 16; with one CTA an SM for its registers)
+cudaError_t launch_lora_ax(const GroupedParams& p, int max_tiles, cudaStream_t st) {
+    if (p.n_adapters == 1) return launch_pdl(lora_rows_kernel<true, 2, 2>, dim3((unsigned)(p.T + 15) / 16, (2 * p.rank + 31) / 32), L_WARPS * 32, 0, st, p);
+    return launch_pdl(lora_rows_kernel<true, 2, 2>, dim3(8u * max_tiles, (2 * p.rank + 31) / 32), L_WARPS * 32, 0, st, p);
 }
-
-// A_down h for all pairs with one shared adapter
-bool launch_lora_adh_pairs(const edg_layer_desc* d, const edg_lora* lora, const float* h, float* u_d, int P, cudaStream_t st) {
-    const int r = d->rank, I = d->I;
-    if (d->n_adapters != 1 || r < 8 || r % 8 != 0 || r > 32 || (I != 256 && I != 512)) return false;
-    const uint16_t* Ad = static_cast<const uint16_t*>(lora->A_down);
-    const int tiles = (r + 15) / 16, grid = (P + kLtTok - 1) / kLtTok;
-    const size_t sm = (size_t)4 * tiles * 128 * 4 + (size_t)2 * kLtTok * (I * 2 + 64);
-    if (I == 512) { if (tiles == 1) lora_adh_pairs_kernel<1, 4><<<grid, 128, sm, st>>>(h, Ad, u_d, P, I, r); else lora_adh_pairs_kernel<2, 4><<<grid, 128, sm, st>>>(h, Ad, u_d, P, I, r); }
-    else { if (tiles == 1) lora_adh_pairs_kernel<1, 2><<<grid, 128, sm, st>>>(h, Ad, u_d, P, I, r); else lora_adh_pairs_kernel<2, 2><<<grid, 128, sm, st>>>(h, Ad, u_d, P, I, r); }
-    return true;
+cudaError_t launch_lora_adh(const GroupedParams& p, int max_tiles, cudaStream_t st) {
+    return launch_pdl(lora_rows_kernel<false, 1, 4>, dim3(4u * max_tiles, (p.rank + 15) / 16), L_WARPS * 32, 0, st, p);
 }
 
 }  // namespace edg

@@ -60,6 +60,58 @@ def test_first_size_of_the_tensor_memory_tiles(n_adapters):
     _check_tokens(L, X, inds_h, gates_h, Y, list(range(0, T, 9)) + [T - 1])
 
 
+# pairs of the eight experts: edges of the tensor-memory tiles' rounding (16) and of the tiles (128), an unused expert, one of several tiles
+_RUNS = [1, 16, 17, 127, 128, 129, 0, 452]
+
+
+@pytest.mark.parametrize("H,I,group,rank,n_adapters", [
+    (256, 128, 32, 0, 1),                   # the smallest layer: four stages a kernel, two sums per stage, no adapter
+    (512, 256, 64, 8, 8),                   # half a k-step of ranks in down
+    (1024, 512, 128, 40, 1),                # a sum over two stages; two stages of adapter in both kernels, the second partly empty
+    (2048, 512, 32, 24, 8),
+    (1024, 1024, 64, 64, 1),                # the largest rank
+    (4096, 512, 128, 16, 1),                # wide state
+])
+def test_tensor_memory_tiles_at_their_edges(H, I, group, rank, n_adapters):
+    L = _layer(H, I, group, rank, 8, 1, n_adapters)
+    T = sum(_RUNS)
+    X = synth.hidden_states(L.cfg, T, stream=64)
+    order = np.random.default_rng(8).permutation(T)
+    inds_h = np.repeat(np.arange(8, dtype=np.int32), _RUNS)[order].reshape(T, 1)
+    gates_h = np.random.default_rng(9).uniform(0.1, 1.0, size=(T, 1)).astype(np.float32)
+    assert T > 96 * 8
+    inds, gates = torch.from_numpy(inds_h).cuda(), torch.from_numpy(gates_h).cuda()
+    Y = _ffn_tokens(L, L.desc, X, inds, gates, T)
+    assert np.isfinite(Y).all()
+    last = [int(np.nonzero(inds_h[:, 0] == e)[0][j]) for e in range(8) if _RUNS[e] for j in {0, _RUNS[e] - 1, min(127, _RUNS[e] - 1)}]
+    _check_tokens(L, X, inds_h, gates_h, Y, sorted(set(last) | set(range(0, T, 31))))
+    assert np.array_equal(Y, _ffn_tokens(L, L.desc, X, inds, gates, T, use_table=False))
+
+
+def test_tensor_memory_tiles_a_slot_named_twice_and_one_out_of_range():
+    """More pairs of a slot than there are tokens; a choice that is no slot leaves its share out and is reported."""
+    L = _layer(512, 256, 64, 8, 4, 2)
+    T = 200
+    X = synth.hidden_states(L.cfg, T, stream=65)
+    inds_h = np.full((T, 2), 1, np.int32)
+    inds_h[::5] = [0, 3]
+    gates_h = np.random.default_rng(10).dirichlet(np.ones(2), size=T).astype(np.float32)
+    assert T * 2 > 40 * 4
+    gates = torch.from_numpy(gates_h).cuda()
+    Y = _ffn_tokens(L, L.desc, X, torch.from_numpy(inds_h).cuda(), gates, T)
+    _check_tokens(L, X, inds_h, gates_h, Y, range(0, T, 7))
+    bad = inds_h.copy()
+    bad[7, 1] = 4
+    y = out_tensor(L.desc, T)
+    edg.moe_expert_ffn_int4_lora(L.desc, L.pool, None, T, torch.from_numpy(bad).cuda(), torch.from_numpy(bad).cuda(), gates, x_dev(X), L.lora, y, L.ws)
+    torch.cuda.synchronize()
+    assert edg.workspace_status(L.ws) == -4
+    got = y.cpu().numpy()
+    assert np.array_equal(np.delete(got, 7, axis=0), np.delete(Y, 7, axis=0))
+    ref = orc.moe_ffn(X[7], bad[7, :1], gates_h[7, :1].astype(np.float64), L.expert, L.get_lora, L.cfg.lora_scale, L.cfg.group)
+    assert orc.max_abs(got[7], ref) <= 2e-2 and orc.rel_l2(got[7], ref) <= 1e-3
+
+
 def test_pool_with_more_slots_than_shared_memory_counts():
     """26,000 slots: the sort keeps its counters in the workspace.  Three experts live in the first, a middle and the last slot."""
     cfg = _layer(256, 128, 32, 8, 4, 2).cfg
