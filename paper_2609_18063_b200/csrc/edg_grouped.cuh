@@ -48,20 +48,4 @@ cudaError_t launch_sum_choices(const GroupedParams& p, cudaStream_t st);
 cudaError_t launch_lora_ax(const GroupedParams& p, int max_tiles, cudaStream_t st);
 cudaError_t launch_lora_adh(const GroupedParams& p, int max_tiles, cudaStream_t st);
 
-// a launch that may begin while the kernel before it runs (it waits for its end by itself)
-template <typename... Params, typename... Args>
-cudaError_t launch_pdl(void (*kern)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 }  // namespace edg
