@@ -245,6 +245,7 @@ struct FusedExtras {
     int dep_wait = -1;                     // ring slot whose flag announces this step's x (chained dependent steps)
     const void* shared_rec = nullptr;      // device record of the layer's shared expert: runs as one more expert with gate 1
     const edg_lora* shared_lora = nullptr; // its adapter (leading dimension 1), or null
+    int run = 0;                           // 1: steps that need nothing of this one follow it; 2: this step needs nothing of the one before it
     bool slot_until_end = false;           // the step before is of the latency form: it writes to the ring slot it hands on until it ends
 };
 

@@ -20,7 +20,9 @@
 //   * A dependent chain hands x + y on, unnormalised, in band as well: every CTA of the next step, resident and
 //     with its weights in shared memory by then, polls it, forms the norm and its bf16 state by itself.  Eight copies: 148
 //     pollers of the same lines held the writes up by 2-4 us.  A CTA without expert work writes the caller's x_next meanwhile.
-// Two launches of this form fit an SM side by side (64 registers x 512 threads, under 113 KB of shared memory).
+// Two launches of this form fit an SM side by side (64 registers x 512 threads, under 113 KB of shared memory).  So do two steps that need
+// nothing of one another (the layers of a token whose inputs are all given): such a run waits for what came before it once, in its first
+// step; the others start beside their predecessor and leave after it.
 //
 // Measured (H 2048, I 512, E 256, K 8, groups of 64, rank 16; the four-CTA clusters per expert quarter it replaces first): a link of
 // a chain 20.4 -> 12.1 us, a step alone 24 -> 14.1 us (12 layers of K = 4 through the resident stack, host loop included: 295 -> 154 us).
@@ -85,6 +87,7 @@ struct StepParams {
     int n_gu, n_dn, n_exp, n_head, n_headc;   // CTAs with gate/up, with down work, the larger of both; tiles of the head, CTAs for them
     int head_tile;                            // rows of a tile of the head
     int flag_in, flag_out, dep;               // dep: x arrives in band from the step before
+    int run;                                  // of independent steps: 1 begins one, 2 goes on with it
     float sigma, eps;
     RecordLayout L;
     StepSmem S;
@@ -221,7 +224,7 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         return hx + p.ux_off + (size_t)set * 8 * p.rmax + (q & 3) * 2 * p.rmax + (q >> 2);
     };
     // ---- start (warp 1): count this CTA in, let the next kernel come; "not yet" into every word this CTA will publish, and say so
-    const bool links = p.flag_in >= 0 || p.flag_out >= 0;                // the next kernel may be a link that does not wait for this one's end
+    const bool links = p.flag_in >= 0 || p.flag_out >= 0 || p.run != 0;  // the next kernel may be one that does not wait for this one's end
     if (tid == 32) {
         uint32_t old;
         asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(p.starts) : "memory");
@@ -236,7 +239,8 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         s_misc[1] = last ? 1 : 0;
         if (!links) pdl_launch_dependents();
     }
-    if (p.flag_in < 0) pdl_wait_prior_grid();                            // a step on its own: everything queued before it has happened
+    // a step on its own: everything queued before it has happened (of a run of independent steps the first has seen to that)
+    if (p.flag_in < 0 && p.run != 2) pdl_wait_prior_grid();
     if (warp == 1) {
         const uint4 none = make_uint4(kNotYet, kNotYet, kNotYet, kNotYet);
         if (has_gu) {
@@ -915,6 +919,8 @@ __global__ void __launch_bounds__(TThreads, 2) step_kernel(const __grid_constant
         __syncthreads();
         if (unit < 0) break;
     }
+    // ---- independent steps complete in order, too, and for the reason given below: none meets the step four before it in their buffer
+    if (p.run == 2) pdl_wait_prior_grid();
     // ---- a link of a chain: the last CTA to have read the routing resets its ring slot; kernels of a chain complete in order
     if (p.flag_in >= 0) {
         // No CTA leaves before the kernel before this one has: the CTAs of the next one but one take over from that kernel, one on
@@ -992,7 +998,7 @@ cudaError_t launch_step(const StepParams& p, int grid, cudaStream_t st) {
     // A step that does not start a chain asks for more than half an SM: with two such launches in flight, the CTAs of one that find an
     // SM free twice would share it (30 SMs of 148 did, once started so: 17.4 us a step instead of 14.4; without the
     // programmatic launch, 17.3).
-    cfg.dynamicSmemBytes = p.flag_in < 0 && p.x_next == nullptr && grid <= sm_count() ? max(p.S.total, (uint32_t)kStepSmemLone) : p.S.total;
+    cfg.dynamicSmemBytes = p.flag_in < 0 && p.x_next == nullptr && p.run == 0 && grid <= sm_count() ? max(p.S.total, (uint32_t)kStepSmemLone) : p.S.total;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1080,6 +1086,7 @@ int32_t run_step(const edg_layer_desc* d, const void* slot_pool, const int32_t* 
     p.cta_route = W_pre == nullptr ? -1 : (idle < grid ? idle : idle - 1);
     p.cta_state = p.x_next == nullptr ? -1 : (W_pre == nullptr ? p.n_exp : (idle + 1 < grid ? idle + 1 : p.n_exp));
     p.flag_in = flag_in; p.flag_out = W_pre != nullptr ? flag_out : -1;
+    p.run = flag_in < 0 && ex.x_next == nullptr ? ex.run : 0;
     p.dep = flag_in >= 0 && ex.dep_wait >= 0;
     p.S = step_smem(*d, p.Kt, p.rmax);
     const cudaError_t e = d->H == 2048 ? (d->I == 512 ? launch_shape<4, 4>(p, grid, st) : launch_shape<4, 2>(p, grid, st))

@@ -67,3 +67,71 @@ def test_stack_decode_matches_oracle(n_slots, prefetch):
         eos, soe = store.snapshot(l)
         assert eos.tolist() == allocs[l].expert_of_slot and soe.tolist() == allocs[l].slot_of_expert
     store.close()
+
+
+def _resident_stack(cfg, n_layers, stream):
+    """A store of resident layers, its decoder's heads, and per-layer inputs of a few tokens."""
+    d = edg.make_desc(cfg, n_slots=cfg.E)
+    host = layer_io.host_layer(d, lambda e: synth.expert_tensors(cfg, 0, e))
+    slots = torch.zeros((n_layers, cfg.E, edg.record_bytes(d)), dtype=torch.uint8, device="cuda")
+    tables = torch.zeros((n_layers, cfg.E), dtype=torch.int32, device="cuda")
+    loras, keep = zip(*[layer_io.lora_to_device(d, [synth.lora_tensors(cfg, l, a) for a in range(cfg.n_adapters)]) for l in range(n_layers)])
+    store = edg.Store(d, [host] * n_layers, slots, tables, list(loras), torch.cuda.Stream())
+    for l in range(n_layers):
+        store.load_whole_layer(l)
+        store.wait_staged(l)
+    W = torch.from_numpy(np.stack([synth.prerouter_weights(cfg, l) for l in range(n_layers)])).cuda()
+    X = layer_io.bits_to_device(np.stack([synth.hidden_states(cfg, 9, layer=l, stream=stream) for l in range(n_layers)], axis=1), torch.bfloat16)
+    torch.cuda.synchronize()
+    return d, store, W, X, (slots, tables, keep)
+
+
+@pytest.mark.parametrize("name,kw,n_layers", [
+    ("cfg1", {}, 7),                                            # more layers than a workspace has exchange buffers, fp32 head
+    ("cfg2", dict(E=32, K=4, n_slots=32), 6),
+    ("cfg2", dict(E=32, K=8, n_slots=32, n_adapters=32), 3),    # all SMs in gate/up, an adapter per expert
+    ("cfg2", dict(E=32, K=12, n_slots=32, rank=0), 5),          # more CTAs than SMs
+])
+def test_layers_of_a_token_side_by_side_are_the_layer_steps(name, kw, n_layers):
+    """Resident layers run beside one another; every output is that of one moe_layer_decode after the other, bit for bit, with two
+    stacks at once on two streams as well."""
+    cfg = synth.CONFIGS[name].with_(**kw)
+    stacks = [_resident_stack(cfg, n_layers, 71 + i) for i in range(2)]
+    want = []
+    for d, store, W, X, _ in stacks:
+        ref = StackDecoder(d, store, W)
+        ref.prime(X[8])
+        rows = []
+        for t in range(8):
+            cur, nxt = t % 2, (t + 1) % 2
+            y, lg = torch.zeros((n_layers, cfg.H), device="cuda"), torch.zeros((n_layers, cfg.E), device="cuda")
+            for l in range(n_layers):
+                n = (l + 1) % n_layers
+                edg.moe_layer_decode(store, l, X[t, l], ref.inds[cur, l], ref.gates[cur, l], W[l], ref.inds[nxt, n], ref.gates[nxt, n], lg[n], y[l], ref.ws)
+            rows.append((y, lg, ref.inds[nxt].clone(), ref.gates[nxt].clone()))
+        torch.cuda.synchronize()
+        assert edg.workspace_status(ref.ws) == 0
+        want.append(rows)
+    for both in (False, True):
+        decs, got = [], [[], []]
+        for d, store, W, X, _ in stacks:
+            decs.append(StackDecoder(d, store, W))
+            decs[-1].prime(X[8])
+        streams = [torch.cuda.Stream() for _ in stacks]
+        torch.cuda.synchronize()
+        for t in range(8):
+            for i, (d, store, W, X, _) in enumerate(stacks):
+                if i == 1 and not both:
+                    continue
+                with torch.cuda.stream(streams[i]):
+                    y, lg = torch.zeros((n_layers, cfg.H), device="cuda"), torch.zeros((n_layers, cfg.E), device="cuda")
+                    decs[i].step(t, X[t], y, lg)
+                    got[i].append((y, lg, decs[i].inds[(t + 1) % 2].clone(), decs[i].gates[(t + 1) % 2].clone()))
+        torch.cuda.synchronize()
+        for i in range(1 + both):
+            assert edg.workspace_status(decs[i].ws) == 0
+            for t in range(8):
+                for a, b in zip(got[i][t], want[i][t]):
+                    assert torch.equal(a, b), (i, t)
+    for _, store, _, _, _ in stacks:
+        store.close()
