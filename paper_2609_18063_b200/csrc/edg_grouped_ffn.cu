@@ -4,7 +4,8 @@
 //
 // A call is four kernels, launched as programmatic dependents of one another:
 //   group_pairs_kernel    one CTA: resolves every pair's slot, sorts the pairs by slot (stable, so a second run is
-//                         bit-identical) and cuts each slot's run into tiles of up to `cap` pairs
+//                         bit-identical) and cuts each slot's run into tiles of up to `cap` pairs; up to 128 pairs the next
+//                         kernel's CTAs do that, each for its tile
 //   tile_operands_kernel  per tile: the tokens' states as fp16 B words in the order the ring stages read them, and the
 //                         adapter projections sigma A_gate x, sigma A_up x (bf16 MMA, fp32 sums)
 //   grouped_ffn_kernel    see below
@@ -15,7 +16,8 @@
 // has a ring of stages of its own, a producer lane that feeds it and a warp for the rank-r projections of h.  Work
 // units come from a ticket counter (all gate/up units of all tiles, then all down units), so ragged tiles balance
 // themselves and the weights of the first down units are on their way while the last gate/up units are computed:
-//   gate/up unit: 8 row tiles (16 rows each) of gate and of up, one per warp, over all of K = H;
+//   gate/up unit: 8 row tiles (16 rows each) of gate and of up, one per warp, over all of K = H (with few tiles: 4, a warp for each
+//                 of gate and of up);
 //   down unit:    16 row tiles of the output, two per warp, over all of K = I.
 // A stage is 128 k for every warp of a group: its codes are ONE tensor copy of 16 KB (the record's tile-major sections seen
 // as an array of runs, row tiles, matrices or column slices, and slots), the (scale, zero) pairs one more (2 KB at groups
@@ -28,11 +30,14 @@
 // Measured (B200, H 2048, I 512, 256 experts, top 8, groups of 64, rank 16; the whole call with its routing), against the
 // kernels before it (clusters of 4 CTAs x 4 warps with sixteen copies per 36 KB, five barriers an item and
 // eight launches; above 8 pairs per slot the tcgen05 path):
-//   5 tokens  80 -> 62 us a layer, 64 tokens 195 -> 134 us (3.6 TB/s in the kernel), 333 tokens 580 -> 250 us.
+//   5 tokens  80 -> 62 us a layer, 64 tokens 195 -> 134 us (3.6 TB/s in the kernel), 333 tokens 580 -> 250 us;
+// then, with narrow units and without the kernel that sorts where there are few pairs, 5 tokens 59 -> 46, 2 tokens 53 -> 41.
 // With the arithmetic left out the 64-token kernel takes 80 of its 109 us, with the copies left out 100: what bounds it now
 // is the issue rate of sixteen warps (nine instructions per eight codes) next to the memory system.  Three groups of
 // eight warps (72 registers) lose more to spills than they gain (113 us).
 #include <cuda.h>
+
+#include <cmath>
 
 #include "edg_grouped.cuh"
 #include "edg_ptx.cuh"
@@ -73,6 +78,7 @@ struct GffnParams {
     int sp, cps, csh;             // down: slices per stage, 32-code chunks of a stage in one slice, log2 of that
     float sigma;
     int evict_first;
+    int rows1;                    // row tiles of gate and of up in a unit: 8, or 4
     GffnSmem S;
 };
 
@@ -105,17 +111,17 @@ struct WarpRuns {
 };
 
 // one stage: acc[m][nt] += W_m[16 rows x 128 k] . act[128 k x 8 tokens]; LO: act carries values and residuals
-template <int NT, int CPB, bool LO>
-__device__ __forceinline__ void mma_stage(float (&acc)[2][NT][4], const uint8_t* st, const WarpRuns& R, const uint8_t* act, int gshift) {
+template <int NT, int CPB, bool LO, int NM>
+__device__ __forceinline__ void mma_stage(float (&acc)[NM][NT][4], const uint8_t* st, const WarpRuns& R, const uint8_t* act, int gshift) {
     const int lane = threadIdx.x & 31, g8 = lane >> 2, t4 = lane & 3;
     const uint32_t lane_c = g8 * 16 + t4 * 4, lane_b = g8 * 64 + t4 * 16;
     constexpr int kTok = 8 * NT * 64;              // bytes of one chunk of token words
 #pragma unroll NT == 1 ? 4 / CPB : 1
     for (int b = 0; b < 4 / CPB; ++b) {
-        float sf[2][2];
-        __half2 mz[2][2];
+        float sf[NM][2];
+        __half2 mz[NM][2];
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
+        for (int m = 0; m < NM; ++m) {
             const int i = b * CPB, part = i >> R.csh, gi = ((i - (part << R.csh)) * 32) >> gshift;
             const uint8_t* z = st + R.sz[m] + part * R.sz_part + gi * 64 + g8 * 4;
 #pragma unroll
@@ -125,12 +131,12 @@ __device__ __forceinline__ void mma_stage(float (&acc)[2][NT][4], const uint8_t*
                 mz[m][hh] = neg_zero_x(v);
             }
         }
-        uint32_t a[CPB][2][2][4];
+        uint32_t a[CPB][NM][2][4];
 #pragma unroll
         for (int u = 0; u < CPB; ++u) {
             const int i = b * CPB + u, part = i >> R.csh;
 #pragma unroll
-            for (int m = 0; m < 2; ++m) {
+            for (int m = 0; m < NM; ++m) {
                 const uint8_t* w = st + R.code[m] + part * R.code_part + (i - (part << R.csh)) * 256 + lane_c;
                 dequant_word_x(*reinterpret_cast<const uint32_t*>(w), mz[m][0], a[u][m][0]);
                 dequant_word_x(*reinterpret_cast<const uint32_t*>(w + 128), mz[m][1], a[u][m][1]);
@@ -138,7 +144,7 @@ __device__ __forceinline__ void mma_stage(float (&acc)[2][NT][4], const uint8_t*
         }
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
-            float c[2][4];
+            float c[NM][4];
 #pragma unroll
             for (int u = 0; u < CPB; ++u) {
                 const uint8_t* bp = act + (LO ? 2 : 1) * (b * CPB + u) * kTok + nt * 512 + lane_b;
@@ -146,16 +152,16 @@ __device__ __forceinline__ void mma_stage(float (&acc)[2][NT][4], const uint8_t*
                 for (int lo = 0; lo < (LO ? 2 : 1); ++lo) {
                     const uint4 v = *reinterpret_cast<const uint4*>(bp + lo * kTok);
 #pragma unroll
-                    for (int m = 0; m < 2; ++m) {
+                    for (int m = 0; m < NM; ++m) {
                         if (u == 0 && lo == 0) mma16816_zero(c[m], a[u][m][0][0], a[u][m][1][0], a[u][m][0][1], a[u][m][1][1], v.x, v.y);
                         else mma16816(c[m], a[u][m][0][0], a[u][m][1][0], a[u][m][0][1], a[u][m][1][1], v.x, v.y);
                     }
 #pragma unroll
-                    for (int m = 0; m < 2; ++m) mma16816(c[m], a[u][m][0][2], a[u][m][1][2], a[u][m][0][3], a[u][m][1][3], v.z, v.w);
+                    for (int m = 0; m < NM; ++m) mma16816(c[m], a[u][m][0][2], a[u][m][1][2], a[u][m][0][3], a[u][m][1][3], v.z, v.w);
                 }
             }
 #pragma unroll
-            for (int m = 0; m < 2; ++m) {
+            for (int m = 0; m < NM; ++m) {
                 fma2(acc[m][nt][0], acc[m][nt][1], sf[m][0], c[m][0], c[m][1]);
                 fma2(acc[m][nt][2], acc[m][nt][3], sf[m][1], c[m][2], c[m][3]);
             }
@@ -195,20 +201,20 @@ struct Gffn {
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[rp.st]);
     }
-    template <int NT>
-    static __device__ __forceinline__ void clear(float (&acc)[2][NT][4]) {
+    template <int NT, int NM>
+    static __device__ __forceinline__ void clear(float (&acc)[NM][NT][4]) {
 #pragma unroll
-        for (int m = 0; m < 2; ++m)
+        for (int m = 0; m < NM; ++m)
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
                 for (int q = 0; q < 4; ++q) acc[m][nt][q] = 0.f;
     }
     // the MMA has seen (q - z) * 2^-9
-    template <int NT>
-    static __device__ __forceinline__ void unscale(float (&acc)[2][NT][4]) {
+    template <int NT, int NM>
+    static __device__ __forceinline__ void unscale(float (&acc)[NM][NT][4]) {
 #pragma unroll
-        for (int m = 0; m < 2; ++m)
+        for (int m = 0; m < NM; ++m)
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -226,7 +232,7 @@ struct Gffn {
     __device__ __forceinline__ void gate_up(int tile, int sub, int ad, RingPos& rp) {
         const int row0 = (sub * GW + warp) * 16;
         float acc[2][NT][4];
-        clear<NT>(acc);
+        clear(acc);
         // the adapter's operands (first 16 ranks) are asked for now and used behind the main loop, where registers allow it
         const bool lora = p.rank > 0 && row0 < p.I;
         constexpr bool ahead = NT <= 2;
@@ -262,7 +268,7 @@ struct Gffn {
             rp.next(p.S.stages);
         }
         if (row0 >= p.I) return;                                         // (the last unit of a narrow layer)
-        unscale<NT>(acc);
+        unscale(acc);
         if (lora) {
             if (!ahead) lora_load();
 #pragma unroll
@@ -282,15 +288,21 @@ struct Gffn {
                 }
             }
         }
-        // h of 16 rows x 8 tokens through the warp's own shared memory: lane = (token, 8 rows, value / residual)
+        store_h<NT>(tile, row0, [&](int nt, int q) { return silu_f(acc[0][nt][q]) * acc[1][nt][q]; });
+    }
+
+    // h of 16 rows and the tile's tokens to global in operand order; value(nt, q): what this lane holds of it, as the accumulators lie
+    template <int NT, typename V>
+    __device__ __forceinline__ void store_h(int tile, int row0, V value) {
+        // 16 rows x 8 tokens through the warp's own shared memory: lane = (token, 8 rows, value / residual)
         float* hs = reinterpret_cast<float*>(smem + p.S.h) + warp * (8 * 20);
         const int tok = lane >> 2, r8 = (lane >> 1) & 1, lo = lane & 1, n = row0 + r8 * 8, c = n >> 5;
         uint8_t* dst = p.hq + (size_t)tile * p.cap * p.I * 4 + ((size_t)(c * 2 + lo) * (8 * NT) + tok) * 64 + ((n & 31) >> 3) * 16;
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
             float* q = hs + (2 * t4) * 20 + g8;
-            q[0] = silu_f(acc[0][nt][0]) * acc[1][nt][0]; q[20] = silu_f(acc[0][nt][1]) * acc[1][nt][1];
-            q[8] = silu_f(acc[0][nt][2]) * acc[1][nt][2]; q[28] = silu_f(acc[0][nt][3]) * acc[1][nt][3];
+            q[0] = value(nt, 0); q[20] = value(nt, 1);
+            q[8] = value(nt, 2); q[28] = value(nt, 3);
             __syncwarp();
             const float4 va = *reinterpret_cast<const float4*>(hs + tok * 20 + r8 * 8), vb = *reinterpret_cast<const float4*>(hs + tok * 20 + r8 * 8 + 4);
             const float f[8] = {va.x, va.y, va.z, va.w, vb.x, vb.y, vb.z, vb.w};
@@ -303,12 +315,59 @@ struct Gffn {
         if (lane == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.done + tile) : "memory");
     }
 
+    // ---- gate/up, narrow units (a column of 8 pairs): four row tiles, a warp for each of gate and of up; the up warp hands its sums over
+    template <int CPB>
+    __device__ __forceinline__ void gate_up_narrow(int tile, int sub, int ad, RingPos& rp) {
+        const int rt = warp >> 1, m = warp & 1, row0 = (sub * (GW / 2) + rt) * 16;
+        float acc[1][1][4];
+        clear(acc);
+        const uint16_t* B = static_cast<const uint16_t*>(m ? p.lora.B_up : p.lora.B_gate) + ((size_t)ad * p.I + row0 + g8) * p.rank;
+        const __half* u = p.u + ((size_t)tile * 2 + m) * p.cap * p.r16 + (size_t)g8 * p.r16 + 2 * t4;
+        uint32_t lb[4], lu[2];
+        if (p.rank > 0) {                                                // (first 16 ranks: asked for now, used behind the main loop)
+            lora_rows(B, 0, lb);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) lu[q] = __ldg(reinterpret_cast<const uint32_t*>(u + 8 * q));
+        }
+        WarpRuns R;
+        R.code[0] = R.code[1] = (uint32_t)(m * (GW / 2) + rt) * 1024;
+        R.sz[0] = R.sz[1] = p.S.sz0 + (uint32_t)(m * (GW / 2) + rt) * (uint32_t)(GStageK >> p.gshift) * 64;
+        R.code_part = R.sz_part = 0; R.csh = 2;
+#pragma unroll 1
+        for (int s = 0; s < p.ns1; ++s) {
+            if (s > 0) ring_wait(&full[rp.st], rp.phase, p.status);
+            const uint8_t* sb = stage(rp.st);
+            mma_stage<1, CPB, false>(acc, sb, R, sb + p.S.act0, p.gshift);
+            release(rp);
+            rp.next(p.S.stages);
+        }
+        unscale(acc);
+        if (p.rank > 0) {
+            mma16816(acc[0][0], lb[0], lb[1], lb[2], lb[3], lu[0], lu[1]);
+            for (int kr = 16; kr < p.rank; kr += 16) {
+                uint32_t a[4];
+                lora_rows(B, kr, a);
+                mma16816(acc[0][0], a[0], a[1], a[2], a[3], __ldg(reinterpret_cast<const uint32_t*>(u + kr)), __ldg(reinterpret_cast<const uint32_t*>(u + kr + 8)));
+            }
+        }
+        float4* up = reinterpret_cast<float4*>(smem + p.S.h + (warp | 1) * (8 * 20 * 4)) + lane;      // (the up warp's part)
+        const int bar = 1 + (int)(threadIdx.x >> 6);                     // of the two warps
+        if (m) *up = make_float4(acc[0][0][0], acc[0][0][1], acc[0][0][2], acc[0][0][3]);
+        asm volatile("bar.sync %0, 64;" ::"r"(bar) : "memory");
+        if (!m) {
+            const float4 v = *up;
+            const float w[4] = {v.x, v.y, v.z, v.w};
+            store_h<1>(tile, row0, [&](int, int q) { return silu_f(acc[0][0][q]) * w[q]; });
+        }
+        asm volatile("bar.sync %0, 64;" ::"r"(bar) : "memory");
+    }
+
     // ---- down: two output row tiles of this warp; o[pair][row] = gate (W h + B (sigma A h))
     template <int NT, int CPB>
     __device__ __forceinline__ void down(int sub, int ad, uint32_t count, RingPos& rp) {
         const int row0 = (sub * GW + warp) * 32;
         float acc[2][NT][4];
-        clear<NT>(acc);
+        clear(acc);
         const bool lora = p.rank > 0 && row0 < p.H;
         constexpr bool ahead = NT <= 2;
         const uint16_t* B = static_cast<const uint16_t*>(p.lora.B_down) + ((size_t)ad * p.H + row0 + g8) * p.rank;
@@ -333,7 +392,7 @@ struct Gffn {
             release(rp);
             rp.next(p.S.stages);
         }
-        unscale<NT>(acc);
+        unscale(acc);
         // the projections of h, pairs and gates, as the group's projection warp has left them
         const uint32_t par = count & 1;
         const __half* s_ud = reinterpret_cast<const __half*>(smem + p.S.ud) + par * p.cap * p.r16;
@@ -445,7 +504,6 @@ struct Gffn {
             const int t = t_next;
             const int4 ti = ti_next;
             if (t >= total) break;
-            t_next = atomicAdd(p.ticket, 1);                             // (the unit after this one: on its way while this one is issued)
             const bool gu = t < u1;
             const int tile = tile_of(t), sub = gu ? t - tile * p.n1 : t - u1 - tile * p.n2;
             const int nt = (ti.z + 7) >> 3, ns = gu ? p.ns1 : p.ns2;
@@ -459,10 +517,10 @@ struct Gffn {
                     s_info[2 * rp.st] = make_int4(gu ? 1 : 2, tile, sub, nt);
                     s_info[2 * rp.st + 1] = make_int4(ti.w, 0, 0, 0);
                 }
-                mbar_expect_tx(bar, GCodeBytes + p.S.sz_bytes + act);
+                mbar_expect_tx(bar, (gu ? (GCodeBytes + p.S.sz_bytes) / GW * p.rows1 : GCodeBytes + p.S.sz_bytes) + act);
                 if (gu) {
-                    tma_load_5d(sb, m_cgu, s * GStageK, sub * GW, 0, ti.x, 0, bar, polw);
-                    tma_load_5d(sb + p.S.sz0, m_zgu, ((s * GStageK) >> p.gshift) * 8, sub * GW, 0, ti.x, 0, bar, polw);
+                    tma_load_5d(sb, m_cgu, s * GStageK, sub * p.rows1, 0, ti.x, 0, bar, polw);
+                    tma_load_5d(sb + p.S.sz0, m_zgu, ((s * GStageK) >> p.gshift) * 8, sub * p.rows1, 0, ti.x, 0, bar, polw);
                 } else {
                     const int sw = p.I / kDownSlices, kk = s * GStageK;
                     const int sl = p.sp > 1 ? s * p.sp : kk / sw, x = p.sp > 1 ? 0 : kk % sw;
@@ -482,7 +540,10 @@ struct Gffn {
                 }
                 bulk_g2s_hint(sb + p.S.act0, asrc + (size_t)s * act, act, bar, pola);
                 advance();
-                if (s == 0 && t_next < total) ti_next = __ldg(p.tiles + tile_of(t_next));
+                // The unit after this one is taken near the end of this one's copies, six stages ahead of its arithmetic: at its start, CTAs
+                // that begin two microseconds before the others (where no CTA of the kernel before holds the SM) took two units each.
+                if (s == max(0, ns - 3)) t_next = atomicAdd(p.ticket, 1);
+                if (s == ns - 1 && t_next < total) ti_next = __ldg(p.tiles + tile_of(t_next));
             }
         }
         acquire();
@@ -494,7 +555,7 @@ struct Gffn {
 
 // Warps: GGroups groups of GW consumers, then a producer warp per group, then a projection warp per group.  NTMAX: columns of 8
 // pairs a tile may have; the form for one column keeps its registers free of the code for more.
-template <int CPB, int NTMAX>
+template <int CPB, int NTMAX, bool NARROW>
 __global__ void __launch_bounds__(GThreads, 1)
 grouped_ffn_kernel(const __grid_constant__ GffnParams p, const __grid_constant__ CUtensorMap m_cgu, const __grid_constant__ CUtensorMap m_zgu,
                    const __grid_constant__ CUtensorMap m_cd, const __grid_constant__ CUtensorMap m_zd) {
@@ -529,7 +590,8 @@ grouped_ffn_kernel(const __grid_constant__ GffnParams p, const __grid_constant__
         const int ad = s_info[2 * rp.st + 1].x;
         if (a.x == 0) break;
         if (a.x == 1) {
-            if (NTMAX == 1 || a.w == 1) k.gate_up<1, CPB>(a.y, a.z, ad, rp);
+            if (NARROW) k.gate_up_narrow<CPB>(a.y, a.z, ad, rp);
+            else if (NTMAX == 1 || a.w == 1) k.gate_up<1, CPB>(a.y, a.z, ad, rp);
             else if (a.w == 2) k.gate_up<(NTMAX < 2 ? 1 : 2), CPB>(a.y, a.z, ad, rp);
             else if (a.w == 3) k.gate_up<(NTMAX < 3 ? 1 : 3), CPB>(a.y, a.z, ad, rp);
             else k.gate_up<(NTMAX < 4 ? 1 : 4), CPB>(a.y, a.z, ad, rp);
@@ -649,29 +711,99 @@ struct TileArgs {
     edg_lora lora;
     int H, K, rank, r16, cap, adapters;
     float sigma;
+    GroupArgs group;                      // (for the form that sorts)
 };
+
+// Up to kSortPairs pairs every CTA finds its tile by itself -- each pair counts the pairs before it in slot order -- and the kernel
+// that sorts is spared: 5 of the 62 us of 5 tokens.  Each CTA reads all pairs, in the square of their number: 1 us at 128, 25 at 512.
+// Same tiles in the same order.  Returns the tile, with `s_pair` its pairs; z = 0: there is none.
+constexpr int kSortPairs = 128;
+__device__ __forceinline__ int4 find_tile(const GroupArgs& g, int tile, int* s_pair) {
+    __shared__ __align__(16) int s_slot[kSortPairs];
+    __shared__ int s_nt[kSortPairs], s_ti[3], s_n;
+    const int i = threadIdx.x;                                           // this thread's pair
+    const bool lead = blockIdx.x == 0 && blockIdx.y == 0;
+    int slot = -1;
+    if (i < g.P) {
+        int e = g.slots[i];
+        slot = e;
+        if (g.table != nullptr) slot = (e >= 0 && e < g.E) ? g.table[e] : -1;
+        else if (g.experts != nullptr) e = g.experts[i];
+        else e = 0;
+        if (slot < 0 || slot >= g.n_slots || (g.adapters && (e < 0 || e >= g.E))) {
+            slot = -1;
+            if (lead) atomicExch(g.status, EDG_E_RANGE);
+        }
+        if (lead) g.pair_slot[i] = slot;
+    }
+    if (i < kSortPairs) s_slot[i] = slot;
+    if (i == 0) { s_ti[0] = -1; s_ti[2] = 0; s_n = 0; }
+    __syncthreads();
+    int pos = 0, before = 0, all = 0, nt = 0;
+    if (slot >= 0) {
+        for (int j = 0; j < g.P; ++j) {
+            const int v = s_slot[j];
+            pos += (unsigned)v < (unsigned)slot;
+            before += v == slot && j < i;
+            all += v == slot;
+        }
+        pos += before;
+        if (before == 0) nt = (all + g.cap - 1) / g.cap;
+    }
+    if (i < kSortPairs) s_nt[i] = nt;
+    __syncthreads();
+    if (nt > 0) {
+        int base = 0;
+        for (int j = 0; j < g.P; ++j) base += (unsigned)s_slot[j] < (unsigned)slot ? s_nt[j] : 0;
+        if (tile >= base && tile < base + nt) {
+            const int f = (tile - base) * g.cap;
+            s_ti[0] = slot; s_ti[1] = pos + f; s_ti[2] = min(g.cap, all - f);
+        }
+        atomicAdd(&s_n, nt);
+    }
+    __syncthreads();
+    const int4 ti = make_int4(s_ti[0], s_ti[1], s_ti[2], 0);
+    if (slot >= 0 && slot == ti.x && pos >= ti.y && pos < ti.y + ti.z) {
+        s_pair[pos - ti.y] = i;
+        if (blockIdx.y == 0) g.order[pos] = i;
+    }
+    if (lead && i == 0) { *g.n_tiles = s_n; *g.ticket = 0; }
+    if (blockIdx.y == 0 && i == 0 && ti.z > 0) g.done[tile] = 0;
+    __syncthreads();
+    return ti;
+}
 
 // blockIdx.y < cap / 8: eight of the tile's token states as fp16 B words, chunk by chunk as the ring reads them (and, for the
 // first, the tile's adapter); the rest: 16 rows each of u = (sigma A_gate x, sigma A_up x) for every token of the tile.
+template <bool SORT>
 __global__ void __launch_bounds__(256) tile_operands_kernel(TileArgs a) {
-    __shared__ int s_tok[32];
+    __shared__ int s_tok[32], s_pair[32];
     __shared__ float s_red[8 * 16 * 32];
     pdl_launch_dependents();
     pdl_wait_prior_grid();
     const int tile = blockIdx.x;
-    if (tile >= *a.n_tiles) return;
-    const int4 ti = a.tiles[tile];
+    int4 ti;
+    if constexpr (SORT) {
+        ti = find_tile(a.group, tile, s_pair);
+        if (ti.z == 0) return;
+    } else {
+        if (tile >= *a.n_tiles) return;
+        ti = a.tiles[tile];
+    }
     const int tid = threadIdx.x, nt = (ti.z + 7) >> 3, ntok = nt * 8, nx = a.cap / 8;
     if ((int)blockIdx.y < nx && (int)blockIdx.y >= nt) return;
-    if (tid < 32) s_tok[tid] = tid < ti.z ? a.order[ti.y + tid] / a.K : -1;
+    if (tid < 32) s_tok[tid] = tid < ti.z ? (SORT ? s_pair[tid] : a.order[ti.y + tid]) / a.K : -1;
     int ad = 0;
     if (a.adapters && ((int)blockIdx.y >= nx || (blockIdx.y == 0 && tid == 0))) {
-        const int pr0 = a.order[ti.y];
+        const int pr0 = SORT ? s_pair[0] : a.order[ti.y];
         ad = a.table != nullptr ? a.slots[pr0] : (a.experts != nullptr ? a.experts[pr0] : 0);
     }
     __syncthreads();
     if ((int)blockIdx.y < nx) {
-        if (blockIdx.y == 0 && tid == 0) a.tiles[tile].w = ad;
+        if (blockIdx.y == 0 && tid == 0) {
+            if (SORT) a.tiles[tile] = make_int4(ti.x, ti.y, ti.z, ad);
+            else a.tiles[tile].w = ad;
+        }
         uint8_t* out = a.xq + (size_t)tile * a.cap * a.H * 2;
         const int t0 = blockIdx.y * 8, q = tid & 3, tok = t0 + ((tid >> 2) & 7), st = s_tok[tok];
         const uint16_t* src = a.x + (size_t)(st < 0 ? 0 : st) * a.H + q * 8;
@@ -829,7 +961,14 @@ int32_t run_grouped_ffn(const edg_layer_desc* d, const GroupedParams& g, const W
     p.H = H; p.I = I; p.rank = g.rank; p.r16 = (g.rank + 15) / 16 * 16; p.cap = cap;
     while ((1 << p.gshift) < g.group) ++p.gshift;
     p.sigma = g.sigma;
-    p.n1 = (I / 16 + GW - 1) / GW; p.n2 = (H / 16 + 2 * GW - 1) / (2 * GW);
+    // Gate/up units of four row tiles (11 us instead of 20: what bounds a unit is its warps' instructions) while those of eight would leave
+    // groups without one.  By the tiles that evenly spread pairs make; eight : four, four layers of 256 experts, top 8, us: 2 tokens 189 : 162,
+    // 5 214 : 185, 8 247 : 229, 9 242 : 244, 15 303 : 312.
+    const int sms = sm_count(), wide1 = (I / 16 + GW - 1) / GW;
+    const double tiles_est = d->n_slots * (1.0 - std::pow(1.0 - 1.0 / d->n_slots, P));
+    const bool narrow = cap == 8 && tiles_est * 2 * wide1 <= 1.65 * GGroups * sms;
+    p.rows1 = narrow ? GW / 2 : GW;
+    p.n1 = (I / 16 + p.rows1 - 1) / p.rows1; p.n2 = (H / 16 + 2 * GW - 1) / (2 * GW);
     p.ns1 = H / GStageK; p.ns2 = I / GStageK;
     const int sw = I / kDownSlices;                // columns of a down slice; a stage takes part of one, or several
     p.sp = sw >= GStageK ? 1 : GStageK / sw;
@@ -862,9 +1001,9 @@ int32_t run_grouped_ffn(const edg_layer_desc* d, const GroupedParams& g, const W
     const uint32_t kc_el = (uint32_t)(sw < GStageK ? sw : GStageK);
     // (run of a row tile, row tile, matrix or slice, slot; the fifth dimension is not used)
     bool ok = tensor_map(&cgu, pool + g.L.codes_gate, {(uint64_t)H, (uint64_t)I / 16, 2, slots, 1}, {(uint64_t)H * 8, (uint64_t)H * I / 2, R, R * slots},
-                         {GStageK, GW, 2, 1, 1});
+                         {GStageK, (uint32_t)p.rows1, 2, 1, 1});
     ok = ok && tensor_map(&zgu, pool + g.L.sz_gate, {gpr * 8, (uint64_t)I / 16, 2, slots, 1}, {gpr * 64, gpr * I * 4, R, R * slots},
-                          {(uint32_t)(GStageK / g.group * 8), GW, 2, 1, 1});
+                          {(uint32_t)(GStageK / g.group * 8), (uint32_t)p.rows1, 2, 1, 1});
     ok = ok && tensor_map(&cd, pool + g.L.codes_down, {(uint64_t)sw, (uint64_t)H / 16, 4, slots, 1}, {(uint64_t)sw * 8, (uint64_t)H * sw / 2, R, R * slots},
                           {kc_el, 2 * GW, (uint32_t)p.sp, 1, 1});
     ok = ok && tensor_map(&zd, pool + g.L.sz_down, {gps * 8, (uint64_t)H / 16, 4, slots, 1}, {gps * 64, (uint64_t)H * gps * 4, R, R * slots},
@@ -873,7 +1012,8 @@ int32_t run_grouped_ffn(const edg_layer_desc* d, const GroupedParams& g, const W
 
     static OncePerDevice once;
     EDG_CUDA_TRY(once([] {
-        const cudaError_t e = allow_smem(GSmemLimit, grouped_ffn_kernel<1, 1>, grouped_ffn_kernel<2, 1>, grouped_ffn_kernel<1, 4>, grouped_ffn_kernel<2, 4>);
+        const cudaError_t e = allow_smem(GSmemLimit, grouped_ffn_kernel<1, 1, false>, grouped_ffn_kernel<2, 1, false>, grouped_ffn_kernel<1, 4, false>,
+                                        grouped_ffn_kernel<2, 4, false>, grouped_ffn_kernel<1, 1, true>, grouped_ffn_kernel<2, 1, true>);
         return e != cudaSuccess ? e : allow_smem(210 * 1024, group_pairs_kernel);
     }));
     GroupArgs ga{};
@@ -885,15 +1025,19 @@ int32_t run_grouped_ffn(const edg_layer_desc* d, const GroupedParams& g, const W
     while (ga.nw > 1 && (size_t)(ga.nw + 1) * d->n_slots * 4 > 200 * 1024) ga.nw /= 2;
     size_t cnt_bytes = (size_t)(ga.nw + 1) * d->n_slots * 4;
     if (cnt_bytes > 200 * 1024) { ga.cnt_g = reinterpret_cast<int32_t*>(ws + W.g_cnt); cnt_bytes = 0; }
-    EDG_CUDA_TRY(launch_pdl(group_pairs_kernel, dim3(1), 1024, cnt_bytes, st, ga));
+    const bool sort = P <= kSortPairs;
+    if (!sort) EDG_CUDA_TRY(launch_pdl(group_pairs_kernel, dim3(1), 1024, cnt_bytes, st, ga));
     TileArgs ta{};
+    ta.group = ga;
     ta.tiles = tiles; ta.n_tiles = n_tiles; ta.order = order;
     ta.slots = g.slots; ta.table = g.table; ta.experts = g.experts; ta.x = g.x; ta.xq = xq; ta.u = u; ta.lora = g.lora;
     ta.H = H; ta.K = g.K; ta.rank = g.rank; ta.r16 = p.r16; ta.cap = cap; ta.adapters = ga.adapters; ta.sigma = g.sigma;
-    EDG_CUDA_TRY(launch_pdl(tile_operands_kernel, dim3((unsigned)grouped_max_tiles(*d, g.T), cap / 8 + 2 * p.r16 / 16), 256, 0, st, ta));
-    const int sms = sm_count();
-    if (cap == 8) EDG_CUDA_TRY(launch_pdl(g.group >= 64 ? grouped_ffn_kernel<2, 1> : grouped_ffn_kernel<1, 1>, dim3(sms), GThreads, smem, st, p, cgu, zgu, cd, zd));
-    else EDG_CUDA_TRY(launch_pdl(g.group >= 64 ? grouped_ffn_kernel<2, 4> : grouped_ffn_kernel<1, 4>, dim3(sms), GThreads, smem, st, p, cgu, zgu, cd, zd));
+    EDG_CUDA_TRY(launch_pdl(sort ? tile_operands_kernel<true> : tile_operands_kernel<false>, dim3((unsigned)grouped_max_tiles(*d, g.T), cap / 8 + 2 * p.r16 / 16), 256, 0, st, ta));
+    const bool wide = g.group >= 64;
+    const auto kern = narrow ? (wide ? grouped_ffn_kernel<2, 1, true> : grouped_ffn_kernel<1, 1, true>)
+                    : cap == 8 ? (wide ? grouped_ffn_kernel<2, 1, false> : grouped_ffn_kernel<1, 1, false>)
+                               : (wide ? grouped_ffn_kernel<2, 4, false> : grouped_ffn_kernel<1, 4, false>);
+    EDG_CUDA_TRY(launch_pdl(kern, dim3(sms), GThreads, smem, st, p, cgu, zgu, cd, zd));
     EDG_CUDA_TRY(launch_sum_choices(g, st));
     return EDG_OK;
 }

@@ -48,6 +48,42 @@ def test_streaming_form_at_tile_edges(H, I, group, rank, E, K, n_adapters, T):
     assert np.array_equal(Y, _ffn_tokens(L, L.desc, X, torch.from_numpy(inds_h).cuda(), torch.from_numpy(gates_h).cuda(), T))
 
 
+@pytest.mark.parametrize("H,I,group,rank,E,K,n_adapters,T", [
+    (512, 256, 32, 8, 32, 2, 32, 63),       # 126 pairs: the tiles find themselves
+    (512, 256, 64, 24, 32, 2, 1, 64),       # 128: the last size that does
+    (512, 256, 64, 24, 32, 2, 1, 65),       # 130: sorted
+    (2048, 512, 64, 0, 64, 1, 1, 61),       # 61 pairs: the last narrow units of the larger layer, about
+    (2048, 128, 32, 16, 64, 1, 64, 40),     # two narrow units a matrix
+])
+def test_few_pairs_find_their_tiles(H, I, group, rank, E, K, n_adapters, T):
+    """Up to 128 pairs, tiles of 8: a slot of 20 pairs, single ones, a choice that is no slot, one named twice by a token."""
+    L = _layer(H, I, group, rank, E, K, n_adapters)
+    X = synth.hidden_states(L.cfg, T, stream=66)
+    rng = np.random.default_rng(11)
+    inds_h, gates_h = _routing(rng, T, E, K)
+    inds_h[5:25, 0] = E - 2
+    if K > 1:
+        inds_h[5:25, 1] = E - 1
+        inds_h[30] = 3
+    inds, gates = torch.from_numpy(inds_h).cuda(), torch.from_numpy(gates_h).cuda()
+    Y = _ffn_tokens(L, L.desc, X, inds, gates, T)
+    _check_tokens(L, X, inds_h, gates_h, Y, range(T))
+    assert np.array_equal(Y, _ffn_tokens(L, L.desc, X, inds, gates, T, use_table=False))
+    bad = inds_h.copy()
+    bad[7, K - 1] = -3
+    y = out_tensor(L.desc, T)
+    table = torch.arange(E, dtype=torch.int32, device="cuda")
+    edg.moe_expert_ffn_int4_lora(L.desc, L.pool, table, T, torch.from_numpy(bad).cuda(), None, gates, x_dev(X), L.lora, y, L.ws)
+    torch.cuda.synchronize()
+    assert edg.workspace_status(L.ws) == -4
+    got = y.cpu().numpy()
+    assert np.array_equal(np.delete(got, 7, axis=0), np.delete(Y, 7, axis=0))
+    if K > 1:
+        _check_tokens(L, X, inds_h[:, :1], gates_h[:, :1], got, [7])
+    else:
+        assert not got[7].any()
+
+
 @pytest.mark.parametrize("n_adapters", [1, 16])
 def test_first_size_of_the_tensor_memory_tiles(n_adapters):
     """97 pairs per slot on the small layer: groups of 32, rank 8, ragged tiles, an expert that spans many tiles."""
