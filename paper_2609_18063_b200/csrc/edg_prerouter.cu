@@ -320,6 +320,120 @@ __global__ void __launch_bounds__(kPreWarps * 32) prerouter_tokens_mma_kernel(Pr
     }
 }
 
+// Many tokens of a head that the kernel above does not take (fp32, or rows that do not split into eight whole tiles): a CTA computes all rows
+// for 16 tokens on the tensor cores, K split over its warps, and does their softmax and top-k; no cluster.  Products are exact: the
+// states are bf16 as they are, an fp32 weight is the sum of three bf16 (8 of its 24 bits each), an fp16 one of two.  Every 32 k start a
+// fresh accumulator, the large parts apart from the small ones, and are added in fp32.
+__device__ __forceinline__ void mma16816_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// eight weights of a row as words of two bf16, part by part
+template <int PARTS>
+__device__ __forceinline__ void bf16_parts(const float (&w)[8], uint32_t (&out)[PARTS][4]) {
+    float r[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) r[i] = w[i];
+#pragma unroll
+    for (int q = 0; q < PARTS; ++q)
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {
+            const uint32_t a = __float_as_uint(r[i]) & 0xFFFF0000u, b = __float_as_uint(r[i + 1]) & 0xFFFF0000u;
+            out[q][i / 2] = (a >> 16) | b;
+            r[i] -= __uint_as_float(a);
+            r[i + 1] -= __uint_as_float(b);
+        }
+}
+__device__ __forceinline__ void load8(const float* w, float (&f)[8]) {
+    const uint4 a = ld_stream16(w), b = ld_stream16(w + 4);
+    f[0] = __uint_as_float(a.x); f[1] = __uint_as_float(a.y); f[2] = __uint_as_float(a.z); f[3] = __uint_as_float(a.w);
+    f[4] = __uint_as_float(b.x); f[5] = __uint_as_float(b.y); f[6] = __uint_as_float(b.z); f[7] = __uint_as_float(b.w);
+}
+__device__ __forceinline__ void load8(const __half* w, float (&f)[8]) {
+    const uint4 a = ld_stream16(w);
+    const float2 x = __half22float2(u32_as_h2(a.x)), y = __half22float2(u32_as_h2(a.y)), z = __half22float2(u32_as_h2(a.z)), v = __half22float2(u32_as_h2(a.w));
+    f[0] = x.x; f[1] = x.y; f[2] = y.x; f[3] = y.y; f[4] = z.x; f[5] = z.y; f[6] = v.x; f[7] = v.y;
+}
+constexpr int kRowTok = 16;
+// From how many tokens on it is ahead of the clusters of FMA warps (us a call, those : this; H 2048).  64 rows fp32: 5 tokens 17 : 18, 16 21 : 20,
+// 1024 66 : 20, 4096 221 : 29; 256 rows fp32: 333 52 : 62, 1024 136 : 63, 4096 439 : 91; 160 rows fp16: 64 31 : 31, 128 41 : 31, 4096
+// 587 : 46; 16 rows of H 1024: 5 tokens 10.6 : 5.4.  Its error against 64 bits is below theirs (8.3e-8 and 1.4e-7 rms, 256 rows).
+inline int rows_mma_tokens(const edg_layer_desc& d) { return d.E < 64 ? 2 : (d.E == 64 ? 16 : (d.pre_dtype == EDG_F16 ? 96 : 512)); }
+inline size_t rows_mma_smem(int E, int H) { return (size_t)kRowTok * E * 4 + kPreWarps * 256 * 4 + (size_t)kRowTok * (H * 2 + 64); }
+
+template <typename WT>
+__global__ void __launch_bounds__(kPreWarps * 32) prerouter_rows_mma_kernel(PreParams p, int T) {
+    constexpr int PARTS = sizeof(WT) == 4 ? 3 : 2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t4 = lane & 3, t0 = blockIdx.x * kRowTok;
+    extern __shared__ float smem[];
+    float* s_logits = smem;                                             // [kRowTok][E]
+    float* s_red = smem + kRowTok * p.E;                                // [kPreWarps][16 rows][16 tokens]
+    const int xs = p.H * 2 + 64;                                        // bytes per token row (padded against bank conflicts)
+    uint8_t* s_x = reinterpret_cast<uint8_t*>(s_red + kPreWarps * 256);
+    pdl_wait_prior_grid();
+    pdl_launch_dependents();
+    for (int i = threadIdx.x; i < kRowTok * (p.H / 8); i += kPreWarps * 32) {
+        const int tt = i / (p.H / 8), c = i % (p.H / 8), t = t0 + tt;
+        *reinterpret_cast<uint4*>(s_x + tt * xs + c * 16) = t < T ? *reinterpret_cast<const uint4*>(p.s + (size_t)t * p.H + c * 8) : make_uint4(0, 0, 0, 0);
+    }
+    __syncthreads();
+    const int ksl = p.H / kPreWarps;                                    // k per warp: a multiple of 32
+    const uint8_t* xb = s_x + g * xs + (warp * ksl + 8 * t4) * 2;
+    for (int r0 = 0; r0 < p.E; r0 += 16) {
+        const WT* w = static_cast<const WT*>(p.W) + (size_t)(r0 + g) * p.H + warp * ksl + 8 * t4;
+        float sum[2][4] = {};
+#pragma unroll 2
+        for (int k = 0; k < ksl; k += 32) {
+            float lo[8], hi[8];
+            load8(w + k, lo);
+            load8(w + (size_t)8 * p.H + k, hi);
+            uint32_t a[PARTS][4], b[PARTS][4];
+            bf16_parts<PARTS>(lo, a);
+            bf16_parts<PARTS>(hi, b);
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                const uint4 v = *reinterpret_cast<const uint4*>(xb + n * 8 * xs + k * 2);
+                float c[2][4] = {};
+#pragma unroll
+                for (int q = PARTS - 1; q >= 0; --q) {
+                    mma16816_bf16(c[q > 0], a[q][0], b[q][0], a[q][1], b[q][1], v.x, v.y);
+                    mma16816_bf16(c[q > 0], a[q][2], b[q][2], a[q][3], b[q][3], v.z, v.w);
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sum[n][e] += c[0][e] + c[1][e];
+            }
+        }
+        float* mine = s_red + warp * 256;                               // rows g / g + 8, tokens 8 n + 2 t4, + 1
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            mine[g * 16 + n * 8 + 2 * t4] = sum[n][0]; mine[g * 16 + n * 8 + 2 * t4 + 1] = sum[n][1];
+            mine[(g + 8) * 16 + n * 8 + 2 * t4] = sum[n][2]; mine[(g + 8) * 16 + n * 8 + 2 * t4 + 1] = sum[n][3];
+        }
+        __syncthreads();
+        double v = 0.0;
+#pragma unroll
+        for (int q = 0; q < kPreWarps; ++q) v += s_red[q * 256 + threadIdx.x];
+        float l = (float)v;
+        if (!(fabsf(l) <= 3.4e38f)) {                                   // (the parts of an infinity, or zero parts times one, are not numbers: as it is)
+            const WT* row = static_cast<const WT*>(p.W) + (size_t)(r0 + (threadIdx.x >> 4)) * p.H;
+            const uint16_t* x = reinterpret_cast<const uint16_t*>(s_x + (threadIdx.x & 15) * xs);
+            l = 0.f;
+            for (int k = 0; k < p.H; ++k) l = fmaf((float)row[k], bf16_bits_to_float(x[k]), l);
+        }
+        s_logits[(threadIdx.x & 15) * p.E + r0 + (threadIdx.x >> 4)] = l;
+        __syncthreads();
+    }
+    for (int tt = warp; tt < kRowTok; tt += kPreWarps) {
+        const int t = t0 + tt;
+        if (t >= T) break;
+        float* row = s_logits + tt * p.E;
+        if (p.logits != nullptr)
+            for (int e = lane; e < p.E; e += 32) p.logits[(size_t)t * p.E + e] = row[e];
+        __syncwarp();
+        warp_softmax_topk(row, p.E, p.K, lane, p.inds + (size_t)t * p.K, p.gates + (size_t)t * p.K);
+    }
+}
+
 // a2 alone: one warp per row of given logits.
 __global__ void __launch_bounds__(128) softmax_topk_rows_kernel(const float* logits, int T, int E, int K,
                                                                 int32_t* inds, float* gates) {
@@ -804,12 +918,21 @@ int32_t run_prerouter(const edg_layer_desc* d, const void* W_pre, const void* s,
     auto launch = [&](auto kern, size_t bytes, auto... args) { return launch_pdl_cluster(kPreCluster, kern, grid, kPreWarps * 32, bytes, st, args...); };
     if (batched) {
         static OncePerDevice once;
-        EDG_CUDA_TRY(once([] { return allow_smem(200 * 1024, prerouter_tokens_kernel<__half>, prerouter_tokens_kernel<float>, prerouter_tokens_mma_kernel); }));
+        EDG_CUDA_TRY(once([] {
+            return allow_smem(200 * 1024, prerouter_tokens_kernel<__half>, prerouter_tokens_kernel<float>, prerouter_tokens_mma_kernel,
+                              prerouter_rows_mma_kernel<__half>, prerouter_rows_mma_kernel<float>);
+        }));
         if (smem > 200 * 1024) return EDG_E_SHAPE;
         // an fp16 head whose rows and columns split into whole MMA tiles goes to the tensor cores
         if (d->pre_dtype == EDG_F16 && d->E % (16 * kPreCluster) == 0 && d->H % (32 * kPreWarps) == 0) {
             const size_t bytes = (size_t)kTokBlock * d->E * 4 + kPreWarps * 256 * 4 + (size_t)kTokBlock * (d->H * 2 + 64);
             EDG_CUDA_TRY(launch(prerouter_tokens_mma_kernel, bytes, p, (int)n_heads));
+            return EDG_OK;
+        }
+        const size_t rows_smem = rows_mma_smem(d->E, d->H);
+        if (n_heads >= rows_mma_tokens(*d) && d->E % 16 == 0 && d->H % (32 * kPreWarps) == 0 && rows_smem <= 200 * 1024) {
+            EDG_CUDA_TRY(launch_pdl(d->pre_dtype == EDG_F16 ? prerouter_rows_mma_kernel<__half> : prerouter_rows_mma_kernel<float>,
+                                    dim3((unsigned)(n_heads + kRowTok - 1) / kRowTok), kPreWarps * 32, rows_smem, st, p, (int)n_heads));
             return EDG_OK;
         }
         if (d->pre_dtype == EDG_F16) EDG_CUDA_TRY(launch(prerouter_tokens_kernel<__half>, smem, p, (int)n_heads));

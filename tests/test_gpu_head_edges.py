@@ -88,3 +88,47 @@ def test_full_head_whose_copies_do_not_come_in_time(tmp_path, pre, variant):
     for a, b in zip(*out):
         assert torch.equal(a, b)
     assert out[0][2].abs().max() > 0
+
+
+@pytest.mark.parametrize("H,E,K,dtype", [(256, 16, 3, "f32"), (1024, 48, 4, "f16"), (2048, 64, 8, "f32"), (512, 160, 2, "f16"), (2048, 160, 6, "f32")])
+@pytest.mark.parametrize("T", [2, 15, 16, 17, 95, 96, 97, 517])
+def test_many_tokens_of_a_head_in_sixteens(H, E, K, dtype, T):
+    """Blocks of 16 tokens, ragged, around the sizes where the form changes, states from 1e-20 to 1e6: fp32 weights are summed from three bf16
+    parts without loss.  Bar: sums of H products in fp32, 2^-24 of the sum of their magnitudes each way of adding."""
+    d = edg.make_desc(None, H=H, I=128, E=E, K=K, group=32, rank=0, n_adapters=1, n_slots=E, pre_dtype=dtype, lora_scale=1.0, out_dtype="f32")
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(T)
+    W = torch.randn((E, H), generator=gen, device="cuda") * 0.02
+    if dtype == "f16":
+        W = W.half()
+    mag = 10.0 ** (torch.arange(T, device="cuda") % 27 - 20).double()
+    X = (torch.randn((T, H), generator=gen, device="cuda").double() * mag[:, None]).bfloat16()
+    inds, gates, logits = torch.full((T, K), -1, dtype=torch.int32, device="cuda"), torch.zeros((T, K), device="cuda"), torch.zeros((T, E), device="cuda")
+    edg.prerouter_topk_tokens(d, W, X, T, inds, gates, logits)
+    torch.cuda.synchronize()
+    want, size = X.double() @ W.double().T, X.double().abs() @ W.double().abs().T
+    assert ((logits.double() - want).abs() <= 4 * 2.0 ** -24 * size).all()
+    top = torch.topk(logits, K).indices.sort(-1).values
+    assert torch.equal(inds.long(), top)
+    picked = torch.gather(logits.double(), 1, top)
+    assert torch.allclose(gates.double(), torch.softmax(picked, -1), rtol=2e-5, atol=1e-7)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+def test_infinities_in_a_head_of_many_tokens(dtype):
+    """An infinite weight or state makes the logits it makes in plain arithmetic, and no others."""
+    H, E, T = 512, 32, 33
+    d = edg.make_desc(None, H=H, I=128, E=E, K=2, group=32, rank=0, n_adapters=1, n_slots=E, pre_dtype=dtype, lora_scale=1.0, out_dtype="f32")
+    W = torch.randn((E, H), device="cuda") * 0.02
+    W[3, 5], W[9, 40] = float("inf"), -float("inf")
+    W = W.half() if dtype == "f16" else W
+    X = torch.randn((T, H), device="cuda").bfloat16()
+    X[7, 11], X[20, 5] = float("inf"), 0.0
+    inds, gates, logits = torch.zeros((T, 2), dtype=torch.int32, device="cuda"), torch.zeros((T, 2), device="cuda"), torch.zeros((T, E), device="cuda")
+    edg.prerouter_topk_tokens(d, W, X, T, inds, gates, logits)
+    torch.cuda.synchronize()
+    want = (X.double().cpu()[:, None, :] * W.double().cpu()[None]).sum(-1)
+    got = logits.double().cpu()
+    assert torch.equal(torch.isnan(got), torch.isnan(want)) and torch.equal(torch.isinf(got), torch.isinf(want))
+    inf, fin = torch.isinf(want), torch.isfinite(want)
+    assert torch.equal(got[inf], want[inf]) and (got[fin] - want[fin]).abs().max() <= 1e-5
