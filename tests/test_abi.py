@@ -56,6 +56,20 @@ def test_record_bytes_and_desc_checks(lib):
     assert lib.ffn_workspace_bytes(d2, 64) > lib.ffn_workspace_bytes(d2, 1)
 
 
+@pytest.mark.parametrize("H,I,group,rank,per_expert", [(256, 128, 32, 0, False), (2048, 512, 32, 16, False), (2048, 512, 64, 16, True),
+                                                       (1024, 1024, 128, 64, False), (512, 256, 64, 8, True), (256, 256, 32, 5, False)])
+@pytest.mark.parametrize("K,slots", [(1, 1), (1, 2), (2, 1), (3, 5), (8, 1), (8, 64), (2, 300), (32, 256), (8, 1100), (1, 9000)])
+def test_a_workspace_serves_every_smaller_call(lib, H, I, group, rank, per_expert, K, slots):
+    """The bytes asked for never fall as T grows, around the sizes where tiles and kernels change and in between."""
+    E = max(K, min(slots, 1024), 16)
+    d = lib.make_desc(None, H=H, I=I, E=E, K=K, group=group, rank=rank, n_adapters=E if per_expert else 1, n_slots=slots, pre_dtype="f16",
+                      lora_scale=1.0, out_dtype="f32")
+    lines = [n * slots // K for n in (4, 8, 40, 96)]
+    Ts = set(range(1, 200)) | {t + i for t in lines for i in range(-3, 4)} | {t + t // q for t in lines for q in (4, 8)}
+    size = [lib.ffn_workspace_bytes(d, T) for T in sorted(t for t in Ts if 1 <= t <= 65535)]
+    assert all(a <= b for a, b in zip(size, size[1:]))
+
+
 def test_pack_unpack_identity_and_layout(lib):
     cfg = synth.CONFIGS["cfg1"]
     d = lib.make_desc(cfg)
