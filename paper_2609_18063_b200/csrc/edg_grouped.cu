@@ -98,7 +98,7 @@ bool grouped_use_umma(const edg_layer_desc& d, int T) {
     return (int64_t)T * d.K > grouped_streaming_pairs(d) && umma_grouped_supported(d);
 }
 int64_t grouped_streaming_pairs(const edg_layer_desc& d) {
-    return (int64_t)(d.group >= 64 ? kUmmaPairsPerSlot : kUmmaPairsPerSlot32) * d.n_slots;
+    return (int64_t)(d.group >= 64 && d.n_slots <= kUmmaSlots ? kUmmaPairsPerSlot : kUmmaPairsPerSlot32) * d.n_slots;
 }
 
 int32_t run_grouped(const edg_layer_desc* d, const void* slot_pool, int32_t T, const int32_t* slots, const int32_t* table,

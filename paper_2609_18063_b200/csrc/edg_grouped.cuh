@@ -36,7 +36,9 @@ constexpr int kUmmaTokens = 128;
 // nothing else is said).  256 experts, top 8: 32 422 : 452, 64 706 : 561; 64 experts: 42 161 : 145, 80 238 : 197; groups of 128: 21
 // 185 : 220, 40 263 : 249; H 1024, I 256, 16 experts: 42 59.4 : 60.2, 128 92 : 66.  With groups of 32 the sums leave tensor memory twice
 // as often: 64 214 : 230, 128 322 : 296.
-constexpr int kUmmaPairsPerSlot = 40, kUmmaPairsPerSlot32 = 96;
+// Beyond 1024 slots (no table names more) the line stays where it was: what is counted per slot of the pool says nothing about the slots
+// in use then, each slot has a CTA that reads all pairs, and with 65,535 tokens of 32 choices the tiles would not fit a grid.
+constexpr int kUmmaPairsPerSlot = 40, kUmmaPairsPerSlot32 = 96, kUmmaSlots = 1024;
 bool umma_grouped_supported(const edg_layer_desc& d);
 cudaError_t launch_umma(const GroupedParams& p, bool down, int max_tiles, cudaStream_t st);
 

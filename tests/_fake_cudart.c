@@ -1,5 +1,6 @@
 /* A CUDA runtime of two devices for host code that launches kernels: nothing runs; a launch that asks for more dynamic shared memory than
- * its function has been allowed on the current device (48 KB, unless an attribute says more) is refused, as the real one does. */
+ * its function has been allowed on the current device (48 KB, unless an attribute says more), or for more than 65,535 blocks along y or z, is
+ * refused, as the real one does. */
 #include <stddef.h>
 
 enum { OK = 0, INVALID = 1, MAX_FN = 256 };
@@ -19,7 +20,7 @@ int fake_launches(void) { return launches; }
 
 struct config { unsigned grid[3], block[3]; size_t smem; void* stream; void* attrs; unsigned n_attrs; };
 int cudaLaunchKernelExC(const struct config* c, const void* fn, void** args) {
-    if (c->smem > (size_t)*allowed(fn)) return INVALID;
+    if (c->smem > (size_t)*allowed(fn) || c->grid[1] > 65535 || c->grid[2] > 65535) return INVALID;
     ++launches;
     return OK;
 }
@@ -33,3 +34,8 @@ void** __cudaRegisterFatBinary(void* p) { static void* h; return &h; }
 void __cudaRegisterFatBinaryEnd(void** h) {}
 void __cudaUnregisterFatBinary(void** h) {}
 void __cudaRegisterFunction(void** h, const char* f, char* d, const char* n, int l, void* a, void* b, void* c, void* e, int* w) {}
+
+int cudaDeviceGetAttribute(int* v, int attr, int d) { *v = 148; return OK; }
+static int encode_tiled(void) { return OK; }
+int cudaGetDriverEntryPoint(const char* name, void** fn, unsigned long long flags, int* found) { *fn = (void*)encode_tiled; *found = 0; return OK; }
+size_t _ZN3edg17step_region_wordsERK14edg_layer_desc(const void* d) { return 0; }     /* (edg_step.cu, which is not part of this) */

@@ -1,5 +1,5 @@
 """Kernels that need more than 48 KB of shared memory, on the second device of a process: the host code against a runtime of two devices
-in which nothing runs (tests/_fake_cudart.c)."""
+in which nothing runs (tests/_fake_cudart.c).  And grids that no device takes."""
 import ctypes as C
 import os
 import shutil
@@ -14,15 +14,24 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(ROOT, "paper_2609_18063_b200", "csrc")
 
 
-@pytest.fixture(scope="module")
-def lib(tmp_path_factory):
-    out = str(tmp_path_factory.mktemp("fake") / "libhost.so")
+def _host_lib(out, sources):
     fake = out[:-3] + "_rt.o"
     subprocess.run([shutil.which("gcc"), "-c", "-fPIC", "-o", fake, os.path.join(HERE, "_fake_cudart.c")], check=True)
     subprocess.run([shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc", "-gencode", "arch=compute_100a,code=compute_100a", "-std=c++17", "-shared",
                     "-Xcompiler", "-fPIC", "-Xlinker", "-Bsymbolic", "-cudart", "none", "-I", os.path.join(ROOT, "include"), "-o", out,
-                    os.path.join(CSRC, "edg_prerouter.cu"), os.path.join(CSRC, "edg_pack.cu"), fake], check=True)
+                    "--threads", "0", *[os.path.join(CSRC, f) for f in sources], fake], check=True)
     return C.CDLL(out, mode=os.RTLD_LAZY)
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return _host_lib(str(tmp_path_factory.mktemp("fake") / "libhost.so"), ["edg_prerouter.cu", "edg_pack.cu"])
+
+
+@pytest.fixture(scope="module")
+def grouped(tmp_path_factory):
+    return _host_lib(str(tmp_path_factory.mktemp("fake") / "libgrouped.so"),
+                     ["edg_ffn.cu", "edg_grouped.cu", "edg_grouped_ffn.cu", "edg_grouped_umma.cu", "edg_lora_tokens.cu", "edg_pack.cu"])
 
 
 def _desc(**kw):
@@ -51,3 +60,17 @@ def test_every_device_launches(lib, call, dtype):
         before = lib.fake_launches()
         assert call(lib, dtype) == 0, device
         assert lib.fake_launches() == before + 1
+
+
+@pytest.mark.parametrize("slots", [1, 1024, 1025, 21845, 40000, 49152, 49153, 50000, 52427, 60000])
+def test_the_largest_calls_fit_a_grid(grouped, slots):
+    """65,535 tokens of 32 choices, whatever the pool: every form's tiles stay within what a launch may have."""
+    d = _desc(H=256, I=256, E=32, K=32, rank=8, n_slots=slots)
+    p = C.c_void_p(P)
+    lora = edg.binding.Lora(*[P] * 6)
+    n = C.c_size_t()
+    for T in (65535, 40 * slots // 32 + 1, 96 * slots // 32 + 1):
+        if not 2 <= T <= 65535:
+            continue
+        assert grouped.edg_ffn_workspace_bytes(C.byref(d), T, C.byref(n)) == 0
+        assert grouped.moe_expert_ffn_int4_lora(C.byref(d), p, p, T, p, p, p, p, C.byref(lora), p, p, n, None) == 0, T
