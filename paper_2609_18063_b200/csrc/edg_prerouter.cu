@@ -7,8 +7,9 @@
 // softmax + top-k with warp shuffles.  No global scratch, no atomics, one launch.
 //
 // All kernels of this file are launched as programmatic dependents: a call's launch is under way while the kernel before it
-// ends, and the kernel behind it is let go as soon as that one has (4096 rows of sigmoid-group routing, call after call, 8.2 -> 6.8 us;
-// 40 full heads 39.0 -> 37.1).  Every thread waits before it reads or writes global memory.
+// ends (4096 rows of sigmoid-group routing, call after call, 8.2 -> 5.8 us; 40 full heads 39.0 -> 37.2).  Every thread waits before it
+// reads or writes global memory.  None lets the kernel behind it come before it has ended itself: a link of a chain does not wait for
+// what was queued before it, and may write what these kernels read or write (let go at once, the two took 6.3 and 37.1 us).
 #include <cooperative_groups.h>
 #include <math_constants.h>
 
@@ -93,7 +94,6 @@ __global__ void __launch_bounds__(kPreWarps * 32) prerouter_kernel(PreParams p) 
     float* s_x = smem + p.E;            // [H]   hidden state widened to fp32
 
     pdl_wait_prior_grid();
-    pdl_launch_dependents();
     const uint16_t* sv = p.s + (size_t)head * p.H;
     for (int i = threadIdx.x; i < p.H; i += blockDim.x) s_x[i] = bf16_bits_to_float(sv[i]);
     __syncthreads();
@@ -138,7 +138,6 @@ __global__ void __launch_bounds__(kPreWarps * 32) prerouter_tokens_kernel(PrePar
     float* s_logits = smem;                         // [kTokBlock][E]  (the leader's copy collects every CTA's rows)
     float* s_x = smem + kTokBlock * p.E;            // [kTokBlock][H]  hidden states widened to fp32
     pdl_wait_prior_grid();
-    pdl_launch_dependents();
     for (int tt = 0; tt < kTokBlock; ++tt) {
         const int t = t0 + tt;
         for (int i = threadIdx.x; i < p.H; i += blockDim.x)
@@ -255,7 +254,6 @@ __global__ void __launch_bounds__(kPreWarps * 32) prerouter_tokens_mma_kernel(Pr
         }
     };
     pdl_wait_prior_grid();
-    pdl_launch_dependents();
     const int r_first = crank * per;
     load_a(r_first, 0, r_first + 16 < (crank + 1) * per);
     for (int i = threadIdx.x; i < kTokBlock * (p.H / 8); i += blockDim.x) {
@@ -371,7 +369,6 @@ __global__ void __launch_bounds__(kPreWarps * 32) prerouter_rows_mma_kernel(PreP
     const int xs = p.H * 2 + 64;                                        // bytes per token row (padded against bank conflicts)
     uint8_t* s_x = reinterpret_cast<uint8_t*>(s_red + kPreWarps * 256);
     pdl_wait_prior_grid();
-    pdl_launch_dependents();
     for (int i = threadIdx.x; i < kRowTok * (p.H / 8); i += kPreWarps * 32) {
         const int tt = i / (p.H / 8), c = i % (p.H / 8), t = t0 + tt;
         *reinterpret_cast<uint4*>(s_x + tt * xs + c * 16) = t < T ? *reinterpret_cast<const uint4*>(p.s + (size_t)t * p.H + c * 8) : make_uint4(0, 0, 0, 0);
@@ -440,7 +437,6 @@ __global__ void __launch_bounds__(128) softmax_topk_rows_kernel(const float* log
     extern __shared__ float smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_wait_prior_grid();
-    pdl_launch_dependents();
     const int t = blockIdx.x * 4 + warp;
     if (t >= T) return;
     float* work = smem + warp * E;
@@ -610,7 +606,6 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(const __g
         }
     };
     pdl_wait_prior_grid();
-    pdl_launch_dependents();
     if (lane == 0)
         for (int i = 0; i < min(total, kMlpSlots); ++i) fetch();
 
@@ -717,7 +712,7 @@ __global__ void __launch_bounds__(kMlpWarps * 32) prerouter_mlp_kernel(const __g
 // lane l holds the V = E / 32 consecutive entries from l V on, so a group is a run of lanes and everything stays in registers;
 // order by (lane, entry) is order by index, so the first lane that holds a round's best key has the winner, ties included.
 // The form over shared memory below spends its time on instructions too, three times as many: a call on 4096 rows of 128, one after
-// the other, 11.1 us, here 8.2, and 6.8 since the next call's launch is under way beside it (6 of them are the host's).
+// the other, 11.1 us, here 8.2 with ordinary launches and 5.8 as programmatic dependents (the host's share is about as long).
 // Same values in the same order as that form.
 template <int V>
 __global__ void __launch_bounds__(256) sigmoid_group_topk_lanes_kernel(const float* logits, const float* bias, int T, int K, int n, int keep,
@@ -728,7 +723,6 @@ __global__ void __launch_bounds__(256) sigmoid_group_topk_lanes_kernel(const flo
     __shared__ float s_g[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_wait_prior_grid();
-    pdl_launch_dependents();
     const int t = blockIdx.x * 8 + warp;
     if (t >= T) return;
     float sg[V], sel[V];
@@ -818,7 +812,6 @@ __global__ void __launch_bounds__(128) sigmoid_group_topk_rows_kernel(const floa
     const unsigned full = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_wait_prior_grid();
-    pdl_launch_dependents();
     const int t = blockIdx.x * 4 + warp;
     if (t >= T) return;
     float* sig = smem + warp * 2 * E;          // [E] raw sigmoid

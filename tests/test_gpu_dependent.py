@@ -199,3 +199,46 @@ def test_dependent_chain_with_the_state_produced_inside_the_layer_kernel(name, s
             _assert_close(yh[t], ref)
     assert len({tuple(r) for r in ih.tolist()}) > min(steps // 2, 60)       # (cfg1 has only 120 possible routings)
     store.close()
+
+
+@pytest.mark.parametrize("form", ["dependent", "routing"])
+def test_a_call_between_two_links_is_done_with_its_buffers_when_the_later_one_writes(form):
+    """The heads of a stack, 15 us of them, queued between two links of a chain: their logits go to memory that the later link writes as well, a
+    few microseconds after it starts, and the stream's order says whose stay."""
+    cfg = synth.CONFIGS["cfg2"].with_(E=32, n_slots=32)
+    store, d, _, _, _, _, _ = _make_store(cfg, n_slots=32)
+    edg.stage_experts_to_slots(store, 0, np.arange(32, dtype=np.int32))
+    n, D, H, E, K = 40, 512, cfg.H, cfg.E, cfg.K
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    rnd = lambda *shape: (torch.randn(shape, generator=gen, device="cuda") * 0.02).half()
+    W1, b1, W2, b2, Wr = rnd(n, D, H + 2 * E), rnd(n, D), rnd(n, E, D), rnd(n, E), rnd(n, E, H)
+    heads_x = torch.randn((n, H), generator=gen, device="cuda").bfloat16()
+    cur = torch.arange(K, dtype=torch.int32, device="cuda").repeat(n, 1)
+    hi, hg = torch.zeros((n, K), dtype=torch.int32, device="cuda"), torch.zeros((n, K), device="cuda")
+    W = torch.from_numpy(synth.prerouter_weights(cfg)).cuda()
+    X = x_dev(synth.hidden_states(cfg, 3, stream=68))
+    inds, gates = torch.zeros((3, K), dtype=torch.int32, device="cuda"), torch.zeros((3, K), device="cuda")
+    y, xn = torch.zeros((2, H), device="cuda"), torch.zeros((2, H), dtype=torch.bfloat16, device="cuda")
+    logits, ws = torch.zeros((n, E), device="cuda"), layer_io.new_workspace(d)
+    edg.prerouter_topk(d, W, X[2], 1, inds[0], gates[0], None)
+
+    def links(between):
+        for t in range(2):
+            out = (W, inds[t + 1], gates[t + 1], logits[n - 1] if t else None, y[t])
+            if form == "dependent":
+                edg.moe_layer_decode_dependent(store, 0, X[0] if t == 0 else xn[0], inds[t], gates[t], *out, xn[t], ws)
+            else:
+                edg.moe_layer_decode(store, 0, X[t], inds[t], gates[t], *out, ws)
+            if t == 0 and between:
+                edg.prerouter_mlp_topk(d, W1, b1, W2, b2, Wr, D, heads_x, cur, cur, n, hi, hg, logits)
+        torch.cuda.synchronize()
+        assert edg.workspace_status(ws) == 0
+        return logits[n - 1].clone()
+    links(True)
+    want = links(False)
+    assert (want - logits[n - 2]).abs().max() > 0.1                   # (the heads' own are others)
+    store.set_chaining(2)
+    for _ in range(5):
+        assert torch.allclose(links(True), want, rtol=1e-3, atol=1e-3)
+    store.close()
