@@ -157,6 +157,7 @@ struct WorkspaceLayout {
     size_t tiles;     // {slot, first position, pairs, adapter} of every tile of 128 pairs
     size_t order;     // [T*K] int32                : pairs sorted by slot
     size_t hq;        // [tiles][I/32][2][4][pairs, up to 128][8] fp16: h of every tile as tensor-core operand tiles (value, residual)
+    size_t hf;        // [tiles][I/8][pairs, up to 128][8] float: h as it is, for the adapters that grouped_wide_h names
     size_t xq;        // [tiles][H/64][8][pairs, up to 128][8] fp16: the gathered token states of every tile as operand tiles
     // streaming form of the grouped path (run_grouped_ffn):
     size_t g_tiles;   // [tiles] {slot, first position, pairs, adapter}
@@ -188,6 +189,9 @@ inline size_t umma_max_tiles(const edg_layer_desc& d, int T) {
 // Whether T tokens go through the tcgen05 tiles (umma_*) or through the streaming form; up to how many pairs the latter is taken.
 bool grouped_use_umma(const edg_layer_desc& d, int T);
 int64_t grouped_streaming_pairs(const edg_layer_desc& d);
+// Which adapters' A_down h the tcgen05 path forms from h in fp32 and adapter rows in bf16, of any magnitude; of the others it takes h as fp16 value
+// and residual and the rows as fp16, as the down kernel does.  (h in fp32 is 64 MB more to write for 4096 tokens of 8 choices at I 512.)
+inline bool grouped_wide_h(const edg_layer_desc& d) { return d.rank > 0 && (d.n_adapters != 1 || d.rank > 32 || (d.I != 256 && d.I != 512)); }
 
 __host__ __device__ inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -206,7 +210,7 @@ inline WorkspaceLayout workspace_layout(const edg_layer_desc& d, int T) {
     W.h = round_up(W.u_gu + (size_t)T * n_sets * 2 * r * sizeof(float), 256);
     W.u_d = round_up(W.h + (T > 1 ? 0 : (size_t)d.K * d.I * sizeof(float)), 256);
     size_t end = round_up(W.u_d + (size_t)T * d.K * r * sizeof(float), 256);
-    W.o = W.pair_slot = W.n_tiles = W.tiles = W.order = W.hq = W.xq = end;
+    W.o = W.pair_slot = W.n_tiles = W.tiles = W.order = W.hq = W.hf = W.xq = end;
     W.g_tiles = W.g_done = W.g_order = W.g_cnt = W.g_u = W.g_xq = W.g_hq = end;
     if (T > 1) {
         const size_t P = (size_t)T * d.K;
@@ -218,6 +222,7 @@ inline WorkspaceLayout workspace_layout(const edg_layer_desc& d, int T) {
             W.tiles = end;         end = round_up(W.tiles + tiles * 16, 256);
             W.order = end;         end = round_up(W.order + P * 4, 256);
             W.hq = end;            end = round_up(W.hq + tiles * d.I * 512, 256);
+            W.hf = end;            end = round_up(W.hf + (grouped_wide_h(d) ? tiles * d.I * 512 : 0), 256);
             W.xq = end;            end = round_up(W.xq + tiles * d.H * 256, 256);
         } else {
             const size_t tiles = grouped_max_tiles(d, T), cap = (size_t)grouped_tile_cap(d, T), r16 = (r + 15) / 16 * 16;

@@ -131,6 +131,7 @@ int32_t run_grouped(const edg_layer_desc* d, const void* slot_pool, int32_t T, c
     p.tiles = reinterpret_cast<int4*>(ws + W.tiles);
     p.order = reinterpret_cast<int32_t*>(ws + W.order);
     p.hq = ws + W.hq;
+    p.hf = has_lora && grouped_wide_h(*d) ? reinterpret_cast<float*>(ws + W.hf) : nullptr;
     p.xq = ws + W.xq;
     const size_t P = (size_t)T * d->K;
     const int max_tiles = (int)umma_max_tiles(*d, T);

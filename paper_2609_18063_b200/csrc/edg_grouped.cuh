@@ -24,6 +24,7 @@ struct GroupedParams {
     int4* tiles;              // {slot, first position in order, pairs, adapter} of every tile of 128 pairs
     int32_t* n_tiles;
     uint8_t* hq;              // h of every tile as fp16 operand tiles, value and residual
+    float* hf;                // h as it is, [tile][8 rows of h][pair][8], or null
     uint8_t* xq;              // the gathered token states of every tile as fp16 operand tiles
     int T, H, I, E, K, group, gshift, rank, n_adapters, n_slots, out_dtype;
     float sigma;

@@ -339,6 +339,11 @@ __global__ void __launch_bounds__(U_THREADS, 2) umma_tile_kernel(const __grid_co
                             uint8_t* w = p.hq + (size_t)tile * p.I * 512 + ((size_t)(k >> 5) * 8 + ((k & 31) >> 3)) * n16 * 16 + (c0 + tok) * 16;
                             *reinterpret_cast<uint4*>(w) = permute8(f);
                             *reinterpret_cast<uint4*>(w + (size_t)n16 * 64) = permute8_lo(f);
+                            if (p.hf != nullptr) {
+                                float4* v = reinterpret_cast<float4*>(p.hf + (size_t)tile * p.I * 128 + ((size_t)(k >> 3) * n16 + c0 + tok) * 8);
+                                v[0] = make_float4(f[0], f[1], f[2], f[3]);
+                                v[1] = make_float4(f[4], f[5], f[6], f[7]);
+                            }
                         }
                     }
                     asm volatile("bar.sync 1, 128;" ::: "memory");

@@ -1,9 +1,11 @@
 // The rank-r projections of the unmerged adapter (Sec. 3.3: delta = sigma * B (A v)) for the tcgen05 tiles of many tokens:
 // u = sigma A_gate x and sigma A_up x before gate/up, u_d = sigma A_down h before down, fp16 as the tiles' operands take them.  Adapter
-// rows are the rows of m16n8k16 tiles, 32 tokens (or pairs) their columns, so an A row is read once per 32; K is split over the warps
-// and summed through shared memory, in fixed order.  With one adapter per layer A x is computed per token, with one per expert per
-// pair, tile by tile (all pairs of a tile have one expert).  x and its adapter rows are bf16 as they are; h is the tiles' fp16 value
-// and residual (two MMAs), its adapter rows fp16 (exact in the normal range); accumulation is fp32.
+// rows are the rows of m16n8k16 tiles, tokens (16 for A x) or pairs (32 for A_down h) their columns, so an A row is read once per 16 or 32;
+// K is split over the warps and summed through shared memory, in fixed order.  With one adapter per layer A x is computed per token, with one per expert per
+// pair, tile by tile (all pairs of a tile have one expert).  x and its adapter rows are bf16 as they are.  h of one adapter of
+// up to 32 ranks (I 256 or 512) is the tiles' fp16 value and residual (two MMAs), the adapter rows are fp16 (exact in the normal range);
+// otherwise h is fp32, the exact sum of three bf16 (three MMAs), the rows are bf16 as they are, and any magnitude keeps its bits.
+// Accumulation is fp32.
 #include "edg_grouped.cuh"
 #include "edg_ptx.cuh"
 
@@ -22,10 +24,27 @@ __device__ __forceinline__ uint4 bf16x8_core(uint4 v) {
     return permute8(f);
 }
 
+// eight values as words of two bf16, part by part: their sum is the value, 8 of its 24 bits each
+__device__ __forceinline__ void bf16_parts(float4 v, float4 w, uint4 (&out)[3]) {
+    float r[8] = {v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        uint32_t o[4];
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {
+            const uint32_t a = __float_as_uint(r[i]) & 0xFFFF0000u, b = __float_as_uint(r[i + 1]) & 0xFFFF0000u;
+            o[i / 2] = (a >> 16) | b;
+            r[i] -= __uint_as_float(a);
+            r[i + 1] -= __uint_as_float(b);
+        }
+        out[q] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+}
+
 // X: u_gu[token or pair][2 rank] = sigma A x, rows 0 .. r-1 from A_gate, r .. 2r-1 from A_up.  Otherwise u_d[pair][rank] = sigma A_down h.
-// blockIdx.x: 8 N tokens, or that part of a tile; blockIdx.y: 16 M rows.
-template <bool X, int M, int N>
-__global__ void __launch_bounds__(L_WARPS * 32, M == 1 ? 3 : 2) lora_rows_kernel(const __grid_constant__ GroupedParams p) {
+// blockIdx.x: 8 N tokens, or that part of a tile; blockIdx.y: 16 M rows.  WIDE: h from p.hf.
+template <bool X, int M, int N, bool WIDE>
+__global__ void __launch_bounds__(L_WARPS * 32, M == 1 && !WIDE ? 3 : 2) lora_rows_kernel(const __grid_constant__ GroupedParams p) {
     constexpr int L_ROWS = 16 * M, L_TOK = 8 * N, SUBS = kUmmaTokens / L_TOK;
     __shared__ float s_red[L_WARPS * L_ROWS * (L_TOK + 1)];
     __shared__ int s_id[L_TOK];                                          // where a column's results go: a token or a pair, or -1
@@ -74,10 +93,11 @@ __global__ void __launch_bounds__(L_WARPS * 32, M == 1 ? 3 : 2) lora_rows_kernel
             xr[n] = id < 0 ? nullptr : p.x + (size_t)(by_token ? id : id / p.K) * p.H + 8 * t4;
         }
     const uint8_t* hq = p.hq + (size_t)tile * p.I * 512 + (size_t)t4 * n16 * 16 + (sub * L_TOK + g8) * 16;
+    const float* hf = WIDE ? p.hf + (size_t)tile * p.I * 128 + ((size_t)t4 * n16 + sub * L_TOK + g8) * 8 : nullptr;
     // X: the warp's eighth of K, 32 k at a time; h: every eighth chunk of 32
 #pragma unroll X ? 4 : 2
     for (int kb = X ? warp * (K / L_WARPS) : warp * 32; kb < (X ? (warp + 1) * (K / L_WARPS) : K); kb += X ? 32 : L_WARPS * 32) {
-        uint4 a[M][2], b[N], bl[N];
+        uint4 a[M][2], b[N], bl[N];                                      // (WIDE: b, bl are the bits of the eight floats)
 #pragma unroll
         for (int m = 0; m < M; ++m)
 #pragma unroll
@@ -87,6 +107,10 @@ __global__ void __launch_bounds__(L_WARPS * 32, M == 1 ? 3 : 2) lora_rows_kernel
             b[n] = zero; bl[n] = zero;
             if (X) {
                 if (xr[n] != nullptr) b[n] = __ldg(reinterpret_cast<const uint4*>(xr[n] + kb));
+            } else if (WIDE && sub * L_TOK + n * 8 < n16) {
+                const uint4* q = reinterpret_cast<const uint4*>(hf + (size_t)(kb >> 3) * n16 * 8 + n * 64);
+                b[n] = __ldcg(q);
+                bl[n] = __ldcg(q + 1);
             } else if (sub * L_TOK + n * 8 < n16) {
                 const uint8_t* q = hq + (size_t)(kb >> 5) * n16 * 128 + n * 128;
                 b[n] = __ldcg(reinterpret_cast<const uint4*>(q));
@@ -95,13 +119,21 @@ __global__ void __launch_bounds__(L_WARPS * 32, M == 1 ? 3 : 2) lora_rows_kernel
         }
 #pragma unroll
         for (int m = 0; m < M; ++m) {
-            if (!X) { a[m][0] = bf16x8_core(a[m][0]); a[m][1] = bf16x8_core(a[m][1]); }
+            if (!X && !WIDE) { a[m][0] = bf16x8_core(a[m][0]); a[m][1] = bf16x8_core(a[m][1]); }
 #pragma unroll
             for (int n = 0; n < N; ++n) {
                 if (n >= nt) continue;
                 if (X) {
                     mma16816_bf16(c[m][n], a[m][0].x, a[m][1].x, a[m][0].y, a[m][1].y, b[n].x, b[n].y);
                     mma16816_bf16(c[m][n], a[m][0].z, a[m][1].z, a[m][0].w, a[m][1].w, b[n].z, b[n].w);
+                } else if (WIDE) {
+                    uint4 part[3];
+                    bf16_parts(*reinterpret_cast<const float4*>(&b[n]), *reinterpret_cast<const float4*>(&bl[n]), part);
+#pragma unroll
+                    for (int q = 2; q >= 0; --q) {
+                        mma16816_bf16(c[m][n], a[m][0].x, a[m][1].x, a[m][0].y, a[m][1].y, part[q].x, part[q].y);
+                        mma16816_bf16(c[m][n], a[m][0].z, a[m][1].z, a[m][0].w, a[m][1].w, part[q].z, part[q].w);
+                    }
                 } else {
                     mma16816(c[m][n], a[m][0].x, a[m][1].x, a[m][0].y, a[m][1].y, b[n].x, b[n].y);
                     mma16816(c[m][n], a[m][0].z, a[m][1].z, a[m][0].w, a[m][1].w, b[n].z, b[n].w);
@@ -135,11 +167,11 @@ __global__ void __launch_bounds__(L_WARPS * 32, M == 1 ? 3 : 2) lora_rows_kernel
 
 // (32 tokens and 32 rows a CTA, whatever the rank: 27 and 77 us for 4096 tokens of 8 choices, rank 16; with one CTA an SM for its registers)
 cudaError_t launch_lora_ax(const GroupedParams& p, int max_tiles, cudaStream_t st) {
-    if (p.n_adapters == 1) return launch_pdl(lora_rows_kernel<true, 2, 2>, dim3((unsigned)(p.T + 15) / 16, (2 * p.rank + 31) / 32), L_WARPS * 32, 0, st, p);
-    return launch_pdl(lora_rows_kernel<true, 2, 2>, dim3(8u * max_tiles, (2 * p.rank + 31) / 32), L_WARPS * 32, 0, st, p);
+    if (p.n_adapters == 1) return launch_pdl(lora_rows_kernel<true, 2, 2, false>, dim3((unsigned)(p.T + 15) / 16, (2 * p.rank + 31) / 32), L_WARPS * 32, 0, st, p);
+    return launch_pdl(lora_rows_kernel<true, 2, 2, false>, dim3(8u * max_tiles, (2 * p.rank + 31) / 32), L_WARPS * 32, 0, st, p);
 }
 cudaError_t launch_lora_adh(const GroupedParams& p, int max_tiles, cudaStream_t st) {
-    return launch_pdl(lora_rows_kernel<false, 1, 4>, dim3(4u * max_tiles, (p.rank + 15) / 16), L_WARPS * 32, 0, st, p);
+    return launch_pdl(p.hf != nullptr ? lora_rows_kernel<false, 1, 4, true> : lora_rows_kernel<false, 1, 4, false>, dim3(4u * max_tiles, (p.rank + 15) / 16), L_WARPS * 32, 0, st, p);
 }
 
 }  // namespace edg

@@ -148,6 +148,37 @@ def test_tensor_memory_tiles_a_slot_named_twice_and_one_out_of_range():
     assert orc.max_abs(got[7], ref) <= 2e-2 and orc.rel_l2(got[7], ref) <= 1e-3
 
 
+@pytest.mark.parametrize("x_exp,a_exp,b_exp", [(5, -19, 13), (-12, 22, 0)])
+@pytest.mark.parametrize("I,rank,n_adapters", [(256, 8, 4), (256, 40, 1), (1024, 8, 1)])
+def test_tensor_memory_tiles_and_the_magnitude_of_h_and_its_adapter(I, rank, n_adapters, x_exp, a_exp, b_exp):
+    """Adapters per expert, of more than 32 ranks, or of layers that are not 256 or 512 wide: rows of A_down near 2^-19 beside an h near 2^11, and
+    near 2^22 beside an h near 2^-23, keep the bits that fp16 would take from them.  The adapter's share is the larger one; what is left is
+    the fp16 of sigma A h, 2^-12 of each rank's share."""
+    L = _layer(512, I, 64, rank, 4, 1, n_adapters)
+    two = lambda bits, e: synth.f32_to_bf16_bits(np.ldexp(synth.bf16_bits_to_f32(bits), e))
+    unit = {p: 1 / s for p, s in (("A", 0.02), ("B", 0.01))}         # synth's standard deviations
+    ident = lambda bits, k: synth.f32_to_bf16_bits(synth.bf16_bits_to_f32(bits) * np.float32(unit[k]))
+    for ad in L.adapters:
+        ad["down"] = (two(ident(ad["down"][0], "A"), a_exp), two(ident(ad["down"][1], "B"), b_exp))
+    L.lora, L._keep = layer_io.lora_to_device(L.desc, L.adapters)
+    for e in range(4):
+        codes, scales, zeros = L.expert(e)["down"]
+        L.expert(e)["down"] = (codes, (scales / 64).astype(np.float16), zeros)
+    L.pool = layer_io.host_layer(L.desc, L.expert).cuda()
+    T = 200
+    X = two(synth.hidden_states(L.cfg, T, stream=67), x_exp)
+    inds_h = np.random.default_rng(12).integers(0, 4, size=(T, 1)).astype(np.int32)
+    gates_h = np.ones((T, 1), np.float32)
+    assert T > 40 * 4
+    Y = _ffn_tokens(L, L.desc, X, torch.from_numpy(inds_h).cuda(), torch.from_numpy(gates_h).cuda(), T)
+    for t in range(0, T, 9):
+        ref = orc.moe_ffn(X[t], inds_h[t], [1.0], L.expert, L.get_lora, L.cfg.lora_scale, L.cfg.group)
+        bare = orc.moe_ffn(X[t], inds_h[t], [1.0], L.expert, lambda e: {**L.get_lora(e), "down": (L.get_lora(e)["down"][0], np.zeros_like(L.get_lora(e)["down"][1]))},
+                           L.cfg.lora_scale, L.cfg.group)
+        assert np.linalg.norm(ref - bare) > 0.5 * np.linalg.norm(ref)
+        assert orc.rel_l2(Y[t], ref) <= 2.0 ** -11
+
+
 def test_pool_with_more_slots_than_shared_memory_counts():
     """26,000 slots: the sort keeps its counters in the workspace.  Three experts live in the first, a middle and the last slot."""
     cfg = _layer(256, 128, 32, 8, 4, 2).cfg
