@@ -411,11 +411,31 @@ __global__ void __launch_bounds__(kPreWarps * 32) prerouter_rows_mma_kernel(PreP
 #pragma unroll
         for (int q = 0; q < kPreWarps; ++q) v += s_red[q * 256 + threadIdx.x];
         float l = (float)v;
-        if (!(fabsf(l) <= 3.4e38f)) {                                   // (the parts of an infinity, or zero parts times one, are not numbers: as it is)
-            const WT* row = static_cast<const WT*>(p.W) + (size_t)(r0 + (threadIdx.x >> 4)) * p.H;
-            const uint16_t* x = reinterpret_cast<const uint16_t*>(s_x + (threadIdx.x & 15) * xs);
-            l = 0.f;
-            for (int k = 0; k < p.H; ++k) l = fmaf((float)row[k], bf16_bits_to_float(x[k]), l);
+        // The parts of an infinity, or zero parts times one, are not numbers: the warp forms such a logit from what is given, and leaves those
+        // of a state that is not a number as they are.  (By one thread each, 1024 tokens of which 64 are padding that is not a number, 160
+        // rows: 361 us instead of 39.)
+        for (unsigned odd = __ballot_sync(0xFFFFFFFFu, !(fabsf(l) <= 3.4e38f)); odd != 0; odd &= odd - 1) {
+            const int src = __ffs(odd) - 1;
+            const WT* row = static_cast<const WT*>(p.W) + (size_t)(r0 + warp * 2 + (src >> 4)) * p.H;
+            const uint8_t* x = s_x + (src & 15) * xs;
+            bool nan = false;
+            for (int k = lane * 8; k < p.H; k += 256) {
+                const uint4 u = *reinterpret_cast<const uint4*>(x + k * 2);
+                const uint32_t most = __vmaxu2(__vmaxu2(u.x & 0x7FFF7FFFu, u.y & 0x7FFF7FFFu), __vmaxu2(u.z & 0x7FFF7FFFu, u.w & 0x7FFF7FFFu));
+                nan |= (most & 0xFFFFu) > 0x7F80u || (most >> 16) > 0x7F80u;
+            }
+            if (__any_sync(0xFFFFFFFFu, nan)) continue;
+            float a = 0.f;
+            for (int k = lane * 8; k < p.H; k += 256) {
+                float f[8];
+                load8(row + k, f);
+                const uint4 u = *reinterpret_cast<const uint4*>(x + k * 2);
+                const uint32_t xw[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) a = fmaf(f[2 * i + 1], bf16_hi(xw[i]), fmaf(f[2 * i], bf16_lo(xw[i]), a));
+            }
+            a = warp_sum(a);
+            if (lane == src) l = a;
         }
         s_logits[(threadIdx.x & 15) * p.E + r0 + (threadIdx.x >> 4)] = l;
         __syncthreads();

@@ -132,3 +132,41 @@ def test_infinities_in_a_head_of_many_tokens(dtype):
     assert torch.equal(torch.isnan(got), torch.isnan(want)) and torch.equal(torch.isinf(got), torch.isinf(want))
     inf, fin = torch.isinf(want), torch.isfinite(want)
     assert torch.equal(got[inf], want[inf]) and (got[fin] - want[fin]).abs().max() <= 1e-5
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+def test_padding_that_is_not_a_number_in_a_head_of_many_tokens(dtype):
+    """States and weights that are no numbers make the logits that are none, and such a state in every block of tokens costs next to nothing
+    (at most the time of the call once more)."""
+    H, E, T = 2048, 160, 1024
+    d = edg.make_desc(None, H=H, I=128, E=E, K=2, group=32, rank=0, n_adapters=1, n_slots=E, pre_dtype=dtype, lora_scale=1.0, out_dtype="f32")
+    W = torch.randn((E, H), device="cuda") * 0.02
+    W = W.half() if dtype == "f16" else W
+    X = torch.randn((T, H), device="cuda").bfloat16()
+    inds, gates, logits = torch.zeros((T, 2), dtype=torch.int32, device="cuda"), torch.zeros((T, 2), device="cuda"), torch.zeros((T, E), device="cuda")
+
+    def us():
+        call = lambda: edg.prerouter_topk_tokens(d, W, X, T, inds, gates, logits)
+        call()
+        times = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            a.record()
+            for _ in range(10):
+                call()
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        return sorted(times)[3]
+    plain, clean = us(), logits.clone()
+    X[11::16, 77] = float("nan")
+    assert us() <= 2 * plain
+    pad = torch.arange(T, device="cuda") % 16 == 11
+    assert torch.isnan(logits[pad]).all() and torch.equal(logits[~pad], clean[~pad])
+    W[37, 1203] = float("nan")
+    edg.prerouter_topk_tokens(d, W, X, T, inds, gates, logits)
+    torch.cuda.synchronize()
+    assert torch.isnan(logits[:, 37]).all()
+    rest = torch.arange(E, device="cuda") != 37
+    assert torch.equal(logits[~pad][:, rest], clean[~pad][:, rest]) and not (inds[~pad] == 37).any()
