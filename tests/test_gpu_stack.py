@@ -135,3 +135,92 @@ def test_layers_of_a_token_side_by_side_are_the_layer_steps(name, kw, n_layers):
                     assert torch.equal(a, b), (i, t)
     for _, store, _, _, _ in stacks:
         store.close()
+
+
+def _tokens(cfg, n_layers, n, stream):
+    """Layer inputs of n tokens of which three in a row are the same: the second and third of each find their experts where the first has put them."""
+    X = np.stack([synth.hidden_states(cfg, (n + 2) // 3, layer=l, stream=stream) for l in range(n_layers)], axis=1)
+    return layer_io.bits_to_device(np.repeat(X, 3, axis=0)[:n], torch.bfloat16)
+
+
+def _shared(store, cfg, layers):
+    d = edg.make_desc(cfg, n_slots=cfg.E)
+    rec = torch.from_numpy(edg.pack_expert(d, synth.expert_tensors(cfg, 1, 0))).cuda()
+    for l in layers:
+        store.set_shared_expert(l, rec)
+
+
+@pytest.mark.parametrize("n_slots,shared", [(8, ()), (5, ()), (8, (0, 2)), (32, (1, 3, 4))])
+def test_layers_side_by_side_in_a_pool_that_evicts_and_beside_shared_experts(n_slots, shared):
+    """Tokens that copy experts and tokens that find them, in pools smaller than the layer, shared experts on some layers: every output is that
+    of one layer-step after the other over resident layers, bit for bit."""
+    cfg, n_layers, T = synth.CONFIGS["cfg2"].with_(E=32, K=4, n_slots=32), 5, 18
+    d, store, W, _, keep = _resident_stack(cfg, n_layers, 81)
+    _shared(store, cfg, shared)
+    X = _tokens(cfg, n_layers, T + 1, 82)
+    ref, want = StackDecoder(d, store, W), []
+    ref.prime(X[T])
+    for t in range(T):
+        cur, nxt = t % 2, (t + 1) % 2
+        y, lg = torch.zeros((n_layers, cfg.H), device="cuda"), torch.zeros((n_layers, cfg.E), device="cuda")
+        for l in range(n_layers):
+            n = (l + 1) % n_layers
+            edg.moe_layer_decode(store, l, X[t, l], ref.inds[cur, l], ref.gates[cur, l], W[l], ref.inds[nxt, n], ref.gates[nxt, n], lg[n], y[l], ref.ws)
+        want.append((y, lg, ref.inds[nxt].clone(), ref.gates[nxt].clone()))
+    torch.cuda.synchronize()
+    store.close()
+    d = edg.make_desc(cfg, n_slots=n_slots)
+    host = layer_io.host_layer(d, lambda e: synth.expert_tensors(cfg, 0, e))
+    slots = torch.zeros((n_layers, n_slots, edg.record_bytes(d)), dtype=torch.uint8, device="cuda")
+    tables = torch.zeros((n_layers, cfg.E), dtype=torch.int32, device="cuda")
+    loras, keep2 = zip(*[layer_io.lora_to_device(d, [synth.lora_tensors(cfg, l, 0)]) for l in range(n_layers)])
+    store = edg.Store(d, [host] * n_layers, slots, tables, list(loras), torch.cuda.Stream())
+    _shared(store, cfg, shared)
+    dec, got, found = StackDecoder(d, store, W), [], 0
+    dec.prime(X[T])
+    for t in range(T):
+        before = dec.misses
+        y, lg = torch.zeros((n_layers, cfg.H), device="cuda"), torch.zeros((n_layers, cfg.E), device="cuda")
+        dec.step(t, X[t], y, lg)
+        found += dec.misses == before
+        got.append((y, lg, dec.inds[(t + 1) % 2].clone(), dec.gates[(t + 1) % 2].clone()))
+    torch.cuda.synchronize()
+    assert edg.workspace_status(dec.ws) == 0
+    assert 4 <= found < T and dec.misses > n_layers * cfg.K
+    for t in range(T):
+        for a, b in zip(got[t], want[t]):
+            assert torch.equal(a, b), t
+    store.close()
+
+
+def test_a_token_whose_outputs_lie_on_inputs_that_have_been_used():
+    """y of a layer on the input of the layer before it: the layers then run one after the other, with the results of separate buffers."""
+    cfg, n_layers, T = synth.CONFIGS["cfg2"].with_(E=32, K=4, n_slots=32), 5, 6
+    d, store, W, _, keep = _resident_stack(cfg, n_layers, 83)
+    store.close()
+    d = edg.make_desc(cfg, n_slots=32, out_dtype="bf16")
+    slots, tables, kept = keep
+    host = layer_io.host_layer(d, lambda e: synth.expert_tensors(cfg, 0, e))
+    loras, keep2 = zip(*[layer_io.lora_to_device(d, [synth.lora_tensors(cfg, l, 0)]) for l in range(n_layers)])
+    store = edg.Store(d, [host] * n_layers, slots, tables, list(loras), torch.cuda.Stream())
+    for l in range(n_layers):
+        store.load_whole_layer(l)
+        store.wait_staged(l)
+    X = _tokens(cfg, n_layers, T + 1, 84)
+    rows = []
+    for apart in (True, False):
+        dec = StackDecoder(d, store, W)
+        dec.prime(X[T])
+        out = []
+        for t in range(T):
+            both = torch.zeros((n_layers + 1, cfg.H), dtype=torch.bfloat16, device="cuda")
+            both[1:] = X[t]
+            y = torch.zeros((n_layers, cfg.H), dtype=torch.bfloat16, device="cuda") if apart else both[:n_layers]
+            dec.step(t, both[1:], y)
+            out.append((y, dec.inds[(t + 1) % 2].clone()))
+        torch.cuda.synchronize()
+        assert edg.workspace_status(dec.ws) == 0
+        rows.append(out)
+    for a, b in zip(*rows):
+        assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+    store.close()
