@@ -85,6 +85,18 @@ __device__ __forceinline__ bool elect_one() {
 }
 __device__ __forceinline__ void fence_to_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// v / (1 + e^-v), the bits of silu_f without the branch that its division has per element (with silu_f itself 874 us for 4096 tokens, so
+// 793, as with an approximate division): the product with an approximate reciprocal, corrected by its remainder (Markstein, Computation of elementary functions on the
+// IBM RISC System/6000 processor, 1990).  A quarter of both sides: the reciprocal of a denominator beyond 2^126 would be subnormal.  Where the
+// denominator is infinite the reciprocal is zero, as the quotient is.
+__device__ __forceinline__ float silu_corrected(float v) {
+    const float d = fminf(fmaf(__expf(-v), 0.25f, 0.25f), 3.402823466e38f), n = 0.25f * v;
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(d));
+    const float q = n * y;
+    return fmaf(fmaf(-d, q, n), y, q);
+}
+
 // The states of a tile's pairs as the gate/up kernel's B operand, [stage of 64 k][8 k cores][pairs rounded to 16][8 k]: a stage is one bulk
 // copy then.  (Gathered by 16-byte copies of the tiles' own CTAs, the bursts held up every other access to shared memory.)
 // Consecutive threads take consecutive pairs of four k cores: their 16-byte pieces are adjacent in the tile; the reads are 64 bytes
@@ -323,7 +335,7 @@ __global__ void __launch_bounds__(U_THREADS, 2) umma_tile_kernel(const __grid_co
 #pragma unroll
                     for (int j = 0; j < half; ++j) {
                         const float mine = is_gate ? acc[c0 + j] : acc[c0 + half + j], gv = is_gate ? mine : o[j];
-                        q[j * U_HS] = __fdividef(gv, 1.f + __expf(-gv)) * (is_gate ? o[j] : mine);
+                        q[j * U_HS] = silu_corrected(gv) * (is_gate ? o[j] : mine);
                     }
                     asm volatile("bar.sync 1, 128;" ::: "memory");
 #pragma unroll

@@ -179,6 +179,28 @@ def test_tensor_memory_tiles_and_the_magnitude_of_h_and_its_adapter(I, rank, n_a
         assert orc.rel_l2(Y[t], ref) <= 2.0 ** -11
 
 
+def test_both_forms_activate_alike():
+    """One code per row that is not its zero point: gate, up and down are single exact products, so what is left is silu(gate) up, and the
+    128-token tiles give the bits of the streaming form."""
+    L = _layer(512, 256, 64, 0, 4, 1)
+    def one_hot(n, kd, first):
+        q = np.full((n, kd), 8, np.uint8)
+        q[np.arange(n), (np.arange(n) + first) % kd] = 9
+        return q[:, 0::2] | q[:, 1::2] << 4, np.ones((n, kd // 64), np.float16), np.full((n, kd // 64), 8, np.float16)
+    for e in range(4):
+        L._experts[e] = {"gate": one_hot(256, 512, e), "up": one_hot(256, 512, 100 + e), "down": one_hot(512, 256, e)}
+    L.pool = layer_io.host_layer(L.desc, L.expert).cuda()
+    T, rng = 200, np.random.default_rng(13)
+    X = synth.f32_to_bf16_bits(rng.uniform(-30, 30, size=(T, 512)).astype(np.float32))
+    inds_h = rng.integers(0, 4, size=(T, 1)).astype(np.int32)
+    inds, gates = torch.from_numpy(inds_h).cuda(), torch.ones((T, 1), device="cuda")
+    assert T > 40 * 4
+    Y = _ffn_tokens(L, L.desc, X, inds, gates, T)
+    _check_tokens(L, X, inds_h, np.ones((T, 1), np.float32), Y, range(0, T, 50))
+    few = np.concatenate([_ffn_tokens(L, L.desc, X[t:t + 50], inds[t:t + 50].contiguous(), gates[t:t + 50], 50) for t in range(0, T, 50)])
+    assert np.array_equal(Y, few)
+
+
 def test_pool_with_more_slots_than_shared_memory_counts():
     """26,000 slots: the sort keeps its counters in the workspace.  Three experts live in the first, a middle and the last slot."""
     cfg = _layer(256, 128, 32, 8, 4, 2).cfg
