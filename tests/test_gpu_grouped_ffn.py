@@ -37,12 +37,19 @@ def _routing(rng, T, E, K, pop=None):
     (2048, 512, 128, 16, 4, 2, 4, 50),      # tiles of up to 32: three columns and a remainder of one pair
     (1024, 1024, 64, 64, 4, 1, 1, 97),      # slices of two stages, the largest rank
     (4096, 512, 64, 0, 4, 2, 1, 70),        # wide state, no adapter
+    # beyond 128 pairs, where a kernel sorts:
+    (512, 256, 64, 24, 32, 2, 32, 100),     # tiles of up to 16, an adapter per expert
+    (1024, 256, 32, 8, 32, 2, 1, 120),      # and one for all
+    (512, 256, 64, 8, 8, 2, 8, 150),        # tiles of up to 32
+    (2048, 512, 32, 16, 4, 2, 1, 150),
+    (512, 256, 64, 16, 8, 1, 8, 320),       # the last size before the tcgen05 tiles
+    (512, 512, 128, 16, 8, 1, 1, 320),
 ])
 def test_streaming_form_at_tile_edges(H, I, group, rank, E, K, n_adapters, T):
     L = _layer(H, I, group, rank, E, K, n_adapters)
     X = synth.hidden_states(L.cfg, T, stream=61)
     inds_h, gates_h = _routing(np.random.default_rng(5), T, E, K, np.array([0.6] + [0.4 / (E - 1)] * (E - 1)))
-    assert T * K <= 96 * E
+    assert T * K <= (40 if group >= 64 else 96) * E                  # (the streaming form's line)
     Y = _ffn_tokens(L, L.desc, X, torch.from_numpy(inds_h).cuda(), torch.from_numpy(gates_h).cuda(), T)
     _check_tokens(L, X, inds_h, gates_h, Y, range(T))
     assert np.array_equal(Y, _ffn_tokens(L, L.desc, X, torch.from_numpy(inds_h).cuda(), torch.from_numpy(gates_h).cuda(), T))
@@ -94,6 +101,35 @@ def test_first_size_of_the_tensor_memory_tiles(n_adapters):
     assert T * 2 > 96 * 16
     Y = _ffn_tokens(L, L.desc, X, torch.from_numpy(inds_h).cuda(), torch.from_numpy(gates_h).cuda(), T)
     _check_tokens(L, X, inds_h, gates_h, Y, list(range(0, T, 9)) + [T - 1])
+
+
+@pytest.mark.parametrize("I,group,rank,n_adapters", [(256, 64, 16, 8), (512, 128, 16, 1)])
+def test_first_size_of_the_tensor_memory_tiles_in_wide_groups(I, group, rank, n_adapters):
+    """41 pairs in a slot of eight and 40 in the others: one pair beyond the line of groups of 64 and more."""
+    L = _layer(512, I, group, rank, 8, 1, n_adapters)
+    T = 40 * 8 + 1
+    X = synth.hidden_states(L.cfg, T, stream=69)
+    inds_h = np.random.default_rng(14).permutation(np.arange(T, dtype=np.int32) % 8).reshape(T, 1)
+    gates_h = np.random.default_rng(15).uniform(0.1, 1.0, size=(T, 1)).astype(np.float32)
+    Y = _ffn_tokens(L, L.desc, X, torch.from_numpy(inds_h).cuda(), torch.from_numpy(gates_h).cuda(), T)
+    _check_tokens(L, X, inds_h, gates_h, Y, list(range(0, T, 5)) + [T - 1])
+
+
+def test_states_that_are_no_numbers_stay_in_their_rows_of_the_tensor_memory_tiles():
+    """An infinity, a NaN and states whose h leaves fp16: their tokens' outputs are not finite, every other token's are the same bits."""
+    L = _layer(512, 256, 64, 8, 4, 1)
+    T = 300
+    X = synth.hidden_states(L.cfg, T, stream=70)
+    inds_h = np.random.default_rng(16).integers(0, 4, size=(T, 1)).astype(np.int32)
+    inds, gates = torch.from_numpy(inds_h).cuda(), torch.ones((T, 1), device="cuda")
+    clean = _ffn_tokens(L, L.desc, X, inds, gates, T)
+    bad = X.copy()
+    bad[17, 3], bad[120, 500] = 0x7F80, 0x7FC0
+    bad[299] = synth.f32_to_bf16_bits(synth.bf16_bits_to_f32(X[299]) * np.float32(2.0 ** 12))
+    Y = _ffn_tokens(L, L.desc, bad, inds, gates, T)
+    odd = [17, 120, 299]
+    assert not np.isfinite(Y[odd]).any()
+    assert np.array_equal(np.delete(Y, odd, axis=0), np.delete(clean, odd, axis=0))
 
 
 # pairs of the eight experts: edges of the tensor-memory tiles' rounding (16) and of the tiles (128), an unused expert, one of several tiles
@@ -201,10 +237,12 @@ def test_both_forms_activate_alike():
     assert np.array_equal(Y, few)
 
 
-def test_pool_with_more_slots_than_shared_memory_counts():
-    """26,000 slots: the sort keeps its counters in the workspace.  Three experts live in the first, a middle and the last slot."""
+@pytest.mark.parametrize("T", [9, 70])
+def test_pool_with_more_slots_than_shared_memory_counts(T):
+    """26,000 slots: the sort of 140 pairs keeps its counters in the workspace (18 pairs find their tiles without one, as up to 128 do).  The
+    experts live in the first, a middle, the last and another slot."""
     cfg = _layer(256, 128, 32, 8, 4, 2).cfg
-    S, T = 26000, 9
+    S = 26000
     desc = edg.make_desc(cfg, n_slots=S)
     R = edg.record_bytes(desc)
     pool = torch.empty((S, R), dtype=torch.uint8, device="cuda")
