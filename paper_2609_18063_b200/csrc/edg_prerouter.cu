@@ -353,10 +353,29 @@ __device__ __forceinline__ void load8(const __half* w, float (&f)[8]) {
     f[0] = x.x; f[1] = x.y; f[2] = y.x; f[3] = y.y; f[4] = z.x; f[5] = z.y; f[6] = v.x; f[7] = v.y;
 }
 constexpr int kRowTok = 16;
-// From how many tokens on it is ahead of the clusters of FMA warps (us a call, those : this; H 2048).  64 rows fp32: 5 tokens 17 : 18, 16 21 : 20,
-// 1024 66 : 20, 4096 221 : 29; 256 rows fp32: 333 52 : 62, 1024 136 : 63, 4096 439 : 91; 160 rows fp16: 64 31 : 31, 128 41 : 31, 4096
-// 587 : 46; 16 rows of H 1024: 5 tokens 10.6 : 5.4.  Its error against 64 bits is below theirs (8.3e-8 and 1.4e-7 rms, 256 rows).
-inline int rows_mma_tokens(const edg_layer_desc& d) { return d.E < 64 ? 2 : (d.E == 64 ? 16 : (d.pre_dtype == EDG_F16 ? 96 : 512)); }
+// Whether T tokens are ahead here of the clusters of FMA warps.  Both times (us a call, those : this) are flat until a form's CTAs fill the GPU a second
+// time: here beyond 2368 tokens, there the sooner the longer the state is (128 tokens at H 4096, 256 at 2048, 384 at 1024); until
+// then a block of 16 rows costs more here (0.6 + 1.26 H / 1024, fp16 0.5 + 0.95) and the start less.  So few rows come here
+// from the start, the more of them the longer the state; others where the clusters begin their second or third round, more
+// rows later.  Fitted to 2240 points (H 256 to 4096, 16 to 1008 rows, 2 to 1024 tokens), of which four are more than 2 % slower than the other form,
+// by 0.3 us at most.  H 2048, fp32: 48 rows 2 tokens 11.1 : 13.6, 8 18.2 : 14.3; 64 rows 96 tokens 19.5 : 19.9, 128 21.3 : 20.1; 256 rows 320
+// tokens 49 : 58, 512 86 : 59; 4096 tokens, 64 rows 218 : 30.  H 256: 64 rows 64 tokens 6.8 : 9.7, 512 12.9 : 10.
+// Its error against 64 bits is below theirs (8.3e-8 and 1.4e-7 rms, 256 rows).
+inline bool rows_mma_ahead(const edg_layer_desc& d, int T) {
+    const bool half = d.pre_dtype == EDG_F16;
+    const int n = d.E / 16, parts = n * (half ? 2 : 3);                  // blocks of 16 rows, bf16 parts of them
+    int lg = 0;                                                          // log2(H / 256)
+    while ((512 << lg) <= d.H) ++lg;
+    if (half ? 2 * n <= 5 * lg : n <= lg) return T >= (parts <= 6 ? 2 : (parts <= 10 ? 4 : 8));
+    if (T <= 8) return T >= 6 && (half ? 2 * n <= 5 * lg + 3 : n <= lg + 1);     // (one column of tokens instead of two)
+    if (half) {
+        if (lg == 0) return T >= (n == 1 ? 96 : (n <= 12 ? 256 : 320));
+        return T >= (lg == 4 || n <= (5 << lg) / 2 + 4 ? 128 : 256);
+    }
+    if (lg == 4) return T >= (n <= 16 ? 128 : (n <= 24 ? 256 : (n <= 32 ? 384 : 768)));
+    const int over = lg == 0 ? n + 3 : n - lg;
+    return T >= (over <= 1 ? 128 : (over == 2 ? 256 : (over <= 4 ? 320 : (over <= 11 ? 384 : (over <= 20 || lg >= 2 ? 512 : 768)))));
+}
 inline size_t rows_mma_smem(int E, int H) { return (size_t)kRowTok * E * 4 + kPreWarps * 256 * 4 + (size_t)kRowTok * (H * 2 + 64); }
 
 template <typename WT>
@@ -943,7 +962,7 @@ int32_t run_prerouter(const edg_layer_desc* d, const void* W_pre, const void* s,
             return EDG_OK;
         }
         const size_t rows_smem = rows_mma_smem(d->E, d->H);
-        if (n_heads >= rows_mma_tokens(*d) && d->E % 16 == 0 && d->H % (32 * kPreWarps) == 0 && rows_smem <= 200 * 1024) {
+        if (d->E % 16 == 0 && d->H % (32 * kPreWarps) == 0 && rows_mma_ahead(*d, n_heads) && rows_smem <= 200 * 1024) {
             EDG_CUDA_TRY(launch_pdl(d->pre_dtype == EDG_F16 ? prerouter_rows_mma_kernel<__half> : prerouter_rows_mma_kernel<float>,
                                     dim3((unsigned)(n_heads + kRowTok - 1) / kRowTok), kPreWarps * 32, rows_smem, st, p, (int)n_heads));
             return EDG_OK;

@@ -93,7 +93,7 @@ def test_full_head_whose_copies_do_not_come_in_time(tmp_path, pre, variant):
 @pytest.mark.parametrize("H,E,K,dtype", [(256, 16, 3, "f32"), (1024, 48, 4, "f16"), (2048, 64, 8, "f32"), (512, 160, 2, "f16"), (2048, 160, 6, "f32")])
 @pytest.mark.parametrize("T", [2, 15, 16, 17, 95, 96, 97, 517])
 def test_many_tokens_of_a_head_in_sixteens(H, E, K, dtype, T):
-    """Blocks of 16 tokens, ragged, around the sizes where the form changes, states from 1e-20 to 1e6: fp32 weights are summed from three bf16
+    """Blocks of 16 tokens, ragged, and the form for other sizes, states from 1e-20 to 1e6: fp32 weights are summed from three bf16
     parts without loss.  Bar: sums of H products in fp32, 2^-24 of the sum of their magnitudes each way of adding."""
     d = edg.make_desc(None, H=H, I=128, E=E, K=K, group=32, rank=0, n_adapters=1, n_slots=E, pre_dtype=dtype, lora_scale=1.0, out_dtype="f32")
     gen = torch.Generator(device="cuda")
@@ -112,6 +112,15 @@ def test_many_tokens_of_a_head_in_sixteens(H, E, K, dtype, T):
     assert torch.equal(inds.long(), top)
     picked = torch.gather(logits.double(), 1, top)
     assert torch.allclose(gates.double(), torch.softmax(picked, -1), rtol=2e-5, atol=1e-7)
+
+
+@pytest.mark.parametrize("H,E,K,dtype,line", [(256, 16, 3, "f32", 320), (256, 48, 4, "f16", 256), (512, 32, 2, "f32", 6), (1024, 48, 4, "f32", 128), (1024, 64, 4, "f16", 4),
+                                              (1024, 160, 6, "f32", 384), (2048, 64, 8, "f32", 128), (2048, 144, 2, "f16", 6), (4096, 64, 3, "f32", 8),
+                                              (4096, 320, 8, "f32", 256), (4096, 320, 8, "f16", 128)])
+def test_a_head_on_both_sides_of_the_line_between_its_forms(H, E, K, dtype, line):
+    """The last number of tokens of one form and the first of the other."""
+    for T in (line - 1, line):
+        test_many_tokens_of_a_head_in_sixteens(H, E, K, dtype, T)
 
 
 @pytest.mark.parametrize("dtype", ["f32", "f16"])
