@@ -143,9 +143,9 @@ static_assert(kCtrlStarts % 128 == 0 && kCtrlDefer + kStepBufs * kStepDeferWords
 
 struct WorkspaceLayout {
     size_t ctrl;      // kCtrlBytes control block
-    size_t u_gu;      // [T][n_sets][2][rank] float : A_gate x and A_up x
-    size_t h;         // [K][I] float               : silu(gate) * up (T = 1)
-    size_t u_d;       // [T][K][rank] float         : A_down h
+    size_t u_gu;      // T = 1: [n_sets][2][rank] float : A_gate x and A_up x; tcgen05 tiles: [T][n_sets][2][rank] fp16 : the same times sigma
+    size_t h;         // T = 1: [K][I] float        : silu(gate) * up
+    size_t u_d;       // T = 1: [K][rank] float     : A_down h; tcgen05 tiles: [T][K][rank] fp16 : the same times sigma
     size_t logits;    // [ring][E + 64] float     : next-step head logits, then the (expert, gate) pairs chosen from them, handed to the chained next step; one set per ring slot
     size_t partial;   // [ring][4(K+1)][H] float  : gate-weighted partial expert outputs of the fused batch-1 kernel, one set per ring slot
     size_t dep;       // [ring][8] float          : dependent chain: kC partial sums of squares of x + y, then the "next state written" flag
@@ -207,9 +207,10 @@ inline WorkspaceLayout workspace_layout(const edg_layer_desc& d, int T) {
     W.lone_bytes = W.partial + one_set;
     W.step_x = round_up(W.partial + (size_t)kHandoffRing * one_set, 256);
     W.u_gu = round_up(W.step_x + step_region_words(d) * sizeof(float), 256);
-    W.h = round_up(W.u_gu + (size_t)T * n_sets * 2 * r * sizeof(float), 256);
+    const size_t u_bytes = T == 1 ? sizeof(float) : (grouped_use_umma(d, T) ? sizeof(uint16_t) : 0);     // (the streaming form has its own)
+    W.h = round_up(W.u_gu + (size_t)T * n_sets * 2 * r * u_bytes, 256);
     W.u_d = round_up(W.h + (T > 1 ? 0 : (size_t)d.K * d.I * sizeof(float)), 256);
-    size_t end = round_up(W.u_d + (size_t)T * d.K * r * sizeof(float), 256);
+    size_t end = round_up(W.u_d + (size_t)T * d.K * r * u_bytes, 256);
     W.o = W.pair_slot = W.n_tiles = W.tiles = W.order = W.hq = W.hf = W.xq = end;
     W.g_tiles = W.g_done = W.g_order = W.g_cnt = W.g_u = W.g_xq = W.g_hq = end;
     if (T > 1) {

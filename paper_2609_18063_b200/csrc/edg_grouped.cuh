@@ -34,9 +34,10 @@ struct GroupedParams {
 // tcgen05 path for large groups (prefill): tiles of 128 tokens
 constexpr int kUmmaTokens = 128;
 // Where the 128-token tiles overtake the streaming form, in pairs per slot (us, streaming : tcgen05; H 2048, I 512, groups of 64 where
-// nothing else is said).  256 experts, top 8: 32 422 : 452, 64 706 : 561; 64 experts: 42 161 : 145, 80 238 : 197; groups of 128: 21
-// 185 : 220, 40 263 : 249; H 1024, I 256, 16 experts: 42 59.4 : 60.2, 128 92 : 66.  With groups of 32 the sums leave tensor memory twice
-// as often: 64 214 : 230, 128 322 : 296.
+// nothing else is said).  256 experts, top 8: 32 422 : 452, 64 701 : 454; 64 experts: 41 156 : 132, 64 200 : 149; 2 experts: 42 79 : 54;
+// groups of 128: 21 185 : 220, 40 263 : 249; H 1024, I 256, 16 experts: 41 54.5 : 44.7, 64 56 : 48.  The average says enough of steeper and
+// sparser routing, where the tiles gain less and more: Zipf(2.0) over 256 experts 41 483 : 443, 64 698 : 538, over 64 of H 512, I 256 64
+// 45.7 : 45.3; 32 of 256 slots in use 41 422 : 240.  With groups of 32 the sums leave tensor memory twice as often: 64 214 : 230, 128 322 : 296.
 // Beyond 1024 slots (no table names more) the line stays where it was: what is counted per slot of the pool says nothing about the slots
 // in use then, each slot has a CTA that reads all pairs, and with 65,535 tokens of 32 choices the tiles would not fit a grid.
 constexpr int kUmmaPairsPerSlot = 40, kUmmaPairsPerSlot32 = 96, kUmmaSlots = 1024;

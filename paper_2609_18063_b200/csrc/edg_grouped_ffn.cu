@@ -98,11 +98,6 @@ __device__ __forceinline__ void ring_wait(uint64_t* bar, uint32_t parity, int32_
         if (++i >= kSpinLimit) { atomicExch(status, EDG_E_TIMEOUT); break; }
 }
 
-__device__ __forceinline__ void mma16816_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
 // where a warp finds its two runs (matrices of gate/up, neighbouring row tiles of down) inside a stage
 struct WarpRuns {
     uint32_t code[2], sz[2];      // first byte of each run
@@ -178,12 +173,6 @@ __device__ __forceinline__ uint32_t bf16_pair(const uint16_t* row, int k, int n)
     const float a = k < n ? bf16_bits_to_float(row[k]) : 0.f, b = k + 1 < n ? bf16_bits_to_float(row[k + 1]) : 0.f;
     return h2_as_u32(__floats2half2_rn(a, b));
 }
-// 16 bytes of an adapter row (8 bf16) as fp16 words in k-slot order
-__device__ __forceinline__ uint4 bf16x8_slots(uint4 v) {
-    const float f[8] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y), bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w)};
-    return permute8(f);
-}
-
 struct RingPos {
     int st;
     uint32_t phase;
@@ -461,7 +450,7 @@ struct Gffn {
                             const uint4 rb = hi_ok ? __ldg(reinterpret_cast<const uint4*>(A + (size_t)8 * p.I + c * 32)) : z;
                             const uint8_t* hb = hq + (size_t)c * 2 * nt_all * 512 + nt * 512;
                             const uint4 hv = __ldcg(reinterpret_cast<const uint4*>(hb)), hl = __ldcg(reinterpret_cast<const uint4*>(hb + nt_all * 512));
-                            const uint4 a = bf16x8_slots(ra), b = bf16x8_slots(rb);
+                            const uint4 a = bf16x8_permute8(ra), b = bf16x8_permute8(rb);
                             mma16816(cc, a.x, b.x, a.y, b.y, hv.x, hv.y);
                             mma16816(cc, a.z, b.z, a.w, b.w, hv.z, hv.w);
                             mma16816(cc, a.x, b.x, a.y, b.y, hl.x, hl.y);
@@ -817,9 +806,7 @@ __global__ void __launch_bounds__(256) tile_operands_kernel(TileArgs a) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 if (c0 + 8 * u >= a.H >> 5) break;
-                const float f[8] = {bf16_lo(v[u].x), bf16_hi(v[u].x), bf16_lo(v[u].y), bf16_hi(v[u].y),
-                                    bf16_lo(v[u].z), bf16_hi(v[u].z), bf16_lo(v[u].w), bf16_hi(v[u].w)};
-                *reinterpret_cast<uint4*>(out + ((size_t)(c0 + 8 * u) * ntok + tok) * 64 + q * 16) = permute8(f);
+                *reinterpret_cast<uint4*>(out + ((size_t)(c0 + 8 * u) * ntok + tok) * 64 + q * 16) = bf16x8_permute8(v[u]);
             }
         }
         return;

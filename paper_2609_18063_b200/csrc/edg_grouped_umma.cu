@@ -20,13 +20,13 @@
 // activations, one bulk copy a stage.  Two CTAs share an SM: one's prologue and epilogue run beside the other's main loop.  Every wait
 // is bounded: a wait that gives up raises the status word and the kernel still frees its tensor memory and returns.
 //
-// Measured (4096 tokens, top 8 of 256 by Zipf(1.1), H 2048, I 512, groups of 64, rank 16): gate/up 413 -> 368 us, down 323 -> 302, the
-// whole call with its routing 904 -> 795; with an adapter per expert 1190 -> 839; 2048 tokens (streaming form before) 706 -> 561.
-// Tensor pipe 13 and 23 % active: the limiter is the rate at which lone warps run their instructions (a stage of gate/up takes a
-// CTA 2000 cycles; without the trips to tensor memory it would be 333 us, the operand traffic alone 110).  Found on the way: MMAs issued by one of
+// Measured (4096 tokens, top 8 of 256 by Zipf(1.1), H 2048, I 512, groups of 64, rank 16): gate/up 413 -> 363 us, down 323 -> 310 (under ncu), the
+// whole call with its routing 904 -> 782; with an adapter per expert 1190 -> 855; 2048 tokens (streaming form before) 706 -> 549.
+// Tensor pipe 20 and 23 % active, schedulers issuing in 44 and 41 % of all cycles: the limiter is the rate at which lone warps run their
+// instructions in roles that wait for one another (1024 tokens, 64 experts).  Found on the way: MMAs issued by one of
 // the warps that take sums out, in between: 1020 us for gate/up; sums out 16 columns at a time: 577; states gathered by 16-byte copies
-// of this kernel, without a pass that gathers them: 554, the copies' bursts hold up every other access to shared memory; four row
-// blocks per CTA one after the other: down 302 -> 400.
+// of this kernel, without a pass that gathers them: 554, the copies' bursts hold up every other access to shared memory (333 without
+// the trips to tensor memory); four row blocks per CTA one after the other: down 302 -> 400.
 #include "edg_grouped.cuh"
 #include "edg_ptx.cuh"
 
@@ -118,22 +118,8 @@ __global__ void __launch_bounds__(256) umma_gather_x_kernel(const __grid_constan
             for (int j = 0; j < 4; ++j) raw[j] = __ldg(src + j);
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float f[8] = {bf16_lo(raw[j].x), bf16_hi(raw[j].x), bf16_lo(raw[j].y), bf16_hi(raw[j].y),
-                                bf16_lo(raw[j].z), bf16_hi(raw[j].z), bf16_lo(raw[j].w), bf16_hi(raw[j].w)};
-            *reinterpret_cast<uint4*>(out + ((size_t)(c * 4 + j) * n16 + tok) * 16) = permute8(f);
-        }
+        for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4*>(out + ((size_t)(c * 4 + j) * n16 + tok) * 16) = bf16x8_permute8(raw[j]);
     }
-}
-
-// 8 bf16 -> 8 fp16 in natural order (adapter matrices)
-__device__ __forceinline__ uint4 bf16x8_to_f16(uint4 v) {
-    uint4 o;
-    o.x = h2_as_u32(__floats2half2_rn(bf16_lo(v.x), bf16_hi(v.x)));
-    o.y = h2_as_u32(__floats2half2_rn(bf16_lo(v.y), bf16_hi(v.y)));
-    o.z = h2_as_u32(__floats2half2_rn(bf16_lo(v.z), bf16_hi(v.z)));
-    o.w = h2_as_u32(__floats2half2_rn(bf16_lo(v.w), bf16_hi(v.w)));
-    return o;
 }
 
 // One tile: DOWN = false: h = silu(gate) up for 64 rows of the intermediate dimension (rows 0..63 of the tile are gate rows, 64..127

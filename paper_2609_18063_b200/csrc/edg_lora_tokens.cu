@@ -14,33 +14,6 @@ namespace {
 
 constexpr int L_WARPS = 8;
 
-__device__ __forceinline__ void mma16816_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-// 16 bytes of an adapter row (8 bf16) as fp16 words in the order of a core row
-__device__ __forceinline__ uint4 bf16x8_core(uint4 v) {
-    const float f[8] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y), bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w)};
-    return permute8(f);
-}
-
-// eight values as words of two bf16, part by part: their sum is the value, 8 of its 24 bits each
-__device__ __forceinline__ void bf16_parts(float4 v, float4 w, uint4 (&out)[3]) {
-    float r[8] = {v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w};
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        uint32_t o[4];
-#pragma unroll
-        for (int i = 0; i < 8; i += 2) {
-            const uint32_t a = __float_as_uint(r[i]) & 0xFFFF0000u, b = __float_as_uint(r[i + 1]) & 0xFFFF0000u;
-            o[i / 2] = (a >> 16) | b;
-            r[i] -= __uint_as_float(a);
-            r[i + 1] -= __uint_as_float(b);
-        }
-        out[q] = make_uint4(o[0], o[1], o[2], o[3]);
-    }
-}
-
 // X: u_gu[token or pair][2 rank] = sigma A x, rows 0 .. r-1 from A_gate, r .. 2r-1 from A_up.  Otherwise u_d[pair][rank] = sigma A_down h.
 // blockIdx.x: 8 N tokens, or that part of a tile; blockIdx.y: 16 M rows.  WIDE: h from p.hf.
 template <bool X, int M, int N, bool WIDE>
@@ -119,7 +92,7 @@ __global__ void __launch_bounds__(L_WARPS * 32, M == 1 && !WIDE ? 3 : 2) lora_ro
         }
 #pragma unroll
         for (int m = 0; m < M; ++m) {
-            if (!X && !WIDE) { a[m][0] = bf16x8_core(a[m][0]); a[m][1] = bf16x8_core(a[m][1]); }
+            if (!X && !WIDE) { a[m][0] = bf16x8_permute8(a[m][0]); a[m][1] = bf16x8_permute8(a[m][1]); }
 #pragma unroll
             for (int n = 0; n < N; ++n) {
                 if (n >= nt) continue;
@@ -127,12 +100,14 @@ __global__ void __launch_bounds__(L_WARPS * 32, M == 1 && !WIDE ? 3 : 2) lora_ro
                     mma16816_bf16(c[m][n], a[m][0].x, a[m][1].x, a[m][0].y, a[m][1].y, b[n].x, b[n].y);
                     mma16816_bf16(c[m][n], a[m][0].z, a[m][1].z, a[m][0].w, a[m][1].w, b[n].z, b[n].w);
                 } else if (WIDE) {
-                    uint4 part[3];
-                    bf16_parts(*reinterpret_cast<const float4*>(&b[n]), *reinterpret_cast<const float4*>(&bl[n]), part);
+                    const float4 v = *reinterpret_cast<const float4*>(&b[n]), w = *reinterpret_cast<const float4*>(&bl[n]);
+                    const float f[8] = {v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w};
+                    uint32_t part[3][4];
+                    bf16_parts(f, part);
 #pragma unroll
                     for (int q = 2; q >= 0; --q) {
-                        mma16816_bf16(c[m][n], a[m][0].x, a[m][1].x, a[m][0].y, a[m][1].y, part[q].x, part[q].y);
-                        mma16816_bf16(c[m][n], a[m][0].z, a[m][1].z, a[m][0].w, a[m][1].w, part[q].z, part[q].w);
+                        mma16816_bf16(c[m][n], a[m][0].x, a[m][1].x, a[m][0].y, a[m][1].y, part[q][0], part[q][1]);
+                        mma16816_bf16(c[m][n], a[m][0].z, a[m][1].z, a[m][0].w, a[m][1].w, part[q][2], part[q][3]);
                     }
                 } else {
                     mma16816(c[m][n], a[m][0].x, a[m][1].x, a[m][0].y, a[m][1].y, b[n].x, b[n].y);
@@ -165,7 +140,7 @@ __global__ void __launch_bounds__(L_WARPS * 32, M == 1 && !WIDE ? 3 : 2) lora_ro
 
 }  // namespace
 
-// (32 tokens and 32 rows a CTA, whatever the rank: 27 and 77 us for 4096 tokens of 8 choices, rank 16; with one CTA an SM for its registers)
+// 4096 tokens of 8 choices, rank 16: 9 and 23 us.  (Not kept: 32 tokens or pairs and 32 rows a CTA in both, one CTA an SM for its registers: 27 and 77.)
 cudaError_t launch_lora_ax(const GroupedParams& p, int max_tiles, cudaStream_t st) {
     if (p.n_adapters == 1) return launch_pdl(lora_rows_kernel<true, 2, 2, false>, dim3((unsigned)(p.T + 15) / 16, (2 * p.rank + 31) / 32), L_WARPS * 32, 0, st, p);
     return launch_pdl(lora_rows_kernel<true, 2, 2, false>, dim3(8u * max_tiles, (2 * p.rank + 31) / 32), L_WARPS * 32, 0, st, p);

@@ -322,26 +322,6 @@ __global__ void __launch_bounds__(kPreWarps * 32) prerouter_tokens_mma_kernel(Pr
 // for 16 tokens on the tensor cores, K split over its warps, and does their softmax and top-k; no cluster.  Products are exact: the
 // states are bf16 as they are, an fp32 weight is the sum of three bf16 (8 of its 24 bits each), an fp16 one of two.  Every 32 k start a
 // fresh accumulator, the large parts apart from the small ones, and are added in fp32.
-__device__ __forceinline__ void mma16816_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-// eight weights of a row as words of two bf16, part by part
-template <int PARTS>
-__device__ __forceinline__ void bf16_parts(const float (&w)[8], uint32_t (&out)[PARTS][4]) {
-    float r[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) r[i] = w[i];
-#pragma unroll
-    for (int q = 0; q < PARTS; ++q)
-#pragma unroll
-        for (int i = 0; i < 8; i += 2) {
-            const uint32_t a = __float_as_uint(r[i]) & 0xFFFF0000u, b = __float_as_uint(r[i + 1]) & 0xFFFF0000u;
-            out[q][i / 2] = (a >> 16) | b;
-            r[i] -= __uint_as_float(a);
-            r[i + 1] -= __uint_as_float(b);
-        }
-}
 __device__ __forceinline__ void load8(const float* w, float (&f)[8]) {
     const uint4 a = ld_stream16(w), b = ld_stream16(w + 4);
     f[0] = __uint_as_float(a.x); f[1] = __uint_as_float(a.y); f[2] = __uint_as_float(a.z); f[3] = __uint_as_float(a.w);
